@@ -169,8 +169,11 @@ def _inputs(case, wl, seed):
         R = np.tile(np.eye(3), (P, 1, 1)) if wl.quats is None else _rotations(wl.quats)
         x = torch.tensor(np.concatenate([wl.shapes[s].colloc @ R[k].T + wl.centres[k]
                                          for k, s in enumerate(wl.shape_id)]), device=DEV)
-        wave, phase = _randn(g, nrhs, 3, d, dtype=x.dtype), _randn(g, nrhs, 1, d, dtype=x.dtype)
-        inp["gamma"] = (torch.sin(x @ wave + 3.0 * phase) + 1e-6 * _randn(g, nrhs, len(x), d, dtype=x.dtype)).to(dt)
+        # plane waves; vector ones are transverse, as a flow has no net flux through a body's surface
+        k, phase, a = (_randn(g, nrhs, 3, dtype=x.dtype) for _ in range(3))
+        a = torch.linalg.cross(k, a) if d == 3 else a[:, :1]
+        rough = 1e-6 * _randn(g, nrhs, len(x), d, dtype=x.dtype)
+        inp["gamma"] = (torch.sin(x @ k.T + 3.0 * phase[:, 0]).T[:, :, None] * a[:, None, :] + rough).to(dt)
     elif case["op"] == "elastance":
         inp["q"] = _randn(g, nrhs, P, dtype=dt)
     else:
