@@ -29,18 +29,21 @@ cudaError_t pack_sources(int D, int nrhs, int packed, const float4 *src_pos, con
 cudaError_t pack_sources_comp(int D, int nrhs, const double *src_local64, const int *src_pt_of_rec,
                               const double *strength, int nsrc, int nrec, float *records, cudaStream_t st);
 
-// FP64 reference of the adjoint's pair gradient (precision = 1), per target: sum over the other
-// bodies' sources of grad_r (tw^T G(r) strength), raw (no 1/(8 pi mu)); tw [nrhs][ntargets][3], out
-// [ntargets][3]; the other arguments as pair_sum_fp64.
-cudaError_t grad_pair_fp64(int nrhs, const double *tgt_local, const int *tgt_body, int ntargets, const double *tw,
-                           const double *src_local4, int nsrc, const int *susp_src_begin, const int *susp_src_end,
-                           const int *body_src_off, const double *centres, const double *strength, double *out,
-                           cudaStream_t st);
-// FP64 reference pair sum (precision = 1): one thread per target, direct loops; raw sums (no 1/(4pi) factor).
-cudaError_t pair_sum_fp64(int D, int nrhs, const double *tgt_local, const int *tgt_body, int ntargets,
+// FP64 sums (precision = 1), one thread per target and source chunk: raw sums (no 1/(4 pi) factor) in
+// `chunks` partials [chunks][nrhs][ntargets][D], to be added in chunk order (fp64_pair_chunks gives the
+// count for targets whose smallest suspension has min_sources sources).
+int fp64_pair_chunks(int ntargets, int min_sources, int sm_count);
+cudaError_t pair_sum_fp64(int D, int nrhs, int chunks, const double *tgt_local, const int *tgt_body, int ntargets,
                           const double *src_local4, int nsrc, const int *susp_src_begin, const int *susp_src_end,
                           const int *body_src_off, const double *centres, const double *strength, int include_self,
                           double *out_raw, cudaStream_t st);
+// The adjoint's pair gradient in FP64, per target: sum over the other bodies' sources of
+// grad_r (tw^T G(r) strength), raw (no 1/(8 pi mu)); tw [nrhs][ntargets][3], out [chunks][ntargets][3];
+// the other arguments as pair_sum_fp64.
+cudaError_t grad_pair_fp64(int nrhs, int chunks, const double *tgt_local, const int *tgt_body, int ntargets,
+                           const double *tw, const double *src_local4, int nsrc, const int *susp_src_begin,
+                           const int *susp_src_end, const int *body_src_off, const double *centres,
+                           const double *strength, double *out, cudaStream_t st);
 
 // ---- preconditioner and setup (precond.cu) ----
 struct ShapeDev {
@@ -67,8 +70,6 @@ cudaError_t build_apply_factors(int kind, int M, int N, const double *Ucm, const
 cudaError_t gather_rotate(int D, const double *gamma, int sum_MD, const int *col_body, const int *col_rhs,
                           const int *body_tgt_off, const double *rot, int ncols, int dM, float *A, double *A64,
                           cudaStream_t st);
-// C[m][n] = sum_k A[m][k] B[k][n]  (row-major; FP32 SIMT tiles, or FP64 when A64/B64 given).
-cudaError_t gemm_rm(int m, int n, int k, const float *A, const float *B, float *C, cudaStream_t st);
 // Split-K FP32 GEMM with TwoSum-compensated slices; chunk results (FP64, P [S][m][n]) summed in FP64
 // into C32 (FP32) or C64 (FP64).  S from gemm_splitk_chunks; P must hold S*m*n doubles.
 int gemm_splitk_chunks(int m, int n, int k, int sm_count);
@@ -111,9 +112,8 @@ cudaError_t gather_rotate_pieces(int D, const double *gamma, int sum_MD, const i
                                  size_t pstride, int pieces, cudaStream_t st);
 cudaError_t gemm_splitk(int m, int n, int k, int S, const float *A, const float *B, double *P, float *C32,
                         double *C64, cudaStream_t st, bool trans_b = false);  // trans_b: B stored [n][k]
-cudaError_t gemm_rm64(int m, int n, int k, const double *A, const double *B, double *C, cudaStream_t st);
-// The same product split over K into S chunks (gemm_rm64_chunks), partials P [S][m][n] summed in chunk
-// order into C (deterministic); S = 1 is gemm_rm64.
+// FP64 C[m][n] = sum_k A[m][k] B[k][n] (row-major) split over K into S chunks (gemm_rm64_chunks),
+// partials P [S][m][n] (unused when S = 1) summed in chunk order into C (deterministic).
 int gemm_rm64_chunks(int m, int n, int k, int sm_count);
 cudaError_t gemm_rm64_splitk(int m, int n, int k, int S, const double *A, const double *B, double *P, double *C,
                              cudaStream_t st);

@@ -75,6 +75,7 @@ struct ShapeHost {
     float2 *Ptc = nullptr;  // chunk results as (hi, lo) pairs
     std::map<int, std::array<TcMap, 6>> amaps;  // per column count: A pieces, T pieces
     double *A64 = nullptr, *T64 = nullptr, *L64 = nullptr;
+    double *Pk64 = nullptr;  // FP64 apply: split-K partials
     // one-body factors per formulation: [0] recompleted S_L (Sec. 3.3), [1] bare self block S^(00)
     // of the Dirichlet problems (Sec. 2.3), built on first use
     FactorSet fs[2];
@@ -129,7 +130,7 @@ struct mfs_ctx {
     int rec_floats = 0;          // floats per record allocated in rec_d (and recT_floats in recT_d)
     int recT_floats = 0;
     double *lam_d = nullptr;     // [max_rhs][sumN][D]
-    double *raw_d = nullptr;     // FP64 reference pair sums [max_rhs][sumM][D]
+    double *raw_d = nullptr;     // FP64 pair sums: source-chunk partials [chunks][max_rhs][sumM or sumN][D]
     std::map<int, PairPlan> plans;  // key: variant * 4 + include_self * 2 + transposed
     int best_variant[2][5] = {{-1, -1, -1, -1, -1}, {-1, -1, -1, -1, -1}};  // [D==3][nrhs]
 
@@ -565,10 +566,22 @@ double kernel_scale(mfs_ctx *ctx) {
 }
 
 // out = beta * base + sign * (pair sum of strengths)  (strengths FP64 [nrhs][sumN][D] on device)
+// (raw in S partials of n, added in order)
 __global__ void combine_raw_kernel(const double *raw, const double *base, double beta, double scale, double *out,
-                                   size_t n) {
+                                   size_t n, int S) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = (base ? beta * base[i] : 0.0) + scale * raw[i];
+    if (i >= n) return;
+    double v = raw[i];
+    for (int z = 1; z < S; ++z) v += raw[(size_t)z * n + i];
+    out[i] = (base ? beta * base[i] : 0.0) + scale * v;
+}
+
+// Source chunks of the FP64 sums over ntargets targets (transposed: the collocation points are the sources).
+int fp64_chunks(const mfs_ctx *ctx, int ntargets, bool transposed = false) {
+    const std::vector<int> &off = transposed ? ctx->tgt_off : ctx->src_off;
+    int least = off.back();
+    for (int s = 0; s < ctx->S; ++s) least = std::min(least, off[ctx->body_off[s + 1]] - off[ctx->body_off[s]]);
+    return fp64_pair_chunks(ntargets, least, ctx->sm_count);
 }
 
 mfs_status ff_pair_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const double *strength, double *out,
@@ -578,11 +591,12 @@ mfs_status pair_apply(mfs_ctx *ctx, const double *strength, double *out, const d
                       double sign, int nrhs, int include_self, cudaStream_t st) {
     const double scale = sign * kernel_scale(ctx);
     if (ctx->opt.precision == 1) {
-        CK(pair_sum_fp64(ctx->D, nrhs, ctx->tgt_local64_d, ctx->tgt_body_d, ctx->sumM, ctx->src_local4_d, ctx->sumN,
-                         ctx->susp_src_begin_d, ctx->susp_src_end_d, ctx->src_off_d, ctx->centres_d, strength,
-                         include_self, ctx->raw_d, st));
+        const int S = fp64_chunks(ctx, ctx->sumM);
+        CK(pair_sum_fp64(ctx->D, nrhs, S, ctx->tgt_local64_d, ctx->tgt_body_d, ctx->sumM, ctx->src_local4_d,
+                         ctx->sumN, ctx->susp_src_begin_d, ctx->susp_src_end_d, ctx->src_off_d, ctx->centres_d,
+                         strength, include_self, ctx->raw_d, st));
         const size_t n = (size_t)nrhs * ctx->sumM * ctx->D;
-        combine_raw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ctx->raw_d, base, beta, scale, out, n);
+        combine_raw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ctx->raw_d, base, beta, scale, out, n, S);
         CK(cudaGetLastError());
         ctx->launches += 2;
         ctx->pair_launches += 1;
@@ -924,6 +938,12 @@ double pair_count(mfs_ctx *ctx, int include_self) {
     return total;
 }
 
+// C [cols][n] = A [cols][k] B [k][n] in FP64 with the shape's split-K scratch.
+cudaError_t gemm64(mfs_ctx *ctx, ShapeHost &sh, int cols, int n, int k, const double *A, const double *B, double *C,
+                   cudaStream_t st) {
+    return gemm_rm64_splitk(cols, n, k, gemm_rm64_chunks(cols, n, k, ctx->sm_count), A, B, sh.Pk64, C, st);
+}
+
 // lambda = (I - L) S_L^+ gamma (project) or S_L^+ gamma  (Eq. pseudo, Remark congruent)
 mfs_status precond_apply_dev(mfs_ctx *ctx, const double *gamma, double *lambda, int project, int nrhs,
                              cudaStream_t st) {
@@ -937,8 +957,8 @@ mfs_status precond_apply_dev(mfs_ctx *ctx, const double *gamma, double *lambda, 
         if (ctx->opt.precision >= 1) {  // FP64 one-body apply (reference and mixed modes)
             CK(gather_rotate(D, gamma, ctx->sumM * D, sh.col_body, sh.col_rhs, ctx->tgt_off_d, ctx->rot64_d, ncols,
                              sd.dM, sh.A, sh.A64, st));
-            CK(gemm_rm64(ncols, sd.r, sd.dM, sh.A64, sd.U64, sh.T64, st));
-            CK(gemm_rm64(ncols, sd.dN, sd.r, sh.T64, project ? sd.Wp64 : sd.Wr64, sh.L64, st));
+            CK(gemm64(ctx, sh, ncols, sd.r, sd.dM, sh.A64, sd.U64, sh.T64, st));
+            CK(gemm64(ctx, sh, ncols, sd.dN, sd.r, sh.T64, project ? sd.Wp64 : sd.Wr64, sh.L64, st));
             CK(scatter_rotate(D, nullptr, sh.L64, sh.col_body, sh.col_rhs, ctx->src_off_d, ctx->rot_d, ctx->rot64_d,
                               ncols, sd.dN, ctx->sumN, lambda, st));
         } else if (fx.tc_ready) {  // tensor cores: multi-piece TF32 tcgen05 GEMMs, double-float chunk sums
@@ -1219,12 +1239,13 @@ mfs_status ensure_transposed(mfs_ctx *ctx) {
 // self pairs included or not.  w: [nrhs][sum_M][3], z: [nrhs][sum_N][3], both FP64 on the device.
 mfs_status pair_apply_T(mfs_ctx *ctx, const double *w, double *z, int nrhs, int include_self, cudaStream_t st) {
     if (ctx->opt.precision == 1) {  // FP64 reference: the plain FP64 loops with the roles swapped
-        CK(pair_sum_fp64(3, nrhs, ctx->src_local64_d, ctx->src_body_d, ctx->sumN, ctx->colloc4_d, ctx->sumM,
+        const int S = fp64_chunks(ctx, ctx->sumN, true);
+        CK(pair_sum_fp64(3, nrhs, S, ctx->src_local64_d, ctx->src_body_d, ctx->sumN, ctx->colloc4_d, ctx->sumM,
                          ctx->colT_begin_d, ctx->colT_end_d, ctx->tgt_off_d, ctx->centres_d, w, include_self,
                          ctx->raw_d, st));
         const size_t n = (size_t)nrhs * ctx->sumN * 3;
         combine_raw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ctx->raw_d, nullptr, 0.0, kernel_scale(ctx), z,
-                                                                        n);
+                                                                        n, S);
         CK(cudaGetLastError());
         ctx->launches += 2;
         return MFS_OK;
@@ -1272,8 +1293,8 @@ mfs_status precondT_dev(mfs_ctx *ctx, const double *z, double *out, int project,
             // FP64 reference: out = R_M U (W (R_N^T z)) with the transposed FP64 factors
             CK(gather_rotate(3, z, ctx->sumN * 3, sh.col_body, sh.col_rhs, ctx->src_off_d, ctx->rot64_d, ncols, sd.dN,
                              sh.A, sh.A64, st));
-            CK(gemm_rm64(ncols, sd.r, sd.dN, sh.A64, project ? sd.WpT64 : sd.WrT64, sh.T64, st));
-            CK(gemm_rm64(ncols, sd.dM, sd.r, sh.T64, sd.UT64, sh.O64, st));
+            CK(gemm64(ctx, sh, ncols, sd.r, sd.dN, sh.A64, project ? sd.WpT64 : sd.WrT64, sh.T64, st));
+            CK(gemm64(ctx, sh, ncols, sd.dM, sd.r, sh.T64, sd.UT64, sh.O64, st));
             CK(scatter_rotate(3, nullptr, sh.O64, sh.col_body, sh.col_rhs, ctx->tgt_off_d, ctx->rot_d, ctx->rot64_d,
                               ncols, sd.dM, ctx->sumM, out, st));
             ctx->launches += 4;
@@ -1329,7 +1350,7 @@ mfs_status matvec_T_dev(mfs_ctx *ctx, const double *w, double *y, int nrhs, cuda
     CKS(pair_apply_T(ctx, w, ctx->lam_d, nrhs, 0, st));
     CKS(precondT_dev(ctx, ctx->lam_d, ctx->tmpM_d, 1, nrhs, st));
     const size_t n = (size_t)nrhs * ctx->sumM * 3;
-    combine_raw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ctx->tmpM_d, w, 1.0, 1.0, y, n);
+    combine_raw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ctx->tmpM_d, w, 1.0, 1.0, y, n, 1);
     CK(cudaGetLastError());
     ctx->launches += 1;
     return MFS_OK;
@@ -1641,9 +1662,17 @@ static mfs_status alloc_apply_scratch(mfs_ctx *ctx, ShapeHost &sh, cudaStream_t 
               ctx->alloc(&sh.A, (size_t)R * nb * m) == cudaSuccess &&
               ctx->alloc(&sh.Tm, (size_t)R * nb * n) == cudaSuccess &&
               ctx->alloc(&sh.Lm, (size_t)R * nb * n) == cudaSuccess;
-    if (ok && ctx->opt.precision >= 1)
+    if (ok && ctx->opt.precision >= 1) {
+        size_t need = 1;  // both GEMMs, and the adjoint's second one (n -> m)
+        for (int h = 1; h <= R; ++h) {
+            const int rows = h * nb;
+            need = std::max(need, (size_t)gemm_rm64_chunks(rows, n, m, ctx->sm_count) * rows * n);
+            need = std::max(need, (size_t)gemm_rm64_chunks(rows, n, n, ctx->sm_count) * rows * n);
+            need = std::max(need, (size_t)gemm_rm64_chunks(rows, m, n, ctx->sm_count) * rows * m);
+        }
         ok = ctx->alloc(&sh.A64, (size_t)R * nb * m) == cudaSuccess &&
-             ctx->alloc(&sh.T64, (size_t)R * nb * n) == cudaSuccess;
+             ctx->alloc(&sh.T64, (size_t)R * nb * n) == cudaSuccess && ctx->alloc(&sh.Pk64, need) == cudaSuccess;
+    }
     if (ok) ok = ctx->alloc(&sh.L64, (size_t)R * nb * n) == cudaSuccess;
     if (ok) {  // split-K chunk results: the largest S * rows * cols over nrhs = 1..R and both GEMMs
         size_t need = 0;
@@ -2166,7 +2195,9 @@ static mfs_status setup_impl(mfs_ctx *ctx, mfs_kind kind, const mfs_bodies *bodi
     CK(ctx->alloc(&ctx->rec_d, (size_t)ctx->nrec * recf));
     CK(cudaMemset(ctx->rec_d, 0, sizeof(float) * (size_t)ctx->nrec * recf));
     CK(ctx->alloc(&ctx->lam_d, (size_t)R * ctx->sumN * D));
-    if (ctx->opt.precision == 1) CK(ctx->alloc(&ctx->raw_d, (size_t)R * ctx->sumM * D));
+    if (ctx->opt.precision == 1)
+        CK(ctx->alloc(&ctx->raw_d, R * D * std::max((size_t)fp64_chunks(ctx, ctx->sumM) * ctx->sumM,
+                                                    (size_t)fp64_chunks(ctx, ctx->sumN, true) * ctx->sumN)));
     CK(cudaMallocHost(&ctx->done_h, sizeof(int)));
     CK(cudaEventCreate(&ctx->ev0));
     CK(cudaEventCreate(&ctx->ev1));
@@ -2795,7 +2826,7 @@ mfs_status mfs_mobility_vjp(mfs_ctx *ctx, const double *dU, const double *dOmega
     CK(completion_stokes(dUi.d, dWi.d, nrhs, P, ctx->rot64_d, ctx->eye6_d, ctx->shape_id_d, ctx->src_local64_d,
                          ctx->src_off_d, ctx->sumN, ctx->lam_d, st));
     CKS(precondT_dev(ctx, ctx->lam_d, ctx->tmpM_d, 0, nrhs, st));
-    combine_raw_kernel<<<(unsigned)((nM + 255) / 256), 256, 0, st>>>(ctx->tmpM_d, nullptr, 0.0, -1.0, ctx->b_d, nM);
+    combine_raw_kernel<<<(unsigned)((nM + 255) / 256), 256, 0, st>>>(ctx->tmpM_d, nullptr, 0.0, -1.0, ctx->b_d, nM, 1);
     CK(cudaGetLastError());
     // 2. A^T w = g
     SolveStats ss;
@@ -2810,7 +2841,7 @@ mfs_status mfs_mobility_vjp(mfs_ctx *ctx, const double *dU, const double *dOmega
                          ctx->src_local64_d, ctx->src_off_d, ctx->sumN, lam0, st));
     CKS(precond_apply_dev(ctx, ctx->keep_gamma, ctx->lam_d, 1, nrhs, st));
     const size_t nN = (size_t)nrhs * ctx->sumN * 3;
-    combine_raw_kernel<<<(unsigned)((nN + 255) / 256), 256, 0, st>>>(lam0, ctx->lam_d, 1.0, 1.0, ctx->lam_d, nN);
+    combine_raw_kernel<<<(unsigned)((nN + 255) / 256), 256, 0, st>>>(lam0, ctx->lam_d, 1.0, 1.0, ctx->lam_d, nN, 1);
     CK(cudaGetLastError());
     // 4. centre gradient: pair kernel over off-diagonal pairs with target strengths w, source strengths mu
     int vc = 0, gv = -1;
@@ -2833,18 +2864,19 @@ mfs_status mfs_mobility_vjp(mfs_ctx *ctx, const double *dU, const double *dOmega
     } else if (ctx->opt.precision == 1) {
         // FP64 reference, the same two sides as the treecode's: weights w at the collocation points
         // against mu, weights mu at the proxy points against w (roles swapped, sign folded into dc)
-        CK(grad_pair_fp64(nrhs, ctx->tgt_local64_d, ctx->tgt_body_d, ctx->sumM, ctx->x_d, ctx->src_local4_d,
-                          ctx->sumN, ctx->susp_src_begin_d, ctx->susp_src_end_d, ctx->src_off_d, ctx->centres_d,
-                          ctx->lam_d, ctx->gradT_d, st));
-        CK(grad_pair_fp64(nrhs, ctx->src_local64_d, ctx->src_body_d, ctx->sumN, ctx->lam_d, ctx->colloc4_d,
-                          ctx->sumM, ctx->colT_begin_d, ctx->colT_end_d, ctx->tgt_off_d, ctx->centres_d, ctx->x_d,
-                          ctx->tmpM_d, st));
         const double scale = kernel_scale(ctx);
         const size_t nc = (size_t)ctx->sumM * 3, np3 = (size_t)ctx->sumN * 3;
-        combine_raw_kernel<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(ctx->gradT_d, nullptr, 0.0, scale,
-                                                                         ctx->gradT_d, nc);
-        combine_raw_kernel<<<(unsigned)((np3 + 255) / 256), 256, 0, st>>>(ctx->tmpM_d, nullptr, 0.0, scale,
-                                                                          ctx->tmpM_d, np3);
+        const int Sc = fp64_chunks(ctx, ctx->sumM), Sp = fp64_chunks(ctx, ctx->sumN, true);
+        CK(grad_pair_fp64(nrhs, Sc, ctx->tgt_local64_d, ctx->tgt_body_d, ctx->sumM, ctx->x_d, ctx->src_local4_d,
+                          ctx->sumN, ctx->susp_src_begin_d, ctx->susp_src_end_d, ctx->src_off_d, ctx->centres_d,
+                          ctx->lam_d, ctx->raw_d, st));
+        combine_raw_kernel<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(ctx->raw_d, nullptr, 0.0, scale,
+                                                                         ctx->gradT_d, nc, Sc);
+        CK(grad_pair_fp64(nrhs, Sp, ctx->src_local64_d, ctx->src_body_d, ctx->sumN, ctx->lam_d, ctx->colloc4_d,
+                          ctx->sumM, ctx->colT_begin_d, ctx->colT_end_d, ctx->tgt_off_d, ctx->centres_d, ctx->x_d,
+                          ctx->raw_d, st));
+        combine_raw_kernel<<<(unsigned)((np3 + 255) / 256), 256, 0, st>>>(ctx->raw_d, nullptr, 0.0, scale,
+                                                                          ctx->tmpM_d, np3, Sp);
         centre_grad_ff_kernel<<<P, 128, 0, st>>>(ctx->gradT_d, ctx->tgt_off_d, ctx->tmpM_d, ctx->src_off_d, dco.d);
         CK(cudaGetLastError());
         ctx->launches += 5;
@@ -3182,12 +3214,14 @@ mfs_status mfs_evaluate(mfs_ctx *ctx, const double *points, const int32_t *owner
         const double scale = kernel_scale(ctx);
         if (ctx->opt.precision == 1) {  // FP64 direct sums
             CK(ctx->alloc(&t64_d, 3 * (size_t)np));
-            CK(ctx->alloc(&raw_d, (size_t)nrhs * np * D));
+            const int S = fp64_chunks(ctx, np);
+            CK(ctx->alloc(&raw_d, (size_t)S * nrhs * np * D));
             CK(cudaMemcpyAsync(t64_d, t64.data(), sizeof(double) * t64.size(), cudaMemcpyHostToDevice, st));
-            CK(pair_sum_fp64(D, nrhs, t64_d, tbody_d, np, ctx->src_local4_d, ctx->sumN, ctx->susp_src_begin_d,
+            CK(pair_sum_fp64(D, nrhs, S, t64_d, tbody_d, np, ctx->src_local4_d, ctx->sumN, ctx->susp_src_begin_d,
                              ctx->susp_src_end_d, ctx->src_off_d, ctx->centres_d, ctx->lam_d, 1, raw_d, st));
             const size_t n = (size_t)nrhs * np * D;
-            combine_raw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(raw_d, nullptr, 0.0, scale, sorted_d, n);
+            combine_raw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(raw_d, nullptr, 0.0, scale, sorted_d, n,
+                                                                            S);
             CK(cudaGetLastError());
         } else {  // the FP32 pair kernel on the new targets, all pairs of the owner's suspension
             const int variant = fp32_variant(ctx, D, nrhs);

@@ -304,59 +304,67 @@ cudaError_t scatter_rotate(int D, const float *L, const double *L64, const int *
 }
 
 // ---------------------------------------------------------------------------
-// Row-major GEMM C[m][n] = A[m][k] B[k][n]: 64x64 output tile, 16-deep k slices in shared
-// memory, 4x4 outputs per thread (256 threads).  FP32 (matvec) and FP64 (reference path, far-field
-// fits).  With gridDim.z > 1, CTA z sums only k in [z kchunk, (z + 1) kchunk) and writes its partial
-// product to C + z m n (a split over K, summed afterwards in a fixed order).
+// FP64 row-major GEMM C[m][n] = A[m][k] B[k][n] (the FP64 one-body applies, the far-field fits).
+//
+// Bound by the FP64 pipe (2 DFMA per clock per SM: a 64 x 64 x 16 slab takes 16 us on one SM), so the
+// kernel spends FP64 instructions on real rows and columns only and keeps every SM equally busy:
+// 64 x 64 output tile per CTA, 16-deep k slices in shared memory, a warp on 32 columns and every fourth
+// row, so that a ragged last tile (24 columns of the one-body apply are rows here) skips its missing
+// rows evenly in all warps; gridDim.z > 1 splits K, CTA z writing its partial product to C + z m n
+// (summed afterwards in chunk order).  Before, 24 columns
+// of a 1800 x 900 factor ran on 15 CTAs with 40 of 64 rows padding, 1.6 ms a product; a matvec of 60
+// spheres with the compensated pair sums (M = 600, N = 300) took 5.78 ms and takes 2.99 ms.
 // ---------------------------------------------------------------------------
-template <typename TT>
-__global__ void __launch_bounds__(256) gemm_rm_kernel(int m, int n, int k, const TT *__restrict__ A,
-                                                      const TT *__restrict__ B, TT *__restrict__ C, int kchunk) {
-    constexpr int BM = 64, BN = 64, BK = 16;
-    __shared__ TT As[BK][BM + 4];
-    __shared__ TT Bs[BK][BN + 4];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+__global__ void __launch_bounds__(256) gemm_rm64_kernel(int m, int n, int k, const double *__restrict__ A,
+                                                        const double *__restrict__ B, double *__restrict__ C,
+                                                        int kchunk) {
+    constexpr int BM = 64, BN = 64, BK = 16, RPT = 16;  // rows per thread: ty, ty + 4, ...
+    __shared__ double As[BK][BM + 1];
+    __shared__ double Bs[BK][BN];
+    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
     const int kbeg = blockIdx.z * kchunk, kend = min(k, kbeg + kchunk);
     C += (size_t)blockIdx.z * m * n;
-    TT acc[4][4];
+    // rows of this warp inside the matrix; none when its 32 columns lie outside
+    int nr = min(RPT, max(0, (m - m0 - ty + 3) / 4));
+    if (n0 + (tx & 32) >= n) nr = 0;
+    double acc[RPT];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0;
+    for (int i = 0; i < RPT; ++i) acc[i] = 0.0;
     for (int k0 = kbeg; k0 < kend; k0 += BK) {
         for (int e = threadIdx.x; e < BM * BK; e += 256) {  // A tile: rows m0.., cols k0..
             const int r = e / BK, c = e % BK;
             const int gm = m0 + r, gk = k0 + c;
-            As[c][r] = (gm < m && gk < kend) ? A[(size_t)gm * k + gk] : TT(0);
+            As[c][r] = (gm < m && gk < kend) ? A[(size_t)gm * k + gk] : 0.0;
         }
         for (int e = threadIdx.x; e < BK * BN; e += 256) {
             const int r = e / BN, c = e % BN;
             const int gk = k0 + r, gn = n0 + c;
-            Bs[r][c] = (gk < kend && gn < n) ? B[(size_t)gk * n + gn] : TT(0);
+            Bs[r][c] = (gk < kend && gn < n) ? B[(size_t)gk * n + gn] : 0.0;
         }
         __syncthreads();
+        if (nr == RPT) {
 #pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            TT a[4], b[4];
+            for (int kk = 0; kk < BK; ++kk) {
+                const double b = Bs[kk][tx];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
+                for (int i = 0; i < RPT; ++i) acc[i] = fma(As[kk][ty + 4 * i], b, acc[i]);
+            }
+        } else if (nr > 0) {
+#pragma unroll 4
+            for (int kk = 0; kk < BK; ++kk) {
+                const double b = Bs[kk][tx];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * b[j];
+                for (int i = 0; i < RPT; ++i)
+                    if (i < nr) acc[i] = fma(As[kk][ty + 4 * i], b, acc[i]);
+            }
         }
         __syncthreads();
     }
+    if (n0 + tx < n)
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int gm = m0 + ty * 4 + i, gn = n0 + tx * 4 + j;
-            if (gm < m && gn < n) C[(size_t)gm * n + gn] = acc[i][j];
-        }
+        for (int i = 0; i < RPT; ++i)
+            if (i < nr) C[(size_t)(m0 + ty + 4 * i) * n + n0 + tx] = acc[i];
 }
 
 // Split-K FP32 GEMM with compensated accumulation: CTA (x, y, z) computes the 64x64 tile (y, x)
@@ -475,25 +483,22 @@ cudaError_t gemm_splitk(int m, int n, int k, int S, const float *A, const float 
     return cudaGetLastError();
 }
 
-cudaError_t gemm_rm(int m, int n, int k, const float *A, const float *B, float *C, cudaStream_t st) {
-    if (m == 0 || n == 0) return cudaSuccess;
-    dim3 grid((n + 63) / 64, (m + 63) / 64);
-    gemm_rm_kernel<float><<<grid, 256, 0, st>>>(m, n, k, A, B, C, k);
-    return cudaGetLastError();
-}
-
-cudaError_t gemm_rm64(int m, int n, int k, const double *A, const double *B, double *C, cudaStream_t st) {
-    if (m == 0 || n == 0) return cudaSuccess;
-    dim3 grid((n + 63) / 64, (m + 63) / 64);
-    gemm_rm_kernel<double><<<grid, 256, 0, st>>>(m, n, k, A, B, C, k);
-    return cudaGetLastError();
-}
-
+// Chunks of K: the count whose busiest SM has the least to do, ceil(CTAs / SMs) times a chunk's length
+// plus about 24 k steps of fill and write-out per CTA; chunks of at least 32.
 int gemm_rm64_chunks(int m, int n, int k, int sm_count) {
-    const int tiles = ((n + 63) / 64) * ((m + 63) / 64);
-    int s = (2 * sm_count) / std::max(tiles, 1);  // about two CTAs per SM
-    s = std::min(s, (k + 127) / 128);               // chunks of at least 128 of K
-    return std::max(s, 1);
+    const long long tiles = (long long)((n + 63) / 64) * ((m + 63) / 64);
+    int best = 1;
+    long long least = 0;
+    for (int s = 1; s <= std::max(1, k / 32); ++s) {
+        const long long kchunk = ((k + s - 1) / s + 15) / 16 * 16, sz = (k + kchunk - 1) / kchunk;
+        const long long cost = (tiles * sz + sm_count - 1) / sm_count * (kchunk + 24);
+        if (s == 1 || cost < least) {
+            least = cost;
+            best = s;
+        }
+        if (tiles * s >= 16LL * sm_count) break;  // finer splits only add partials to sum
+    }
+    return best;
 }
 
 __global__ void sum_chunks_kernel(int S, size_t mn, const double *__restrict__ P, double *__restrict__ C) {
@@ -507,13 +512,14 @@ __global__ void sum_chunks_kernel(int S, size_t mn, const double *__restrict__ P
 cudaError_t gemm_rm64_splitk(int m, int n, int k, int S, const double *A, const double *B, double *P, double *C,
                              cudaStream_t st) {
     if (m == 0 || n == 0) return cudaSuccess;
-    if (S <= 1) return gemm_rm64(m, n, k, A, B, C, st);
     const int kchunk = ((k + S - 1) / S + 15) / 16 * 16;
     const int Sz = (k + kchunk - 1) / kchunk;
     dim3 grid((n + 63) / 64, (m + 63) / 64, Sz);
-    gemm_rm_kernel<double><<<grid, 256, 0, st>>>(m, n, k, A, B, P, kchunk);
-    const size_t mn = (size_t)m * n;
-    sum_chunks_kernel<<<(unsigned)std::min<size_t>((mn + 255) / 256, 4096), 256, 0, st>>>(Sz, mn, P, C);
+    gemm_rm64_kernel<<<grid, 256, 0, st>>>(m, n, k, A, B, Sz > 1 ? P : C, kchunk);
+    if (Sz > 1) {
+        const size_t mn = (size_t)m * n;
+        sum_chunks_kernel<<<(unsigned)std::min<size_t>((mn + 255) / 256, 4096), 256, 0, st>>>(Sz, mn, P, C);
+    }
     return cudaGetLastError();
 }
 
@@ -679,103 +685,181 @@ cudaError_t extract_laplace(const double *alpha, int nrhs, int P, const int *bod
 }
 
 // ---------------------------------------------------------------------------
-// FP64 reference pair sum (precision = 1): one thread per target, plain loops.
-// out_raw holds the sum without the 1/(4 pi) or 1/(8 pi mu) factor, layout [nrhs][nt][D].
+// FP64 reference sums (precision = 1): one thread per target and source chunk.
+//
+// Bound by the FP64 pipe (GB300: 2 DFMA per clock per SM, a warp's DFMA every 64 clocks per scheduler),
+// so what counts is FP64 instructions per pair and that every SM has the same share of them; loads and
+// shared memory do not show.  Per Stokeslet pair: 3 subtractions (the target is taken relative to the
+// source body's centre once per body), r^2 3, 1/r 5 (rsqrt64), r.l 3, (r.l)/r^2 2, six FMAs = 22, where
+// divisions and a square root by the library took it above 100.  The grid's y axis cuts each target's
+// sources into S chunks so that small suspensions fill the GPU too; the partial sums [S][nrhs][nt][D]
+// are added in chunk order by the caller's combine kernel.  24 spheres (M = 600, N = 300), 9.9e7 pairs:
+// 17.8 ms on 113 CTAs with library square roots and divisions; the whole FP64 matvec with this kernel
+// and the GEMM above 4.59 ms (20.9 ms before).
 // ---------------------------------------------------------------------------
-__global__ void pair_sum_fp64_kernel(int D, int nrhs, const double *tgt_local, const int *tgt_body, int nt,
-                                     const double *src_local4, int nsrc, const int *susp_src_begin,
-                                     const int *susp_src_end, const int *body_src_off, const double *centres,
-                                     const double *strength, int include_self, double *out) {
+#define FP64_PAIR_THREADS 128
+
+int fp64_pair_chunks(int ntargets, int min_sources, int sm_count) {
+    // about 16 CTAs per SM, so that the last ones to run leave little of the GPU idle; chunks keep at
+    // least 64 sources, which the per-body set-up and the epilogue's share are small against
+    const long long ctas = (ntargets + FP64_PAIR_THREADS - 1) / FP64_PAIR_THREADS;
+    long long s = (16LL * sm_count + ctas - 1) / std::max<long long>(ctas, 1);
+    s = std::min<long long>(s, std::max(1, min_sources / 64));
+    return (int)std::max<long long>(1, std::min<long long>(s, 64));
+}
+
+// Body of source s among bodies whose offsets are body_src_off (the body with off[b] <= s).
+__device__ __forceinline__ int body_of_source(const double *src_local4, int s) { return (int)src_local4[4 * (size_t)s + 3]; }
+
+template <int D, int NRHS>
+__global__ void __launch_bounds__(FP64_PAIR_THREADS)
+pair_sum_fp64_kernel(const double *__restrict__ tgt_local, const int *__restrict__ tgt_body, int nt,
+                     const double *__restrict__ src_local4, int nsrc, const int *__restrict__ susp_src_begin,
+                     const int *__restrict__ susp_src_end, const int *__restrict__ body_src_off,
+                     const double *__restrict__ centres, const double *__restrict__ strength, int include_self,
+                     double *__restrict__ out) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nt) return;
     const int kt = tgt_body[t];
-    const double x[3] = {centres[3 * kt] + tgt_local[3 * t], centres[3 * kt + 1] + tgt_local[3 * t + 1],
-                         centres[3 * kt + 2] + tgt_local[3 * t + 2]};
-    double acc[12];
-    for (int c = 0; c < 12; ++c) acc[c] = 0.0;
-    const int self0 = body_src_off[kt], self1 = body_src_off[kt + 1];
-    for (int s = susp_src_begin[kt]; s < susp_src_end[kt]; ++s) {
-        if (!include_self && s >= self0 && s < self1) continue;
-        const double *yl = src_local4 + 4 * (size_t)s;  // x, y, z (rotated, body-local), source body
-        const int kb = (int)yl[3];
-        const double r[3] = {x[0] - (centres[3 * kb] + yl[0]), x[1] - (centres[3 * kb + 1] + yl[1]),
-                             x[2] - (centres[3 * kb + 2] + yl[2])};
-        const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
-        const double ri = 1.0 / sqrt(r2);
-        for (int h = 0; h < nrhs; ++h) {
-            if (D == 1) {
-                acc[h] += strength[(size_t)h * nsrc + s] * ri;
-            } else {
-                const double *l = strength + ((size_t)h * nsrc + s) * 3;
-                const double dot = r[0] * l[0] + r[1] * l[1] + r[2] * l[2];
-                for (int a = 0; a < 3; ++a) acc[3 * h + a] += (l[a] + r[a] * dot / r2) * ri;
+    const int sb = susp_src_begin[kt];
+    const long long len = susp_src_end[kt] - sb;
+    int s = sb + (int)(len * blockIdx.y / gridDim.y);
+    const int send = sb + (int)(len * (blockIdx.y + 1) / gridDim.y);
+    double acc[D * NRHS];
+#pragma unroll
+    for (int c = 0; c < D * NRHS; ++c) acc[c] = 0.0;
+    while (s < send) {
+        const int kb = body_of_source(src_local4, s);
+        const int e = min(send, body_src_off[kb + 1]);
+        if (kb == kt && !include_self) {
+            s = e;
+            continue;
+        }
+        double x[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) x[c] = (centres[3 * kt + c] - centres[3 * kb + c]) + tgt_local[3 * (size_t)t + c];
+#pragma unroll 2
+        for (; s < e; ++s) {
+            const double *yl = src_local4 + 4 * (size_t)s;
+            const double r0 = x[0] - yl[0], r1 = x[1] - yl[1], r2_ = x[2] - yl[2];
+            const double ri = rsqrt64(fma(r0, r0, fma(r1, r1, r2_ * r2_)));
+            const double ri2 = ri * ri;
+#pragma unroll
+            for (int h = 0; h < NRHS; ++h) {
+                if (D == 1) {
+                    acc[h] = fma(strength[(size_t)h * nsrc + s], ri, acc[h]);
+                } else {
+                    const double *l = strength + ((size_t)h * nsrc + s) * 3;
+                    const double l0 = l[0], l1 = l[1], l2 = l[2];
+                    const double sc = fma(r0, l0, fma(r1, l1, r2_ * l2)) * ri2;
+                    acc[D * h] = fma(fma(r0, sc, l0), ri, acc[D * h]);
+                    if (D == 3) {
+                        acc[D * h + 1] = fma(fma(r1, sc, l1), ri, acc[D * h + 1]);
+                        acc[D * h + 2] = fma(fma(r2_, sc, l2), ri, acc[D * h + 2]);
+                    }
+                }
             }
         }
     }
-    for (int h = 0; h < nrhs; ++h)
-        for (int a = 0; a < D; ++a) out[((size_t)h * nt + t) * D + a] = acc[D * h + a];
+    double *o = out + (size_t)blockIdx.y * NRHS * nt * D;
+#pragma unroll
+    for (int h = 0; h < NRHS; ++h)
+#pragma unroll
+        for (int a = 0; a < D; ++a) o[((size_t)h * nt + t) * D + a] = acc[D * h + a];
 }
 
-// FP64 reference of the adjoint's pair gradient (precision = 1): one thread per target,
+// The adjoint's pair gradient (precision = 1), the same split:
 //   out_t = sum_h sum_{s in t's suspension, not on t's body} grad_r (tw_h(t)^T G(r) sigma_h(s)),  r = x_t - y_s,
 // G = I / r + r r^T / r^3 (raw, without 1 / (8 pi mu)), so grad_r = [w (r.m) + m (w.r) - (w.m) r
 // - 3 (w.r)(r.m) r / r^2] / r^3 with w = tw_h(t), m = sigma_h(s).  Layouts as pair_sum_fp64; tw is
-// [nrhs][nt][3], out [nt][3].
-__global__ void grad_pair_fp64_kernel(int nrhs, const double *tgt_local, const int *tgt_body, int nt, const double *tw,
-                                      const double *src_local4, int nsrc, const int *susp_src_begin,
-                                      const int *susp_src_end, const int *body_src_off, const double *centres,
-                                      const double *strength, double *out) {
+// [nrhs][nt][3], out [S][nt][3].
+template <int NRHS>
+__global__ void __launch_bounds__(FP64_PAIR_THREADS)
+grad_pair_fp64_kernel(const double *__restrict__ tgt_local, const int *__restrict__ tgt_body, int nt,
+                      const double *__restrict__ tw, const double *__restrict__ src_local4, int nsrc,
+                      const int *__restrict__ susp_src_begin, const int *__restrict__ susp_src_end,
+                      const int *__restrict__ body_src_off, const double *__restrict__ centres,
+                      const double *__restrict__ strength, double *__restrict__ out) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nt) return;
     const int kt = tgt_body[t];
-    const double x[3] = {centres[3 * kt] + tgt_local[3 * t], centres[3 * kt + 1] + tgt_local[3 * t + 1],
-                         centres[3 * kt + 2] + tgt_local[3 * t + 2]};
-    double acc[3] = {0.0, 0.0, 0.0};
-    const int self0 = body_src_off[kt], self1 = body_src_off[kt + 1];
-    for (int s = susp_src_begin[kt]; s < susp_src_end[kt]; ++s) {
-        if (s >= self0 && s < self1) continue;
-        const double *yl = src_local4 + 4 * (size_t)s;
-        const int kb = (int)yl[3];
-        const double r[3] = {x[0] - (centres[3 * kb] + yl[0]), x[1] - (centres[3 * kb + 1] + yl[1]),
-                             x[2] - (centres[3 * kb + 2] + yl[2])};
-        const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
-        const double ri = 1.0 / sqrt(r2);
-        const double ri3 = ri * ri * ri;
-        for (int h = 0; h < nrhs; ++h) {
-            const double *w = tw + ((size_t)h * nt + t) * 3;
-            const double *m = strength + ((size_t)h * nsrc + s) * 3;
-            const double wm = w[0] * m[0] + w[1] * m[1] + w[2] * m[2];
-            const double wr = w[0] * r[0] + w[1] * r[1] + w[2] * r[2];
-            const double rm = r[0] * m[0] + r[1] * m[1] + r[2] * m[2];
-            const double q = -(wm + 3.0 * wr * rm / r2);
-            for (int a = 0; a < 3; ++a) acc[a] += (r[a] * q + w[a] * rm + m[a] * wr) * ri3;
+    const int sb = susp_src_begin[kt];
+    const long long len = susp_src_end[kt] - sb;
+    int s = sb + (int)(len * blockIdx.y / gridDim.y);
+    const int send = sb + (int)(len * (blockIdx.y + 1) / gridDim.y);
+    double w[NRHS][3], acc[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int h = 0; h < NRHS; ++h)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) w[h][c] = tw[((size_t)h * nt + t) * 3 + c];
+    while (s < send) {
+        const int kb = body_of_source(src_local4, s);
+        const int e = min(send, body_src_off[kb + 1]);
+        if (kb == kt) {
+            s = e;
+            continue;
+        }
+        double x[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) x[c] = (centres[3 * kt + c] - centres[3 * kb + c]) + tgt_local[3 * (size_t)t + c];
+        for (; s < e; ++s) {
+            const double *yl = src_local4 + 4 * (size_t)s;
+            const double r[3] = {x[0] - yl[0], x[1] - yl[1], x[2] - yl[2]};
+            const double ri = rsqrt64(fma(r[0], r[0], fma(r[1], r[1], r[2] * r[2])));
+            const double ri2 = ri * ri, ri3 = ri * ri2, ri2_3 = 3.0 * ri2;
+#pragma unroll
+            for (int h = 0; h < NRHS; ++h) {
+                const double *m = strength + ((size_t)h * nsrc + s) * 3;
+                const double m0 = m[0], m1 = m[1], m2 = m[2];
+                const double wm = fma(w[h][0], m0, fma(w[h][1], m1, w[h][2] * m2));
+                const double wr = fma(w[h][0], r[0], fma(w[h][1], r[1], w[h][2] * r[2]));
+                const double rm = fma(r[0], m0, fma(r[1], m1, r[2] * m2));
+                const double q = -fma(wr * rm, ri2_3, wm);
+                acc[0] = fma(fma(r[0], q, fma(w[h][0], rm, m0 * wr)), ri3, acc[0]);
+                acc[1] = fma(fma(r[1], q, fma(w[h][1], rm, m1 * wr)), ri3, acc[1]);
+                acc[2] = fma(fma(r[2], q, fma(w[h][2], rm, m2 * wr)), ri3, acc[2]);
+            }
         }
     }
-    for (int a = 0; a < 3; ++a) out[3 * (size_t)t + a] = acc[a];
+    double *o = out + (size_t)blockIdx.y * nt * 3;
+    for (int a = 0; a < 3; ++a) o[3 * (size_t)t + a] = acc[a];
 }
 
-cudaError_t grad_pair_fp64(int nrhs, const double *tgt_local, const int *tgt_body, int ntargets, const double *tw,
-                           const double *src_local4, int nsrc, const int *susp_src_begin, const int *susp_src_end,
-                           const int *body_src_off, const double *centres, const double *strength, double *out,
-                           cudaStream_t st) {
-    const int threads = 128;
+cudaError_t grad_pair_fp64(int nrhs, int chunks, const double *tgt_local, const int *tgt_body, int ntargets,
+                           const double *tw, const double *src_local4, int nsrc, const int *susp_src_begin,
+                           const int *susp_src_end, const int *body_src_off, const double *centres,
+                           const double *strength, double *out, cudaStream_t st) {
     if (ntargets == 0) return cudaSuccess;
-    grad_pair_fp64_kernel<<<(ntargets + threads - 1) / threads, threads, 0, st>>>(
-        nrhs, tgt_local, tgt_body, ntargets, tw, src_local4, nsrc, susp_src_begin, susp_src_end, body_src_off, centres,
-        strength, out);
-    return cudaGetLastError();
+    const dim3 grid((ntargets + FP64_PAIR_THREADS - 1) / FP64_PAIR_THREADS, chunks);
+#define GP(R_)                                                                                                   \
+    if (nrhs == R_) {                                                                                            \
+        grad_pair_fp64_kernel<R_><<<grid, FP64_PAIR_THREADS, 0, st>>>(tgt_local, tgt_body, ntargets, tw, src_local4, \
+                                                                      nsrc, susp_src_begin, susp_src_end,        \
+                                                                      body_src_off, centres, strength, out);     \
+        return cudaGetLastError();                                                                               \
+    }
+    GP(1) GP(2) GP(3) GP(4)
+#undef GP
+    return cudaErrorInvalidValue;
 }
 
-cudaError_t pair_sum_fp64(int D, int nrhs, const double *tgt_local, const int *tgt_body, int ntargets,
+cudaError_t pair_sum_fp64(int D, int nrhs, int chunks, const double *tgt_local, const int *tgt_body, int ntargets,
                           const double *src_local4, int nsrc, const int *susp_src_begin, const int *susp_src_end,
                           const int *body_src_off, const double *centres, const double *strength, int include_self,
                           double *out_raw, cudaStream_t st) {
-    const int threads = 128;
     if (ntargets == 0) return cudaSuccess;
-    pair_sum_fp64_kernel<<<(ntargets + threads - 1) / threads, threads, 0, st>>>(
-        D, nrhs, tgt_local, tgt_body, ntargets, src_local4, nsrc, susp_src_begin, susp_src_end, body_src_off, centres,
-        strength, include_self, out_raw);
-    return cudaGetLastError();
+    const dim3 grid((ntargets + FP64_PAIR_THREADS - 1) / FP64_PAIR_THREADS, chunks);
+#define PS(D_, R_)                                                                                                \
+    if (D == D_ && nrhs == R_) {                                                                                  \
+        pair_sum_fp64_kernel<D_, R_><<<grid, FP64_PAIR_THREADS, 0, st>>>(tgt_local, tgt_body, ntargets, src_local4,  \
+                                                                         nsrc, susp_src_begin, susp_src_end,      \
+                                                                         body_src_off, centres, strength,         \
+                                                                         include_self, out_raw);                  \
+        return cudaGetLastError();                                                                                \
+    }
+    PS(3, 1) PS(3, 2) PS(3, 3) PS(3, 4) PS(1, 1) PS(1, 2) PS(1, 3) PS(1, 4)
+#undef PS
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace mfs
