@@ -110,7 +110,10 @@ typedef struct {
                              points) / 0.83, fitted in FP64 by least squares to its proxies' field at 392
                              check points at 2.5 r_e; targets at least 3 r_e from a node's centre see it
                              through those points, nearer ones its children, down to the proxy points of the
-                             near bodies (direct, FP32 pair kernel).  Relative accuracy of the sums about
+                             near bodies (direct, FP32 pair kernel).  Targets further away use 128, 96 or 64
+                             points matched to the 196 (from 4, 5 and 8 radii on), and bodies with many
+                             collocation points receive what lies 5 of their radii away through 96 local
+                             sources fitted around them.  Relative accuracy of the sums about
                              1e-7; the pair work drops from O(P^2) to about O(P log P).  Needs precision 0 or
                              2.  Every forward pair sum uses it (the solves, mfs_matvec, mfs_pair_sum); the
                              transposed sums of mfs_matvec_transposed and mfs_mobility_vjp use a second tree

@@ -154,6 +154,87 @@ void ff_interaction_list(const FFTree &t, int root, const std::vector<int> &tbod
     }
 }
 
+int ff_order(double ratio, double kappa0) {
+    const double f = std::max(1.0, kappa0 / FF_ORD_KAPPA[0]);
+    if (!(ratio >= kappa0)) return -1;
+    int o = 0;
+    while (o + 1 < FF_NORD && ratio >= f * FF_ORD_KAPPA[o + 1]) ++o;
+    return o;
+}
+
+static double distance_to(const FFNode &n, const double *c) {
+    double d2 = 0.0;
+    for (int a = 0; a < 3; ++a) d2 += (c[a] - n.c[a]) * (c[a] - n.c[a]);
+    return std::sqrt(d2);
+}
+
+void ff_ordered_list(const FFTree &t, int root, const std::vector<int> &tbodies, const double *centres,
+                     const double *rtgt, double kappa0, int self_skip, std::vector<int> &segs) {
+    const int P = (int)t.order.size(), nodes = (int)t.nodes.size();
+    std::vector<int> stack{root};
+    while (!stack.empty()) {
+        const int ni = stack.back();
+        stack.pop_back();
+        const FFNode &n = t.nodes[ni];
+        double near = 1e300;  // the nearest target point to the node's centre, at least
+        for (int b : tbodies) near = std::min(near, distance_to(n, centres + 3 * b) - rtgt[b]);
+        const int o = ff_order(near / n.re, kappa0);
+        if (o >= 0) {
+            segs.push_back(P + o * nodes + ni);
+        } else if (n.body >= 0) {
+            if (!(self_skip && tbodies.size() == 1 && tbodies[0] == n.body)) segs.push_back(t.pos[n.body]);
+        } else {
+            for (int i = n.nchild - 1; i >= 0; --i) stack.push_back(n.child[i]);
+        }
+    }
+}
+
+void ff_cell_lists(const FFTree &t, int root, const std::vector<int> &tbodies, const double *centres,
+                   const double *rtgt, double kappa0, double targets_per_body, std::vector<int> &local,
+                   std::vector<std::vector<int>> &direct) {
+    const int P = (int)t.order.size(), nodes = (int)t.nodes.size(), nt = (int)tbodies.size();
+    const double gap = FF_LOC_GAP * std::max(1.0, kappa0 / FF_ORD_KAPPA[0]);
+    local.clear();
+    direct.assign(nt, {});
+    double points = 0.0;  // equivalent points in `local`
+    std::vector<int> stack{root};
+    while (!stack.empty()) {
+        const int ni = stack.back();
+        stack.pop_back();
+        const FFNode &n = t.nodes[ni];
+        bool all = true;
+        double near = 1e300;
+        for (int b : tbodies) {
+            const double d = distance_to(n, centres + 3 * b);
+            near = std::min(near, d - FF_LOC_CHECK * rtgt[b]);  // its check points
+            all = all && d - n.re >= gap * rtgt[b];
+            if (!all) break;
+        }
+        const int o = all ? ff_order(near / n.re, kappa0) : -1;
+        if (o >= 0) {
+            local.push_back(P + o * nodes + ni);
+            points += FF_ORD_N[o];
+        } else if (n.body < 0) {
+            for (int i = n.nchild - 1; i >= 0; --i) stack.push_back(n.child[i]);
+        } else {
+            for (int i = 0; i < nt; ++i) {  // one source body: each target body by its own distance
+                if (tbodies[i] == n.body) continue;
+                const double ratio = (distance_to(n, centres + 3 * tbodies[i]) - rtgt[tbodies[i]]) / n.re;
+                const int oi = ff_order(ratio, kappa0);
+                direct[i].push_back(oi >= 0 ? P + oi * nodes + ni : t.pos[n.body]);
+            }
+        }
+    }
+    if (local.empty()) return;
+    const bool pays = points * targets_per_body >
+                      points * FF_LOC_NC + targets_per_body * FF_LOC_N + FF_LOC_FIT_PAIRS;
+    for (int i = 0; i < nt; ++i) {
+        if (pays) direct[i].push_back(P + FF_NORD * nodes + t.pos[tbodies[i]]);
+        else direct[i].insert(direct[i].end(), local.begin(), local.end());
+    }
+    if (!pays) local.clear();
+}
+
 __global__ void ff_scale_kernel(double *mu, const double *re, int nodes, int per_node, size_t n) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         mu[i] *= re[(i / per_node) % nodes];

@@ -156,6 +156,32 @@ constexpr double FF_CHECK = 2.5;      // check radius / equivalent radius
 constexpr double FF_SRC_RATIO = 0.83; // a node's source radius / its equivalent radius
 // (a target at least mfs_options.farfield_separation equivalent radii from a node's centre sees the node
 // through its equivalent points)
+// Lower orders of the same equivalent sources, for targets further away: order o has FF_ORD_N[o] points
+// on the node's equivalent sphere and serves targets at least FF_ORD_KAPPA[o] equivalent radii from the
+// node's centre (order 0 from farfield_separation on).  Its strengths are the least-squares match of the
+// next higher order's field at FF_ORD_NC[o] points at FF_ORD_CHECK[o] radii, where the high-degree part
+// that the smaller set cannot hold has already decayed.  White-noise sources at the edge of the node,
+// relative field error: 196 points 1.9e-7 at 3 radii and 3e-8 at 4; 128 points 6e-8 at 4; 96 points
+// 5e-8 at 5; 64 points 3e-8 at 8 (each falling further out).
+constexpr int FF_NORD = 4;
+constexpr int FF_ORD_N[FF_NORD] = {FF_NE, 128, 96, 64};
+constexpr int FF_ORD_NC[FF_NORD] = {FF_NC, 192, 160, 128};
+constexpr double FF_ORD_CHECK[FF_NORD] = {FF_CHECK, 4.0, 5.0, 8.0};
+constexpr double FF_ORD_KAPPA[FF_NORD] = {3.0, 4.0, 5.0, 8.0};
+// Singular values kept relative to the largest.  The last order's and the local match are cut at 1e-8:
+// below it they only amplify FP32 rounding of the check field into strengths twice as large, whose own
+// FP32 rounding then shows (field of 400 ellipsoids, white-noise strengths: 3.6e-7 uncut, 2.0e-7 cut,
+// 2.1e-7 without local expansions or lower orders).
+constexpr double FF_ORD_TRUNC[FF_NORD] = {1e-12, 1e-12, 1e-12, 1e-8}, FF_LOC_TRUNC = 1e-8;
+// Local expansions: the field of the sources whose equivalent spheres stay FF_LOC_GAP target radii
+// (rt, a body's farthest target point) away from a body's centre is evaluated at FF_LOC_NC points at
+// FF_LOC_CHECK rt, matched by FF_LOC_N sources at FF_LOC_EQ rt around the body, and those are summed at
+// the body's targets (1.5e-7 at the gap's edge, 3e-8 one radius further, 1e-8 at twice the distance).
+constexpr int FF_LOC_N = 96, FF_LOC_NC = 128;
+constexpr double FF_LOC_CHECK = 1.1, FF_LOC_EQ = 6.0, FF_LOC_GAP = 5.0;
+// The match of one body's local sources (3 FF_LOC_NC x 3 FF_LOC_N FP64 FMAs at 2 per clock per SM) in
+// pairs of the pair kernel (5.8 per clock per SM).
+constexpr double FF_LOC_FIT_PAIRS = 3.2e5;
 struct FFNode {
     double c[3] = {0, 0, 0};  // centre
     double rs = 0.0;          // radius of the node's proxy sources about c
@@ -178,6 +204,23 @@ void ff_build_tree(int P, const double *centres, const double *rsrc, int S, cons
 // self_skip, a single target body's own proxy points are left out.
 void ff_interaction_list(const FFTree &t, int root, const std::vector<int> &tbodies, const double *centres,
                          const double *rtgt, double kappa, int self_skip, std::vector<int> &segs);
+// Segment ids of the sums over several orders: proxies of tree position q: q; order o of node n:
+// P + o nodes + n; local sources of tree position q: P + FF_NORD nodes + q.
+// The highest order index whose distance rule holds at `ratio` = distance to the nearest target over
+// r_e, -1 when none does; kappa0 = farfield_separation (orders keep their distances when it is below 3
+// and move out in proportion above).
+int ff_order(double ratio, double kappa0);
+// Segments of the targets of the body set `tbodies` (one list for all of them): near bodies' proxies,
+// far nodes at their order; self_skip as ff_interaction_list.
+void ff_ordered_list(const FFTree &t, int root, const std::vector<int> &tbodies, const double *centres,
+                     const double *rtgt, double kappa0, int self_skip, std::vector<int> &segs);
+// The same cover split for local expansions: `local` gets the nodes that every body of the cell
+// `tbodies` sees through its local expansion; direct[i] the remaining segments of tbodies[i] itself (its
+// own proxies left out), among them its own local segment when `local` is not empty.  `local` stays
+// empty where summing those nodes at the bodies' targets (targets_per_body of them) is less work.
+void ff_cell_lists(const FFTree &t, int root, const std::vector<int> &tbodies, const double *centres,
+                   const double *rtgt, double kappa0, double targets_per_body, std::vector<int> &local,
+                   std::vector<std::vector<int>> &direct);
 // mu[h][node][e][d] *= re[node] (the fit was made on the unit sphere; the kernels are homogeneous of
 // degree -1).
 cudaError_t ff_scale(double *mu, const double *re, int nodes, int per_node, int nrhs, cudaStream_t st);

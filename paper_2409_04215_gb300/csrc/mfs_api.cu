@@ -200,15 +200,38 @@ struct mfs_ctx {
         int rec_floats = 0;
         double *ucheck = nullptr;                    // [max_rhs][nodes FF_NC][D]
         double *mu = nullptr;                        // [max_rhs][nodes FF_NE][D]
-        double *fit_chunks = nullptr;                // split-K partials of the fit product
+        double *fit_chunks = nullptr;                // split-K partials of the fit products
         float *wt = nullptr;                         // [max_rhs][ntgt][3] target weights in tree order (gradient)
-        struct Plan {
-            PairPlan up, ev;
-            int *lst_seg_up = nullptr, *lst_seg_ev = nullptr;
-            long long *lst_cum_up = nullptr, *lst_cum_ev = nullptr;
-            double pairs_up = 0.0, pairs_ev = 0.0;   // target-source pairs one application evaluates
+        // lower orders of the equivalent sources (index 1 .. FF_NORD - 1): the map from the next higher
+        // order's strengths, the points about their node's centre, the strengths
+        double *ordT[FF_NORD] = {};                  // [D FF_ORD_N[o - 1]][D FF_ORD_N[o]]
+        float4 *ord_pos[FF_NORD] = {};               // [nodes FF_ORD_N[o]]
+        double *ord_mu[FF_NORD] = {};                // [max_rhs][nodes FF_ORD_N[o]][D]
+        size_t ord_rec[FF_NORD] = {};                // first record of the order's segments
+        // local expansions of the bodies (tree order)
+        bool use_local = false;
+        double *locT = nullptr;                      // [D FF_LOC_NC][D FF_LOC_N]: check -> local sources, unit radius
+        double *rloc = nullptr;                      // [P] target radii
+        float4 *loc_pos = nullptr, *lchk_pos = nullptr;  // [P FF_LOC_N], [P FF_LOC_NC] about the body's centre
+        double *ulocal = nullptr, *nu = nullptr;     // [max_rhs][P FF_LOC_NC][D], [max_rhs][P FF_LOC_N][D]
+        size_t loc_rec = 0;
+        struct ListPlan {
+            PairPlan p;
+            int *seg = nullptr;
+            long long *cum = nullptr;
+            double pairs = 0.0;                      // target-source pairs one application evaluates
         };
-        std::map<int, Plan> plans;                   // key: variant * 2 + include_self
+        std::map<int, ListPlan> up;                  // upward sums, key: variant
+        std::map<int, ListPlan> ev;                  // order-0 lists at the targets (gradient), key: variant
+        std::map<int, ListPlan> loc;                 // local check points, key: variant
+        std::map<int, ListPlan> direct;              // targets, all orders, key: variant * 2 + include_self
+        struct Cells {                               // ff_cell_lists of every cell of `size` tree positions
+            std::vector<int> first;                  // first tree position of each cell, then P
+            std::vector<int> cell_of;                // tree position -> cell
+            std::vector<std::vector<int>> local;     // per cell
+            std::vector<std::vector<int>> direct;    // per tree position
+        };
+        std::map<int, Cells> cells;                  // key: cell size
     } ff, ffT;                                       // forward sums; transposed sums (adjoint)
 
     int sm_count = 0;
@@ -730,61 +753,175 @@ mfs_status build_plan_lists(mfs_ctx *ctx, int variant, int include_self, const s
     return MFS_OK;
 }
 
-// The far-field plans of one pair-kernel variant: the upward sums (each node's check points against
-// its descendant bodies' proxy points) and the evaluation (targets in tree order against their
-// interaction lists).
-mfs_status ff_get_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, int include_self,
-                       mfs_ctx::FarField::Plan **out) {
-    const int key = variant * 2 + include_self;
-    auto it = F.plans.find(key);
-    if (it != F.plans.end()) {
-        *out = &it->second;
-        return MFS_OK;
+// Records and blocks of every far-field segment.
+static void ff_segments(const mfs_ctx::FarField &F, std::vector<long long> &blocks, std::vector<int> &recs) {
+    const size_t n = F.seg_rec0_h.size();
+    blocks.resize(n);
+    recs.resize(n);
+    for (size_t sg = 0; sg < n; ++sg) {
+        recs[sg] = F.seg_rec1_h[sg] - F.seg_rec0_h[sg];
+        blocks[sg] = (recs[sg] + MFS_BS - 1) / MFS_BS;
     }
-    mfs_ctx::FarField::Plan pl;
-    const int P = ctx->P, nodes = F.nodes;
-    std::vector<long long> seg_blocks(P + nodes);
-    std::vector<int> seg_recs(P + nodes);
-    for (int sg = 0; sg < P + nodes; ++sg) {
-        seg_recs[sg] = F.seg_rec1_h[sg] - F.seg_rec0_h[sg];
-        seg_blocks[sg] = (seg_recs[sg] + MFS_BS - 1) / MFS_BS;
-    }
-    // upward: one group per node, tiles never span two nodes
-    std::vector<int> toff_up(nodes + 1), cuts_up(nodes + 1);
-    for (int n = 0; n <= nodes; ++n) {
-        toff_up[n] = n * FF_NC;
-        cuts_up[n] = n;
-    }
-    CKS(build_plan_lists(ctx, variant, 1, toff_up, P, cuts_up, seg_blocks, seg_recs,
-                         [&](int g0, int g1, std::vector<int> &segs) {
-                             for (int n = g0; n <= g1; ++n)
-                                 for (int q = F.tree.nodes[n].first; q < F.tree.nodes[n].first + F.tree.nodes[n].count;
-                                      ++q)
-                                     segs.push_back(q);
-                         },
-                         pl.up, &pl.lst_seg_up, &pl.lst_cum_up, pl.pairs_up));
-    // evaluation: groups are the bodies in tree order; tiles stay inside a suspension
-    std::vector<int> toff_ev(P + 1, 0);
-    for (int q = 0; q < P; ++q) {
-        const int b = F.tree.order[q];
-        toff_ev[q + 1] = toff_ev[q] + ((*F.tgt_off)[b + 1] - (*F.tgt_off)[b]);
-    }
-    std::vector<int> cuts_ev(ctx->S + 1);
-    for (int sp = 0; sp <= ctx->S; ++sp) cuts_ev[sp] = ctx->body_off[sp];
-    std::vector<int> suspension_of(P);
+}
+
+static std::vector<int> suspension_of_bodies(const mfs_ctx *ctx) {
+    std::vector<int> sus(ctx->P);
     for (int sp = 0; sp < ctx->S; ++sp)
-        for (int b = ctx->body_off[sp]; b < ctx->body_off[sp + 1]; ++b) suspension_of[b] = sp;
+        for (int b = ctx->body_off[sp]; b < ctx->body_off[sp + 1]; ++b) sus[b] = sp;
+    return sus;
+}
+
+using FFListPlan = mfs_ctx::FarField::ListPlan;
+
+// The plan of the upward sums for one pair-kernel variant: each node's check points against its
+// descendant bodies' proxy points (one group per node, tiles never span two nodes).
+mfs_status ff_up_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, FFListPlan **out) {
+    auto it = F.up.find(variant);
+    if (it == F.up.end()) {
+        FFListPlan lp;
+        const int nodes = F.nodes;
+        std::vector<long long> blocks;
+        std::vector<int> recs, toff(nodes + 1), cuts(nodes + 1);
+        ff_segments(F, blocks, recs);
+        for (int n = 0; n <= nodes; ++n) {
+            toff[n] = n * FF_NC;
+            cuts[n] = n;
+        }
+        CKS(build_plan_lists(ctx, variant, 1, toff, ctx->P, cuts, blocks, recs,
+                             [&](int g0, int g1, std::vector<int> &segs) {
+                                 for (int n = g0; n <= g1; ++n)
+                                     for (int q = F.tree.nodes[n].first;
+                                          q < F.tree.nodes[n].first + F.tree.nodes[n].count; ++q)
+                                         segs.push_back(q);
+                             },
+                             lp.p, &lp.seg, &lp.cum, lp.pairs));
+        it = F.up.emplace(variant, lp).first;
+    }
+    *out = &it->second;
+    return MFS_OK;
+}
+
+// The order-0 plan at the targets in tree order (the centre gradient's kernels): tiles stay inside a
+// suspension and may span bodies, self pairs left out.
+mfs_status ff_ev_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, FFListPlan **out) {
+    auto it = F.ev.find(variant);
+    if (it == F.ev.end()) {
+        FFListPlan lp;
+        const int P = ctx->P;
+        std::vector<long long> blocks;
+        std::vector<int> recs, toff(P + 1, 0), cuts(ctx->body_off.begin(), ctx->body_off.end()), tb;
+        ff_segments(F, blocks, recs);
+        for (int q = 0; q < P; ++q) {
+            const int b = F.tree.order[q];
+            toff[q + 1] = toff[q] + ((*F.tgt_off)[b + 1] - (*F.tgt_off)[b]);
+        }
+        const std::vector<int> sus = suspension_of_bodies(ctx);
+        CKS(build_plan_lists(ctx, variant, 0, toff, 0, cuts, blocks, recs,
+                             [&](int g0, int g1, std::vector<int> &segs) {
+                                 tb.clear();
+                                 for (int q = g0; q <= g1; ++q) tb.push_back(F.tree.order[q]);
+                                 ff_interaction_list(F.tree, F.tree.roots[sus[tb[0]]], tb, ctx->centres.data(),
+                                                     F.rtgt.data(), ctx->opt.farfield_separation, 1, segs);
+                             },
+                             lp.p, &lp.seg, &lp.cum, lp.pairs));
+        it = F.ev.emplace(variant, lp).first;
+    }
+    *out = &it->second;
+    return MFS_OK;
+}
+
+// The cells of `size` consecutive tree positions (cut at suspensions) and their lists.
+static const mfs_ctx::FarField::Cells &ff_cells(mfs_ctx *ctx, mfs_ctx::FarField &F, int size) {
+    auto it = F.cells.find(size);
+    if (it != F.cells.end()) return it->second;
+    mfs_ctx::FarField::Cells &c = F.cells[size];
+    c.cell_of.resize(ctx->P);
+    c.direct.resize(ctx->P);
     std::vector<int> tb;
-    CKS(build_plan_lists(ctx, variant, include_self, toff_ev, 0, cuts_ev, seg_blocks, seg_recs,
-                         [&](int g0, int g1, std::vector<int> &segs) {
-                             tb.clear();
-                             for (int q = g0; q <= g1; ++q) tb.push_back(F.tree.order[q]);
-                             ff_interaction_list(F.tree, F.tree.roots[suspension_of[tb[0]]], tb, ctx->centres.data(),
-                                                 F.rtgt.data(), ctx->opt.farfield_separation, !include_self, segs);
-                         },
-                         pl.ev, &pl.lst_seg_ev, &pl.lst_cum_ev, pl.pairs_ev));
-    pl.ev.include_self = include_self;
-    it = F.plans.emplace(key, pl).first;
+    std::vector<std::vector<int>> direct;
+    for (int sp = 0; sp < ctx->S; ++sp)
+        for (int q0 = ctx->body_off[sp]; q0 < ctx->body_off[sp + 1]; q0 += size) {
+            const int q1 = std::min(q0 + size, ctx->body_off[sp + 1]);
+            tb.clear();
+            for (int q = q0; q < q1; ++q) tb.push_back(F.tree.order[q]);
+            c.local.emplace_back();
+            ff_cell_lists(F.tree, F.tree.roots[sp], tb, ctx->centres.data(), F.rtgt.data(),
+                          ctx->opt.farfield_separation, (double)F.ntgt / ctx->P, c.local.back(), direct);
+            for (int q = q0; q < q1; ++q) {
+                c.cell_of[q] = (int)c.first.size();
+                c.direct[q].swap(direct[q - q0]);
+            }
+            c.first.push_back(q0);
+        }
+    c.first.push_back(ctx->P);
+    return c;
+}
+
+// Bodies whose local check points share one tile of the variant.
+static int ff_cell_size(int variant) {
+    int vc = 0;
+    return std::max(1, pair_variants(&vc)[variant].tile_targets / FF_LOC_NC);
+}
+
+// The plan of the sums at the bodies' local check points (one tile and one list per cell).
+mfs_status ff_loc_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, FFListPlan **out) {
+    auto it = F.loc.find(variant);
+    if (it == F.loc.end()) {
+        FFListPlan lp;
+        const int P = ctx->P;
+        const auto &cells = ff_cells(ctx, F, ff_cell_size(variant));
+        std::vector<long long> blocks;
+        std::vector<int> recs, toff(P + 1);
+        ff_segments(F, blocks, recs);
+        for (int q = 0; q <= P; ++q) toff[q] = q * FF_LOC_NC;
+        CKS(build_plan_lists(ctx, variant, 1, toff, 0, cells.first, blocks, recs,
+                             [&](int g0, int, std::vector<int> &segs) { segs = cells.local[cells.cell_of[g0]]; }, lp.p,
+                             &lp.seg, &lp.cum, lp.pairs));
+        it = F.loc.emplace(variant, lp).first;
+    }
+    *out = &it->second;
+    return MFS_OK;
+}
+
+// The plan of the final sums at the targets (tree order).  With local expansions every tile holds one
+// body's targets and that body's own list; without, tiles span bodies and share the list of them all.
+mfs_status ff_direct_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, int include_self, FFListPlan **out) {
+    const int key = variant * 2 + include_self;
+    auto it = F.direct.find(key);
+    if (it == F.direct.end()) {
+        FFListPlan lp;
+        const int P = ctx->P;
+        std::vector<long long> blocks;
+        std::vector<int> recs, toff(P + 1, 0), cuts, tb;
+        ff_segments(F, blocks, recs);
+        for (int q = 0; q < P; ++q) {
+            const int b = F.tree.order[q];
+            toff[q + 1] = toff[q] + ((*F.tgt_off)[b + 1] - (*F.tgt_off)[b]);
+        }
+        if (F.use_local) {
+            const auto &cells = ff_cells(ctx, F, ff_cell_size(variant));
+            for (int q = 0; q <= P; ++q) cuts.push_back(q);
+            CKS(build_plan_lists(ctx, variant, include_self, toff, 0, cuts, blocks, recs,
+                                 [&](int g0, int, std::vector<int> &segs) {
+                                     segs = cells.direct[g0];
+                                     if (include_self) segs.push_back(g0);
+                                 },
+                                 lp.p, &lp.seg, &lp.cum, lp.pairs));
+        } else {
+            cuts.assign(ctx->body_off.begin(), ctx->body_off.end());
+            const std::vector<int> sus = suspension_of_bodies(ctx);
+            CKS(build_plan_lists(ctx, variant, include_self, toff, 0, cuts, blocks, recs,
+                                 [&](int g0, int g1, std::vector<int> &segs) {
+                                     tb.clear();
+                                     for (int q = g0; q <= g1; ++q) tb.push_back(F.tree.order[q]);
+                                     ff_ordered_list(F.tree, F.tree.roots[sus[tb[0]]], tb, ctx->centres.data(),
+                                                     F.rtgt.data(), ctx->opt.farfield_separation, !include_self,
+                                                     segs);
+                                 },
+                                 lp.p, &lp.seg, &lp.cum, lp.pairs));
+        }
+        it = F.direct.emplace(key, lp).first;
+    }
     *out = &it->second;
     return MFS_OK;
 }
@@ -809,8 +946,10 @@ mfs_status ff_launch(mfs_ctx *ctx, int variant, const PairGeom &g, const PairWor
 }
 
 // The geometry of a far-field launch: the tree-ordered centres and the segments' record ranges.
-static PairGeom ff_geom(const mfs_ctx::FarField &F) {
+static PairGeom ff_geom(const mfs_ctx::FarField &F, const FFListPlan &lp) {
     PairGeom g;
+    g.lst_seg = lp.seg;
+    g.lst_cum = lp.cum;
     g.src = F.rec;
     g.src_off = nullptr;
     g.blk_off = nullptr;
@@ -820,11 +959,21 @@ static PairGeom ff_geom(const mfs_ctx::FarField &F) {
     return g;
 }
 
+// C [rows][D n] = A [rows][D k] B [D k][D n] in FP64 (the far field's fits; the context's D).
+static cudaError_t ff_fit(mfs_ctx *ctx, mfs_ctx::FarField &F, int rows, int n, int k, const double *A, const double *B,
+                          double *C, cudaStream_t st) {
+    const int D = ctx->D;
+    return gemm_rm64_splitk(rows, D * n, D * k, gemm_rm64_chunks(rows, D * n, D * k, ctx->sm_count), A, B,
+                            F.fit_chunks, C, st);
+}
+
 // The upward step of the treecode: the sources (records in the layout of `variant`, packed into
 // F.rec) summed at every node's check points over the node's descendant bodies, then the node's
 // equivalent strengths F.mu = (FP64 product with the pseudo-inverse) scaled by the radius.
-static mfs_status ff_upward(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const mfs_ctx::FarField::Plan *pl,
-                            const double *strength, int nrhs, cudaStream_t st) {
+static mfs_status ff_upward(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const double *strength, int nrhs,
+                            cudaStream_t st) {
+    FFListPlan *pl = nullptr;
+    CKS(ff_up_plan(ctx, F, variant, &pl));
     int vc = 0;
     const PairVariant *vv = pair_variants(&vc);
     const int D = ctx->D, nodes = F.nodes;
@@ -833,45 +982,68 @@ static mfs_status ff_upward(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, con
         return MFS_ERR_INVALID_ARG;
     }
     CK(pack_sources(D, nrhs, vv[variant].packed, F.src_pos, F.rec_pt, strength, F.nsrc, F.nrec, F.rec, st));
-    PairGeom g = ff_geom(F);
-    g.lst_seg = pl->lst_seg_up;
-    g.lst_cum = pl->lst_cum_up;
+    PairGeom g = ff_geom(F, *pl);
     g.tgt = F.chk_pos;
     g.ntargets = nodes * FF_NC;
-    const PairWork wu = work_of(pl->up);
+    const PairWork wu = work_of(pl->p);
     CKS(ff_launch(ctx, variant, g, wu, st));
     CK(pair_epilogue(D, nrhs, wu, nullptr, 0.0, 1.0, F.ucheck, nodes * FF_NC, st));
-    const int Sk = gemm_rm64_chunks(nrhs * nodes, D * FF_NE, D * FF_NC, ctx->sm_count);
-    CK(gemm_rm64_splitk(nrhs * nodes, D * FF_NE, D * FF_NC, Sk, F.ucheck, F.PinvT, F.fit_chunks, F.mu, st));
+    CK(ff_fit(ctx, F, nrhs * nodes, FF_NE, FF_NC, F.ucheck, F.PinvT, F.mu, st));
     CK(ff_scale(F.mu, F.re, nodes, D * FF_NE, nrhs, st));
     ctx->launches += 4;
     return MFS_OK;
 }
 
-// out = beta * base + scale * (pair sum of strengths) through the treecode: the upward step, the
-// equivalent strengths' records, then the evaluation over the interaction lists (results written
-// back in the caller's target order).
+// out = beta * base + scale * (pair sum of strengths) through the treecode, results in the caller's
+// target order: the upward step, the lower orders of the equivalent strengths, the far cells' field at
+// the bodies' local check points and the local sources that match it, then the sums at the targets.
+//
+// What bounds it is the number of pairs.  With order-0 lists at all targets a body of 2000 Type T
+// ellipsoids (839 targets) saw about 850 nodes x 196 points: 1.4e8 pairs, 96 % of a matvec's 162 ms.
+// Fewer points for distant nodes (FF_ORD_*) and 128 check points in place of the body's targets for
+// everything beyond FF_LOC_GAP leave 2.1e10 pairs per sum for 1000 ellipsoids (1.0e11 before), and a
+// matvec of 2000 takes 38.5 ms (163.7); the result is as close to the direct sum as before (white-noise
+// strengths, 1000 ellipsoids: 1.3e-7, 1.5e-7 before).
 mfs_status ff_pair_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const double *strength, double *out,
                          const double *base, double beta, double scale, int nrhs, int include_self, cudaStream_t st) {
-    mfs_ctx::FarField::Plan *pl = nullptr;
-    CKS(ff_get_plan(ctx, F, variant, include_self, &pl));
+    FFListPlan *pl = nullptr, *ll = nullptr;
+    CKS(ff_direct_plan(ctx, F, variant, include_self, &pl));
     int vc = 0;
     const PairVariant *vv = pair_variants(&vc);
-    const int D = ctx->D, nodes = F.nodes;
-    const int REC = pair_record_floats(D, nrhs, vv[variant].packed);
-    CKS(ff_upward(ctx, F, variant, pl, strength, nrhs, st));
-    CK(pack_sources(D, nrhs, vv[variant].packed, F.eq_pos, F.eq_pt, F.mu, nodes * FF_NE, nodes * FF_NE,
-                    F.rec + (size_t)F.nrec * REC, st));
-    PairGeom g = ff_geom(F);
-    g.lst_seg = pl->lst_seg_ev;
-    g.lst_cum = pl->lst_cum_ev;
+    const int D = ctx->D, nodes = F.nodes, P = ctx->P, layout = vv[variant].packed;
+    const size_t REC = pair_record_floats(D, nrhs, layout);
+    CKS(ff_upward(ctx, F, variant, strength, nrhs, st));
+    for (int o = 0; o < FF_NORD; ++o) {
+        const int n = FF_ORD_N[o];
+        if (o > 0)
+            CK(ff_fit(ctx, F, nrhs * nodes, n, FF_ORD_N[o - 1], o == 1 ? F.mu : F.ord_mu[o - 1], F.ordT[o],
+                      F.ord_mu[o], st));
+        CK(pack_sources(D, nrhs, layout, o == 0 ? F.eq_pos : F.ord_pos[o], F.eq_pt, o == 0 ? F.mu : F.ord_mu[o],
+                        nodes * n, nodes * n, F.rec + F.ord_rec[o] * REC, st));
+    }
+    ctx->launches += 2 * FF_NORD - 1;
+    if (F.use_local) {
+        CKS(ff_loc_plan(ctx, F, variant, &ll));
+        PairGeom g = ff_geom(F, *ll);
+        g.tgt = F.lchk_pos;
+        g.ntargets = P * FF_LOC_NC;
+        const PairWork wl = work_of(ll->p);
+        CKS(ff_launch(ctx, variant, g, wl, st));
+        CK(pair_epilogue(D, nrhs, wl, nullptr, 0.0, 1.0, F.ulocal, P * FF_LOC_NC, st));
+        CK(ff_fit(ctx, F, nrhs * P, FF_LOC_N, FF_LOC_NC, F.ulocal, F.locT, F.nu, st));
+        CK(ff_scale(F.nu, F.rloc, P, D * FF_LOC_N, nrhs, st));
+        CK(pack_sources(D, nrhs, layout, F.loc_pos, F.eq_pt, F.nu, P * FF_LOC_N, P * FF_LOC_N, F.rec + F.loc_rec * REC,
+                        st));
+        ctx->launches += 4;
+    }
+    PairGeom g = ff_geom(F, *pl);
     g.tgt = F.tgt;
     g.ntargets = F.ntgt;
-    PairWork we = work_of(pl->ev);
+    PairWork we = work_of(pl->p);
     we.tperm = F.tperm;
     CKS(ff_launch(ctx, variant, g, we, st));
     CK(pair_epilogue(D, nrhs, we, base, beta, scale, out, F.ntgt, st));
-    ctx->launches += 3;
+    ctx->launches += 2;
     return MFS_OK;
 }
 
@@ -895,10 +1067,9 @@ static __global__ void ff_gather_weights_kernel(const double *v, const int *perm
 mfs_status ff_grad_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int gv, const double *sigma, const double *tw, int nrhs,
                          double *out, cudaStream_t st) {
     const int fv = fp32_variant(ctx, 3, nrhs);  // the upward sums: the forward pair kernel
-    mfs_ctx::FarField::Plan *pu = nullptr, *pg = nullptr;
-    CKS(ff_get_plan(ctx, F, fv, 1, &pu));
-    CKS(ff_get_plan(ctx, F, gv, 0, &pg));
-    CKS(ff_upward(ctx, F, fv, pu, sigma, nrhs, st));
+    FFListPlan *pg = nullptr;
+    CKS(ff_ev_plan(ctx, F, gv, &pg));
+    CKS(ff_upward(ctx, F, fv, sigma, nrhs, st));
     // records of the gradient kernel (plain layout): the sources, then the equivalent points
     const int REC = pair_record_floats(3, nrhs, 0), nodes = F.nodes;
     CK(pack_sources(3, nrhs, 0, F.src_pos, F.rec_pt, sigma, F.nsrc, F.nrec, F.rec, st));
@@ -907,13 +1078,11 @@ mfs_status ff_grad_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int gv, const doubl
     if (!F.wt) CK(ctx->alloc(&F.wt, (size_t)ctx->opt.max_rhs * F.ntgt * 3));
     ff_gather_weights_kernel<<<1024, 256, 0, st>>>(tw, F.tperm, F.ntgt, nrhs, F.wt);
     CK(cudaGetLastError());
-    PairGeom g = ff_geom(F);
-    g.lst_seg = pg->lst_seg_ev;
-    g.lst_cum = pg->lst_cum_ev;
+    PairGeom g = ff_geom(F, *pg);
     g.tgt = F.tgt;
     g.ntargets = F.ntgt;
     g.tgt_w = F.wt;
-    PairWork we = work_of(pg->ev);
+    PairWork we = work_of(pg->p);
     we.tperm = F.tperm;
     we.src_grad = nullptr;  // segments are bodies and nodes here: no per-source-body reduction
     CKS(ff_launch(ctx, gv, g, we, st));
@@ -1743,93 +1912,144 @@ static void unit_fibonacci(int n, std::vector<double> &p) {
     }
 }
 
-// The transposed pseudo-inverse of the check <- equivalent map on the unit sphere (raw kernel: 1/r or
-// (I + r r^T / r^2) / r), FP64, truncated at 1e-12 of the largest singular value; least squares
-// (FF_NC > FF_NE).  It depends on the kernel only, so a context computes it once.
-static mfs_status ff_unit_pinv(mfs_ctx *ctx, mfs_ctx::FarField &F, const std::vector<double> &ue,
-                               const std::vector<double> &uc, cudaStream_t st) {
-    const int D = ctx->D;
-    const int m = D * FF_NC, n = D * FF_NE;
-    std::vector<double> A((size_t)m * n);
-    for (int i = 0; i < FF_NC; ++i)
-        for (int j = 0; j < FF_NE; ++j) {
+// The raw kernel (1/r or (I + r r^T / r^2) / r) between two scaled point sets, column-major
+// [D nt][D ns] (read row-major: its transpose).
+static std::vector<double> ff_map(int D, const std::vector<double> &tgt, double rt, const std::vector<double> &src,
+                                  double rs) {
+    const int nt = (int)tgt.size() / 3, ns = (int)src.size() / 3;
+    const int m = D * nt;
+    std::vector<double> A((size_t)m * D * ns);
+    for (int j = 0; j < ns; ++j)
+        for (int i = 0; i < nt; ++i) {
             double r[3], r2 = 0.0;
             for (int a = 0; a < 3; ++a) {
-                r[a] = FF_CHECK * uc[3 * i + a] - ue[3 * j + a];
+                r[a] = rt * tgt[3 * i + a] - rs * src[3 * j + a];
                 r2 += r[a] * r[a];
             }
             const double ri = 1.0 / std::sqrt(r2);
-            for (int a = 0; a < D; ++a)
-                for (int b = 0; b < D; ++b) {
-                    const double v = D == 1 ? ri : ((a == b ? ri : 0.0) + r[a] * r[b] * ri * ri * ri);
-                    A[(size_t)(D * j + b) * m + (D * i + a)] = v;
-                }
+            for (int b = 0; b < D; ++b)
+                for (int a = 0; a < D; ++a)
+                    A[(size_t)(D * j + b) * m + (D * i + a)] =
+                        D == 1 ? ri : ((a == b ? ri : 0.0) + r[a] * r[b] * ri * ri * ri);
         }
+    return A;
+}
+
+// V[j][k] *= 1 / s_k over the singular values kept (s_k > trunc s_0), 0 for the others.
+static __global__ void ff_scale_columns_kernel(double *V, const double *s, int n, double trunc) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n * n) return;
+    const int k = i % n;
+    V[i] *= s[k] > trunc * s[0] ? 1.0 / s[k] : 0.0;
+}
+
+// The transposed pseudo-inverse [m][n] (device, row-major, owned by the caller through ctx->alloc) of a
+// column-major m x n matrix, m >= n, in FP64, truncated at `trunc` of the largest singular value.
+static mfs_status ff_pinvT(mfs_ctx *ctx, cusolverDnHandle_t solver, int m, int n, const std::vector<double> &A,
+                           double trunc, double **out, cudaStream_t st) {
+    double *A_d = nullptr, *U_d = nullptr, *S_d = nullptr, *VT_d = nullptr, *work = nullptr, *P_d = nullptr;
+    int *info_d = nullptr, lwork = 0, info_h = 0;
+    double s0 = 0.0;
+    CK(ctx->alloc(out, (size_t)m * n));
+    bool ok = cudaMalloc(&A_d, sizeof(double) * A.size()) == cudaSuccess &&
+              cudaMalloc(&U_d, sizeof(double) * (size_t)m * n) == cudaSuccess &&
+              cudaMalloc(&S_d, sizeof(double) * n) == cudaSuccess &&
+              cudaMalloc(&VT_d, sizeof(double) * (size_t)n * n) == cudaSuccess &&
+              cudaMalloc(&P_d, sizeof(double) * (size_t)n * m) == cudaSuccess &&
+              cudaMalloc(&info_d, sizeof(int)) == cudaSuccess &&
+              cudaMemcpyAsync(A_d, A.data(), sizeof(double) * A.size(), cudaMemcpyHostToDevice, st) == cudaSuccess &&
+              cusolverDnDgesvd_bufferSize(solver, m, n, &lwork) == CUSOLVER_STATUS_SUCCESS &&
+              cudaMalloc(&work, sizeof(double) * std::max(lwork, 1)) == cudaSuccess;
+    signed char jobu = 'S', jobvt = 'S';
+    ok = ok && cusolverDnDgesvd(solver, jobu, jobvt, m, n, A_d, m, S_d, U_d, m, VT_d, n, work, lwork, nullptr,
+                                info_d) == CUSOLVER_STATUS_SUCCESS;
+    if (ok) {  // pinv [n][m] = (V S^+) U^T: column-major V^T read row-major is V, column-major U is U^T
+        ff_scale_columns_kernel<<<(n * n + 255) / 256, 256, 0, st>>>(VT_d, S_d, n, trunc);
+        ok = gemm_rm64_splitk(n, m, n, 1, VT_d, U_d, nullptr, P_d, st) == cudaSuccess;
+        transpose64_kernel<<<1024, 256, 0, st>>>(P_d, n, m, *out);
+        ok = ok && cudaGetLastError() == cudaSuccess &&
+             cudaMemcpyAsync(&info_h, info_d, sizeof(int), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+             cudaMemcpyAsync(&s0, S_d, sizeof(double), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+             cudaStreamSynchronize(st) == cudaSuccess && info_h == 0;
+    }
+    cudaFree(A_d); cudaFree(U_d); cudaFree(S_d); cudaFree(VT_d); cudaFree(P_d); cudaFree(work); cudaFree(info_d);
+    if (!ok || !(s0 > 0.0)) {
+        cudaGetLastError();
+        ctx->last_error = "far field: SVD of a check <- equivalent map failed";
+        return MFS_ERR_CUDA;
+    }
+    return MFS_OK;
+}
+
+// The matrices on the unit sphere: check field -> order-0 strengths (PinvT), each order's strengths ->
+// the next lower order's (ordT), local check field -> local sources (locT).  They depend on the kernel
+// only, so a context computes them once.
+static mfs_status ff_unit_matrices(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStream_t st) {
+    const int D = ctx->D;
     cusolverDnHandle_t solver = nullptr;
     if (cusolverDnCreate(&solver) != CUSOLVER_STATUS_SUCCESS) {
         ctx->last_error = "cusolverDnCreate failed";
         return MFS_ERR_CUDA;
     }
     cusolverDnSetStream(solver, st);
-    double *A_d = nullptr, *U_d = nullptr, *S_d = nullptr, *VT_d = nullptr, *work = nullptr;
-    int *info_d = nullptr, lwork = 0, info_h = 0;
-    bool ok = cudaMalloc(&A_d, sizeof(double) * A.size()) == cudaSuccess &&
-              cudaMalloc(&U_d, sizeof(double) * (size_t)m * n) == cudaSuccess &&
-              cudaMalloc(&S_d, sizeof(double) * n) == cudaSuccess &&
-              cudaMalloc(&VT_d, sizeof(double) * (size_t)n * n) == cudaSuccess &&
-              cudaMalloc(&info_d, sizeof(int)) == cudaSuccess &&
-              cudaMemcpy(A_d, A.data(), sizeof(double) * A.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
-              cusolverDnDgesvd_bufferSize(solver, m, n, &lwork) == CUSOLVER_STATUS_SUCCESS &&
-              cudaMalloc(&work, sizeof(double) * std::max(lwork, 1)) == cudaSuccess;
-    signed char jobu = 'S', jobvt = 'S';
-    ok = ok && cusolverDnDgesvd(solver, jobu, jobvt, m, n, A_d, m, S_d, U_d, m, VT_d, n, work, lwork, nullptr,
-                                info_d) == CUSOLVER_STATUS_SUCCESS;
-    std::vector<double> U((size_t)m * n), S(n), VT((size_t)n * n);
-    ok = ok && cudaMemcpy(&info_h, info_d, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess && info_h == 0 &&
-         cudaMemcpy(U.data(), U_d, sizeof(double) * U.size(), cudaMemcpyDeviceToHost) == cudaSuccess &&
-         cudaMemcpy(S.data(), S_d, sizeof(double) * n, cudaMemcpyDeviceToHost) == cudaSuccess &&
-         cudaMemcpy(VT.data(), VT_d, sizeof(double) * VT.size(), cudaMemcpyDeviceToHost) == cudaSuccess;
-    cudaFree(A_d); cudaFree(U_d); cudaFree(S_d); cudaFree(VT_d); cudaFree(work); cudaFree(info_d);
-    cusolverDnDestroy(solver);
-    if (!ok || !(S[0] > 0.0)) {
-        cudaGetLastError();
-        ctx->last_error = "far field: SVD of the check <- equivalent map failed";
-        return MFS_ERR_CUDA;
-    }
-    // PinvT[i][j] = sum_k U[i][k] / s_k VT[k][j] (row-major m x n) over the kept singular values
-    std::vector<double> PinvT((size_t)m * n, 0.0), row(n);
-    for (int k = 0; k < n; ++k) {
-        if (!(S[k] > 1e-12 * S[0])) continue;
-        const double inv = 1.0 / S[k];
-        for (int j = 0; j < n; ++j) row[j] = inv * VT[(size_t)j * n + k];
-        for (int i = 0; i < m; ++i) {
-            const double u = U[(size_t)k * m + i];
-            double *o = &PinvT[(size_t)i * n];
-            for (int j = 0; j < n; ++j) o[j] += u * row[j];
+    auto build = [&]() -> mfs_status {
+        std::vector<double> e[FF_NORD], c;
+        for (int o = 0; o < FF_NORD; ++o) {
+            unit_fibonacci(FF_ORD_N[o], e[o]);
+            unit_fibonacci(FF_ORD_NC[o], c);
+            const int m = D * FF_ORD_NC[o], n = D * FF_ORD_N[o];
+            double *pinvT = nullptr;
+            CKS(ff_pinvT(ctx, solver, m, n, ff_map(D, c, FF_ORD_CHECK[o], e[o], 1.0), FF_ORD_TRUNC[o], &pinvT, st));
+            if (o == 0) {
+                F.PinvT = pinvT;
+                continue;
+            }
+            // ordT = (previous order's field at this order's check points)^T pinvT
+            const int np = D * FF_ORD_N[o - 1];
+            const std::vector<double> G = ff_map(D, c, FF_ORD_CHECK[o], e[o - 1], 1.0);
+            double *G_d = nullptr;
+            CK(ctx->alloc(&G_d, G.size()));
+            CK(ctx->alloc(&F.ordT[o], (size_t)np * n));
+            CK(cudaMemcpyAsync(G_d, G.data(), sizeof(double) * G.size(), cudaMemcpyHostToDevice, st));
+            CK(gemm_rm64_splitk(np, n, m, 1, G_d, pinvT, nullptr, F.ordT[o], st));
+            CK(cudaStreamSynchronize(st));
+            ctx->release(G_d);
+            ctx->release(pinvT);
         }
-    }
-    CK(ctx->alloc(&F.PinvT, PinvT.size()));
-    CK(cudaMemcpy(F.PinvT, PinvT.data(), sizeof(double) * PinvT.size(), cudaMemcpyHostToDevice));
-    return MFS_OK;
+        std::vector<double> l;
+        unit_fibonacci(FF_LOC_N, l);
+        unit_fibonacci(FF_LOC_NC, c);
+        return ff_pinvT(ctx, solver, D * FF_LOC_NC, D * FF_LOC_N, ff_map(D, c, FF_LOC_CHECK, l, FF_LOC_EQ),
+                        FF_LOC_TRUNC, &F.locT, st);
+    };
+    const mfs_status rc = build();
+    cusolverDnDestroy(solver);
+    return rc;
 }
 
 // Frees the far-field structures that depend on the body centres (all but the pseudo-inverse) and
 // drops the captured graphs that hold their addresses.
 static void ff_release_geometry(mfs_ctx *ctx, mfs_ctx::FarField &F) {
     ctx->drop_graphs();
-    for (auto &kv : F.plans) {
-        auto &pl = kv.second;
-        for (PairPlan *pp : {&pl.up, &pl.ev}) {
-            ctx->release(pp->tiles);
-            ctx->release(pp->partial);
-            ctx->release(pp->direct);
+    for (auto *plans : {&F.up, &F.ev, &F.loc, &F.direct}) {
+        for (auto &kv : *plans) {
+            release_plan(ctx, kv.second.p);
+            ctx->release(kv.second.seg);
+            ctx->release(kv.second.cum);
         }
-        ctx->release(pl.lst_seg_up);
-        ctx->release(pl.lst_cum_up);
-        ctx->release(pl.lst_seg_ev);
-        ctx->release(pl.lst_cum_ev);
+        plans->clear();
     }
-    F.plans.clear();
+    F.cells.clear();
+    for (int o = 1; o < FF_NORD; ++o) {
+        ctx->release(F.ord_pos[o]);
+        ctx->release(F.ord_mu[o]);
+        F.ord_pos[o] = nullptr;
+        F.ord_mu[o] = nullptr;
+    }
+    for (void *p : {(void *)F.rloc, (void *)F.loc_pos, (void *)F.lchk_pos, (void *)F.ulocal, (void *)F.nu})
+        ctx->release(p);
+    F.rloc = F.ulocal = F.nu = nullptr;
+    F.loc_pos = F.lchk_pos = nullptr;
     ctx->release(F.centres);
     ctx->release(F.re);
     ctx->release(F.eq_pos);
@@ -1877,34 +2097,52 @@ static mfs_status ff_setup(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStream_t st) 
     unit_fibonacci(FF_NC, uc);
     if (!F.PinvT) {  // independent of the centres (kept across moves) and of the roles (shared)
         const auto &other = &F == &ctx->ff ? ctx->ffT : ctx->ff;
-        if (other.PinvT) F.PinvT = other.PinvT;
-        else CKS(ff_unit_pinv(ctx, F, ue, uc, st));
+        if (other.PinvT) {
+            F.PinvT = other.PinvT;
+            F.locT = other.locT;
+            for (int o = 1; o < FF_NORD; ++o) F.ordT[o] = other.ordT[o];
+        } else {
+            CKS(ff_unit_matrices(ctx, F, st));
+        }
     }
+    // Local expansions where a body has clearly more targets than check points: with fewer, the check
+    // sums and the match cost more than the lower orders at the targets themselves (ff_cell_lists then
+    // weighs each cell).
+    F.use_local = F.ntgt >= 160LL * P;
+    for (int k = 0; k < P; ++k) F.use_local = F.use_local && F.rtgt[k] > 0.0;
     // tree-ordered geometry and segments: proxy segment q (tree position) = body order[q], node segment
-    // P + node = its equivalent points
-    std::vector<double> cen(3 * (size_t)(P + nodes)), re(nodes);
-    for (int q = 0; q < P; ++q)
-        for (int a = 0; a < 3; ++a) cen[3 * q + a] = ctx->centres[3 * F.tree.order[q] + a];
+    // P + o nodes + node = order o of its equivalent points, local segment P + FF_NORD nodes + q
+    const int nseg = P + FF_NORD * nodes + (F.use_local ? P : 0);
+    std::vector<double> cen(3 * (size_t)nseg), re(nodes), rloc(P);
+    for (int q = 0; q < P; ++q) {
+        rloc[q] = F.rtgt[F.tree.order[q]];
+        for (int a = 0; a < 3; ++a) {
+            cen[3 * (size_t)q + a] = ctx->centres[3 * F.tree.order[q] + a];
+            if (F.use_local) cen[3 * (size_t)(P + FF_NORD * nodes + q) + a] = ctx->centres[3 * F.tree.order[q] + a];
+        }
+    }
     for (int nd = 0; nd < nodes; ++nd) {
-        for (int a = 0; a < 3; ++a) cen[3 * (P + nd) + a] = F.tree.nodes[nd].c[a];
+        for (int o = 0; o < FF_NORD; ++o)
+            for (int a = 0; a < 3; ++a) cen[3 * (size_t)(P + o * nodes + nd) + a] = F.tree.nodes[nd].c[a];
         re[nd] = F.tree.nodes[nd].re;
     }
-    std::vector<float4> eq((size_t)nodes * FF_NE), chk((size_t)nodes * FF_NC);
-    std::vector<int> eq_pt((size_t)nodes * FF_NE);
-    for (int nd = 0; nd < nodes; ++nd) {
-        float w;
-        const int id = P + nd;
-        std::memcpy(&w, &id, sizeof(float));
-        for (int e = 0; e < FF_NE; ++e) {
-            eq[(size_t)nd * FF_NE + e] = make_float4((float)(re[nd] * ue[3 * e]), (float)(re[nd] * ue[3 * e + 1]),
-                                                     (float)(re[nd] * ue[3 * e + 2]), 0.f);
-            eq_pt[(size_t)nd * FF_NE + e] = nd * FF_NE + e;
+    // unit points scaled by r[i] about their centres, w = id0 + i (int bits)
+    auto scaled = [](const std::vector<double> &unit, double f, const std::vector<double> &r, int id0) {
+        const int n = (int)unit.size() / 3;
+        std::vector<float4> out(r.size() * n);
+        for (size_t i = 0; i < r.size(); ++i) {
+            float w;
+            const int id = id0 + (int)i;
+            std::memcpy(&w, &id, sizeof(float));
+            for (int e = 0; e < n; ++e)
+                out[i * n + e] = make_float4((float)(f * r[i] * unit[3 * e]), (float)(f * r[i] * unit[3 * e + 1]),
+                                             (float)(f * r[i] * unit[3 * e + 2]), w);
         }
-        for (int c = 0; c < FF_NC; ++c)
-            chk[(size_t)nd * FF_NC + c] =
-                make_float4((float)(FF_CHECK * re[nd] * uc[3 * c]), (float)(FF_CHECK * re[nd] * uc[3 * c + 1]),
-                            (float)(FF_CHECK * re[nd] * uc[3 * c + 2]), w);
-    }
+        return out;
+    };
+    const std::vector<float4> eq = scaled(ue, 1.0, re, 0), chk = scaled(uc, FF_CHECK, re, P);
+    std::vector<int> eq_pt((size_t)nodes * FF_NE);  // identity (packing); long enough for every order
+    for (size_t i = 0; i < eq_pt.size(); ++i) eq_pt[i] = (int)i;
     std::vector<float4> tpos(F.ntgt), tff(F.ntgt);
     CK(cudaMemcpy(tpos.data(), F.tgt_pos, sizeof(float4) * F.ntgt, cudaMemcpyDeviceToHost));
     std::vector<int> tperm(F.ntgt);
@@ -1918,16 +2156,29 @@ static mfs_status ff_setup(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStream_t st) 
             tperm[t] = i;
         }
     }
-    F.seg_rec0_h.resize(P + nodes);
-    F.seg_rec1_h.resize(P + nodes);
+    F.seg_rec0_h.resize(nseg);
+    F.seg_rec1_h.resize(nseg);
     for (int q = 0; q < P; ++q) {
         const int b = F.tree.order[q];
         F.seg_rec0_h[q] = (*F.rec_off)[b];
         F.seg_rec1_h[q] = (*F.rec_off)[b + 1];  // padded to a multiple of 4 (zero-strength padding records)
     }
-    for (int nd = 0; nd < nodes; ++nd) {
-        F.seg_rec0_h[P + nd] = F.nrec + nd * FF_NE;
-        F.seg_rec1_h[P + nd] = F.nrec + (nd + 1) * FF_NE;
+    size_t nrec_all = F.nrec;
+    for (int o = 0; o < FF_NORD; ++o) {
+        F.ord_rec[o] = nrec_all;
+        for (int nd = 0; nd < nodes; ++nd) {
+            F.seg_rec0_h[P + o * nodes + nd] = (int)nrec_all + nd * FF_ORD_N[o];
+            F.seg_rec1_h[P + o * nodes + nd] = (int)nrec_all + (nd + 1) * FF_ORD_N[o];
+        }
+        nrec_all += (size_t)nodes * FF_ORD_N[o];
+    }
+    F.loc_rec = nrec_all;
+    if (F.use_local) {
+        for (int q = 0; q < P; ++q) {
+            F.seg_rec0_h[P + FF_NORD * nodes + q] = (int)nrec_all + q * FF_LOC_N;
+            F.seg_rec1_h[P + FF_NORD * nodes + q] = (int)nrec_all + (q + 1) * FF_LOC_N;
+        }
+        nrec_all += (size_t)P * FF_LOC_N;
     }
     const int R = ctx->opt.max_rhs;
     F.rec_floats = std::max(pair_record_floats(D, R, 0), pair_record_floats(D, R, 1));  // plain or f32x2 policies
@@ -1940,14 +2191,41 @@ static mfs_status ff_setup(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStream_t st) 
     CK(ctx->alloc(&F.tperm, tperm.size()));
     CK(ctx->alloc(&F.seg_rec0, F.seg_rec0_h.size()));
     CK(ctx->alloc(&F.seg_rec1, F.seg_rec1_h.size()));
-    CK(ctx->alloc(&F.rec, (size_t)(F.nrec + (size_t)nodes * FF_NE) * F.rec_floats));
+    CK(ctx->alloc(&F.rec, nrec_all * F.rec_floats));
+    auto upload4 = [&](float4 **dst, const std::vector<float4> &v) -> cudaError_t {
+        const cudaError_t e = ctx->alloc(dst, v.size());
+        return e != cudaSuccess ? e
+                                : cudaMemcpy(*dst, v.data(), sizeof(float4) * v.size(), cudaMemcpyHostToDevice);
+    };
+    for (int o = 1; o < FF_NORD; ++o) {
+        std::vector<double> u;
+        unit_fibonacci(FF_ORD_N[o], u);
+        CK(upload4(&F.ord_pos[o], scaled(u, 1.0, re, 0)));
+        CK(ctx->alloc(&F.ord_mu[o], (size_t)R * nodes * FF_ORD_N[o] * D));
+    }
+    if (F.use_local) {
+        std::vector<double> u;
+        unit_fibonacci(FF_LOC_N, u);
+        CK(upload4(&F.loc_pos, scaled(u, FF_LOC_EQ, rloc, 0)));
+        unit_fibonacci(FF_LOC_NC, u);
+        CK(upload4(&F.lchk_pos, scaled(u, FF_LOC_CHECK, rloc, 0)));
+        CK(ctx->alloc(&F.rloc, rloc.size()));
+        CK(cudaMemcpy(F.rloc, rloc.data(), sizeof(double) * P, cudaMemcpyHostToDevice));
+        CK(ctx->alloc(&F.ulocal, (size_t)R * P * FF_LOC_NC * D));
+        CK(ctx->alloc(&F.nu, (size_t)R * P * FF_LOC_N * D));
+    }
     CK(ctx->alloc(&F.ucheck, (size_t)R * nodes * FF_NC * D));
     CK(ctx->alloc(&F.mu, (size_t)R * nodes * FF_NE * D));
     {
         size_t chunk_doubles = 1;
+        auto fit_size = [&](int rows, int n, int k) {
+            const int S = gemm_rm64_chunks(rows, D * n, D * k, ctx->sm_count);
+            if (S > 1) chunk_doubles = std::max(chunk_doubles, (size_t)S * rows * n * D);
+        };
         for (int h = 1; h <= R; ++h) {
-            const int S = gemm_rm64_chunks(h * nodes, D * FF_NE, D * FF_NC, ctx->sm_count);
-            if (S > 1) chunk_doubles = std::max(chunk_doubles, (size_t)S * h * nodes * FF_NE * D);
+            fit_size(h * nodes, FF_NE, FF_NC);
+            for (int o = 1; o < FF_NORD; ++o) fit_size(h * nodes, FF_ORD_N[o], FF_ORD_N[o - 1]);
+            fit_size(h * P, FF_LOC_N, FF_LOC_NC);
         }
         CK(ctx->alloc(&F.fit_chunks, chunk_doubles));
     }
@@ -1960,7 +2238,7 @@ static mfs_status ff_setup(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStream_t st) 
     CK(cudaMemcpy(F.tperm, tperm.data(), sizeof(int) * tperm.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(F.seg_rec0, F.seg_rec0_h.data(), sizeof(int) * F.seg_rec0_h.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(F.seg_rec1, F.seg_rec1_h.data(), sizeof(int) * F.seg_rec1_h.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemset(F.rec, 0, sizeof(float) * (size_t)(F.nrec + (size_t)nodes * FF_NE) * F.rec_floats));
+    CK(cudaMemset(F.rec, 0, sizeof(float) * nrec_all * F.rec_floats));
     F.ready = true;
     return MFS_OK;
 }
@@ -2492,8 +2770,12 @@ static mfs_status finish_info(mfs_ctx *ctx, mfs_solve_info *info, const SolveSta
         info->pairs_evaluated = info->pairs;
         if (ctx->ff.ready) {  // what the treecode's launches evaluated for the same sums
             auto evaluated = [&](int include_self) {
-                const auto it = ctx->ff.plans.find(forward_variant(ctx, nrhs) * 2 + include_self);
-                return it == ctx->ff.plans.end() ? 0.0 : it->second.pairs_up + it->second.pairs_ev;
+                const int v = forward_variant(ctx, nrhs);
+                const auto d = ctx->ff.direct.find(v * 2 + include_self);
+                const auto u = ctx->ff.up.find(v), l = ctx->ff.loc.find(v);
+                return (d == ctx->ff.direct.end() ? 0.0 : d->second.pairs) +
+                       (u == ctx->ff.up.end() ? 0.0 : u->second.pairs) +
+                       (l == ctx->ff.loc.end() ? 0.0 : l->second.pairs);
             };
             info->pairs_evaluated = evaluated(0) * ss.matvecs + (rhs_pairs ? evaluated(1) : 0.0);
         }
@@ -3079,9 +3361,7 @@ static mfs_status ff_points(mfs_ctx *ctx, int variant, const EvalTargets &et, co
     int vc = 0;
     const PairVariant *vv = pair_variants(&vc);
     const int fv = fp32_variant(ctx, D, nrhs);
-    mfs_ctx::FarField::Plan *pu = nullptr;
-    CKS(ff_get_plan(ctx, F, fv, 1, &pu));
-    CKS(ff_upward(ctx, F, fv, pu, ctx->lam_d, nrhs, st));
+    CKS(ff_upward(ctx, F, fv, ctx->lam_d, nrhs, st));
     const int layout = vv[variant].packed, REC = pair_record_floats(D, nrhs, layout);
     if (REC > F.rec_floats) {
         ctx->last_error = "far field: record layout larger than its buffer";
@@ -3110,22 +3390,16 @@ static mfs_status ff_points(mfs_ctx *ctx, int variant, const EvalTargets &et, co
         }
         toff[q + 1] = t;
     }
-    std::vector<long long> seg_blocks(P + nodes);
-    std::vector<int> seg_recs(P + nodes);
-    for (int sg = 0; sg < P + nodes; ++sg) {
-        seg_recs[sg] = F.seg_rec1_h[sg] - F.seg_rec0_h[sg];
-        seg_blocks[sg] = (seg_recs[sg] + MFS_BS - 1) / MFS_BS;
-    }
-    std::vector<int> cuts(ctx->S + 1), suspension_of(P), tb;
-    for (int sp = 0; sp <= ctx->S; ++sp) cuts[sp] = ctx->body_off[sp];
-    for (int sp = 0; sp < ctx->S; ++sp)
-        for (int b = ctx->body_off[sp]; b < ctx->body_off[sp + 1]; ++b) suspension_of[b] = sp;
-    PairPlan plan;
-    int *lst_seg = nullptr, *perm_d = nullptr;
-    long long *lst_cum = nullptr;
+    std::vector<long long> seg_blocks;
+    std::vector<int> seg_recs;
+    ff_segments(F, seg_blocks, seg_recs);
+    std::vector<int> cuts(ctx->body_off.begin(), ctx->body_off.end()), tb;
+    const std::vector<int> suspension_of = suspension_of_bodies(ctx);
+    FFListPlan lp;
+    PairPlan &plan = lp.p;
+    int *perm_d = nullptr;
     float4 *tt_d = nullptr;
     float *tw_d = nullptr;
-    double pairs = 0.0;
     mfs_status rc = build_plan_lists(
         ctx, variant, 1, toff, 0, cuts, seg_blocks, seg_recs,
         [&](int g0, int g1, std::vector<int> &segs) {
@@ -3134,7 +3408,7 @@ static mfs_status ff_points(mfs_ctx *ctx, int variant, const EvalTargets &et, co
             ff_interaction_list(F.tree, F.tree.roots[suspension_of[tb[0]]], tb, ctx->centres.data(), rad.data(),
                                 ctx->opt.farfield_separation, 0, segs);
         },
-        plan, &lst_seg, &lst_cum, pairs);
+        plan, &lp.seg, &lp.cum, lp.pairs);
     if (rc == MFS_OK) {
         rc = [&]() -> mfs_status {
             CK(ctx->alloc(&tt_d, np));
@@ -3145,9 +3419,7 @@ static mfs_status ff_points(mfs_ctx *ctx, int variant, const EvalTargets &et, co
                 CK(ctx->alloc(&tw_d, tw.size()));
                 CK(cudaMemcpyAsync(tw_d, tw.data(), sizeof(float) * tw.size(), cudaMemcpyHostToDevice, st));
             }
-            PairGeom g = ff_geom(F);
-            g.lst_seg = lst_seg;
-            g.lst_cum = lst_cum;
+            PairGeom g = ff_geom(F, lp);
             g.tgt = tt_d;
             g.ntargets = np;
             g.tgt_w = tw_d;
@@ -3162,8 +3434,8 @@ static mfs_status ff_points(mfs_ctx *ctx, int variant, const EvalTargets &et, co
     ctx->release(tt_d);
     ctx->release(tw_d);
     ctx->release(perm_d);
-    ctx->release(lst_seg);
-    ctx->release(lst_cum);
+    ctx->release(lp.seg);
+    ctx->release(lp.cum);
     if (plan.tiles) release_plan(ctx, plan);
     return rc;
 }

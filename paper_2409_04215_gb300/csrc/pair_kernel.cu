@@ -88,6 +88,7 @@ struct Stage {
     int nrec;      // records in this stage (multiple of 4)
     long long u;   // global unit index of the first block
     int nblk;      // blocks in this stage
+    int entry;     // interaction lists: the list entry
 };
 
 // Last tile with u0 <= u (tiles are contiguous in unit space; empty tiles come before the tile they abut).
@@ -100,9 +101,11 @@ __device__ __forceinline__ int tile_of_unit(const PairTile *tiles, int ntiles, l
     return lo;
 }
 
-// The stage that starts at global unit u (u < uend), at most max_blocks blocks long.
+// The stage that starts at global unit u (u < uend), at most max_blocks blocks long.  hint_entry: with
+// interaction lists, the entry of the stage before (the one that ends at u), or -1; the next entry is
+// then the same or the following one, where a search is a chain of about ten dependent loads per stage.
 __device__ __forceinline__ Stage make_stage(const PairTile *tiles, int ntiles, const PairGeom &geo, long long u,
-                                            long long uend, int max_blocks, int hint_tile) {
+                                            long long uend, int max_blocks, int hint_tile, int hint_entry) {
     Stage st;
     int t = hint_tile;
     if (t < 0 || !(tiles[t].u0 <= u && u < tiles[t].u1)) t = tile_of_unit(tiles, ntiles, u);
@@ -110,10 +113,16 @@ __device__ __forceinline__ Stage make_stage(const PairTile *tiles, int ntiles, c
     const long long seg_end_u = tl.u1 < uend ? tl.u1 : uend;
     if (tl.L0 >= 0) {  // interaction list: the entry e with lst_cum[e] <= u < lst_cum[e + 1]
         int lo = tl.L0, hi = tl.L1 - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (geo.lst_cum[mid] <= u) lo = mid; else hi = mid - 1;
+        if (hint_entry >= lo && hint_entry <= hi) {
+            lo = hint_entry;
+            if (geo.lst_cum[lo + 1] <= u) ++lo;
+        } else {
+            while (lo < hi) {
+                int mid = (lo + hi + 1) >> 1;
+                if (geo.lst_cum[mid] <= u) lo = mid; else hi = mid - 1;
+            }
         }
+        st.entry = lo;
         const int seg = geo.lst_seg[lo];
         const int blk = (int)(u - geo.lst_cum[lo]);
         const int seg_blocks = (int)(geo.lst_cum[lo + 1] - geo.lst_cum[lo]);
@@ -130,6 +139,7 @@ __device__ __forceinline__ Stage make_stage(const PairTile *tiles, int ntiles, c
         st.nblk = n;
         return st;
     }
+    st.entry = -1;
     const long long *blk_off = geo.blk_off;
     const int *src_off = geo.src_off;
     long long gbl = blk_off[tl.B0] + (u - tl.u0);
@@ -167,6 +177,8 @@ struct PolicyBase {
     // idx: the target (a clamped duplicate when !valid: computed, never written)
     __device__ __forceinline__ void load_extra(int, int, bool, const PairGeom &) {}
     __device__ __forceinline__ void source_side(int, bool, double *) {}
+    // targets of the tile (CTA-uniform): policies that skip missing target pairs keep it
+    __device__ __forceinline__ void set_count(int) {}
 };
 
 template <int D, int NRHS, int T, int NT>
@@ -283,7 +295,12 @@ struct PackedStokesT : PolicyBase {
     float *sm;
     int tid;
     u64 bsum[TP][C];
+    int pairs;  // target pairs per thread that hold targets (CTA-uniform)
 
+    // Tiles that end with their target group (the treecode's check points and bodies: 392 or 839
+    // targets against 640 per tile) leave whole target pairs of every thread empty; those pairs are
+    // skipped (2000 ellipsoids, M = 839: 1.31 tiles of work per body instead of 2).
+    __device__ __forceinline__ void set_count(int n) { pairs = min(TP, (n + 2 * NT - 1) / (2 * NT)); }
     __device__ __forceinline__ float &at(int f, int j) const { return sm[(f * T + j) * NT + tid]; }
     __device__ __forceinline__ void init(float *base, int t) {
         sm = base;
@@ -308,9 +325,23 @@ struct PackedStokesT : PolicyBase {
     }
     __device__ __forceinline__ void compute(const float *sb, int nrec, const float (*dc)[3], const float (*)[3],
                                             int kb0) {
-        u64 xt[TP][3];
+        if (pairs == TP) compute_pairs<TP>(sb, nrec, dc, kb0);
+        else if constexpr (TP > 1) compute_fewer<TP - 1>(sb, nrec, dc, kb0);
+    }
+    template <int A>
+    __device__ __forceinline__ void compute_fewer(const float *sb, int nrec, const float (*dc)[3], int kb0) {
+        if constexpr (A == 1) {
+            compute_pairs<1>(sb, nrec, dc, kb0);
+        } else {
+            if (pairs == A) compute_pairs<A>(sb, nrec, dc, kb0);
+            else compute_fewer<A - 1>(sb, nrec, dc, kb0);
+        }
+    }
+    template <int A>
+    __device__ __forceinline__ void compute_pairs(const float *sb, int nrec, const float (*dc)[3], int kb0) {
+        u64 xt[A][3];
 #pragma unroll
-        for (int p = 0; p < TP; ++p) {
+        for (int p = 0; p < A; ++p) {
             const int j0 = 2 * p, j1 = 2 * p + 1;
             const int r0 = body(j0) - kb0, r1 = body(j1) - kb0;
             xt[p][0] = f2_pack(dc[r0][0] + at(0, j0), dc[r1][0] + at(0, j1));
@@ -319,9 +350,9 @@ struct PackedStokesT : PolicyBase {
         }
         for (int s0 = 0; s0 < nrec; s0 += MFS_BS) {
             const int s1 = min(s0 + MFS_BS, nrec);
-            u64 blk[TP][C];
+            u64 blk[A][C];
 #pragma unroll
-            for (int p = 0; p < TP; ++p)
+            for (int p = 0; p < A; ++p)
 #pragma unroll
                 for (int c = 0; c < C; ++c) blk[p][c] = 0ull;
             for (int s = s0; s < s1; s += 4) {
@@ -335,7 +366,7 @@ struct PackedStokesT : PolicyBase {
                         rec[2 * v + 1] = f.y;
                     }
 #pragma unroll
-                    for (int p = 0; p < TP; ++p) {
+                    for (int p = 0; p < A; ++p) {
                         const u64 dx = f2_sub(xt[p][0], rec[0]);
                         const u64 dy = f2_sub(xt[p][1], rec[1]);
                         const u64 dz = f2_sub(xt[p][2], rec[2]);
@@ -366,7 +397,7 @@ struct PackedStokesT : PolicyBase {
                 }
             }
 #pragma unroll
-            for (int p = 0; p < TP; ++p)
+            for (int p = 0; p < A; ++p)
 #pragma unroll
                 for (int c = 0; c < C; ++c) bsum[p][c] = f2_add(bsum[p][c], blk[p][c]);
         }
@@ -1086,7 +1117,7 @@ __global__ void __launch_bounds__(NT, MINB) pair_sum_kernel(PairGeom geo, PairWo
     __syncthreads();
 
     const PairTile *tiles = work.tiles;
-    Stage cur = make_stage(tiles, work.ntiles, geo, ubeg, uend, Cfg::STAGE_BLOCKS, -1);
+    Stage cur = make_stage(tiles, work.ntiles, geo, ubeg, uend, Cfg::STAGE_BLOCKS, -1, -1);
     const int first_tile = cur.tile;
     if (tid == 0) {
         mbar_arrive_expect_tx(&bars[0], (uint32_t)(cur.nrec * REC * 4));
@@ -1098,6 +1129,7 @@ __global__ void __launch_bounds__(NT, MINB) pair_sum_kernel(PairGeom geo, PairWo
     PairTile tl = tiles[cur.tile];
     long long seg_begin = ubeg;
     auto load_targets = [&](const PairTile &t_) {
+        pol.set_count(t_.t1 - t_.t0);
 #pragma unroll
         for (int j = 0; j < TPT; ++j) {
             int idx = t_.t0 + tid + j * NT;
@@ -1123,7 +1155,8 @@ __global__ void __launch_bounds__(NT, MINB) pair_sum_kernel(PairGeom geo, PairWo
                 while (hint < work.ntiles && tiles[hint].u1 <= unext) ++hint;
                 if (hint >= work.ntiles) hint = -1;
             }
-            nxt = make_stage(tiles, work.ntiles, geo, unext, uend, Cfg::STAGE_BLOCKS, hint);
+            nxt = make_stage(tiles, work.ntiles, geo, unext, uend, Cfg::STAGE_BLOCKS, hint,
+                             hint == cur.tile ? cur.entry : -1);
             if (tid == 0) {
                 mbar_arrive_expect_tx(&bars[buf ^ 1], (uint32_t)(nxt.nrec * REC * 4));
                 bulk_g2s(smem + (buf ^ 1) * SREC * REC, geo.src + (size_t)nxt.rec0 * REC,
