@@ -107,8 +107,8 @@ typedef struct {
                              GPU counterpart of the far-field acceleration the paper does with an FMM (Sec. 4):
                              an 8-ary tree of median splits over the body centres; every body and every node
                              gets 196 equivalent point sources on a sphere of radius r_e = (radius of its proxy
-                             points) / 0.83, fitted in FP64 by least squares to its proxies' field at 392
-                             check points at 2.5 r_e; targets at least 3 r_e from a node's centre see it
+                             points) / 0.83, fitted in FP64 by least squares to its proxies' field at 256
+                             check points at 2.6 r_e; targets at least 3 r_e from a node's centre see it
                              through those points, nearer ones its children, down to the proxy points of the
                              near bodies (direct, FP32 pair kernel).  Targets further away use 128, 96 or 64
                              points matched to the 196 (from 4, 5 and 8 radii on), and bodies with many
@@ -127,7 +127,7 @@ typedef struct {
                              velocities are matched to about 1e-7; a larger separation tightens both). */
     double farfield_separation; /* farfield = 1: a target uses a node's equivalent points when it is at least
                                    this many equivalent radii from the node's centre; default 3, allowed
-                                   [2.5, 10] (2.5 = the check sphere; smaller is faster and less accurate). */
+                                   [2.5, 10] (smaller is faster and less accurate). */
 } mfs_options;
 
 typedef struct {

@@ -151,8 +151,12 @@ cudaError_t stress_f64(int nrhs, const double *tgt_local, const int *tbody, cons
 
 // ---- far field of the pair sums: equivalent-source treecode (farfield.cu) ----
 constexpr int FF_NE = 196;            // equivalent points per node (a Fibonacci sphere of radius r_e)
-constexpr int FF_NC = 392;            // check points per node (radius FF_CHECK * r_e), least-squares fit
-constexpr double FF_CHECK = 2.5;      // check radius / equivalent radius
+// Check points per node and their radius over r_e, least-squares fit: 256 at 2.6 leave a field error of
+// 1.2e-7 at 3 radii where 392 at 2.5 left 1.6e-7 (white-noise sources), fill two target pairs of every
+// thread of an upward tile exactly and take a third off the FP64 fit.
+constexpr int FF_NC = 256;
+constexpr double FF_CHECK = 2.6;
+constexpr double FF_MIN_SEPARATION = 2.5;  // the smallest mfs_options.farfield_separation
 constexpr double FF_SRC_RATIO = 0.83; // a node's source radius / its equivalent radius
 // (a target at least mfs_options.farfield_separation equivalent radii from a node's centre sees the node
 // through its equivalent points)
@@ -161,7 +165,7 @@ constexpr double FF_SRC_RATIO = 0.83; // a node's source radius / its equivalent
 // node's centre (order 0 from farfield_separation on).  Its strengths are the least-squares match of the
 // next higher order's field at FF_ORD_NC[o] points at FF_ORD_CHECK[o] radii, where the high-degree part
 // that the smaller set cannot hold has already decayed.  White-noise sources at the edge of the node,
-// relative field error: 196 points 1.9e-7 at 3 radii and 3e-8 at 4; 128 points 6e-8 at 4; 96 points
+// relative field error: 196 points 1.2e-7 at 3 radii and 3e-8 at 4; 128 points 6e-8 at 4; 96 points
 // 5e-8 at 5; 64 points 3e-8 at 8 (each falling further out).
 constexpr int FF_NORD = 4;
 constexpr int FF_ORD_N[FF_NORD] = {FF_NE, 128, 96, 64};

@@ -225,13 +225,13 @@ struct mfs_ctx {
         std::map<int, ListPlan> ev;                  // order-0 lists at the targets (gradient), key: variant
         std::map<int, ListPlan> loc;                 // local check points, key: variant
         std::map<int, ListPlan> direct;              // targets, all orders, key: variant * 2 + include_self
-        struct Cells {                               // ff_cell_lists of every cell of `size` tree positions
+        struct Cells {                               // ff_cell_lists of every cell of consecutive tree positions
             std::vector<int> first;                  // first tree position of each cell, then P
             std::vector<int> cell_of;                // tree position -> cell
             std::vector<std::vector<int>> local;     // per cell
             std::vector<std::vector<int>> direct;    // per tree position
         };
-        std::map<int, Cells> cells;                  // key: cell size
+        Cells cells;
     } ff, ffT;                                       // forward sums; transposed sums (adjoint)
 
     int sm_count = 0;
@@ -830,18 +830,24 @@ mfs_status ff_ev_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, FFListPla
     return MFS_OK;
 }
 
-// The cells of `size` consecutive tree positions (cut at suspensions) and their lists.
-static const mfs_ctx::FarField::Cells &ff_cells(mfs_ctx *ctx, mfs_ctx::FarField &F, int size) {
-    auto it = F.cells.find(size);
-    if (it != F.cells.end()) return it->second;
-    mfs_ctx::FarField::Cells &c = F.cells[size];
+// Bodies that share a cell (one list, one tile of FF_LOC_NC check points each).  More bodies fill a tile
+// better (5 or 6 of them with the widest policies), but a node must be far from all of them: with 6 the
+// bodies' own lists take 6.2e6 pairs a body (2000 ellipsoids, near bodies apart), with 2 they take 3.5e6
+// and the two active target pairs per thread cost the cells' sums little (matvec 38.7 ms with 6, 36.4 with
+// 2, 36.8 with 1; 37.3, 35.8 and 36.3 with the 5-pair policy).
+constexpr int FF_CELL = 2;
+
+// The cells of FF_CELL consecutive tree positions (cut at suspensions) and their lists.
+static const mfs_ctx::FarField::Cells &ff_cells(mfs_ctx *ctx, mfs_ctx::FarField &F) {
+    mfs_ctx::FarField::Cells &c = F.cells;
+    if (!c.first.empty()) return c;
     c.cell_of.resize(ctx->P);
     c.direct.resize(ctx->P);
     std::vector<int> tb;
     std::vector<std::vector<int>> direct;
     for (int sp = 0; sp < ctx->S; ++sp)
-        for (int q0 = ctx->body_off[sp]; q0 < ctx->body_off[sp + 1]; q0 += size) {
-            const int q1 = std::min(q0 + size, ctx->body_off[sp + 1]);
+        for (int q0 = ctx->body_off[sp]; q0 < ctx->body_off[sp + 1]; q0 += FF_CELL) {
+            const int q1 = std::min(q0 + FF_CELL, ctx->body_off[sp + 1]);
             tb.clear();
             for (int q = q0; q < q1; ++q) tb.push_back(F.tree.order[q]);
             c.local.emplace_back();
@@ -857,19 +863,13 @@ static const mfs_ctx::FarField::Cells &ff_cells(mfs_ctx *ctx, mfs_ctx::FarField 
     return c;
 }
 
-// Bodies whose local check points share one tile of the variant.
-static int ff_cell_size(int variant) {
-    int vc = 0;
-    return std::max(1, pair_variants(&vc)[variant].tile_targets / FF_LOC_NC);
-}
-
 // The plan of the sums at the bodies' local check points (one tile and one list per cell).
 mfs_status ff_loc_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, FFListPlan **out) {
     auto it = F.loc.find(variant);
     if (it == F.loc.end()) {
         FFListPlan lp;
         const int P = ctx->P;
-        const auto &cells = ff_cells(ctx, F, ff_cell_size(variant));
+        const auto &cells = ff_cells(ctx, F);
         std::vector<long long> blocks;
         std::vector<int> recs, toff(P + 1);
         ff_segments(F, blocks, recs);
@@ -899,7 +899,7 @@ mfs_status ff_direct_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, int i
             toff[q + 1] = toff[q] + ((*F.tgt_off)[b + 1] - (*F.tgt_off)[b]);
         }
         if (F.use_local) {
-            const auto &cells = ff_cells(ctx, F, ff_cell_size(variant));
+            const auto &cells = ff_cells(ctx, F);
             for (int q = 0; q <= P; ++q) cuts.push_back(q);
             CKS(build_plan_lists(ctx, variant, include_self, toff, 0, cuts, blocks, recs,
                                  [&](int g0, int, std::vector<int> &segs) {
@@ -2039,7 +2039,7 @@ static void ff_release_geometry(mfs_ctx *ctx, mfs_ctx::FarField &F) {
         }
         plans->clear();
     }
-    F.cells.clear();
+    F.cells = mfs_ctx::FarField::Cells{};
     for (int o = 1; o < FF_NORD; ++o) {
         ctx->release(F.ord_pos[o]);
         ctx->release(F.ord_mu[o]);
@@ -2589,7 +2589,7 @@ mfs_status mfs_setup(mfs_ctx **out, mfs_kind kind, const mfs_bodies *bodies, int
         g_setup_error = "mfs_setup: farfield must be 0 or 1, and 1 needs precision 0 or 2 (FP32 pair sums)";
         return MFS_ERR_INVALID_ARG;
     }
-    if (ctx->opt.farfield == 1 && !(ctx->opt.farfield_separation >= FF_CHECK && ctx->opt.farfield_separation <= 10.0)) {
+    if (ctx->opt.farfield == 1 && !(ctx->opt.farfield_separation >= FF_MIN_SEPARATION && ctx->opt.farfield_separation <= 10.0)) {
         g_setup_error = "mfs_setup: farfield_separation must lie in [2.5, 10]";
         return MFS_ERR_INVALID_ARG;
     }

@@ -297,7 +297,7 @@ struct PackedStokesT : PolicyBase {
     u64 bsum[TP][C];
     int pairs;  // target pairs per thread that hold targets (CTA-uniform)
 
-    // Tiles that end with their target group (the treecode's check points and bodies: 392 or 839
+    // Tiles that end with their target group (the treecode's check points and bodies: 256 or 839
     // targets against 640 per tile) leave whole target pairs of every thread empty; those pairs are
     // skipped (2000 ellipsoids, M = 839: 1.31 tiles of work per body instead of 2).
     __device__ __forceinline__ void set_count(int n) { pairs = min(TP, (n + 2 * NT - 1) / (2 * NT)); }

@@ -19,7 +19,7 @@ from test_farfield_fit import fibonacci, kernel_matrix
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2409_04215_gb300", "csrc")
-ORD_N, ORD_NC, ORD_CHECK, ORD_KAPPA = (196, 128, 96, 64), (392, 192, 160, 128), (2.5, 4.0, 5.0, 8.0), (3.0, 4.0, 5.0, 8.0)
+ORD_N, ORD_NC, ORD_CHECK, ORD_KAPPA = (196, 128, 96, 64), (256, 192, 160, 128), (2.6, 4.0, 5.0, 8.0), (3.0, 4.0, 5.0, 8.0)
 ORD_TRUNC, LOC_TRUNC = (1e-12, 1e-12, 1e-12, 1e-8), 1e-8
 LOC_N, LOC_NC, LOC_CHECK, LOC_EQ, LOC_GAP = 96, 128, 1.1, 6.0, 5.0
 
