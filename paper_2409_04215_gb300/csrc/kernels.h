@@ -140,6 +140,28 @@ cudaError_t dirichlet_rhs_stokes(const double *U, const double *Om, int nrhs, in
 cudaError_t dirichlet_rhs_laplace(const double *phi, int nrhs, int P, const int *body_tgt_off, int sum_M, double *b,
                                   cudaStream_t st);
 
+// ---- evaluation points grouped by body (eval_group.cu) ----
+// Device pointers.  A point's key is its owner body, or key_of_body[owner] (body_of_key its inverse)
+// when given; grouped point j is the caller's point order[j], keys ascending, the caller's order kept
+// within a key; toff[q] the first grouped point of key q.
+int eval_chunks(int np);
+struct EvalGroup {
+    int np = 0, P = 0;
+    const double *points = nullptr, *normals = nullptr;  // [np][3]; normals may be null
+    const int *owner = nullptr;                          // [np] or null: the nearest centre
+    const double *centres = nullptr;                     // [P][3] by body
+    const int *key_of_body = nullptr, *body_of_key = nullptr;
+    int *key = nullptr, *counts = nullptr, *total = nullptr;  // scratch [np], [eval_chunks(np)][P], [P]
+    int *toff = nullptr, *order = nullptr;               // [P + 1], [np]
+    float4 *t4 = nullptr;                                // [np] relative to the owner's centre, w = key (int bits)
+    float *n32 = nullptr;                                // [np][3] grouped normals (with normals)
+    double *t64 = nullptr, *n64 = nullptr;               // [np][3] FP64 copies, or null
+    int *tbody = nullptr;                                // [np] keys, or null
+    unsigned long long *radius = nullptr;                // [P] largest distance per key (double bits), or null
+    int *err = nullptr;                                  // |= MFS_DEVERR_BADARG
+};
+cudaError_t eval_group(const EvalGroup &e, cudaStream_t st);
+
 // ---- pressure and traction at evaluation points (stress.cu, Eq. traction), FP64 reference ----
 // Points tgt_local (owner-relative) with owners tbody, unit normals nrm [np][3] or null (no traction),
 // FP64 body-local sources and strengths, per-body suspension body range [sb0, sb1); outputs p

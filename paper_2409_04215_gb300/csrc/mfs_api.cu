@@ -193,6 +193,7 @@ struct mfs_ctx {
         int *eq_pt = nullptr;                        // identity record -> point map (packing)
         float4 *chk_pos = nullptr;                   // [nodes FF_NC] check points, w = P + node
         float4 *tgt = nullptr;                       // [sum_M] targets in tree order, w = tree position
+        int *pos = nullptr, *order = nullptr;        // [P] body -> tree position and back (device)
         int *tperm = nullptr;                        // [sum_M] tree-order target -> caller's target index
         int *seg_rec0 = nullptr, *seg_rec1 = nullptr;  // [P + nodes] record range of every segment
         std::vector<int> seg_rec0_h, seg_rec1_h;
@@ -235,6 +236,7 @@ struct mfs_ctx {
     } ff, ffT;                                       // forward sums; transposed sums (adjoint)
 
     int sm_count = 0;
+    cudaMemPool_t pool = nullptr;  // scratch of single calls (Scratch); kept between calls, given back with the context
     std::string last_error;
     std::vector<void *> allocs;
     double ms_setup = 0.0;
@@ -268,6 +270,7 @@ struct mfs_ctx {
         if (evp0) cudaEventDestroy(evp0);
         if (evp1) cudaEventDestroy(evp1);
         for (cudaEvent_t e : pev) cudaEventDestroy(e);
+        if (pool) cudaMemPoolDestroy(pool);
     }
 };
 
@@ -300,6 +303,37 @@ bool is_device_ptr(const void *p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Device scratch of one call on one stream: allocations from the context's pool, freed in stream order
+// when the call returns (no device synchronisation; a cudaMalloc and cudaFree pair per buffer took most
+// of a small evaluation).
+struct Scratch {
+    mfs_ctx *ctx;
+    cudaStream_t st;
+    std::vector<void *> ps;
+    std::vector<std::shared_ptr<void>> host;  // host arrays whose uploads may still be in flight
+    Scratch(mfs_ctx *c, cudaStream_t s) : ctx(c), st(s) {}
+    Scratch(const Scratch &) = delete;
+    ~Scratch() {
+        if (!host.empty()) cudaStreamSynchronize(st);
+        for (void *p : ps) cudaFreeAsync(p, st);
+    }
+    // Upload of a host array that is kept until the stream is done with it.
+    template <typename T>
+    cudaError_t upload(T *dst, std::vector<T> &&src) {
+        auto kept = std::make_shared<std::vector<T>>(std::move(src));
+        host.push_back(kept);
+        return cudaMemcpyAsync(dst, kept->data(), sizeof(T) * kept->size(), cudaMemcpyHostToDevice, st);
+    }
+    template <typename T>
+    cudaError_t alloc(T **p, size_t count) {
+        *p = nullptr;
+        const cudaError_t e =
+            cudaMallocFromPoolAsync((void **)p, sizeof(T) * std::max<size_t>(count, 1), ctx->pool, st);
+        if (e == cudaSuccess) ps.push_back((void *)*p);
+        return e;
+    }
+};
+
 // A device view of a user pointer: either the pointer itself or a staged copy.
 struct Staged {
     mfs_ctx *ctx = nullptr;
@@ -307,8 +341,9 @@ struct Staged {
     const void *user = nullptr;
     size_t count = 0;
     bool owned = false;
+    cudaStream_t st = nullptr;
     ~Staged() {
-        if (owned && d) cudaFree(d);
+        if (owned && d) cudaFreeAsync(d, st);
     }
 };
 
@@ -320,13 +355,14 @@ mfs_status stage_in(mfs_ctx *ctx, Staged &s, const double *user, size_t count, c
         s.d = const_cast<double *>(user);
         return MFS_OK;
     }
-    CK(cudaMalloc(&s.d, sizeof(double) * std::max<size_t>(count, 1)));
+    s.st = st;
+    CK(cudaMallocFromPoolAsync((void **)&s.d, sizeof(double) * std::max<size_t>(count, 1), ctx->pool, st));
     s.owned = true;
     CK(cudaMemcpyAsync(s.d, user, sizeof(double) * count, cudaMemcpyHostToDevice, st));
     return MFS_OK;
 }
 
-mfs_status stage_out_alloc(mfs_ctx *ctx, Staged &s, double *user, size_t count) {
+mfs_status stage_out_alloc(mfs_ctx *ctx, Staged &s, double *user, size_t count, cudaStream_t st) {
     s.ctx = ctx;
     s.user = user;
     s.count = count;
@@ -334,7 +370,8 @@ mfs_status stage_out_alloc(mfs_ctx *ctx, Staged &s, double *user, size_t count) 
         s.d = user;
         return MFS_OK;
     }
-    CK(cudaMalloc(&s.d, sizeof(double) * std::max<size_t>(count, 1)));
+    s.st = st;
+    CK(cudaMallocFromPoolAsync((void **)&s.d, sizeof(double) * std::max<size_t>(count, 1), ctx->pool, st));
     s.owned = true;
     return MFS_OK;
 }
@@ -441,10 +478,10 @@ int fp32_variant(const mfs_ctx *ctx, int D, int nrhs) {
 // sources (the matvec and u_0); transposed = 1: proxy targets, collocation sources (the adjoint's
 // S^T sums).
 // Work list of a pair sum over any target set grouped by body: targets of body k are
-// [toff[k], toff[k+1]) and tbody[t] is the body of target t; source blocks per body from boff.
+// [toff[k], toff[k+1]); source blocks per body from boff.  With `tmp` the plan's device arrays are that
+// call's scratch.
 mfs_status build_plan_for(mfs_ctx *ctx, int variant, int include_self, const std::vector<int> &toff,
-                          const std::vector<int> &tbody, const std::vector<long long> &boff, int ntargets,
-                          PairPlan &plan) {
+                          const std::vector<long long> &boff, int ntargets, PairPlan &plan, Scratch *tmp = nullptr) {
     int count = 0;
     const PairVariant *vv = pair_variants(&count);
     const PairVariant &v = vv[variant];
@@ -455,11 +492,12 @@ mfs_status build_plan_for(mfs_ctx *ctx, int variant, int include_self, const std
     for (int s = 0; s < ctx->S; ++s) {
         const int B0 = ctx->body_off[s], B1 = ctx->body_off[s + 1];
         const int t_end = toff[B1];
-        int t = toff[B0];
+        int t = toff[B0], kb0 = B0;
         while (t < t_end) {
             int t1 = std::min(t + TT, t_end);
-            const int kb0 = tbody[t];
-            int kb1 = tbody[t1 - 1];
+            while (toff[kb0 + 1] <= t) ++kb0;  // the body of target t, then of target t1 - 1
+            int kb1 = kb0;
+            while (toff[kb1 + 1] < t1) ++kb1;
             if (kb1 - kb0 + 1 > MFS_MAX_TILE_BODIES) {
                 kb1 = kb0 + MFS_MAX_TILE_BODIES - 1;
                 t1 = toff[kb1 + 1];
@@ -509,6 +547,13 @@ mfs_status build_plan_for(mfs_ctx *ctx, int variant, int include_self, const std
     plan.ntiles = (int)tiles.size();
     plan.max_share = max_share;
     plan.total_units = units;
+    if (tmp) {
+        CK(tmp->alloc(&plan.tiles, tiles.size()));
+        CK(tmp->alloc(&plan.partial, (size_t)G * 2 * TT * C));
+        CK(tmp->alloc(&plan.direct, (size_t)std::max(ntargets, 1) * C));
+        CK(tmp->upload(plan.tiles, std::move(tiles)));
+        return MFS_OK;
+    }
     CK(ctx->alloc(&plan.tiles, tiles.size()));
     CK(cudaMemcpy(plan.tiles, tiles.data(), sizeof(PairTile) * tiles.size(), cudaMemcpyHostToDevice));
     plan.partial_bytes = sizeof(double) * (size_t)G * 2 * TT * C;
@@ -520,8 +565,7 @@ mfs_status build_plan_for(mfs_ctx *ctx, int variant, int include_self, const std
 
 mfs_status build_plan(mfs_ctx *ctx, int variant, int include_self, int transposed, PairPlan &plan) {
     return build_plan_for(ctx, variant, include_self, transposed ? ctx->src_off : ctx->tgt_off,
-                          transposed ? ctx->src_body : ctx->tgt_body, transposed ? ctx->blkT_off : ctx->blk_off,
-                          transposed ? ctx->sumN : ctx->sumM, plan);
+                          transposed ? ctx->blkT_off : ctx->blk_off, transposed ? ctx->sumN : ctx->sumM, plan);
 }
 
 void release_plan(mfs_ctx *ctx, PairPlan &plan) {
@@ -664,7 +708,7 @@ template <class ListFn>
 mfs_status build_plan_lists(mfs_ctx *ctx, int variant, int include_self, const std::vector<int> &toff, int gid0,
                             const std::vector<int> &cuts, const std::vector<long long> &seg_blocks,
                             const std::vector<int> &seg_recs, ListFn list_of, PairPlan &plan, int **lst_seg_d,
-                            long long **lst_cum_d, double &pairs) {
+                            long long **lst_cum_d, double &pairs, Scratch *tmp = nullptr) {
     int count = 0;
     const PairVariant *vv = pair_variants(&count);
     const PairVariant &v = vv[variant];
@@ -742,12 +786,22 @@ mfs_status build_plan_lists(mfs_ctx *ctx, int variant, int include_self, const s
     plan.ntiles = (int)tiles.size();
     plan.max_share = max_share;
     plan.total_units = units;
-    CK(ctx->alloc(&plan.tiles, std::max<size_t>(tiles.size(), 1)));
+    auto alloc_all = [&](auto &&from) -> cudaError_t {
+        cudaError_t e = from.alloc(&plan.tiles, tiles.size());
+        if (e == cudaSuccess) e = from.alloc(&plan.partial, (size_t)G * 2 * TT * C);
+        if (e == cudaSuccess) e = from.alloc(&plan.direct, (size_t)std::max(toff.back(), 1) * C);
+        if (e == cudaSuccess) e = from.alloc(lst_seg_d, lst.size());
+        if (e == cudaSuccess) e = from.alloc(lst_cum_d, cum.size());
+        return e;
+    };
+    CK(tmp ? alloc_all(*tmp) : alloc_all(*ctx));
+    if (tmp) {
+        CK(tmp->upload(plan.tiles, std::move(tiles)));
+        CK(tmp->upload(*lst_seg_d, std::move(lst)));
+        CK(tmp->upload(*lst_cum_d, std::move(cum)));
+        return MFS_OK;
+    }
     CK(cudaMemcpy(plan.tiles, tiles.data(), sizeof(PairTile) * tiles.size(), cudaMemcpyHostToDevice));
-    CK(ctx->alloc(&plan.partial, (size_t)G * 2 * TT * C));
-    CK(ctx->alloc(&plan.direct, (size_t)std::max(toff.back(), 1) * C));
-    CK(ctx->alloc(lst_seg_d, std::max<size_t>(lst.size(), 1)));
-    CK(ctx->alloc(lst_cum_d, cum.size()));
     if (!lst.empty()) CK(cudaMemcpy(*lst_seg_d, lst.data(), sizeof(int) * lst.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(*lst_cum_d, cum.data(), sizeof(long long) * cum.size(), cudaMemcpyHostToDevice));
     return MFS_OK;
@@ -2057,6 +2111,9 @@ static void ff_release_geometry(mfs_ctx *ctx, mfs_ctx::FarField &F) {
     ctx->release(F.chk_pos);
     ctx->release(F.tgt);
     ctx->release(F.tperm);
+    ctx->release(F.pos);
+    ctx->release(F.order);
+    F.pos = F.order = nullptr;
     ctx->release(F.seg_rec0);
     ctx->release(F.seg_rec1);
     ctx->release(F.rec);
@@ -2189,6 +2246,10 @@ static mfs_status ff_setup(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStream_t st) 
     CK(ctx->alloc(&F.chk_pos, chk.size()));
     CK(ctx->alloc(&F.tgt, tff.size()));
     CK(ctx->alloc(&F.tperm, tperm.size()));
+    CK(ctx->alloc(&F.pos, P));
+    CK(ctx->alloc(&F.order, P));
+    CK(cudaMemcpy(F.pos, F.tree.pos.data(), sizeof(int) * P, cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(F.order, F.tree.order.data(), sizeof(int) * P, cudaMemcpyHostToDevice));
     CK(ctx->alloc(&F.seg_rec0, F.seg_rec0_h.size()));
     CK(ctx->alloc(&F.seg_rec1, F.seg_rec1_h.size()));
     CK(ctx->alloc(&F.rec, nrec_all * F.rec_floats));
@@ -2534,7 +2595,7 @@ static mfs_status autotune(mfs_ctx *ctx, int nrhs, cudaStream_t st) {
         PairPlan local;
         PairPlan *plan = &local;
         if (sample)
-            CKS(build_plan_for(ctx, i, 0, toff_s, ctx->tgt_body, ctx->blk_off, nt_s, local));
+            CKS(build_plan_for(ctx, i, 0, toff_s, ctx->blk_off, nt_s, local));
         else
             CKS(get_plan(ctx, i, 0, &plan));
         struct Release {
@@ -2616,6 +2677,17 @@ mfs_status mfs_setup(mfs_ctx **out, mfs_kind kind, const mfs_bodies *bodies, int
         return MFS_ERR_CUDA;
     }
     cudaStream_t st = (cudaStream_t)stream;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    unsigned long long keep = ~0ull;
+    if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        g_setup_error = "mfs_setup: cannot create a memory pool";
+        return MFS_ERR_CUDA;
+    }
     mfs_status s = setup_impl(ctx.get(), kind, bodies, num_shapes, proxy, colloc, st);
     if (s == MFS_OK && ctx->opt.autotune && ctx->opt.precision != 1 && ctx->best_variant[kind == MFS_STOKES][1] < 0) {
         // tune the single-rhs variant now; other nrhs on first use
@@ -2663,7 +2735,7 @@ mfs_status mfs_matvec(mfs_ctx *ctx, const double *gamma, double *y, int32_t nrhs
     const size_t n = (size_t)nrhs * ctx->sumM * ctx->D;
     Staged gi, yo;
     CKS(stage_in(ctx, gi, gamma, n, st));
-    CKS(stage_out_alloc(ctx, yo, y, n));
+    CKS(stage_out_alloc(ctx, yo, y, n, st));
     CKS(matvec_dev(ctx, gi.d, yo.d, nrhs, st));
     CKS(stage_out_finish(ctx, yo, st));
     return check_device_error(ctx, st);
@@ -2683,7 +2755,7 @@ mfs_status mfs_matvec_transposed(mfs_ctx *ctx, const double *w, double *y, int32
     const size_t n = (size_t)nrhs * ctx->sumM * 3;
     Staged wi, yo;
     CKS(stage_in(ctx, wi, w, n, st));
-    CKS(stage_out_alloc(ctx, yo, y, n));
+    CKS(stage_out_alloc(ctx, yo, y, n, st));
     CKS(matvec_T_dev(ctx, wi.d, yo.d, nrhs, st));
     CKS(stage_out_finish(ctx, yo, st));
     return check_device_error(ctx, st);
@@ -2698,7 +2770,7 @@ mfs_status mfs_precond_apply(mfs_ctx *ctx, const double *gamma, double *lambda, 
     cudaStream_t st = (cudaStream_t)stream;
     Staged gi, lo;
     CKS(stage_in(ctx, gi, gamma, (size_t)nrhs * ctx->sumM * ctx->D, st));
-    CKS(stage_out_alloc(ctx, lo, lambda, (size_t)nrhs * ctx->sumN * ctx->D));
+    CKS(stage_out_alloc(ctx, lo, lambda, (size_t)nrhs * ctx->sumN * ctx->D, st));
     CKS(precond_apply_dev(ctx, gi.d, lo.d, project ? 1 : 0, nrhs, st));
     CKS(stage_out_finish(ctx, lo, st));
     return MFS_OK;
@@ -2713,7 +2785,7 @@ mfs_status mfs_pair_sum(mfs_ctx *ctx, const double *strengths, double *u, int32_
     cudaStream_t st = (cudaStream_t)stream;
     Staged si, uo;
     CKS(stage_in(ctx, si, strengths, (size_t)nrhs * ctx->sumN * ctx->D, st));
-    CKS(stage_out_alloc(ctx, uo, u, (size_t)nrhs * ctx->sumM * ctx->D));
+    CKS(stage_out_alloc(ctx, uo, u, (size_t)nrhs * ctx->sumM * ctx->D, st));
     CKS(pair_apply(ctx, si.d, uo.d, nullptr, 0.0, 1.0, nrhs, include_self ? 1 : 0, st));
     CKS(stage_out_finish(ctx, uo, st));
     return check_device_error(ctx, st);
@@ -2806,8 +2878,8 @@ mfs_status mfs_solve_mobility(mfs_ctx *ctx, const double *F, const double *T, do
     Staged Fi, Ti, Uo, Oo;
     CKS(stage_in(ctx, Fi, F, nb, st));
     CKS(stage_in(ctx, Ti, T, nb, st));
-    CKS(stage_out_alloc(ctx, Uo, U, nb));
-    CKS(stage_out_alloc(ctx, Oo, Omega, nb));
+    CKS(stage_out_alloc(ctx, Uo, U, nb, st));
+    CKS(stage_out_alloc(ctx, Oo, Omega, nb, st));
     if (ctx->opt.autotune && ctx->opt.precision != 1 && ctx->best_variant[1][nrhs] < 0) CKS(autotune(ctx, nrhs, st));
     CKS(ensure_gmres(ctx, nrhs));
     begin_call(ctx);
@@ -2848,7 +2920,7 @@ mfs_status mfs_solve_elastance(mfs_ctx *ctx, const double *Q, double *V, int32_t
     const size_t nb = (size_t)nrhs * ctx->P;
     Staged Qi, Vo;
     CKS(stage_in(ctx, Qi, Q, nb, st));
-    CKS(stage_out_alloc(ctx, Vo, V, nb));
+    CKS(stage_out_alloc(ctx, Vo, V, nb, st));
     if (ctx->opt.autotune && ctx->opt.precision != 1 && ctx->best_variant[0][nrhs] < 0) CKS(autotune(ctx, nrhs, st));
     CKS(ensure_gmres(ctx, nrhs));
     begin_call(ctx);
@@ -2902,7 +2974,7 @@ mfs_status mfs_dirichlet_matvec(mfs_ctx *ctx, const double *gamma, double *y, in
     Staged gi, yo;
     const size_t n = (size_t)nrhs * ctx->sumM * ctx->D;
     CKS(stage_in(ctx, gi, gamma, n, st));
-    CKS(stage_out_alloc(ctx, yo, y, n));
+    CKS(stage_out_alloc(ctx, yo, y, n, st));
     {
         DirichletScope scope(ctx);
         CKS(matvec_dev(ctx, gi.d, yo.d, nrhs, st));
@@ -2920,7 +2992,7 @@ mfs_status mfs_dirichlet_apply(mfs_ctx *ctx, const double *gamma, double *alpha,
     CKS(ensure_dirichlet(ctx, st));
     Staged gi, ao;
     CKS(stage_in(ctx, gi, gamma, (size_t)nrhs * ctx->sumM * ctx->D, st));
-    CKS(stage_out_alloc(ctx, ao, alpha, (size_t)nrhs * ctx->sumN * ctx->D));
+    CKS(stage_out_alloc(ctx, ao, alpha, (size_t)nrhs * ctx->sumN * ctx->D, st));
     {
         DirichletScope scope(ctx);
         CKS(precond_apply_dev(ctx, gi.d, ao.d, 0, nrhs, st));
@@ -2944,8 +3016,8 @@ mfs_status mfs_solve_resistance(mfs_ctx *ctx, const double *U, const double *Ome
     Staged Ui, Oi, Fo, To;
     CKS(stage_in(ctx, Ui, U, nb, st));
     CKS(stage_in(ctx, Oi, Omega, nb, st));
-    CKS(stage_out_alloc(ctx, Fo, F, nb));
-    CKS(stage_out_alloc(ctx, To, T, nb));
+    CKS(stage_out_alloc(ctx, Fo, F, nb, st));
+    CKS(stage_out_alloc(ctx, To, T, nb, st));
     CKS(ensure_dirichlet(ctx, st));
     if (ctx->opt.autotune && ctx->opt.precision != 1 && ctx->best_variant[1][nrhs] < 0) CKS(autotune(ctx, nrhs, st));
     CKS(ensure_gmres(ctx, nrhs));
@@ -2981,7 +3053,7 @@ mfs_status mfs_solve_capacitance(mfs_ctx *ctx, const double *phi, double *q, int
     const size_t nb = (size_t)nrhs * ctx->P;
     Staged Pi, Qo;
     CKS(stage_in(ctx, Pi, phi, nb, st));
-    CKS(stage_out_alloc(ctx, Qo, q, nb));
+    CKS(stage_out_alloc(ctx, Qo, q, nb, st));
     CKS(ensure_dirichlet(ctx, st));
     if (ctx->opt.autotune && ctx->opt.precision != 1 && ctx->best_variant[0][nrhs] < 0) CKS(autotune(ctx, nrhs, st));
     CKS(ensure_gmres(ctx, nrhs));
@@ -3096,10 +3168,10 @@ mfs_status mfs_mobility_vjp(mfs_ctx *ctx, const double *dU, const double *dOmega
     Staged dUi, dWi, dco, dFo, dTo;
     CKS(stage_in(ctx, dUi, dU, nb, st));
     CKS(stage_in(ctx, dWi, dOmega, nb, st));
-    CKS(stage_out_alloc(ctx, dco, dcenters, (size_t)P * 3));
+    CKS(stage_out_alloc(ctx, dco, dcenters, (size_t)P * 3, st));
     if (dF) {
-        CKS(stage_out_alloc(ctx, dFo, dF, nb));
-        CKS(stage_out_alloc(ctx, dTo, dT, nb));
+        CKS(stage_out_alloc(ctx, dFo, dF, nb, st));
+        CKS(stage_out_alloc(ctx, dTo, dT, nb, st));
     }
     CKS(ensure_transposed(ctx));
     CKS(ensure_gmres(ctx, nrhs));
@@ -3233,91 +3305,82 @@ static __global__ void unsort_kernel(const double *in, const int *order, int np,
     }
 }
 
-// Evaluation points grouped by owner body (counting sort): order[j] is the caller's index of the j-th
-// grouped point, toff[k] the first grouped point of body k; t4 / t64 the points relative to their
-// owner's centre (FP32 with the owner id bits / FP64), nrm the grouped unit normals when given.
-struct EvalTargets {
-    std::vector<int> toff, order, tbody;
-    std::vector<float4> t4;
-    std::vector<double> t64;
-    std::vector<float> nrm32;
-    std::vector<double> nrm64;
+// Evaluation points grouped by owner body, or by tree position when `tree` (eval_group.cu); device
+// arrays in the call's scratch, offsets and, for the tree, each key's largest distance on the host.
+struct Grouped {
+    std::vector<int> toff;
+    std::vector<double> radius;
+    float4 *t4 = nullptr;
+    float *n32 = nullptr;
+    double *t64 = nullptr, *n64 = nullptr;
+    int *tbody = nullptr, *order = nullptr;
 };
 
-static mfs_status group_targets(mfs_ctx *ctx, const double *points, const double *normals, const int32_t *owner,
-                                int np, EvalTargets &e) {
+static mfs_status group_points(mfs_ctx *ctx, const double *points, const double *normals, const int32_t *owner, int np,
+                               bool tree, bool want64, Scratch &tmp, Grouped &g) {
     const int P = ctx->P;
+    cudaStream_t st = tmp.st;
     if (!owner && ctx->S > 1) {
         ctx->last_error = "evaluation: owner bodies are required with several suspensions";
         return MFS_ERR_INVALID_ARG;
     }
-    std::vector<double> pts(3 * (size_t)np), nv;
-    std::vector<int> own(np);
-    CK(cudaMemcpy(pts.data(), points, sizeof(double) * pts.size(), cudaMemcpyDefault));
-    if (normals) {
-        nv.resize(3 * (size_t)np);
-        CK(cudaMemcpy(nv.data(), normals, sizeof(double) * nv.size(), cudaMemcpyDefault));
-    }
-    if (owner) {
-        CK(cudaMemcpy(own.data(), owner, sizeof(int) * np, cudaMemcpyDefault));
-    } else {  // nearest body centre (single suspension)
-        for (int i = 0; i < np; ++i) {
-            double best = 1e300;
-            int bk = 0;
-            for (int k = 0; k < P; ++k) {
-                double d2 = 0.0;
-                for (int a = 0; a < 3; ++a) {
-                    const double d = pts[3 * (size_t)i + a] - ctx->centres[3 * (size_t)k + a];
-                    d2 += d * d;
-                }
-                if (d2 < best) {
-                    best = d2;
-                    bk = k;
-                }
-            }
-            own[i] = bk;
+    auto device = [&](auto *user, size_t count, auto **out) -> cudaError_t {  // the pointer or a copy of host data
+        if (is_device_ptr(user)) {
+            *out = user;
+            return cudaSuccess;
         }
+        typename std::remove_const<typename std::remove_pointer<decltype(user)>::type>::type *d = nullptr;
+        cudaError_t e = tmp.alloc(&d, count);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(d, user, sizeof(*user) * count, cudaMemcpyHostToDevice, st);
+        *out = d;
+        return e;
+    };
+    EvalGroup e;
+    e.np = np;
+    e.P = P;
+    CK(device(points, 3 * (size_t)np, &e.points));
+    if (normals) CK(device(normals, 3 * (size_t)np, &e.normals));
+    if (owner) CK(device((const int *)owner, (size_t)np, &e.owner));
+    e.centres = ctx->centres_d;
+    if (tree) {
+        e.key_of_body = ctx->ff.pos;
+        e.body_of_key = ctx->ff.order;
+        CK(tmp.alloc(&e.radius, P));
     }
-    e.toff.assign(P + 1, 0);
-    e.order.resize(np);
-    e.tbody.resize(np);
-    for (int i = 0; i < np; ++i) {
-        bool finite = std::isfinite(pts[3 * (size_t)i]) && std::isfinite(pts[3 * (size_t)i + 1]) &&
-                      std::isfinite(pts[3 * (size_t)i + 2]);
-        if (normals)
-            finite = finite && std::isfinite(nv[3 * (size_t)i]) && std::isfinite(nv[3 * (size_t)i + 1]) &&
-                     std::isfinite(nv[3 * (size_t)i + 2]);
-        if (own[i] < 0 || own[i] >= P || !finite) {
-            ctx->last_error = "evaluation: owner out of range or non-finite point or normal";
-            return MFS_ERR_INVALID_ARG;
-        }
-        e.toff[own[i] + 1]++;
+    CK(tmp.alloc(&e.key, np));
+    CK(tmp.alloc(&e.counts, (size_t)eval_chunks(np) * P));
+    CK(tmp.alloc(&e.total, P));
+    CK(tmp.alloc(&e.toff, P + 1));
+    CK(tmp.alloc(&e.order, np));
+    CK(tmp.alloc(&e.t4, np));
+    CK(tmp.alloc(&e.err, 1));
+    if (normals) CK(tmp.alloc(&e.n32, 3 * (size_t)np));
+    if (want64) {
+        CK(tmp.alloc(&e.t64, 3 * (size_t)np));
+        CK(tmp.alloc(&e.tbody, np));
+        if (normals) CK(tmp.alloc(&e.n64, 3 * (size_t)np));
     }
-    for (int k = 0; k < P; ++k) e.toff[k + 1] += e.toff[k];
-    e.t4.resize(np);
-    e.t64.resize(3 * (size_t)np);
-    if (normals) {
-        e.nrm32.resize(3 * (size_t)np);
-        e.nrm64.resize(3 * (size_t)np);
+    CK(cudaMemsetAsync(e.err, 0, sizeof(int), st));
+    CK(eval_group(e, st));
+    g.toff.resize(P + 1);
+    int bad = 0;
+    CK(cudaMemcpyAsync(g.toff.data(), e.toff, sizeof(int) * (P + 1), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(&bad, e.err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    if (tree) {
+        g.radius.resize(P);
+        CK(cudaMemcpyAsync(g.radius.data(), e.radius, sizeof(double) * P, cudaMemcpyDeviceToHost, st));
     }
-    std::vector<int> fill(e.toff.begin(), e.toff.end() - 1);
-    for (int i = 0; i < np; ++i) {
-        const int k = own[i], j = fill[k]++;
-        e.order[j] = i;
-        e.tbody[j] = k;
-        double x[3];
-        for (int a = 0; a < 3; ++a) {
-            x[a] = pts[3 * (size_t)i + a] - ctx->centres[3 * (size_t)k + a];
-            e.t64[3 * (size_t)j + a] = x[a];
-            if (normals) {
-                e.nrm64[3 * (size_t)j + a] = nv[3 * (size_t)i + a];
-                e.nrm32[3 * (size_t)j + a] = (float)nv[3 * (size_t)i + a];
-            }
-        }
-        float kb;
-        std::memcpy(&kb, &k, sizeof(float));  // body id stored as int bits
-        e.t4[j] = make_float4((float)x[0], (float)x[1], (float)x[2], kb);
+    CK(cudaStreamSynchronize(st));
+    if (bad) {
+        ctx->last_error = "evaluation: owner out of range or non-finite point or normal";
+        return MFS_ERR_INVALID_ARG;
     }
+    g.t4 = e.t4;
+    g.n32 = e.n32;
+    g.t64 = e.t64;
+    g.n64 = e.n64;
+    g.tbody = e.tbody;
+    g.order = e.order;
     return MFS_OK;
 }
 
@@ -3347,17 +3410,17 @@ mfs_status last_strengths(mfs_ctx *ctx, int nrhs, double *tmp, cudaStream_t st) 
 }
 }  // namespace
 
-// Sums at owner-grouped evaluation points through the treecode (farfield = 1): the upward step on the
-// strengths in lam_d (a forward pair-sum entry), the proxy and equivalent records in the layout of
-// `variant` (a pair sum for mfs_evaluate, the stress entry for mfs_evaluate_stress), the points
-// reordered into the tree's body order, one-off interaction lists for them (each owner's radius that
-// of its farthest point), and the launch of `variant` with per-point weights `tw_grouped` (the normals
-// for the stress; may be null); results land in out_grouped [nrhs][np][dout] in the grouped order,
-// scaled by `scale`.
-static mfs_status ff_points(mfs_ctx *ctx, int variant, const EvalTargets &et, const float *tw_grouped, int nrhs,
-                            int dout, double scale, double *out_grouped, cudaStream_t st) {
+// Sums at evaluation points (grouped by tree position) through the treecode (farfield = 1): the upward
+// step on the strengths in lam_d (a forward pair-sum entry), the proxy and equivalent records in the
+// layout of `variant` (a pair sum for mfs_evaluate, the stress entry for mfs_evaluate_stress), one-off
+// interaction lists for the points (each owner's radius that of its farthest point), and the launch of
+// `variant` with the grouped normals as target weights (the stress; null otherwise); results land in out
+// [nrhs][np][dout] in the caller's order, scaled by `scale`.
+static mfs_status ff_points(mfs_ctx *ctx, int variant, const Grouped &gr, int np, int nrhs, int dout, double scale,
+                            double *out, Scratch &tmp) {
     auto &F = ctx->ff;
-    const int P = ctx->P, D = ctx->D, np = (int)et.t4.size(), nodes = F.nodes;
+    cudaStream_t st = tmp.st;
+    const int P = ctx->P, D = ctx->D, nodes = F.nodes;
     int vc = 0;
     const PairVariant *vv = pair_variants(&vc);
     const int fv = fp32_variant(ctx, D, nrhs);
@@ -3370,74 +3433,32 @@ static mfs_status ff_points(mfs_ctx *ctx, int variant, const EvalTargets &et, co
     CK(pack_sources(D, nrhs, layout, F.src_pos, F.rec_pt, ctx->lam_d, F.nsrc, F.nrec, F.rec, st));
     CK(pack_sources(D, nrhs, layout, F.eq_pos, F.eq_pt, F.mu, nodes * FF_NE, nodes * FF_NE,
                     F.rec + (size_t)F.nrec * REC, st));
-    // tree order of the points; w = the owner's tree position; tperm: tree index -> grouped index
-    std::vector<float4> tt(np);
-    std::vector<float> tw(tw_grouped ? 3 * (size_t)np : 0);
-    std::vector<int> tperm(np), toff(P + 1, 0);
-    std::vector<double> rad(P, 0.0);
-    int t = 0;
-    for (int q = 0; q < P; ++q) {
-        const int b = F.tree.order[q];
-        float w;
-        std::memcpy(&w, &q, sizeof(float));
-        for (int j = et.toff[b]; j < et.toff[b + 1]; ++j, ++t) {
-            tt[t] = make_float4(et.t4[j].x, et.t4[j].y, et.t4[j].z, w);
-            if (tw_grouped)
-                for (int a = 0; a < 3; ++a) tw[3 * (size_t)t + a] = tw_grouped[3 * (size_t)j + a];
-            tperm[t] = j;
-            const double *x = &et.t64[3 * (size_t)j];
-            rad[b] = std::max(rad[b], std::sqrt(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]));
-        }
-        toff[q + 1] = t;
-    }
+    std::vector<double> rad(P);  // by body
+    for (int q = 0; q < P; ++q) rad[F.tree.order[q]] = gr.radius[q];
     std::vector<long long> seg_blocks;
     std::vector<int> seg_recs;
     ff_segments(F, seg_blocks, seg_recs);
     std::vector<int> cuts(ctx->body_off.begin(), ctx->body_off.end()), tb;
     const std::vector<int> suspension_of = suspension_of_bodies(ctx);
     FFListPlan lp;
-    PairPlan &plan = lp.p;
-    int *perm_d = nullptr;
-    float4 *tt_d = nullptr;
-    float *tw_d = nullptr;
-    mfs_status rc = build_plan_lists(
-        ctx, variant, 1, toff, 0, cuts, seg_blocks, seg_recs,
+    CKS(build_plan_lists(
+        ctx, variant, 1, gr.toff, 0, cuts, seg_blocks, seg_recs,
         [&](int g0, int g1, std::vector<int> &segs) {
             tb.clear();
             for (int q = g0; q <= g1; ++q) tb.push_back(F.tree.order[q]);
             ff_interaction_list(F.tree, F.tree.roots[suspension_of[tb[0]]], tb, ctx->centres.data(), rad.data(),
                                 ctx->opt.farfield_separation, 0, segs);
         },
-        plan, &lp.seg, &lp.cum, lp.pairs);
-    if (rc == MFS_OK) {
-        rc = [&]() -> mfs_status {
-            CK(ctx->alloc(&tt_d, np));
-            CK(ctx->alloc(&perm_d, np));
-            CK(cudaMemcpyAsync(tt_d, tt.data(), sizeof(float4) * np, cudaMemcpyHostToDevice, st));
-            CK(cudaMemcpyAsync(perm_d, tperm.data(), sizeof(int) * np, cudaMemcpyHostToDevice, st));
-            if (tw_grouped) {
-                CK(ctx->alloc(&tw_d, tw.size()));
-                CK(cudaMemcpyAsync(tw_d, tw.data(), sizeof(float) * tw.size(), cudaMemcpyHostToDevice, st));
-            }
-            PairGeom g = ff_geom(F, lp);
-            g.tgt = tt_d;
-            g.ntargets = np;
-            g.tgt_w = tw_d;
-            PairWork we = work_of(plan);
-            we.tperm = perm_d;
-            CKS(ff_launch(ctx, variant, g, we, st));
-            CK(pair_epilogue(dout, nrhs, we, nullptr, 0.0, scale, out_grouped, np, st));
-            return MFS_OK;
-        }();
-    }
-    cudaStreamSynchronize(st);  // the one-off lists and plan are freed below
-    ctx->release(tt_d);
-    ctx->release(tw_d);
-    ctx->release(perm_d);
-    ctx->release(lp.seg);
-    ctx->release(lp.cum);
-    if (plan.tiles) release_plan(ctx, plan);
-    return rc;
+        lp.p, &lp.seg, &lp.cum, lp.pairs, &tmp));
+    PairGeom g = ff_geom(F, lp);
+    g.tgt = gr.t4;
+    g.ntargets = np;
+    g.tgt_w = gr.n32;
+    PairWork we = work_of(lp.p);
+    we.tperm = gr.order;
+    CKS(ff_launch(ctx, variant, g, we, st));
+    CK(pair_epilogue(dout, nrhs, we, nullptr, 0.0, scale, out, np, st));
+    return MFS_OK;
 }
 
 extern "C" {
@@ -3454,78 +3475,56 @@ mfs_status mfs_evaluate(mfs_ctx *ctx, const double *points, const int32_t *owner
     }
     if (npoints == 0) return MFS_OK;
     cudaStream_t st = (cudaStream_t)stream;
-    const int P = ctx->P, D = ctx->D, np = npoints;
-    EvalTargets et;
-    CKS(group_targets(ctx, points, nullptr, owner, np, et));
-    std::vector<int> &toff = et.toff, &order = et.order, &tbody = et.tbody;
-    std::vector<float4> &t4 = et.t4;
-    std::vector<double> &t64 = et.t64;
-    (void)P;
+    const int D = ctx->D, np = npoints;
+    Scratch tmp(ctx, st);
+    Grouped gr;
+    const bool fp64 = ctx->opt.precision == 1;
+    CKS(group_points(ctx, points, nullptr, owner, np, ctx->ff.ready, fp64, tmp, gr));
     Staged oo;
-    CKS(stage_out_alloc(ctx, oo, out, (size_t)nrhs * np * D));
-    float4 *t4_d = nullptr;
-    int *order_d = nullptr, *tbody_d = nullptr;
-    double *t64_d = nullptr, *sorted_d = nullptr, *tmp_d = nullptr, *raw_d = nullptr;
-    PairPlan plan;
-    auto cleanup = [&]() {
-        cudaStreamSynchronize(st);
-        void *ps[] = {t4_d, order_d, tbody_d, t64_d, sorted_d, tmp_d, raw_d};
-        for (void *p : ps) ctx->release(p);
-        if (plan.tiles) release_plan(ctx, plan);
-    };
-    mfs_status rc = [&]() -> mfs_status {
-        CK(ctx->alloc(&t4_d, np));
-        CK(ctx->alloc(&order_d, np));
-        CK(ctx->alloc(&tbody_d, np));
-        CK(ctx->alloc(&sorted_d, (size_t)nrhs * np * D));
-        CK(ctx->alloc(&tmp_d, (size_t)nrhs * ctx->sumN * D));
-        CK(cudaMemcpyAsync(t4_d, t4.data(), sizeof(float4) * np, cudaMemcpyHostToDevice, st));
-        CK(cudaMemcpyAsync(order_d, order.data(), sizeof(int) * np, cudaMemcpyHostToDevice, st));
-        CK(cudaMemcpyAsync(tbody_d, tbody.data(), sizeof(int) * np, cudaMemcpyHostToDevice, st));
-        CKS(last_strengths(ctx, nrhs, tmp_d, st));
-        const double scale = kernel_scale(ctx);
-        if (ctx->opt.precision == 1) {  // FP64 direct sums
-            CK(ctx->alloc(&t64_d, 3 * (size_t)np));
-            const int S = fp64_chunks(ctx, np);
-            CK(ctx->alloc(&raw_d, (size_t)S * nrhs * np * D));
-            CK(cudaMemcpyAsync(t64_d, t64.data(), sizeof(double) * t64.size(), cudaMemcpyHostToDevice, st));
-            CK(pair_sum_fp64(D, nrhs, S, t64_d, tbody_d, np, ctx->src_local4_d, ctx->sumN, ctx->susp_src_begin_d,
-                             ctx->susp_src_end_d, ctx->src_off_d, ctx->centres_d, ctx->lam_d, 1, raw_d, st));
-            const size_t n = (size_t)nrhs * np * D;
-            combine_raw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(raw_d, nullptr, 0.0, scale, sorted_d, n,
-                                                                            S);
-            CK(cudaGetLastError());
-        } else {  // the FP32 pair kernel on the new targets, all pairs of the owner's suspension
-            const int variant = fp32_variant(ctx, D, nrhs);
-            if (variant < 0) {
-                ctx->last_error = "no pair-kernel variant for this nrhs";
-                return MFS_ERR_INVALID_ARG;
-            }
-            if (ctx->ff.ready) {  // through the treecode
-                CKS(ff_points(ctx, variant, et, nullptr, nrhs, D, scale, sorted_d, st));
-            } else {
-                CKS(build_plan_for(ctx, variant, 1, toff, tbody, ctx->blk_off, np, plan));
-                int vc = 0;
-                const PairVariant *vv = pair_variants(&vc);
-                CK(pack_sources(D, nrhs, vv[variant].packed, ctx->src_pos_d, ctx->rec_pt_d, ctx->lam_d, ctx->sumN,
-                                ctx->nrec, ctx->rec_d, st));
-                PairGeom g = geom_of(ctx);
-                g.tgt = t4_d;
-                g.ntargets = np;
-                const PairWork w = work_of(plan);
-                if (w.total_units > 0) CK(pair_launch(variant, g, w, ctx->err_d, st));
-                CK(pair_epilogue(D, nrhs, w, nullptr, 0.0, scale, sorted_d, np, st));
-            }
-        }
+    CKS(stage_out_alloc(ctx, oo, out, (size_t)nrhs * np * D, st));
+    double *tmp_d = nullptr;
+    CK(tmp.alloc(&tmp_d, (size_t)nrhs * ctx->sumN * D));
+    CKS(last_strengths(ctx, nrhs, tmp_d, st));
+    const double scale = kernel_scale(ctx);
+    if (fp64) {  // FP64 direct sums
+        double *raw_d = nullptr, *sorted_d = nullptr;
+        const int S = fp64_chunks(ctx, np);
+        CK(tmp.alloc(&raw_d, (size_t)S * nrhs * np * D));
+        CK(tmp.alloc(&sorted_d, (size_t)nrhs * np * D));
+        CK(pair_sum_fp64(D, nrhs, S, gr.t64, gr.tbody, np, ctx->src_local4_d, ctx->sumN, ctx->susp_src_begin_d,
+                         ctx->susp_src_end_d, ctx->src_off_d, ctx->centres_d, ctx->lam_d, 1, raw_d, st));
         const size_t n = (size_t)nrhs * np * D;
-        unsort_kernel<<<(unsigned)std::min<size_t>((n + 255) / 256, 4096), 256, 0, st>>>(sorted_d, order_d, np, D,
+        combine_raw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(raw_d, nullptr, 0.0, scale, sorted_d, n, S);
+        CK(cudaGetLastError());
+        unsort_kernel<<<(unsigned)std::min<size_t>((n + 255) / 256, 4096), 256, 0, st>>>(sorted_d, gr.order, np, D,
                                                                                           nrhs, oo.d);
         CK(cudaGetLastError());
-        CKS(stage_out_finish(ctx, oo, st));
-        return check_device_error(ctx, st);
-    }();
-    cleanup();
-    return rc;
+    } else {  // the FP32 pair kernel on the new targets, all pairs of the owner's suspension
+        const int variant = fp32_variant(ctx, D, nrhs);
+        if (variant < 0) {
+            ctx->last_error = "no pair-kernel variant for this nrhs";
+            return MFS_ERR_INVALID_ARG;
+        }
+        if (ctx->ff.ready) {  // through the treecode
+            CKS(ff_points(ctx, variant, gr, np, nrhs, D, scale, oo.d, tmp));
+        } else {
+            int vc = 0;
+            const PairVariant *vv = pair_variants(&vc);
+            PairPlan plan;
+            CKS(build_plan_for(ctx, variant, 1, gr.toff, ctx->blk_off, np, plan, &tmp));
+            CK(pack_sources(D, nrhs, vv[variant].packed, ctx->src_pos_d, ctx->rec_pt_d, ctx->lam_d, ctx->sumN,
+                            ctx->nrec, ctx->rec_d, st));
+            PairGeom g = geom_of(ctx);
+            g.tgt = gr.t4;
+            g.ntargets = np;
+            PairWork w = work_of(plan);
+            w.tperm = gr.order;  // the epilogue writes in the caller's order
+            if (w.total_units > 0) CK(pair_launch(variant, g, w, ctx->err_d, st));
+            CK(pair_epilogue(D, nrhs, w, nullptr, 0.0, scale, oo.d, np, st));
+        }
+    }
+    CKS(stage_out_finish(ctx, oo, st));
+    return check_device_error(ctx, st);
 }
 
 }  // extern "C"
@@ -3550,104 +3549,75 @@ mfs_status mfs_evaluate_stress(mfs_ctx *ctx, const double *points, const double 
     if (npoints == 0) return MFS_OK;
     cudaStream_t st = (cudaStream_t)stream;
     const int P = ctx->P, np = npoints;
-    EvalTargets et;
-    CKS(group_targets(ctx, points, traction ? normals : nullptr, owner, np, et));
-    // per body: the body range of its suspension
-    std::vector<int> sb0(P), sb1(P);
-    for (int s = 0; s < ctx->S; ++s)
-        for (int k = ctx->body_off[s]; k < ctx->body_off[s + 1]; ++k) {
-            sb0[k] = ctx->body_off[s];
-            sb1[k] = ctx->body_off[s + 1];
-        }
+    Scratch tmp(ctx, st);
+    Grouped gr;
+    const bool fp64 = ctx->opt.precision == 1;
+    CKS(group_points(ctx, points, traction ? normals : nullptr, owner, np, ctx->ff.ready, fp64, tmp, gr));
     Staged po, to;
-    if (pressure) CKS(stage_out_alloc(ctx, po, pressure, (size_t)nrhs * np));
-    if (traction) CKS(stage_out_alloc(ctx, to, traction, (size_t)nrhs * np * 3));
-    float4 *t4_d = nullptr;
-    float *n32_d = nullptr;
-    int *order_d = nullptr, *tbody_d = nullptr, *sb0_d = nullptr, *sb1_d = nullptr;
-    double *t64_d = nullptr, *n64_d = nullptr, *ps_d = nullptr, *ts_d = nullptr, *tmp_d = nullptr, *o4_d = nullptr;
-    PairPlan splan;
-    auto cleanup = [&]() {
-        cudaStreamSynchronize(st);
-        void *ps[] = {t4_d, n32_d, order_d, tbody_d, sb0_d, sb1_d, t64_d, n64_d, ps_d, ts_d, tmp_d, o4_d};
-        for (void *p : ps) ctx->release(p);
-        if (splan.tiles) release_plan(ctx, splan);
-    };
-    mfs_status rc = [&]() -> mfs_status {
-        CK(ctx->alloc(&order_d, np));
-        CK(ctx->alloc(&sb0_d, P));
-        CK(ctx->alloc(&sb1_d, P));
-        CK(ctx->alloc(&tmp_d, (size_t)nrhs * ctx->sumN * 3));
-        if (pressure) CK(ctx->alloc(&ps_d, (size_t)nrhs * np));
-        if (traction) CK(ctx->alloc(&ts_d, (size_t)nrhs * np * 3));
-        CK(cudaMemcpyAsync(order_d, et.order.data(), sizeof(int) * np, cudaMemcpyHostToDevice, st));
-        CK(cudaMemcpyAsync(sb0_d, sb0.data(), sizeof(int) * P, cudaMemcpyHostToDevice, st));
-        CK(cudaMemcpyAsync(sb1_d, sb1.data(), sizeof(int) * P, cudaMemcpyHostToDevice, st));
-        CKS(last_strengths(ctx, nrhs, tmp_d, st));
-        if (ctx->opt.precision == 1) {
-            CK(ctx->alloc(&t64_d, 3 * (size_t)np));
-            CK(ctx->alloc(&tbody_d, np));
-            CK(cudaMemcpyAsync(t64_d, et.t64.data(), sizeof(double) * et.t64.size(), cudaMemcpyHostToDevice, st));
-            CK(cudaMemcpyAsync(tbody_d, et.tbody.data(), sizeof(int) * np, cudaMemcpyHostToDevice, st));
-            if (traction) {
-                CK(ctx->alloc(&n64_d, 3 * (size_t)np));
-                CK(cudaMemcpyAsync(n64_d, et.nrm64.data(), sizeof(double) * et.nrm64.size(), cudaMemcpyHostToDevice,
-                                   st));
+    if (pressure) CKS(stage_out_alloc(ctx, po, pressure, (size_t)nrhs * np, st));
+    if (traction) CKS(stage_out_alloc(ctx, to, traction, (size_t)nrhs * np * 3, st));
+    double *tmp_d = nullptr;
+    CK(tmp.alloc(&tmp_d, (size_t)nrhs * ctx->sumN * 3));
+    CKS(last_strengths(ctx, nrhs, tmp_d, st));
+    if (fp64) {
+        // per body: the body range of its suspension
+        std::vector<int> sb0(P), sb1(P);
+        for (int s = 0; s < ctx->S; ++s)
+            for (int k = ctx->body_off[s]; k < ctx->body_off[s + 1]; ++k) {
+                sb0[k] = ctx->body_off[s];
+                sb1[k] = ctx->body_off[s + 1];
             }
-            CK(stress_f64(nrhs, t64_d, tbody_d, n64_d, np, ctx->src_local64_d, ctx->src_off_d, ctx->sumN, ctx->lam_d,
-                          sb0_d, sb1_d, ctx->centres_d, ps_d, ts_d, st));
-        } else {  // the stress entry of the pair kernel (p, T per rhs), directly or through the treecode
-            const int sv = stress_variant(nrhs);
-            if (sv < 0) {
-                ctx->last_error = "no stress kernel for this nrhs";
-                return MFS_ERR_INVALID_ARG;
-            }
-            CK(ctx->alloc(&o4_d, (size_t)nrhs * np * 4));
-            const double scale = 1.0 / (4.0 * MFS_PI);
-            if (ctx->ff.ready) {
-                CKS(ff_points(ctx, sv, et, traction ? et.nrm32.data() : nullptr, nrhs, 4, scale, o4_d, st));
-            } else {
-                CK(ctx->alloc(&t4_d, np));
-                CK(cudaMemcpyAsync(t4_d, et.t4.data(), sizeof(float4) * np, cudaMemcpyHostToDevice, st));
-                if (traction) {
-                    CK(ctx->alloc(&n32_d, 3 * (size_t)np));
-                    CK(cudaMemcpyAsync(n32_d, et.nrm32.data(), sizeof(float) * et.nrm32.size(),
-                                       cudaMemcpyHostToDevice, st));
-                }
-                CKS(build_plan_for(ctx, sv, 1, et.toff, et.tbody, ctx->blk_off, np, splan));
-                CK(pack_sources(3, nrhs, 0, ctx->src_pos_d, ctx->rec_pt_d, ctx->lam_d, ctx->sumN, ctx->nrec,
-                                ctx->rec_d, st));
-                PairGeom g = geom_of(ctx);
-                g.tgt = t4_d;
-                g.ntargets = np;
-                g.tgt_w = n32_d;
-                const PairWork w = work_of(splan);
-                if (w.total_units > 0) CK(pair_launch(sv, g, w, ctx->err_d, st));
-                CK(pair_epilogue(4, nrhs, w, nullptr, 0.0, scale, o4_d, np, st));
-            }
-            const size_t n = (size_t)nrhs * np;
-            split_stress_kernel<<<(unsigned)std::min<size_t>((n + 255) / 256, 4096), 256, 0, st>>>(o4_d, n, ps_d,
-                                                                                                  ts_d);
-            CK(cudaGetLastError());
-        }
-        if (pressure) {
-            const size_t n = (size_t)nrhs * np;
-            unsort_kernel<<<(unsigned)std::min<size_t>((n + 255) / 256, 4096), 256, 0, st>>>(ps_d, order_d, np, 1,
+        int *sb0_d = nullptr, *sb1_d = nullptr;
+        double *ps_d = nullptr, *ts_d = nullptr;
+        CK(tmp.alloc(&sb0_d, P));
+        CK(tmp.alloc(&sb1_d, P));
+        if (pressure) CK(tmp.alloc(&ps_d, (size_t)nrhs * np));
+        if (traction) CK(tmp.alloc(&ts_d, (size_t)nrhs * np * 3));
+        CK(tmp.upload(sb0_d, std::move(sb0)));
+        CK(tmp.upload(sb1_d, std::move(sb1)));
+        CK(stress_f64(nrhs, gr.t64, gr.tbody, gr.n64, np, ctx->src_local64_d, ctx->src_off_d, ctx->sumN, ctx->lam_d,
+                      sb0_d, sb1_d, ctx->centres_d, ps_d, ts_d, st));
+        const size_t n = (size_t)nrhs * np;
+        if (pressure)
+            unsort_kernel<<<(unsigned)std::min<size_t>((n + 255) / 256, 4096), 256, 0, st>>>(ps_d, gr.order, np, 1,
                                                                                               nrhs, po.d);
-            CK(cudaGetLastError());
-            CKS(stage_out_finish(ctx, po, st));
+        if (traction)
+            unsort_kernel<<<(unsigned)std::min<size_t>((3 * n + 255) / 256, 4096), 256, 0, st>>>(ts_d, gr.order, np,
+                                                                                                  3, nrhs, to.d);
+        CK(cudaGetLastError());
+    } else {  // the stress entry of the pair kernel (p, T per rhs), directly or through the treecode
+        const int sv = stress_variant(nrhs);
+        if (sv < 0) {
+            ctx->last_error = "no stress kernel for this nrhs";
+            return MFS_ERR_INVALID_ARG;
         }
-        if (traction) {
-            const size_t n = (size_t)nrhs * np * 3;
-            unsort_kernel<<<(unsigned)std::min<size_t>((n + 255) / 256, 4096), 256, 0, st>>>(ts_d, order_d, np, 3,
-                                                                                              nrhs, to.d);
-            CK(cudaGetLastError());
-            CKS(stage_out_finish(ctx, to, st));
+        double *o4_d = nullptr;
+        CK(tmp.alloc(&o4_d, (size_t)nrhs * np * 4));
+        const double scale = 1.0 / (4.0 * MFS_PI);
+        if (ctx->ff.ready) {
+            CKS(ff_points(ctx, sv, gr, np, nrhs, 4, scale, o4_d, tmp));
+        } else {
+            PairPlan plan;
+            CKS(build_plan_for(ctx, sv, 1, gr.toff, ctx->blk_off, np, plan, &tmp));
+            CK(pack_sources(3, nrhs, 0, ctx->src_pos_d, ctx->rec_pt_d, ctx->lam_d, ctx->sumN, ctx->nrec, ctx->rec_d,
+                            st));
+            PairGeom g = geom_of(ctx);
+            g.tgt = gr.t4;
+            g.ntargets = np;
+            g.tgt_w = gr.n32;
+            PairWork w = work_of(plan);
+            w.tperm = gr.order;
+            if (w.total_units > 0) CK(pair_launch(sv, g, w, ctx->err_d, st));
+            CK(pair_epilogue(4, nrhs, w, nullptr, 0.0, scale, o4_d, np, st));
         }
-        return check_device_error(ctx, st);
-    }();
-    cleanup();
-    return rc;
+        const size_t n = (size_t)nrhs * np;
+        split_stress_kernel<<<(unsigned)std::min<size_t>((n + 255) / 256, 4096), 256, 0, st>>>(
+            o4_d, n, pressure ? po.d : nullptr, traction ? to.d : nullptr);
+        CK(cudaGetLastError());
+    }
+    if (pressure) CKS(stage_out_finish(ctx, po, st));
+    if (traction) CKS(stage_out_finish(ctx, to, st));
+    return check_device_error(ctx, st);
 }
 
 }  // extern "C"
