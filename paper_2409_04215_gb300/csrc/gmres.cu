@@ -4,378 +4,559 @@
 // process, Hessenberg matrix and Givens rotations, so independent problems iterate together
 // and stop separately (converged lanes are masked).  Orthogonalisation is classical
 // Gram-Schmidt applied twice (CGS2); every reduction is deterministic (fixed block partials).
+//
+// Work is cut into blocks of one lane each (GmresDev::blk_*, sized on the host so that all blocks have
+// about the same length whatever the lanes' sizes; with a fixed number of blocks per lane, suspensions
+// of 2 to 64 bodies left most SMs waiting for the longest lane).  What bounds the step is latency and
+// the FP64 pipe (2 DFMA per clock per SM), not bandwidth: an iteration was ten launches, each a chain of
+// dependent loads, so it is five here (dot, update, dot, update, finish), and one for short lanes
+// (gm_arnoldi_cluster_kernel).
 #include <algorithm>
+
+#include <cooperative_groups.h>
 
 #include "common.cuh"
 #include "kernels.h"
 
 namespace mfs {
 
-#define GM_THREADS 256
+#define GM_THREADS 512
+#define GM_WARPS (GM_THREADS / 32)
+#define GM_CLUSTER 16  // blocks per cluster of the short-lane form
+#define GM_CHUNK 1024  // and the entries each of them holds
 
-__device__ __forceinline__ double block_sum(double v, double *sh) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    v = (threadIdx.x < blockDim.x / 32) ? sh[threadIdx.x] : 0.0;
-    if (wid == 0)
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    __syncthreads();
-    return v;  // valid in thread 0
-}
-
-__device__ __forceinline__ void lane_chunk(const GmresDev &gd, int l, int b, long long &e0, long long &e1) {
-    const long long s0 = gd.seg_off[l], s1 = gd.seg_off[l + 1], len = s1 - s0;
-    e0 = s0 + len * b / gd.part_blocks;
-    e1 = s0 + len * (b + 1) / gd.part_blocks;
-}
-
-#define MDOT_THREADS 512
-
-// Columns i0 .. i0+G-1 of one block's chunk: part[l][b][i] = sum over the chunk of V[i][e] * w[e].
-// The loop is bound by memory latency, not by the FP64 pipe: 16 warps per block, four elements per
-// step (4 (G + 1) independent loads in flight per thread).  The block's G x MDOT_THREADS partials go
-// to shared memory and warp g adds column g's values in a fixed order (16 per lane, then a shuffle
-// tree): GB300 executes FP64 at about 2 DFMA per clock per SM, so the reduction costs 21 FP64
-// instructions per column per block rather than a shuffle tree per thread and column.
-template <int G>
-__device__ __forceinline__ void mdot_group(const GmresDev &gd, const double *w, long long e0, long long e1, int i0,
-                                           double *sh, double *dst) {
-    double acc[G];
+// Block-wide dots: out[i] = sum over e in [0, len) of V[i n + e] w[e], i = 0 .. cols - 1, in a fixed
+// order.  A warp takes a group of four columns on a part of the elements (w is read once for the four;
+// with few columns the elements are cut into parts so that all 16 warps work); the lanes' partials go to
+// shared memory and are added there, eight lanes to a column: a shuffle tree per warp and column would
+// cost as many FP64 instructions as the dots themselves.  sh: 4 * GM_THREADS doubles.
+__device__ __forceinline__ void block_dots(const double *V, long long n, const double *w, int len, int cols,
+                                           double *sh, double *out) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ng = (cols + 3) / 4;
+    for (int g0 = 0; g0 < ng; g0 += GM_WARPS) {
+        const int groups = min(ng - g0, GM_WARPS), parts = GM_WARPS / groups;
+        const int g = warp / parts, p = warp % parts;
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        if (g < groups) {
+            const int c0 = 4 * (g0 + g), nc = min(4, cols - c0);
+            const int e1 = (int)((long long)len * (p + 1) / parts);
+            const double *Vc = V + (size_t)c0 * n;
+            for (int e = (int)((long long)len * p / parts) + lane; e < e1; e += 128) {
+                double we[4], v[4][4];
 #pragma unroll
-    for (int g = 0; g < G; ++g) acc[g] = 0.0;
-    const double *V = gd.V + (size_t)i0 * gd.n;
-    const long long step = blockDim.x;
-    long long e = e0 + threadIdx.x;
-    for (; e + 3 * step < e1; e += 4 * step) {
-        double we[4], v[G][4];
+                for (int u = 0; u < 4; ++u) we[u] = e + 32 * u < e1 ? w[e + 32 * u] : 0.0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) we[u] = w[e + u * step];
+                for (int c = 0; c < 4; ++c)
 #pragma unroll
-        for (int g = 0; g < G; ++g)
+                    for (int u = 0; u < 4; ++u)
+                        v[c][u] = (c < nc && e + 32 * u < e1) ? Vc[(size_t)c * n + e + 32 * u] : 0.0;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) v[g][u] = V[(size_t)g * gd.n + e + u * step];
+                for (int c = 0; c < 4; ++c)
+                    if (c < nc)
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int g = 0; g < G; ++g) acc[g] = fma(v[g][u], we[u], acc[g]);
-    }
-    for (; e < e1; e += step) {
-        const double we = w[e];
-#pragma unroll
-        for (int g = 0; g < G; ++g) acc[g] = fma(V[(size_t)g * gd.n + e], we, acc[g]);
-    }
-#pragma unroll
-    for (int g = 0; g < G; ++g) sh[g * MDOT_THREADS + threadIdx.x] = acc[g];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int g = warp; g < G; g += nw) {
-        double r = 0.0;
-        for (int k = lane; k < (int)blockDim.x; k += 32) r += sh[g * MDOT_THREADS + k];
-        for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-        if (lane == 0) dst[i0 + g] = r;
-    }
-    __syncthreads();
-}
-
-// part[l][b][i] = sum over chunk b of lane l of V[i][e] * w[e], i = 0..j  (grid: PB x L, MDOT_THREADS
-// threads): groups of 8 columns, then one group of 4, 2 and 1 for the rest (no predicated-off FP64
-// work).
-__global__ void __launch_bounds__(MDOT_THREADS) mdot_kernel(GmresDev gd, const double *w) {
-    const int b = blockIdx.x, l = blockIdx.y;
-    if (!gd.active[l]) return;
-    const int j = *gd.jcur;
-    __shared__ double sh[8 * MDOT_THREADS];
-    long long e0, e1;
-    lane_chunk(gd, l, b, e0, e1);
-    double *dst = gd.part + ((size_t)l * gd.part_blocks + b) * (gd.m + 1);
-    int i0 = 0;
-    for (; i0 + 8 <= j + 1; i0 += 8) mdot_group<8>(gd, w, e0, e1, i0, sh, dst);
-    if (j + 1 - i0 >= 4) { mdot_group<4>(gd, w, e0, e1, i0, sh, dst); i0 += 4; }
-    if (j + 1 - i0 >= 2) { mdot_group<2>(gd, w, e0, e1, i0, sh, dst); i0 += 2; }
-    if (j + 1 - i0 >= 1) mdot_group<1>(gd, w, e0, e1, i0, sh, dst);
-}
-
-// Sum over the block partials of lane l, entry i, by one warp: each lane adds its blocks (four
-// independent loads per step), then a fixed shuffle tree -- the same order every call.
-__device__ __forceinline__ double warp_part_sum(const GmresDev &gd, int l, int i) {
-    const int lane = threadIdx.x & 31;
-    const double *p = gd.part + (size_t)l * gd.part_blocks * (gd.m + 1) + i;
-    const size_t stride = (size_t)(gd.m + 1);
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    int b = lane;
-    for (; b + 96 < gd.part_blocks; b += 128) {
-        s0 += p[(size_t)b * stride];
-        s1 += p[(size_t)(b + 32) * stride];
-        s2 += p[(size_t)(b + 64) * stride];
-        s3 += p[(size_t)(b + 96) * stride];
-    }
-    for (; b < gd.part_blocks; b += 32) s0 += p[(size_t)b * stride];
-    double s = (s0 + s1) + (s2 + s3);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return s;
-}
-
-// hbuf[l][i] (+)= sum_b part[l][b][i]   (grid: L, one warp per entry i <= j, warps striding)
-__global__ void mdot_reduce_kernel(GmresDev gd, double *htmp, int accumulate) {
-    const int l = blockIdx.x;
-    if (!gd.active[l]) return;
-    const int j = *gd.jcur;
-    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i = warp; i <= j; i += nw) {
-        const double s = warp_part_sum(gd, l, i);
-        if ((threadIdx.x & 31) == 0) {
-            htmp[(size_t)l * (gd.m + 1) + i] = s;
-            if (accumulate) gd.hbuf[(size_t)l * (gd.m + 1) + i] += s;
-            else gd.hbuf[(size_t)l * (gd.m + 1) + i] = s;
+                        for (int u = 0; u < 4; ++u) acc[c] = fma(v[c][u], we[u], acc[c]);
+            }
         }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) sh[(c * GM_WARPS + warp) * 32 + lane] = acc[c];
+        __syncthreads();
+        // column 4 g + c: the `parts` warps of group g, 32 values each; 8 lanes add 4 parts values apiece
+        const int per = GM_THREADS / 8;
+        for (int q = threadIdx.x / 8; q < 4 * groups; q += per) {  // 4 groups <= 64 = per: one round
+            const int gg = q / 4, c = q % 4, s8 = threadIdx.x & 7;
+            double r = 0.0;
+            for (int pp = 0; pp < parts; ++pp) {
+                const double *x = sh + (c * GM_WARPS + gg * parts + pp) * 32 + s8;
+                r += (x[0] + x[8]) + (x[16] + x[24]);
+            }
+            const unsigned mask = 0xffu << (threadIdx.x & 24);
+            for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(mask, r, o);
+            const int col = 4 * (g0 + gg) + c;
+            if (s8 == 0 && col < cols) out[col] = r;
+        }
+        __syncthreads();
     }
 }
 
-// w -= sum_{i<=j} htmp[l][i] V[i]   (grid: PB x L).  Four elements per step and eight columns per
-// inner step, so that 32 independent loads are in flight per thread (the kernel is bound by memory
-// latency); each element's sum runs over the columns in order (one FP64 chain per element).
-__global__ void __launch_bounds__(2 * GM_THREADS) update_kernel(GmresDev gd, double *w, const double *htmp) {
-    const int b = blockIdx.x, l = blockIdx.y;
-    if (!gd.active[l]) return;
-    const int j = *gd.jcur;
-    __shared__ double h[1024];
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) h[i] = htmp[(size_t)l * (gd.m + 1) + i];
-    __syncthreads();
-    long long e0, e1;
-    lane_chunk(gd, l, b, e0, e1);
-    const long long step = blockDim.x;
-    long long e = e0 + threadIdx.x;
-    for (; e + 3 * step < e1; e += 4 * step) {
+// w[e] -= sum_{i < cols} h[i] V[i n + e] over e in [0, len); returns the thread's sum of the new w[e]^2
+// (0 unless NORM).  Four elements per thread and eight columns at a time: 32 loads in flight, the last
+// round guarded instead of a remainder loop; each element's sum runs over the columns in order.
+template <bool NORM>
+__device__ __forceinline__ double block_update(const double *V, long long n, double *w, int len, int cols,
+                                               const double *h) {
+    double nrm = 0.0;
+    for (int e = threadIdx.x; e < len; e += 4 * GM_THREADS) {
         double a[4] = {0.0, 0.0, 0.0, 0.0};
-        int i = 0;
-        for (; i + 8 <= j + 1; i += 8) {
-            const double *V = gd.V + (size_t)i * gd.n + e;
+        bool in[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) in[u] = e + u * GM_THREADS < len;
+        for (int i = 0; i < cols; i += 8) {
             double v[8][4];
 #pragma unroll
             for (int g = 0; g < 8; ++g)
 #pragma unroll
-                for (int u = 0; u < 4; ++u) v[g][u] = V[(size_t)g * gd.n + u * step];
+                for (int u = 0; u < 4; ++u)
+                    v[g][u] = (in[u] && i + g < cols) ? V[(size_t)(i + g) * n + e + u * GM_THREADS] : 0.0;
+#pragma unroll
+            for (int g = 0; g < 8; ++g)
+                if (i + g < cols)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) a[u] = fma(h[i + g], v[g][u], a[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (in[u]) {
+                const double x = w[e + u * GM_THREADS] - a[u];
+                w[e + u * GM_THREADS] = x;
+                if (NORM) nrm = fma(x, x, nrm);
+            }
+    }
+    return nrm;
+}
+
+// Sum over the block in a fixed order, valid in every thread.  sh: GM_WARPS doubles.
+__device__ __forceinline__ double block_sum_all(double v, double *sh) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = 0.0;
+    for (int i = 0; i < (int)blockDim.x / 32; ++i) s += sh[i];
+    return s;
+}
+
+// The Givens update of column j for lane l (one thread): hcol[0 .. j] the column's entries, hn the norm
+// of the new Krylov vector, cs, sn the earlier rotations (hcol, cs and sn preferably in shared memory).
+__device__ void givens_lane(const GmresDev &gd, int l, int j, const double *hcol, const double *cs_, const double *sn_,
+                            double h_next) {
+    const int m = gd.m;
+    double *H = gd.H + (size_t)l * (m + 1) * m;  // H[i][jj] at i*m + jj
+    double *cs = gd.cs + (size_t)l * m, *sn = gd.sn + (size_t)l * m, *g = gd.g + (size_t)l * (m + 1);
+    double carry = hcol[0];  // the rotated entry, carried in a register
+    for (int i = 0; i < j; ++i) {
+        const double c = hcol[i + 1];
+        H[i * m + j] = cs_[i] * carry + sn_[i] * c;
+        carry = -sn_[i] * carry + cs_[i] * c;
+    }
+    const double a = carry, c = h_next;
+    const double den = hypot(a, c);
+    const double cj = den > 0.0 ? a / den : 1.0, sj = den > 0.0 ? c / den : 0.0;
+    cs[j] = cj;
+    sn[j] = sj;
+    H[j * m + j] = den;
+    const double gj = g[j], gn = -sj * gj;
+    g[j + 1] = gn;
+    g[j] = cj * gj;
+    gd.iters[l] = j + 1;
+    const double res = fabs(gn) / gd.beta[l];
+    gd.resid[l] = res;
+    int keep = 1;
+    if (!isfinite(res) || !isfinite(den)) {
+        gd.status[l] = 2;  // breakdown
+        keep = 0;
+    } else if (res <= gd.tol || h_next == 0.0 || j + 1 >= m) {
+        keep = 0;
+    }
+    gd.active[l] = keep;
+}
+
+// Called by one block (all threads): done from the lanes' flags, then j += 1 unless done or the basis is
+// full; with a graph conditional handle sets it to whether another iteration follows.
+__device__ void advance_step(const GmresDev &gd, int j, cudaGraphConditionalHandle cond, int cond_valid) {
+    int any = 0;
+    for (int l = threadIdx.x; l < gd.L; l += blockDim.x) any |= *(volatile int *)&gd.active[l];
+    any = __syncthreads_or(any);
+    if (threadIdx.x == 0) {
+        *gd.done = any ? 0 : 1;
+        const int more = any && (j + 1 < gd.m);
+        if (more) *gd.jcur = j + 1;
+        if (cond_valid) cudaGraphSetConditional(cond, more ? 1u : 0u);
+    }
+}
+
+// True in every thread of the block that arrives last of `total` (whose predecessors' writes it sees).
+__device__ __forceinline__ bool last_to_arrive(const GmresDev &gd, unsigned total) {
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(gd.arrive, total - 1) == total - 1;  // wraps to 0 for the next use
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// part[b][i] = sum over block b's chunk of V[i][e] * w[e], i = 0..j
+__global__ void __launch_bounds__(GM_THREADS) gm_dot_kernel(GmresDev gd, const double *w) {
+    const int b = blockIdx.x, l = gd.blk_lane[b];
+    if (!gd.active[l]) return;
+    __shared__ double sh[4 * GM_THREADS];
+    const long long e0 = gd.blk_off[b];
+    block_dots(gd.V + e0, gd.n, w + e0, (int)(gd.blk_off[b + 1] - e0), *gd.jcur + 1, sh,
+               gd.part + (size_t)b * (gd.m + 1));
+}
+
+// h = the lane's dots (its blocks' partials added in order, eight threads to a column); hbuf = or += h;
+// w -= V h; in the second pass also the block's share of ||w||^2.
+template <int PASS>
+__global__ void __launch_bounds__(GM_THREADS) gm_update_kernel(GmresDev gd, double *w) {
+    const int b = blockIdx.x, l = gd.blk_lane[b];
+    if (!gd.active[l]) return;
+    const int cols = *gd.jcur + 1;
+    __shared__ double h[1024];
+    __shared__ double red[GM_WARPS];
+    const int b0 = gd.lane_blk[l], nb = gd.lane_blk[l + 1] - b0;
+    const size_t ld = gd.m + 1;
+    for (int q0 = 0; q0 < cols; q0 += GM_THREADS / 8) {  // uniform trip count
+        const int q = q0 + threadIdx.x / 8, s8 = threadIdx.x & 7;
+        double r = 0.0;
+        if (q < cols) {
+            const double *p = gd.part + (size_t)b0 * ld + q;
+            int i = s8;
+            for (; i + 24 < nb; i += 32) {
+                const double x0 = p[(size_t)i * ld], x1 = p[(size_t)(i + 8) * ld], x2 = p[(size_t)(i + 16) * ld],
+                             x3 = p[(size_t)(i + 24) * ld];
+                r += (x0 + x1) + (x2 + x3);
+            }
+            for (; i < nb; i += 8) r += p[(size_t)i * ld];
+        }
+        for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+        if (q < cols && s8 == 0) {
+            h[q] = r;
+            if (b == b0) {
+                double *hb = gd.hbuf + (size_t)l * ld + q;
+                *hb = PASS ? *hb + r : r;
+            }
+        }
+    }
+    __syncthreads();
+    const long long e0 = gd.blk_off[b];
+    const double s = block_update<PASS == 1>(gd.V + e0, gd.n, w + e0, (int)(gd.blk_off[b + 1] - e0), cols, h);
+    if (PASS == 1) {
+        const double t = block_sum_all(s, red);
+        if (threadIdx.x == 0) gd.normp[b] = t;
+    }
+}
+
+// normp[b] = block b's share of ||x||^2 (all lanes)
+__global__ void __launch_bounds__(GM_THREADS) gm_norm_kernel(GmresDev gd, const double *x) {
+    const int b = blockIdx.x;
+    __shared__ double red[GM_WARPS];
+    const long long e0 = gd.blk_off[b], e1 = gd.blk_off[b + 1];
+    double s = 0.0;
+    for (long long e = e0 + threadIdx.x; e < e1; e += GM_THREADS) s = fma(x[e], x[e], s);
+    s = block_sum_all(s, red);
+    if (threadIdx.x == 0) gd.normp[b] = s;
+}
+
+// The lane's norm from its blocks' shares, the same in every block of the lane.
+__device__ __forceinline__ double lane_norm(const GmresDev &gd, int l) {
+    __shared__ double nrm;
+    if (threadIdx.x < 32) {
+        double s = 0.0;
+        for (int i = gd.lane_blk[l] + threadIdx.x; i < gd.lane_blk[l + 1]; i += 32) s += gd.normp[i];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) nrm = sqrt(s);
+    }
+    __syncthreads();
+    return nrm;
+}
+
+// The start: v_0 = b / ||b|| (also to vin, the fixed input of the next matvec), the lanes' states,
+// j = 0, done = (no lane active).
+__global__ void __launch_bounds__(GM_THREADS) gm_start_kernel(GmresDev gd, const double *x, double *vin) {
+    const int b = blockIdx.x, l = gd.blk_lane[b];
+    const double nrm = lane_norm(gd, l);
+    const double inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
+    for (long long e = gd.blk_off[b] + threadIdx.x; e < gd.blk_off[b + 1]; e += GM_THREADS) {
+        const double v = x[e] * inv;
+        gd.V[e] = v;
+        vin[e] = v;
+    }
+    if (b == gd.lane_blk[l] && threadIdx.x == 0) {
+        gd.beta[l] = nrm;
+        gd.g[(size_t)l * (gd.m + 1)] = nrm;
+        gd.active[l] = (nrm > 0.0 && isfinite(nrm)) ? 1 : 0;
+        gd.iters[l] = 0;
+        gd.resid[l] = (nrm > 0.0) ? 1.0 : 0.0;
+        gd.status[l] = isfinite(nrm) ? 0 : 2;
+    }
+    if (last_to_arrive(gd, gridDim.x)) {
+        int any = 0;
+        for (int k = threadIdx.x; k < gd.L; k += blockDim.x) any |= *(volatile int *)&gd.active[k];
+        any = __syncthreads_or(any);
+        if (threadIdx.x == 0) {
+            *gd.done = any ? 0 : 1;
+            *gd.jcur = 0;
+        }
+    }
+}
+
+// v_{j+1} = w / ||w|| to the basis and to vin; the first block of each lane updates its Hessenberg column;
+// with `advance` the last block to finish moves to the next column.
+__global__ void __launch_bounds__(GM_THREADS) gm_finish_kernel(GmresDev gd, const double *w, double *vin, int advance) {
+    const int b = blockIdx.x, l = gd.blk_lane[b], j = *gd.jcur;
+    __shared__ double hs[3][1024];
+    // one read for the block: the lane's first block may clear the flag meanwhile
+    const int active = __syncthreads_or(threadIdx.x == 0 ? gd.active[l] : 0);
+    if (active) {
+        const double nrm = lane_norm(gd, l);
+        const bool first = b == gd.lane_blk[l];
+        if (first) {  // the loads of the serial update ahead of it
+            for (int i = threadIdx.x; i <= j; i += GM_THREADS) {
+                hs[0][i] = gd.hbuf[(size_t)l * (gd.m + 1) + i];
+                hs[1][i] = gd.cs[(size_t)l * gd.m + i];
+                hs[2][i] = gd.sn[(size_t)l * gd.m + i];
+            }
+        }
+        const double inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
+        double *v = gd.V + (size_t)(j + 1) * gd.n;
+        for (long long e = gd.blk_off[b] + threadIdx.x; e < gd.blk_off[b + 1]; e += GM_THREADS) {
+            const double x = w[e] * inv;
+            v[e] = x;
+            vin[e] = x;
+        }
+        __syncthreads();
+        // a block of the lane that starts after its flag was cleared here skips its share of v_{j+1}, which
+        // a stopped lane does not use
+        if (first && threadIdx.x == 0) givens_lane(gd, l, j, hs[0], hs[1], hs[2], nrm);
+    }
+    if (advance && last_to_arrive(gd, gridDim.x)) advance_step(gd, j, cudaGraphConditionalHandle(), 0);
+}
+
+// j += 1 or stop, and the while node's condition (a graph iteration's last kernel; one block)
+__global__ void gm_advance_kernel(GmresDev gd, cudaGraphConditionalHandle cond, int cond_valid) {
+    advance_step(gd, *gd.jcur, cond, cond_valid);
+}
+
+// The whole Arnoldi step of one short lane by one cluster of GM_CLUSTER blocks: w stays in shared memory,
+// the dots and the norm are exchanged through distributed shared memory, and the five launches of the
+// long-lane form (each at least a launch and a chain of dependent loads, about 5 us) become one.  For
+// lanes of at most GM_CLUSTER * GM_CHUNK entries: beyond that the FP64 pipes of 16 SMs take longer than
+// the launches saved (at j = 15, 16384 entries: 4 us a pass).
+// Whole solves with this file's kernels against the ten-launch form: two conductors (1200 entries) 709 ->
+// 549 us, six spheres (4320) 1610 -> 1308 us; five launches: 40 spheroids (119 640 entries, 76 columns)
+// 51.8 -> 46.2 ms, 48 uneven lanes 125.0 -> 119.9 ms.
+__global__ void __launch_bounds__(GM_THREADS) gm_arnoldi_cluster_kernel(GmresDev gd, const double *w, double *vin,
+                                                                        int advance) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int l = blockIdx.y, rank = blockIdx.x, j = *gd.jcur, cols = j + 1, m1 = gd.m + 1;
+    extern __shared__ double dyn[];
+    double *sh = dyn, *wb = sh + 4 * GM_THREADS, *pa = wb + GM_CHUNK, *pb = pa + m1, *h = pb + m1, *hc = h + m1,
+           *cs = hc + m1, *sn = cs + m1;
+    __shared__ double red[GM_WARPS], pn;
+    if (gd.active[l]) {
+        const long long s0 = gd.blk_off[gd.lane_blk[l]], s1 = gd.blk_off[gd.lane_blk[l + 1]];
+        const long long e0 = s0 + (s1 - s0) * rank / GM_CLUSTER;
+        const int len = (int)(s0 + (s1 - s0) * (rank + 1) / GM_CLUSTER - e0);
+        const double *V = gd.V + e0;
+        for (int e = threadIdx.x; e < len; e += GM_THREADS) wb[e] = w[e0 + e];
+        if (rank == 0)
+            for (int i = threadIdx.x; i < j; i += GM_THREADS) {
+                cs[i] = gd.cs[(size_t)l * gd.m + i];
+                sn[i] = gd.sn[(size_t)l * gd.m + i];
+            }
+        __syncthreads();
+        block_dots(V, gd.n, wb, len, cols, sh, pa);
+        cl.sync();
+        for (int i = threadIdx.x; i < cols; i += GM_THREADS) {
+            double s = 0.0;
+            for (int r = 0; r < GM_CLUSTER; ++r) s += cl.map_shared_rank(pa, r)[i];
+            h[i] = hc[i] = s;
+        }
+        __syncthreads();
+        block_update<false>(V, gd.n, wb, len, cols, h);
+        __syncthreads();
+        block_dots(V, gd.n, wb, len, cols, sh, pb);
+        cl.sync();
+        for (int i = threadIdx.x; i < cols; i += GM_THREADS) {
+            double s = 0.0;
+            for (int r = 0; r < GM_CLUSTER; ++r) s += cl.map_shared_rank(pb, r)[i];
+            h[i] = s;
+            hc[i] += s;
+        }
+        __syncthreads();
+        const double t = block_sum_all(block_update<true>(V, gd.n, wb, len, cols, h), red);
+        if (threadIdx.x == 0) pn = t;
+        cl.sync();
+        double s = 0.0;
+        for (int r = 0; r < GM_CLUSTER; ++r) s += *cl.map_shared_rank(&pn, r);
+        const double nrm = sqrt(s), inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
+        double *v = gd.V + (size_t)(j + 1) * gd.n + e0;
+        for (int e = threadIdx.x; e < len; e += GM_THREADS) {
+            const double x = wb[e] * inv;
+            v[e] = x;
+            vin[e0 + e] = x;
+        }
+        if (rank == 0 && threadIdx.x == 0) givens_lane(gd, l, j, hc, cs, sn, nrm);
+        cl.sync();  // no block leaves while another reads its shared memory
+    }
+    if (advance && rank == 0 && last_to_arrive(gd, gd.L)) advance_step(gd, j, cudaGraphConditionalHandle(), 0);
+}
+
+// x = sum_{i<k_l} y_l[i] V[i] with H_l y = g_l (upper triangular, k_l columns): every block solves its
+// lane's triangle itself (one warp, the triangle in shared memory, column by column with the diagonal's
+// reciprocals taken beforehand; one thread walking it in global memory took 250 us at 76 columns), then
+// combines its chunk with 32 loads in flight per thread.
+#define GM_TRI 144  // columns whose triangle fits the block's shared memory (83 KB)
+__global__ void __launch_bounds__(GM_THREADS) gm_solution_kernel(GmresDev gd, double *x) {
+    extern __shared__ double tri[];  // row i of the triangle (columns i .. k - 1) packed by column: c (c + 1) / 2 + i
+    __shared__ double y[1024], dinv[1024];
+    const int b = blockIdx.x, l = gd.blk_lane[b], k = gd.iters[l], m = gd.m;
+    const double *H = gd.H + (size_t)l * (m + 1) * m;
+    const bool packed = k <= GM_TRI;
+    for (int i = threadIdx.x; i < k; i += GM_THREADS) {
+        const double d = H[(size_t)i * m + i];
+        dinv[i] = d != 0.0 ? 1.0 / d : 0.0;
+        y[i] = gd.g[(size_t)l * (m + 1) + i];
+    }
+    if (packed)
+        for (int i = threadIdx.x >> 5; i < k; i += GM_WARPS)
+            for (int c = i + (threadIdx.x & 31); c < k; c += 32) tri[c * (c + 1) / 2 + i] = H[(size_t)i * m + c];
+    __syncthreads();
+    if (threadIdx.x < 32)
+        for (int c = k - 1; c >= 0; --c) {
+            const double yc = y[c] * dinv[c];
+            __syncwarp();
+            if (threadIdx.x == 0) y[c] = yc;
+            for (int i = threadIdx.x; i < c; i += 32)
+                y[i] = fma(-(packed ? tri[c * (c + 1) / 2 + i] : H[(size_t)i * m + c]), yc, y[i]);
+            __syncwarp();
+        }
+    __syncthreads();
+    const long long e0 = gd.blk_off[b];
+    const int len = (int)(gd.blk_off[b + 1] - e0);
+    const double *V = gd.V + e0;
+    for (int e = threadIdx.x; e < len; e += 4 * GM_THREADS) {
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
+        bool in[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) in[u] = e + u * GM_THREADS < len;
+        for (int i = 0; i < k; i += 8) {
+            double v[8][4];
 #pragma unroll
             for (int g = 0; g < 8; ++g)
 #pragma unroll
-                for (int u = 0; u < 4; ++u) a[u] = fma(h[i + g], v[g][u], a[u]);
-        }
-        for (; i <= j; ++i) {
-            const double *V = gd.V + (size_t)i * gd.n + e;
+                for (int u = 0; u < 4; ++u)
+                    v[g][u] = (in[u] && i + g < k) ? V[(size_t)(i + g) * gd.n + e + u * GM_THREADS] : 0.0;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) a[u] = fma(h[i], V[u * step], a[u]);
+            for (int g = 0; g < 8; ++g)
+                if (i + g < k)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) a[u] = fma(y[i + g], v[g][u], a[u]);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) w[e + u * step] -= a[u];
-    }
-    for (; e < e1; e += step) {
-        double a = 0.0;
-        for (int i = 0; i <= j; ++i) a = fma(h[i], gd.V[(size_t)i * gd.n + e], a);
-        w[e] -= a;
+        for (int u = 0; u < 4; ++u)
+            if (in[u]) x[e0 + e + u * GM_THREADS] = a[u];
     }
 }
 
-// part[l][b][0] = sum over chunk of x*x  (norms)
-__global__ void norm_part_kernel(GmresDev gd, const double *x, int all_lanes) {
-    const int b = blockIdx.x, l = blockIdx.y;
-    if (!all_lanes && !gd.active[l]) return;
-    __shared__ double sh[32];
-    long long e0, e1;
-    lane_chunk(gd, l, b, e0, e1);
-    // four elements per step: independent loads in flight (the loop is bound by memory latency)
-    const long long step = blockDim.x;
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    long long e = e0 + threadIdx.x;
-    for (; e + 3 * step < e1; e += 4 * step) {
-        const double x0 = x[e], x1 = x[e + step], x2 = x[e + 2 * step], x3 = x[e + 3 * step];
-        a0 = fma(x0, x0, a0);
-        a1 = fma(x1, x1, a1);
-        a2 = fma(x2, x2, a2);
-        a3 = fma(x3, x3, a3);
+bool gmres_plan_blocks(const std::vector<long long> &seg, int sm_count, std::vector<int> &blk_lane,
+                       std::vector<long long> &blk_off, std::vector<int> &lane_blk) {
+    const int L = (int)seg.size() - 1;
+    long long longest = 0;
+    for (int l = 0; l < L; ++l) longest = std::max(longest, seg[l + 1] - seg[l]);
+    auto blocks = [&](long long chunk) {
+        long long t = 0;
+        for (int l = 0; l < L; ++l) t += std::max<long long>(1, (seg[l + 1] - seg[l] + chunk - 1) / chunk);
+        return t;
+    };
+    // the shortest chunk (in steps of 256, at least 2048) whose blocks fill whole waves: one wave, or two
+    // blocks per lane on average when the lanes alone are more than the SMs
+    const long long want = L <= sm_count / 2 ? sm_count : (2LL * L + sm_count - 1) / sm_count * sm_count;
+    long long lo = 8, hi = std::max<long long>(9, (longest + 255) / 256);
+    while (lo < hi) {
+        const long long mid = (lo + hi) / 2;
+        if (blocks(256 * mid) <= want) hi = mid; else lo = mid + 1;
     }
-    for (; e < e1; e += step) a0 = fma(x[e], x[e], a0);
-    double acc = (a0 + a1) + (a2 + a3);
-    acc = block_sum(acc, sh);
-    if (threadIdx.x == 0) gd.part[((size_t)l * gd.part_blocks + b) * (gd.m + 1)] = acc;
-}
-
-// v_dst = x / ||x|| per lane, norm taken from the partials (grid: PB x L); vdst = V[j+1] when null
-__global__ void normalise_kernel(GmresDev gd, const double *x, double *vdst, double *norm_out, int all_lanes) {
-    const int b = blockIdx.x, l = blockIdx.y;
-    if (!all_lanes && !gd.active[l]) return;
-    if (!vdst) vdst = gd.V + (size_t)(*gd.jcur + 1) * gd.n;
-    __shared__ double nrm_sh;
-    if (threadIdx.x < 32) {  // the first warp sums the block partials of the squared norm
-        const double s = warp_part_sum(gd, l, 0);
-        if (threadIdx.x == 0) nrm_sh = sqrt(s);
-    }
-    __syncthreads();
-    const double nrm = nrm_sh;
-    if (b == 0 && threadIdx.x == 0 && norm_out) norm_out[l] = nrm;
-    const double inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
-    long long e0, e1;
-    lane_chunk(gd, l, b, e0, e1);
-    const long long step = blockDim.x;
-    long long e = e0 + threadIdx.x;
-    for (; e + 3 * step < e1; e += 4 * step) {
-        const double x0 = x[e], x1 = x[e + step], x2 = x[e + 2 * step], x3 = x[e + 3 * step];
-        vdst[e] = x0 * inv;
-        vdst[e + step] = x1 * inv;
-        vdst[e + 2 * step] = x2 * inv;
-        vdst[e + 3 * step] = x3 * inv;
-    }
-    for (; e < e1; e += step) vdst[e] = x[e] * inv;
-}
-
-__global__ void init_lanes_kernel(GmresDev gd) {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= gd.L) return;
-    const double b = gd.beta[l];
-    gd.g[(size_t)l * (gd.m + 1)] = b;
-    gd.active[l] = (b > 0.0 && isfinite(b)) ? 1 : 0;
-    gd.iters[l] = 0;
-    gd.resid[l] = (b > 0.0) ? 1.0 : 0.0;
-    gd.status[l] = isfinite(b) ? 0 : 2;
-}
-
-// done = no lane active, j = 0 (one thread)
-__global__ void init_done_kernel(GmresDev gd) {
-    int any = 0;
-    for (int l = 0; l < gd.L; ++l) any |= gd.active[l];
-    *gd.done = any ? 0 : 1;
-    *gd.jcur = 0;
-}
-
-__global__ void load_vj_kernel(GmresDev gd, double *vin) {
-    const double *v = gd.V + (size_t)(*gd.jcur) * gd.n;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < gd.n; e += (long long)gridDim.x * blockDim.x)
-        vin[e] = v[e];
-}
-
-// After column j: continue with j + 1 unless every lane stopped or the basis is full.
-__global__ void advance_kernel(GmresDev gd, cudaGraphConditionalHandle cond, int cond_valid) {
-    const int j = *gd.jcur;
-    const int more = (*gd.done == 0) && (j + 1 < gd.m);
-    if (more) *gd.jcur = j + 1;
-    if (cond_valid) cudaGraphSetConditional(cond, more ? 1u : 0u);
-}
-
-// Givens update of column j for every active lane; sets done when no lane is active.
-__global__ void givens_kernel(GmresDev gd, const double *hn) {
-    const int l = threadIdx.x;
-    const int j = *gd.jcur;
-    __shared__ int any_active;
-    if (l == 0) any_active = 0;
-    __syncthreads();
-    for (int ll = l; ll < gd.L; ll += blockDim.x) {
-        if (!gd.active[ll]) continue;
-        const int m = gd.m;
-        double *H = gd.H + (size_t)ll * (m + 1) * m;  // H[i][jj] at i*m + jj
-        double *cs = gd.cs + (size_t)ll * m, *sn = gd.sn + (size_t)ll * m, *g = gd.g + (size_t)ll * (m + 1);
-        // column j from hbuf, rotated by the previous Givens rotations with one value carried in a
-        // register (the loads of hbuf, cs and sn do not wait on the chain; H is written once)
-        const double *hcol = gd.hbuf + (size_t)ll * (m + 1);
-        const double h_next = hn[ll];
-        double carry = hcol[0];
-        for (int i = 0; i < j; ++i) {
-            const double c = hcol[i + 1];
-            H[i * m + j] = cs[i] * carry + sn[i] * c;
-            carry = -sn[i] * carry + cs[i] * c;
+    const long long chunk = 256 * lo;
+    blk_lane.clear();
+    blk_off.assign(1, seg[0]);
+    lane_blk.assign(1, 0);
+    for (int l = 0; l < L; ++l) {
+        const long long len = seg[l + 1] - seg[l], nb = std::max<long long>(1, (len + chunk - 1) / chunk);
+        for (long long i = 0; i < nb; ++i) {
+            blk_lane.push_back(l);
+            blk_off.push_back(seg[l] + len * (i + 1) / nb);
         }
-        const double a = carry, c = h_next;
-        const double den = hypot(a, c);
-        cs[j] = den > 0.0 ? a / den : 1.0;
-        sn[j] = den > 0.0 ? c / den : 0.0;
-        H[j * m + j] = den;
-        H[(j + 1) * m + j] = 0.0;
-        g[j + 1] = -sn[j] * g[j];
-        g[j] = cs[j] * g[j];
-        gd.iters[ll] = j + 1;
-        const double res = fabs(g[j + 1]) / gd.beta[ll];
-        gd.resid[ll] = res;
-        int keep = 1;
-        if (!isfinite(res) || !isfinite(den)) {
-            gd.status[ll] = 2;  // breakdown
-            keep = 0;
-        } else if (res <= gd.tol || h_next == 0.0 || j + 1 >= m) {
-            keep = 0;
-        }
-        gd.active[ll] = keep;
-        if (keep) atomicOr(&any_active, 1);
+        lane_blk.push_back((int)blk_lane.size());
     }
-    __syncthreads();
-    if (threadIdx.x == 0) *gd.done = any_active ? 0 : 1;
+    return longest <= (long long)GM_CLUSTER * GM_CHUNK;
 }
 
-// y_l solves the k_l x k_l upper-triangular H_l y = g_l (one thread per lane)
-__global__ void trisolve_kernel(GmresDev gd, double *y) {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= gd.L) return;
-    const int m = gd.m, k = gd.iters[l];
-    const double *H = gd.H + (size_t)l * (m + 1) * m;
-    const double *g = gd.g + (size_t)l * (m + 1);
-    double *yl = y + (size_t)l * (m + 1);
-    for (int i = k - 1; i >= 0; --i) {
-        double s = g[i];
-        for (int c = i + 1; c < k; ++c) s -= H[i * m + c] * yl[c];
-        yl[i] = (H[i * m + i] != 0.0) ? s / H[i * m + i] : 0.0;
-    }
+static size_t cluster_smem(const GmresDev &gd) { return sizeof(double) * (4 * GM_THREADS + GM_CHUNK + 6 * (size_t)(gd.m + 1)); }
+static size_t solution_smem(const GmresDev &gd) {
+    const size_t k = std::min(gd.m, GM_TRI);
+    return sizeof(double) * (k * (k + 1) / 2);
 }
 
-// x = sum_{i<k_l} y_l[i] V[i]  (grid: PB x L)
-__global__ void combine_kernel(GmresDev gd, const double *y, double *x) {
-    const int b = blockIdx.x, l = blockIdx.y;
-    const int k = gd.iters[l];
-    long long e0, e1;
-    lane_chunk(gd, l, b, e0, e1);
-    const double *yl = y + (size_t)l * (gd.m + 1);
-    for (long long e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-        double s = 0.0;
-        for (int i = 0; i < k; ++i) s += yl[i] * gd.V[(size_t)i * gd.n + e];
-        x[e] = s;
+cudaError_t gmres_prepare(GmresDev &gd) {
+    cudaError_t e = cudaFuncSetAttribute(gm_solution_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(sizeof(double) * GM_TRI * (GM_TRI + 1) / 2));
+    if (e != cudaSuccess || !gd.clusters) return e;
+    e = cudaFuncSetAttribute(gm_arnoldi_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(sizeof(double) * (4 * GM_THREADS + GM_CHUNK + 6 * 1024)));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(gm_arnoldi_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    // the device must be able to hold one such cluster, else the long-lane form serves
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = GM_CLUSTER;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(GM_CLUSTER, gd.L);
+    cfg.blockDim = dim3(GM_THREADS);
+    cfg.dynamicSmemBytes = cluster_smem(gd);
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, gm_arnoldi_cluster_kernel, &cfg) != cudaSuccess || n < 1) {
+        cudaGetLastError();
+        gd.clusters = 0;
     }
+    return cudaSuccess;
 }
 
-cudaError_t gmres_init(GmresDev &gd, const double *b, cudaStream_t st) {
-    dim3 grid(gd.part_blocks, gd.L);
-    norm_part_kernel<<<grid, GM_THREADS, 0, st>>>(gd, b, 1);
-    normalise_kernel<<<grid, GM_THREADS, 0, st>>>(gd, b, gd.V, gd.beta, 1);
-    cudaMemsetAsync(gd.H, 0, sizeof(double) * (size_t)gd.L * (gd.m + 1) * gd.m, st);
-    cudaMemsetAsync(gd.g, 0, sizeof(double) * (size_t)gd.L * (gd.m + 1), st);
-    init_lanes_kernel<<<(gd.L + 127) / 128, 128, 0, st>>>(gd);
-    init_done_kernel<<<1, 1, 0, st>>>(gd);
+cudaError_t gmres_init(GmresDev &gd, const double *b, double *vin, cudaStream_t st) {
+    gm_norm_kernel<<<gd.nblk, GM_THREADS, 0, st>>>(gd, b);
+    gm_start_kernel<<<gd.nblk, GM_THREADS, 0, st>>>(gd, b, vin);
     return cudaGetLastError();
 }
 
-cudaError_t gmres_arnoldi(GmresDev &gd, double *w, cudaStream_t st) {
-    dim3 grid(gd.part_blocks, gd.L);
-    for (int pass = 0; pass < 2; ++pass) {  // CGS2
-        mdot_kernel<<<grid, MDOT_THREADS, 0, st>>>(gd, w);
-        mdot_reduce_kernel<<<gd.L, 512, 0, st>>>(gd, gd.htmp, pass);  // 16 warps over the entries i <= j
-        update_kernel<<<grid, 2 * GM_THREADS, 0, st>>>(gd, w, gd.htmp);  // latency-bound: more loads in flight
+int gmres_arnoldi_launches(const GmresDev &gd) { return gd.clusters ? 1 : 5; }
+
+cudaError_t gmres_arnoldi(GmresDev &gd, double *w, double *vin, int advance, cudaStream_t st) {
+    if (gd.clusters) {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = GM_CLUSTER;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(GM_CLUSTER, gd.L);
+        cfg.blockDim = dim3(GM_THREADS);
+        cfg.dynamicSmemBytes = cluster_smem(gd);
+        cfg.stream = st;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, gm_arnoldi_cluster_kernel, gd, (const double *)w, vin, advance);
     }
-    norm_part_kernel<<<grid, GM_THREADS, 0, st>>>(gd, w, 0);
-    normalise_kernel<<<grid, GM_THREADS, 0, st>>>(gd, w, nullptr, gd.hn, 0);
-    givens_kernel<<<1, 256, 0, st>>>(gd, gd.hn);
+    gm_dot_kernel<<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);  // CGS2
+    gm_update_kernel<0><<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
+    gm_dot_kernel<<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
+    gm_update_kernel<1><<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
+    gm_finish_kernel<<<gd.nblk, GM_THREADS, 0, st>>>(gd, w, vin, advance);
     return cudaGetLastError();
 }
 
-cudaError_t gmres_load_vj(GmresDev &gd, double *vin, cudaStream_t st) {
-    load_vj_kernel<<<1024, 256, 0, st>>>(gd, vin);
+cudaError_t gmres_advance(GmresDev &gd, cudaGraphConditionalHandle cond, cudaStream_t st) {
+    gm_advance_kernel<<<1, 256, 0, st>>>(gd, cond, 1);
     return cudaGetLastError();
 }
 
-cudaError_t gmres_advance(GmresDev &gd, cudaGraphConditionalHandle cond, int cond_valid, cudaStream_t st) {
-    advance_kernel<<<1, 1, 0, st>>>(gd, cond, cond_valid);
-    return cudaGetLastError();
-}
-
-cudaError_t gmres_solution(GmresDev &gd, double *x, double *y_small, cudaStream_t st) {
-    trisolve_kernel<<<(gd.L + 127) / 128, 128, 0, st>>>(gd, y_small);
-    dim3 grid(gd.part_blocks, gd.L);
-    combine_kernel<<<grid, GM_THREADS, 0, st>>>(gd, y_small, x);
+cudaError_t gmres_solution(GmresDev &gd, double *x, cudaStream_t st) {
+    gm_solution_kernel<<<gd.nblk, GM_THREADS, solution_smem(gd), st>>>(gd, x);
     return cudaGetLastError();
 }
 

@@ -251,18 +251,23 @@ void ff_cell_lists(const FFTree &t, int root, const std::vector<int> &tbodies, c
 // degree -1).
 cudaError_t ff_scale(double *mu, const double *re, int nodes, int per_node, int nrhs, cudaStream_t st);
 
-// ---- GMRES (gmres.cu): L independent lanes, lane l owns vector entries [seg_off[l], seg_off[l+1]) ----
+// ---- GMRES (gmres.cu): L independent lanes, lane l owns vector entries [seg[l], seg[l+1]) ----
 struct GmresDev {
     int L, m;                  // lanes, Krylov basis capacity (m <= 1023)
     long long n;               // vector length (all lanes)
-    const long long *seg_off;  // [L+1] (device)
+    int nblk;                  // blocks of the long-lane kernels, each within one lane
+    const int *blk_lane;       // [nblk] the block's lane
+    const long long *blk_off;  // [nblk+1] its first entry (blocks are contiguous)
+    const int *lane_blk;       // [L+1] the lane's first block
+    int clusters;              // 1: every lane is short enough for the one-launch Arnoldi step
     double *V;                 // [(m+1)][n] basis
     double *H;                 // [L][m+1][m] Hessenberg, rotated to upper triangular
     double *cs, *sn, *g;       // [L][m], [L][m], [L][m+1]
     double *beta;              // [L] ||b||
-    double *hbuf, *htmp;       // [L][m+1] current column, current CGS pass
-    double *hn;                // [L] norm of the new Krylov vector
-    double *part;              // [L][part_blocks][m+1] block partials
+    double *hbuf;              // [L][m+1] current column
+    double *part;              // [nblk][m+1] block partials of the dots
+    double *normp;             // [nblk] block partials of the norm
+    unsigned *arrive;          // [1] blocks done (wraps to 0)
     int *active;               // [L] 1 while the lane iterates
     int *iters;                // [L] iterations done
     int *status;               // [L] 0 ok, 2 breakdown (non-finite)
@@ -270,19 +275,24 @@ struct GmresDev {
     int *done;                 // [1] 1 when no lane is active
     int *jcur;                 // [1] the current Arnoldi column j (device-side, so a graph can loop)
     double tol;
-    int part_blocks;           // blocks per lane in the reductions
 };
-// Start: v_0 = b / ||b|| per lane, lanes with b = 0 inactive, j = 0, done = (no lane active).
-cudaError_t gmres_init(GmresDev &gd, const double *b, cudaStream_t st);
-// Orthogonalise w = A v_j against v_0..v_j (CGS2), append v_{j+1}, Givens-update every active lane;
-// j is read from gd.jcur.
-cudaError_t gmres_arnoldi(GmresDev &gd, double *w, cudaStream_t st);
-// vin = v_j (j from gd.jcur): the input of the next matvec at a fixed address.
-cudaError_t gmres_load_vj(GmresDev &gd, double *vin, cudaStream_t st);
-// j += 1 unless done or the basis is full; with a graph conditional handle (cond_valid), sets it to
-// whether another iteration follows.
-cudaError_t gmres_advance(GmresDev &gd, cudaGraphConditionalHandle cond, int cond_valid, cudaStream_t st);
-// x = V y with H y = g per lane (y_small: [L][m+1] scratch).
-cudaError_t gmres_solution(GmresDev &gd, double *x, double *y_small, cudaStream_t st);
+// The blocks of lanes seg[0..L]: about equal lengths, whole waves of the SMs; returns whether every lane
+// is short enough for the one-launch step.
+bool gmres_plan_blocks(const std::vector<long long> &seg, int sm_count, std::vector<int> &blk_lane,
+                       std::vector<long long> &blk_off, std::vector<int> &lane_blk);
+// Kernel attributes for this basis; clears gd.clusters when the device cannot hold the cluster.
+cudaError_t gmres_prepare(GmresDev &gd);
+// Start (two launches): v_0 = b / ||b|| per lane, also to vin (the matvec's input at a fixed address),
+// lanes with b = 0 inactive, j = 0, done = (no lane active).
+cudaError_t gmres_init(GmresDev &gd, const double *b, double *vin, cudaStream_t st);
+// Orthogonalise w = A v_j against v_0..v_j (CGS2), append v_{j+1} (also to vin), Givens-update every
+// active lane; j is read from gd.jcur and, with advance, increased unless done or the basis is full.
+cudaError_t gmres_arnoldi(GmresDev &gd, double *w, double *vin, int advance, cudaStream_t st);
+int gmres_arnoldi_launches(const GmresDev &gd);
+// The advance as a kernel of its own that also sets a while node's condition to whether another
+// iteration follows.
+cudaError_t gmres_advance(GmresDev &gd, cudaGraphConditionalHandle cond, cudaStream_t st);
+// x = V y with H y = g per lane.
+cudaError_t gmres_solution(GmresDev &gd, double *x, cudaStream_t st);
 
 }  // namespace mfs

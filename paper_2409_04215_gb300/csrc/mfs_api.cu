@@ -93,7 +93,7 @@ struct mfs_ctx {
         int launches = 0, pair_launches = 0;  // per iteration
     };
     std::map<int, SolveGraph> graphs;
-    double *vin_d = nullptr;  // matvec input of a graph iteration (v_j copied to a fixed address)
+    double *vin_d = nullptr;  // matvec input of every iteration (v_j at a fixed address)
     cudaStream_t cap_stream = nullptr;  // capture only (the legacy stream cannot capture); launches use the caller's
     void drop_graphs() {
         for (auto &kv : graphs) {
@@ -138,9 +138,10 @@ struct mfs_ctx {
     GmresDev gd{};
     size_t gd_n = 0;
     int gd_L = 0, gd_m = 0;
-    long long *seg_off_d = nullptr;
-    double *w_d = nullptr, *b_d = nullptr, *x_d = nullptr, *ysmall_d = nullptr;
-    int *done_h = nullptr;
+    double *w_d = nullptr, *b_d = nullptr, *x_d = nullptr;
+    unsigned char *stat_d = nullptr, *stat_h = nullptr;  // the solve's statistics, device and pinned host
+    static size_t stat_bytes(int L) { return sizeof(double) * L + sizeof(int) * (2 * (size_t)L + 4); }
+    int *done_h = nullptr;   // pinned: [0] done, [1] the device error flag
 
     // solution kept for the adjoint
     // the last solve, for mfs_mobility_vjp and mfs_evaluate: which problem, its GMRES solution gamma
@@ -265,6 +266,7 @@ struct mfs_ctx {
         if (cap_stream) cudaStreamDestroy(cap_stream);
         for (void *p : allocs) cudaFree(p);
         if (done_h) cudaFreeHost(done_h);
+        if (stat_h) cudaFreeHost(stat_h);
         if (ev0) cudaEventDestroy(ev0);
         if (ev1) cudaEventDestroy(ev1);
         if (evp0) cudaEventDestroy(evp0);
@@ -1243,59 +1245,66 @@ mfs_status ensure_gmres(mfs_ctx *ctx, int nrhs) {
     const int L = nrhs * ctx->S;
     const int m = std::min(ctx->opt.restart, ctx->opt.max_iter);
     if (ctx->gd.V && ctx->gd_n == (size_t)n && ctx->gd_L == L && ctx->gd_m == m) return MFS_OK;
-    // free old
-    void *olds[] = {ctx->gd.V, ctx->gd.H, ctx->gd.cs, ctx->gd.sn, ctx->gd.g, ctx->gd.beta, ctx->gd.hbuf,
-                    ctx->gd.htmp, ctx->gd.hn, ctx->gd.part, ctx->gd.active, ctx->gd.iters, ctx->gd.status,
-                    ctx->gd.resid, ctx->gd.done, ctx->gd.jcur, ctx->seg_off_d, ctx->w_d, ctx->b_d, ctx->x_d,
-                    ctx->ysmall_d, ctx->vin_d};
+    GmresDev &gd = ctx->gd;
+    void *olds[] = {gd.V, gd.H, gd.cs, gd.sn, gd.g, gd.beta, gd.hbuf, gd.part, gd.normp, gd.active, (void *)gd.blk_lane,
+                    (void *)gd.blk_off, (void *)gd.lane_blk, ctx->stat_d, ctx->w_d, ctx->b_d, ctx->x_d, ctx->vin_d};
     ctx->drop_graphs();  // they hold the old buffers' addresses
     for (void *p : olds) ctx->release(p);
-    ctx->vin_d = nullptr;
-    GmresDev &gd = ctx->gd;
+    if (ctx->stat_h) cudaFreeHost(ctx->stat_h);
+    ctx->vin_d = ctx->w_d = ctx->b_d = ctx->x_d = nullptr;
+    ctx->stat_d = ctx->stat_h = nullptr;
     gd = GmresDev{};
     gd.L = L;
     gd.m = m;
     gd.n = n;
     gd.tol = ctx->opt.gmres_tol;
-    // blocks per lane: one wave over all lanes (SMs / L, so that no SM runs two blocks while others
-    // run one), but at least ~2048 elements per block (8 per thread), so that the FP64 work of the dot
-    // products outweighs their block reductions
-    const long long per_lane = n / std::max(L, 1);
-    gd.part_blocks = (int)std::max<long long>(1, std::min<long long>((long long)ctx->sm_count / std::max(L, 1),
-                                                                     (per_lane + 2047) / 2048));
-    gd.part_blocks = std::min(gd.part_blocks, 512);
-    std::vector<long long> seg(L + 1);
+    std::vector<long long> seg(L + 1), blk_off;
+    std::vector<int> blk_lane, lane_blk;
     for (int h = 0; h < nrhs; ++h)
         for (int s = 0; s < ctx->S; ++s) {
             const int l = h * ctx->S + s;
             seg[l] = (long long)h * ctx->sumM * ctx->D + (long long)ctx->tgt_off[ctx->body_off[s]] * ctx->D;
         }
     seg[L] = n;
-    CK(ctx->alloc(&ctx->seg_off_d, L + 1));
-    CK(cudaMemcpy(ctx->seg_off_d, seg.data(), sizeof(long long) * (L + 1), cudaMemcpyHostToDevice));
-    gd.seg_off = ctx->seg_off_d;
+    gd.clusters = gmres_plan_blocks(seg, ctx->sm_count, blk_lane, blk_off, lane_blk) ? 1 : 0;
+    gd.nblk = (int)blk_lane.size();
+    int *bl = nullptr, *lb = nullptr;
+    long long *bo = nullptr;
+    CK(ctx->alloc(&bl, blk_lane.size()));
+    CK(ctx->alloc(&bo, blk_off.size()));
+    CK(ctx->alloc(&lb, lane_blk.size()));
+    gd.blk_lane = bl;
+    gd.blk_off = bo;
+    gd.lane_blk = lb;
+    CK(cudaMemcpy(bl, blk_lane.data(), sizeof(int) * blk_lane.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(bo, blk_off.data(), sizeof(long long) * blk_off.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(lb, lane_blk.data(), sizeof(int) * lane_blk.size(), cudaMemcpyHostToDevice));
     CK(ctx->alloc(&gd.V, (size_t)(m + 1) * n));
-    CK(cudaMemset(gd.V, 0, sizeof(double) * (size_t)(m + 1) * n));
     CK(ctx->alloc(&gd.H, (size_t)L * (m + 1) * m));
     CK(ctx->alloc(&gd.cs, (size_t)L * m));
     CK(ctx->alloc(&gd.sn, (size_t)L * m));
     CK(ctx->alloc(&gd.g, (size_t)L * (m + 1)));
     CK(ctx->alloc(&gd.beta, L));
     CK(ctx->alloc(&gd.hbuf, (size_t)L * (m + 1)));
-    CK(ctx->alloc(&gd.htmp, (size_t)L * (m + 1)));
-    CK(ctx->alloc(&gd.hn, L));
-    CK(ctx->alloc(&gd.part, (size_t)L * gd.part_blocks * (m + 1)));
+    CK(ctx->alloc(&gd.part, (size_t)gd.nblk * (m + 1)));
+    CK(ctx->alloc(&gd.normp, gd.nblk));
     CK(ctx->alloc(&gd.active, L));
-    CK(ctx->alloc(&gd.iters, L));
-    CK(ctx->alloc(&gd.status, L));
-    CK(ctx->alloc(&gd.resid, L));
-    CK(ctx->alloc(&gd.done, 1));
-    CK(ctx->alloc(&gd.jcur, 1));
+    // what a solve reports, in one block (one copy back): resid [L], iters [L], status [L], done, jcur,
+    // and the blocks' arrival counter
+    CK(ctx->alloc(&ctx->stat_d, ctx->stat_bytes(L)));
+    CK(cudaMallocHost((void **)&ctx->stat_h, ctx->stat_bytes(L)));
+    CK(cudaMemset(ctx->stat_d, 0, ctx->stat_bytes(L)));
+    gd.resid = reinterpret_cast<double *>(ctx->stat_d);
+    gd.iters = reinterpret_cast<int *>(gd.resid + L);
+    gd.status = gd.iters + L;
+    gd.done = gd.status + L;
+    gd.jcur = gd.done + 1;
+    gd.arrive = reinterpret_cast<unsigned *>(gd.jcur + 1);
+    CK(gmres_prepare(gd));
     CK(ctx->alloc(&ctx->vin_d, n));
     CK(ctx->alloc(&ctx->w_d, n));
     CK(ctx->alloc(&ctx->b_d, n));
     CK(ctx->alloc(&ctx->x_d, n));
-    CK(ctx->alloc(&ctx->ysmall_d, (size_t)L * (m + 1)));
     ctx->gd_n = n;
     ctx->gd_L = L;
     ctx->gd_m = m;
@@ -1582,6 +1591,8 @@ mfs_status matvec_T_dev(mfs_ctx *ctx, const double *w, double *y, int nrhs, cuda
 struct SolveStats {
     int iters = 0, converged = 1, matvecs = 0, breakdown = 0;
     double resid = 0.0;
+    int host_iters = 0;                              // iterations the host enqueued one by one
+    const mfs_ctx::SolveGraph *graph = nullptr;      // the rest ran in it
 };
 
 // One GMRES iteration's matvec: w = A vin (or A^T vin).
@@ -1590,10 +1601,11 @@ mfs_status iteration_matvec(mfs_ctx *ctx, const double *vin, int nrhs, bool tran
     return matvec_dev(ctx, vin, ctx->w_d, nrhs, st);
 }
 
-// The loop of iterations j >= 1 as a CUDA graph: a while node whose body loads v_j, applies the
-// matvec, orthogonalises (Arnoldi, Givens) and advances j, clearing the node's condition when every
-// lane stopped or the basis is full (at most m - 1 passes).  Built on first use (the first iteration
-// ran on the host loop, so every plan and tensor map the body needs exists) and kept per key.
+// The loop of iterations as a CUDA graph: a while node whose body applies the matvec to vin,
+// orthogonalises (Arnoldi, Givens; v_{j+1} to vin) and advances j, clearing the node's condition when
+// every lane stopped or the basis is full.  Built on first use (the first iteration of that solve ran on
+// the host loop, so every plan and tensor map the body needs exists) and kept per key; later solves run
+// all their iterations in it.
 mfs_status solve_graph(mfs_ctx *ctx, int nrhs, bool transposed, mfs_ctx::SolveGraph **out) {
     const int key = nrhs * 4 + ctx->fset * 2 + (transposed ? 1 : 0);
     auto it = ctx->graphs.find(key);
@@ -1631,13 +1643,13 @@ mfs_status solve_graph(mfs_ctx *ctx, int nrhs, bool transposed, mfs_ctx::SolveGr
     e = cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e != cudaSuccess) return fail(e);
     mfs_status ms = MFS_OK;
-    cudaError_t ce = gmres_load_vj(gd, ctx->vin_d, st);
-    if (ce == cudaSuccess) ms = iteration_matvec(ctx, ctx->vin_d, nrhs, transposed, st);
-    if (ce == cudaSuccess && ms == MFS_OK) ce = gmres_arnoldi(gd, ctx->w_d, st);
-    if (ce == cudaSuccess && ms == MFS_OK) ce = gmres_advance(gd, cond, 1, st);
+    cudaError_t ce = cudaSuccess;
+    ms = iteration_matvec(ctx, ctx->vin_d, nrhs, transposed, st);
+    if (ms == MFS_OK) ce = gmres_arnoldi(gd, ctx->w_d, ctx->vin_d, 0, st);
+    if (ce == cudaSuccess && ms == MFS_OK) ce = gmres_advance(gd, cond, st);
     cudaGraph_t captured = nullptr;
     e = cudaStreamEndCapture(st, &captured);
-    g.launches = ctx->launches - l0 + 11;
+    g.launches = ctx->launches - l0 + gmres_arnoldi_launches(gd) + 1;
     g.pair_launches = ctx->pair_launches - p0;
     ctx->launches = l0;
     ctx->pair_launches = p0;
@@ -1654,50 +1666,62 @@ mfs_status solve_graph(mfs_ctx *ctx, int nrhs, bool transposed, mfs_ctx::SolveGr
     return MFS_OK;
 }
 
-// Solve A x = b (or A^T x = b) with b = ctx->b_d for all lanes; x in ctx->x_d.
-mfs_status gmres_solve(mfs_ctx *ctx, int nrhs, cudaStream_t st, SolveStats &stats, bool transposed = false) {
+// Enqueue the solve of A x = b (or A^T x = b) with b = ctx->b_d for all lanes, x to `x`; gmres_finish
+// waits for it.  Once a solve of this kind has run, its whole iteration loop is one graph launch and
+// nothing here waits for the device.
+mfs_status gmres_solve(mfs_ctx *ctx, int nrhs, cudaStream_t st, double *x, SolveStats &stats,
+                       bool transposed = false) {
     GmresDev &gd = ctx->gd;
-    CK(gmres_init(gd, ctx->b_d, st));
-    ctx->launches += 6;
+    CK(gmres_init(gd, ctx->b_d, ctx->vin_d, st));
+    ctx->launches += 2;
     const bool use_graph = ctx->opt.graphs && !ctx->opt.profile;
-    for (int j = 0; j < gd.m; ++j) {
-        CKS(iteration_matvec(ctx, gd.V + (size_t)j * gd.n, nrhs, transposed, st));
-        CK(gmres_arnoldi(gd, ctx->w_d, st));
-        CK(gmres_advance(gd, cudaGraphConditionalHandle(), 0, st));
-        ctx->launches += 10;
-        CK(cudaMemcpyAsync(ctx->done_h, gd.done, sizeof(int), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        stats.matvecs = j + 1;
-        if (*ctx->done_h || j + 1 >= gd.m) break;
-        if (use_graph) {  // the remaining iterations as one graph launch
-            mfs_ctx::SolveGraph *g = nullptr;
-            CKS(solve_graph(ctx, nrhs, transposed, &g));
-            CK(cudaGraphLaunch(g->exec, st));
-            int jend = 0;
-            CK(cudaMemcpyAsync(&jend, gd.jcur, sizeof(int), cudaMemcpyDeviceToHost, st));
+    const auto have = ctx->graphs.find(nrhs * 4 + ctx->fset * 2 + (transposed ? 1 : 0));
+    if (use_graph && have != ctx->graphs.end()) {
+        stats.graph = &have->second;
+        CK(cudaGraphLaunch(have->second.exec, st));
+    } else {
+        for (int j = 0; j < gd.m; ++j) {
+            CKS(iteration_matvec(ctx, ctx->vin_d, nrhs, transposed, st));
+            CK(gmres_arnoldi(gd, ctx->w_d, ctx->vin_d, 1, st));
+            ctx->launches += gmres_arnoldi_launches(gd);
+            CK(cudaMemcpyAsync(ctx->done_h, gd.done, sizeof(int), cudaMemcpyDeviceToHost, st));
             CK(cudaStreamSynchronize(st));
-            const int extra = jend - j;  // iterations the graph ran (j advanced from j + 1 to jend)
-            ctx->launches += extra * g->launches;
-            ctx->pair_launches += extra * g->pair_launches;
-            stats.matvecs = jend + 1;
-            break;
+            stats.host_iters = j + 1;
+            if (*ctx->done_h || j + 1 >= gd.m) break;
+            if (use_graph) {  // the remaining iterations as one graph launch
+                mfs_ctx::SolveGraph *g = nullptr;
+                CKS(solve_graph(ctx, nrhs, transposed, &g));
+                stats.graph = g;
+                CK(cudaGraphLaunch(g->exec, st));
+                break;
+            }
         }
     }
-    CK(gmres_solution(gd, ctx->x_d, ctx->ysmall_d, st));
-    ctx->launches += 2;
-    std::vector<int> it(gd.L), status(gd.L), active(gd.L);
-    std::vector<double> res(gd.L);
-    CK(cudaMemcpyAsync(it.data(), gd.iters, sizeof(int) * gd.L, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(status.data(), gd.status, sizeof(int) * gd.L, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(res.data(), gd.resid, sizeof(double) * gd.L, cudaMemcpyDeviceToHost, st));
+    CK(gmres_solution(gd, x, st));
+    ctx->launches += 1;
+    CK(cudaMemcpyAsync(ctx->stat_h, ctx->stat_d, ctx->stat_bytes(gd.L), cudaMemcpyDeviceToHost, st));
+    return MFS_OK;
+}
+
+// Wait for the stream and read the solve's statistics and the device error flag.
+mfs_status gmres_finish(mfs_ctx *ctx, cudaStream_t st, SolveStats &stats) {
+    const GmresDev &gd = ctx->gd;
+    CK(cudaMemcpyAsync(ctx->done_h + 1, ctx->err_d, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    const double *res = reinterpret_cast<const double *>(ctx->stat_h);
+    const int *it = reinterpret_cast<const int *>(res + gd.L), *status = it + gd.L, jend = status[gd.L + 1];
     for (int l = 0; l < gd.L; ++l) {
         stats.iters = std::max(stats.iters, it[l]);
         stats.resid = std::max(stats.resid, res[l]);
         if (status[l] == 2) stats.breakdown = 1;
         if (!(res[l] <= gd.tol)) stats.converged = 0;
     }
-    CKS(check_device_error(ctx, st));
+    stats.matvecs = jend + 1;
+    if (stats.graph) {
+        ctx->launches += (stats.matvecs - stats.host_iters) * stats.graph->launches;
+        ctx->pair_launches += (stats.matvecs - stats.host_iters) * stats.graph->pair_launches;
+    }
+    if (ctx->done_h[1]) return check_device_error(ctx, st);
     return MFS_OK;
 }
 
@@ -2537,7 +2561,7 @@ static mfs_status setup_impl(mfs_ctx *ctx, mfs_kind kind, const mfs_bodies *bodi
     if (ctx->opt.precision == 1)
         CK(ctx->alloc(&ctx->raw_d, R * D * std::max((size_t)fp64_chunks(ctx, ctx->sumM) * ctx->sumM,
                                                     (size_t)fp64_chunks(ctx, ctx->sumN, true) * ctx->sumN)));
-    CK(cudaMallocHost(&ctx->done_h, sizeof(int)));
+    CK(cudaMallocHost(&ctx->done_h, 2 * sizeof(int)));
     CK(cudaEventCreate(&ctx->ev0));
     CK(cudaEventCreate(&ctx->ev1));
     CK(cudaEventCreate(&ctx->evp0));
@@ -2791,16 +2815,19 @@ mfs_status mfs_pair_sum(mfs_ctx *ctx, const double *strengths, double *u, int32_
     return check_device_error(ctx, st);
 }
 
-// Keep the GMRES solution gamma (ctx->x_d) and the inputs a (and b), n doubles each, of the solve
-// just run (kind: 1 mobility, 2 elastance, 3 resistance, 4 capacitance).
+// Where a solve's gamma goes: it is kept for mfs_mobility_vjp and mfs_evaluate.
+static mfs_status keep_buffers(mfs_ctx *ctx) {
+    ctx->last_solve = 0;  // until this one is done
+    if (ctx->keep_gamma) return MFS_OK;
+    CK(ctx->alloc(&ctx->keep_gamma, (size_t)ctx->opt.max_rhs * ctx->sumM * ctx->D));
+    CK(ctx->alloc(&ctx->keep_lam0, (size_t)ctx->opt.max_rhs * ctx->P * 6));
+    return MFS_OK;
+}
+
+// Keep the inputs a (and b), n doubles each, of the solve just run (kind: 1 mobility, 2 elastance,
+// 3 resistance, 4 capacitance), whose gamma is in keep_gamma.
 static mfs_status keep_solution(mfs_ctx *ctx, int kind, int nrhs, const double *a, const double *b, size_t n,
                                 cudaStream_t st) {
-    if (!ctx->keep_gamma) {
-        CK(ctx->alloc(&ctx->keep_gamma, (size_t)ctx->opt.max_rhs * ctx->sumM * ctx->D));
-        CK(ctx->alloc(&ctx->keep_lam0, (size_t)ctx->opt.max_rhs * ctx->P * 6));
-    }
-    CK(cudaMemcpyAsync(ctx->keep_gamma, ctx->x_d, sizeof(double) * nrhs * ctx->sumM * ctx->D,
-                       cudaMemcpyDeviceToDevice, st));
     if (a) CK(cudaMemcpyAsync(ctx->keep_lam0, a, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
     if (b) CK(cudaMemcpyAsync(ctx->keep_lam0 + n, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
     ctx->last_solve = kind;
@@ -2882,6 +2909,7 @@ mfs_status mfs_solve_mobility(mfs_ctx *ctx, const double *F, const double *T, do
     CKS(stage_out_alloc(ctx, Oo, Omega, nb, st));
     if (ctx->opt.autotune && ctx->opt.precision != 1 && ctx->best_variant[1][nrhs] < 0) CKS(autotune(ctx, nrhs, st));
     CKS(ensure_gmres(ctx, nrhs));
+    CKS(keep_buffers(ctx));
     begin_call(ctx);
     CK(cudaEventRecord(ctx->ev0, st));
     ctx->launches += 1;
@@ -2890,15 +2918,15 @@ mfs_status mfs_solve_mobility(mfs_ctx *ctx, const double *F, const double *T, do
                          ctx->src_off_d, ctx->sumN, ctx->lam_d, st));
     CKS(pair_apply(ctx, ctx->lam_d, ctx->b_d, nullptr, 0.0, -1.0, nrhs, 1, st));
     SolveStats ss;
-    CKS(gmres_solve(ctx, nrhs, st, ss));
+    CKS(gmres_solve(ctx, nrhs, st, ctx->keep_gamma, ss));
     // lambda = S_L^+ gamma, [U; Omega] = -K_N^T lambda (Eq. getU)
-    CKS(precond_apply_dev(ctx, ctx->x_d, ctx->lam_d, 0, nrhs, st));
+    CKS(precond_apply_dev(ctx, ctx->keep_gamma, ctx->lam_d, 0, nrhs, st));
     CK(extract_stokes(ctx->lam_d, nrhs, ctx->P, ctx->src_local64_d, ctx->src_off_d, ctx->sumN, Uo.d, Oo.d, st));
     ctx->launches += 1;
     CK(cudaEventRecord(ctx->ev1, st));
     // keep gamma, F and T for mfs_mobility_vjp and mfs_evaluate (outside the timed region)
     CKS(keep_solution(ctx, 1, nrhs, Fi.d, Ti.d, nb, st));
-    CK(cudaEventSynchronize(ctx->ev1));
+    CKS(gmres_finish(ctx, st, ss));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
     CKS(stage_out_finish(ctx, Uo, st));
@@ -2923,19 +2951,20 @@ mfs_status mfs_solve_elastance(mfs_ctx *ctx, const double *Q, double *V, int32_t
     CKS(stage_out_alloc(ctx, Vo, V, nb, st));
     if (ctx->opt.autotune && ctx->opt.precision != 1 && ctx->best_variant[0][nrhs] < 0) CKS(autotune(ctx, nrhs, st));
     CKS(ensure_gmres(ctx, nrhs));
+    CKS(keep_buffers(ctx));
     begin_call(ctx);
     CK(cudaEventRecord(ctx->ev0, st));
     ctx->launches += 1;
     CK(completion_laplace(Qi.d, nrhs, ctx->P, ctx->src_off_d, ctx->sumN, ctx->lam_d, st));  // Eq. al0
     CKS(pair_apply(ctx, ctx->lam_d, ctx->b_d, nullptr, 0.0, -1.0, nrhs, 1, st));           // b = -u_0, Eq. erhsK
     SolveStats ss;
-    CKS(gmres_solve(ctx, nrhs, st, ss));
-    CKS(precond_apply_dev(ctx, ctx->x_d, ctx->lam_d, 0, nrhs, st));
+    CKS(gmres_solve(ctx, nrhs, st, ctx->keep_gamma, ss));
+    CKS(precond_apply_dev(ctx, ctx->keep_gamma, ctx->lam_d, 0, nrhs, st));
     CK(extract_laplace(ctx->lam_d, nrhs, ctx->P, ctx->src_off_d, ctx->sumN, Vo.d, st));  // Eq. vkal
     ctx->launches += 1;
     CK(cudaEventRecord(ctx->ev1, st));
     CKS(keep_solution(ctx, 2, nrhs, Qi.d, nullptr, nb, st));
-    CK(cudaEventSynchronize(ctx->ev1));
+    CKS(gmres_finish(ctx, st, ss));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
     CKS(stage_out_finish(ctx, Vo, st));
@@ -2956,8 +2985,8 @@ struct DirichletScope {
 // the strengths alpha = S^+ gamma in ctx->lam_d.
 mfs_status dirichlet_solve(mfs_ctx *ctx, int nrhs, cudaStream_t st, SolveStats &ss) {
     DirichletScope scope(ctx);
-    CKS(gmres_solve(ctx, nrhs, st, ss));
-    CKS(precond_apply_dev(ctx, ctx->x_d, ctx->lam_d, 0, nrhs, st));
+    CKS(gmres_solve(ctx, nrhs, st, ctx->keep_gamma, ss));
+    CKS(precond_apply_dev(ctx, ctx->keep_gamma, ctx->lam_d, 0, nrhs, st));
     return MFS_OK;
 }
 }  // namespace
@@ -3021,6 +3050,7 @@ mfs_status mfs_solve_resistance(mfs_ctx *ctx, const double *U, const double *Ome
     CKS(ensure_dirichlet(ctx, st));
     if (ctx->opt.autotune && ctx->opt.precision != 1 && ctx->best_variant[1][nrhs] < 0) CKS(autotune(ctx, nrhs, st));
     CKS(ensure_gmres(ctx, nrhs));
+    CKS(keep_buffers(ctx));
     begin_call(ctx);
     CK(cudaEventRecord(ctx->ev0, st));
     // b = K_M U (Sec. 2.2), then Algorithm 1 and [f; t] = K_N^T lambda (Eq. force_def)
@@ -3031,7 +3061,7 @@ mfs_status mfs_solve_resistance(mfs_ctx *ctx, const double *U, const double *Ome
     ctx->launches += 2;
     CK(cudaEventRecord(ctx->ev1, st));
     CKS(keep_solution(ctx, 3, nrhs, nullptr, nullptr, 0, st));
-    CK(cudaEventSynchronize(ctx->ev1));
+    CKS(gmres_finish(ctx, st, ss));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
     CKS(stage_out_finish(ctx, Fo, st));
@@ -3057,6 +3087,7 @@ mfs_status mfs_solve_capacitance(mfs_ctx *ctx, const double *phi, double *q, int
     CKS(ensure_dirichlet(ctx, st));
     if (ctx->opt.autotune && ctx->opt.precision != 1 && ctx->best_variant[0][nrhs] < 0) CKS(autotune(ctx, nrhs, st));
     CKS(ensure_gmres(ctx, nrhs));
+    CKS(keep_buffers(ctx));
     begin_call(ctx);
     CK(cudaEventRecord(ctx->ev0, st));
     // eta = phi 1_M (Sec. 2.1), then Algorithm 1 and q = sum alpha (Eq. qkgauss)
@@ -3067,7 +3098,7 @@ mfs_status mfs_solve_capacitance(mfs_ctx *ctx, const double *phi, double *q, int
     ctx->launches += 2;
     CK(cudaEventRecord(ctx->ev1, st));
     CKS(keep_solution(ctx, 4, nrhs, nullptr, nullptr, 0, st));
-    CK(cudaEventSynchronize(ctx->ev1));
+    CKS(gmres_finish(ctx, st, ss));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
     CKS(stage_out_finish(ctx, Qo, st));
@@ -3184,7 +3215,8 @@ mfs_status mfs_mobility_vjp(mfs_ctx *ctx, const double *dU, const double *dOmega
     CK(cudaGetLastError());
     // 2. A^T w = g
     SolveStats ss;
-    CKS(gmres_solve(ctx, nrhs, st, ss, true));
+    CKS(gmres_solve(ctx, nrhs, st, ctx->x_d, ss, true));
+    CKS(gmres_finish(ctx, st, ss));
     if (ss.breakdown || !ss.converged) {
         ctx->last_error = "adjoint GMRES did not converge";
         return ss.breakdown ? MFS_ERR_BREAKDOWN : MFS_ERR_NOT_CONVERGED;
