@@ -8,9 +8,11 @@
 // Work is cut into blocks of one lane each (GmresDev::blk_*, sized on the host so that all blocks have
 // about the same length whatever the lanes' sizes; with a fixed number of blocks per lane, suspensions
 // of 2 to 64 bodies left most SMs waiting for the longest lane).  What bounds the step is latency and
-// the FP64 pipe (2 DFMA per clock per SM), not bandwidth: an iteration was ten launches, each a chain of
-// dependent loads, so it is five here (dot, update, dot, update, finish), and one for short lanes
-// (gm_arnoldi_cluster_kernel).
+// the FP64 pipe, not bandwidth: an iteration was ten launches, each a chain of dependent loads, so it is
+// five here (dot, update, dot, update, finish), and one for short lanes (gm_arnoldi_cluster_kernel).  A
+// warp's FP64 instruction holds its scheduler's FP64 pipe for 64 clocks however many of its lanes are
+// active, so scalar FP64 work (norms, rotations, the tails of reductions) is done by one warp and handed
+// on through shared memory, and no warp runs FP64 instructions on elements or columns that do not exist.
 #include <algorithm>
 
 #include <cooperative_groups.h>
@@ -27,22 +29,24 @@ namespace mfs {
 
 // Block-wide dots: out[i] = sum over e in [0, len) of V[i n + e] w[e], i = 0 .. cols - 1, in a fixed
 // order.  A warp takes a group of four columns on a part of the elements (w is read once for the four;
-// with few columns the elements are cut into parts so that all 16 warps work); the lanes' partials go to
-// shared memory and are added there, eight lanes to a column: a shuffle tree per warp and column would
-// cost as many FP64 instructions as the dots themselves.  sh: 4 * GM_THREADS doubles.
+// with few columns the elements are cut into parts, of at least 128 elements each); the lanes' partials
+// go to shared memory and are added there, eight lanes to a column: a shuffle tree per warp and column
+// would cost as many FP64 instructions as the dots themselves.  sh: 4 * GM_THREADS doubles.
 __device__ __forceinline__ void block_dots(const double *V, long long n, const double *w, int len, int cols,
                                            double *sh, double *out) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ng = (cols + 3) / 4;
     for (int g0 = 0; g0 < ng; g0 += GM_WARPS) {
-        const int groups = min(ng - g0, GM_WARPS), parts = GM_WARPS / groups;
+        const int groups = min(ng - g0, GM_WARPS);
+        const int parts = max(1, min(min(GM_WARPS / groups, 8), (len + 127) / 128));
         const int g = warp / parts, p = warp % parts;
-        double acc[4] = {0.0, 0.0, 0.0, 0.0};
         if (g < groups) {
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
             const int c0 = 4 * (g0 + g), nc = min(4, cols - c0);
             const int e1 = (int)((long long)len * (p + 1) / parts);
             const double *Vc = V + (size_t)c0 * n;
-            for (int e = (int)((long long)len * p / parts) + lane; e < e1; e += 128) {
+            for (int eb = (int)((long long)len * p / parts); eb < e1; eb += 128) {
+                const int e = eb + lane;
                 double we[4], v[4][4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) we[u] = e + 32 * u < e1 ? w[e + 32 * u] : 0.0;
@@ -52,26 +56,26 @@ __device__ __forceinline__ void block_dots(const double *V, long long n, const d
                     for (int u = 0; u < 4; ++u)
                         v[c][u] = (c < nc && e + 32 * u < e1) ? Vc[(size_t)c * n + e + 32 * u] : 0.0;
 #pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    if (c < nc)
+                for (int u = 0; u < 4; ++u)
+                    if (eb + 32 * u < e1)
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) acc[c] = fma(v[c][u], we[u], acc[c]);
+                        for (int c = 0; c < 4; ++c)
+                            if (c < nc) acc[c] = fma(v[c][u], we[u], acc[c]);
             }
-        }
 #pragma unroll
-        for (int c = 0; c < 4; ++c) sh[(c * GM_WARPS + warp) * 32 + lane] = acc[c];
+            for (int c = 0; c < 4; ++c) sh[(c * GM_WARPS + warp) * 32 + lane] = acc[c];
+        }
         __syncthreads();
         // column 4 g + c: the `parts` warps of group g, 32 values each; 8 lanes add 4 parts values apiece
-        const int per = GM_THREADS / 8;
-        for (int q = threadIdx.x / 8; q < 4 * groups; q += per) {  // 4 groups <= 64 = per: one round
+        const int q = threadIdx.x / 8;  // 4 groups <= 64 columns = GM_THREADS / 8
+        if ((q & ~3) < 4 * groups) {    // whole warps: four columns each
             const int gg = q / 4, c = q % 4, s8 = threadIdx.x & 7;
             double r = 0.0;
             for (int pp = 0; pp < parts; ++pp) {
                 const double *x = sh + (c * GM_WARPS + gg * parts + pp) * 32 + s8;
                 r += (x[0] + x[8]) + (x[16] + x[24]);
             }
-            const unsigned mask = 0xffu << (threadIdx.x & 24);
-            for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(mask, r, o);
+            for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
             const int col = 4 * (g0 + gg) + c;
             if (s8 == 0 && col < cols) out[col] = r;
         }
@@ -86,7 +90,9 @@ template <bool NORM>
 __device__ __forceinline__ double block_update(const double *V, long long n, double *w, int len, int cols,
                                                const double *h) {
     double nrm = 0.0;
-    for (int e = threadIdx.x; e < len; e += 4 * GM_THREADS) {
+    const int lane = threadIdx.x & 31;
+    for (int eb = threadIdx.x - lane; eb < len; eb += 4 * GM_THREADS) {  // the warp's first element
+        const int e = eb + lane;
         double a[4] = {0.0, 0.0, 0.0, 0.0};
         bool in[4];
 #pragma unroll
@@ -99,31 +105,42 @@ __device__ __forceinline__ double block_update(const double *V, long long n, dou
                 for (int u = 0; u < 4; ++u)
                     v[g][u] = (in[u] && i + g < cols) ? V[(size_t)(i + g) * n + e + u * GM_THREADS] : 0.0;
 #pragma unroll
-            for (int g = 0; g < 8; ++g)
-                if (i + g < cols)
+            for (int u = 0; u < 4; ++u)
+                if (eb + u * GM_THREADS < len)
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) a[u] = fma(h[i + g], v[g][u], a[u]);
+                    for (int g = 0; g < 8; ++g)
+                        if (i + g < cols) a[u] = fma(h[i + g], v[g][u], a[u]);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (in[u]) {
-                const double x = w[e + u * GM_THREADS] - a[u];
-                w[e + u * GM_THREADS] = x;
+            if (eb + u * GM_THREADS < len) {
+                const double x = in[u] ? w[e + u * GM_THREADS] - a[u] : 0.0;
+                if (in[u]) w[e + u * GM_THREADS] = x;
                 if (NORM) nrm = fma(x, x, nrm);
             }
     }
     return nrm;
 }
 
-// Sum over the block in a fixed order, valid in every thread.  sh: GM_WARPS doubles.
-__device__ __forceinline__ double block_sum_all(double v, double *sh) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+// Sum of v over the block in a fixed order, returned in lane 0 of warp 0: through shared memory, one warp
+// adds (threads beyond `threads` hold zeros and are left out).  sh: GM_THREADS doubles.
+__device__ __forceinline__ double block_sum(double v, int threads, double *sh) {
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    sh[threadIdx.x] = v;
     __syncthreads();
     double s = 0.0;
-    for (int i = 0; i < (int)blockDim.x / 32; ++i) s += sh[i];
+    if (threadIdx.x < 32) {
+        for (int i = threadIdx.x; i < threads; i += 32) s += sh[i];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
     return s;
+}
+
+// (||x||, 1 / ||x||) from s = ||x||^2, (0, 0) for 0.
+__device__ __forceinline__ double2 norm_and_inverse(double s) {
+    if (s == 0.0) return make_double2(0.0, 0.0);
+    const double inv = rsqrt64(s);
+    return make_double2(isfinite(s) ? s * inv : sqrt(s), inv);
 }
 
 // The Givens update of column j for lane l (one thread): hcol[0 .. j] the column's entries, hn the norm
@@ -140,8 +157,18 @@ __device__ void givens_lane(const GmresDev &gd, int l, int j, const double *hcol
         carry = -sn_[i] * carry + cs_[i] * c;
     }
     const double a = carry, c = h_next;
-    const double den = hypot(a, c);
-    const double cj = den > 0.0 ? a / den : 1.0, sj = den > 0.0 ? c / den : 0.0;
+    const double r2 = fma(a, a, c * c);
+    double den, cj, sj;
+    if ((unsigned)__double2hiint(r2) - 0x06000000u < 0x72000000u) {  // r2 well inside the normal range
+        const double ri = rsqrt64(r2);
+        den = r2 * ri;
+        cj = a * ri;
+        sj = c * ri;
+    } else {
+        den = hypot(a, c);
+        cj = den > 0.0 ? a / den : 1.0;
+        sj = den > 0.0 ? c / den : 0.0;
+    }
     cs[j] = cj;
     sn[j] = sj;
     H[j * m + j] = den;
@@ -149,7 +176,7 @@ __device__ void givens_lane(const GmresDev &gd, int l, int j, const double *hcol
     g[j + 1] = gn;
     g[j] = cj * gj;
     gd.iters[l] = j + 1;
-    const double res = fabs(gn) / gd.beta[l];
+    const double res = fabs(gn) * gd.ibeta[l];
     gd.resid[l] = res;
     int keep = 1;
     if (!isfinite(res) || !isfinite(den)) {
@@ -204,11 +231,12 @@ __global__ void __launch_bounds__(GM_THREADS) gm_update_kernel(GmresDev gd, doub
     if (!gd.active[l]) return;
     const int cols = *gd.jcur + 1;
     __shared__ double h[1024];
-    __shared__ double red[GM_WARPS];
+    __shared__ double red[GM_THREADS];
     const int b0 = gd.lane_blk[l], nb = gd.lane_blk[l + 1] - b0;
     const size_t ld = gd.m + 1;
-    for (int q0 = 0; q0 < cols; q0 += GM_THREADS / 8) {  // uniform trip count
+    for (int q0 = 0; q0 < cols; q0 += GM_THREADS / 8) {
         const int q = q0 + threadIdx.x / 8, s8 = threadIdx.x & 7;
+        if ((q & ~3) >= cols) break;  // whole warps: four columns each
         double r = 0.0;
         if (q < cols) {
             const double *p = gd.part + (size_t)b0 * ld + q;
@@ -233,7 +261,7 @@ __global__ void __launch_bounds__(GM_THREADS) gm_update_kernel(GmresDev gd, doub
     const long long e0 = gd.blk_off[b];
     const double s = block_update<PASS == 1>(gd.V + e0, gd.n, w + e0, (int)(gd.blk_off[b + 1] - e0), cols, h);
     if (PASS == 1) {
-        const double t = block_sum_all(s, red);
+        const double t = block_sum(s, GM_THREADS, red);
         if (threadIdx.x == 0) gd.normp[b] = t;
     }
 }
@@ -241,22 +269,22 @@ __global__ void __launch_bounds__(GM_THREADS) gm_update_kernel(GmresDev gd, doub
 // normp[b] = block b's share of ||x||^2 (all lanes)
 __global__ void __launch_bounds__(GM_THREADS) gm_norm_kernel(GmresDev gd, const double *x) {
     const int b = blockIdx.x;
-    __shared__ double red[GM_WARPS];
+    __shared__ double red[GM_THREADS];
     const long long e0 = gd.blk_off[b], e1 = gd.blk_off[b + 1];
     double s = 0.0;
     for (long long e = e0 + threadIdx.x; e < e1; e += GM_THREADS) s = fma(x[e], x[e], s);
-    s = block_sum_all(s, red);
+    s = block_sum(s, GM_THREADS, red);
     if (threadIdx.x == 0) gd.normp[b] = s;
 }
 
-// The lane's norm from its blocks' shares, the same in every block of the lane.
-__device__ __forceinline__ double lane_norm(const GmresDev &gd, int l) {
-    __shared__ double nrm;
+// The lane's norm and its inverse from its blocks' shares, the same in every block of the lane.
+__device__ __forceinline__ double2 lane_norm(const GmresDev &gd, int l) {
+    __shared__ double2 nrm;
     if (threadIdx.x < 32) {
         double s = 0.0;
         for (int i = gd.lane_blk[l] + threadIdx.x; i < gd.lane_blk[l + 1]; i += 32) s += gd.normp[i];
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) nrm = sqrt(s);
+        if (threadIdx.x == 0) nrm = norm_and_inverse(s);
     }
     __syncthreads();
     return nrm;
@@ -266,15 +294,15 @@ __device__ __forceinline__ double lane_norm(const GmresDev &gd, int l) {
 // j = 0, done = (no lane active).
 __global__ void __launch_bounds__(GM_THREADS) gm_start_kernel(GmresDev gd, const double *x, double *vin) {
     const int b = blockIdx.x, l = gd.blk_lane[b];
-    const double nrm = lane_norm(gd, l);
-    const double inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
+    const double2 ni = lane_norm(gd, l);
+    const double nrm = ni.x, inv = ni.y;
     for (long long e = gd.blk_off[b] + threadIdx.x; e < gd.blk_off[b + 1]; e += GM_THREADS) {
         const double v = x[e] * inv;
         gd.V[e] = v;
         vin[e] = v;
     }
     if (b == gd.lane_blk[l] && threadIdx.x == 0) {
-        gd.beta[l] = nrm;
+        gd.ibeta[l] = inv;
         gd.g[(size_t)l * (gd.m + 1)] = nrm;
         gd.active[l] = (nrm > 0.0 && isfinite(nrm)) ? 1 : 0;
         gd.iters[l] = 0;
@@ -300,7 +328,8 @@ __global__ void __launch_bounds__(GM_THREADS) gm_finish_kernel(GmresDev gd, cons
     // one read for the block: the lane's first block may clear the flag meanwhile
     const int active = __syncthreads_or(threadIdx.x == 0 ? gd.active[l] : 0);
     if (active) {
-        const double nrm = lane_norm(gd, l);
+        const double2 ni = lane_norm(gd, l);
+        const double nrm = ni.x, inv = ni.y;
         const bool first = b == gd.lane_blk[l];
         if (first) {  // the loads of the serial update ahead of it
             for (int i = threadIdx.x; i <= j; i += GM_THREADS) {
@@ -309,7 +338,6 @@ __global__ void __launch_bounds__(GM_THREADS) gm_finish_kernel(GmresDev gd, cons
                 hs[2][i] = gd.sn[(size_t)l * gd.m + i];
             }
         }
-        const double inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
         double *v = gd.V + (size_t)(j + 1) * gd.n;
         for (long long e = gd.blk_off[b] + threadIdx.x; e < gd.blk_off[b + 1]; e += GM_THREADS) {
             const double x = w[e] * inv;
@@ -334,9 +362,9 @@ __global__ void gm_advance_kernel(GmresDev gd, cudaGraphConditionalHandle cond, 
 // long-lane form (each at least a launch and a chain of dependent loads, about 5 us) become one.  For
 // lanes of at most GM_CLUSTER * GM_CHUNK entries: beyond that the FP64 pipes of 16 SMs take longer than
 // the launches saved (at j = 15, 16384 entries: 4 us a pass).
-// Whole solves with this file's kernels against the ten-launch form: two conductors (1200 entries) 709 ->
-// 549 us, six spheres (4320) 1610 -> 1308 us; five launches: 40 spheroids (119 640 entries, 76 columns)
-// 51.8 -> 46.2 ms, 48 uneven lanes 125.0 -> 119.9 ms.
+// Whole solves with this file's kernels against the ten-launch form: two conductors (1200 entries) 692 ->
+// 445 us, six spheres (4320) 1372 -> 942 us; five launches: 40 spheroids (119 640 entries, 76 columns)
+// 48.1 -> 43.2 ms, 48 uneven lanes 130.7 -> 126.9 ms, solve and gradients of 100 spheres 26.1 -> 25.5 ms.
 __global__ void __launch_bounds__(GM_THREADS) gm_arnoldi_cluster_kernel(GmresDev gd, const double *w, double *vin,
                                                                         int advance) {
     namespace cg = cooperative_groups;
@@ -345,7 +373,8 @@ __global__ void __launch_bounds__(GM_THREADS) gm_arnoldi_cluster_kernel(GmresDev
     extern __shared__ double dyn[];
     double *sh = dyn, *wb = sh + 4 * GM_THREADS, *pa = wb + GM_CHUNK, *pb = pa + m1, *h = pb + m1, *hc = h + m1,
            *cs = hc + m1, *sn = cs + m1;
-    __shared__ double red[GM_WARPS], pn;
+    __shared__ double pn;
+    __shared__ double2 ni;
     if (gd.active[l]) {
         const long long s0 = gd.blk_off[gd.lane_blk[l]], s1 = gd.blk_off[gd.lane_blk[l + 1]];
         const long long e0 = s0 + (s1 - s0) * rank / GM_CLUSTER;
@@ -377,12 +406,16 @@ __global__ void __launch_bounds__(GM_THREADS) gm_arnoldi_cluster_kernel(GmresDev
             hc[i] += s;
         }
         __syncthreads();
-        const double t = block_sum_all(block_update<true>(V, gd.n, wb, len, cols, h), red);
+        const double t = block_sum(block_update<true>(V, gd.n, wb, len, cols, h), min(GM_THREADS, (len + 31) / 32 * 32), sh);
         if (threadIdx.x == 0) pn = t;
         cl.sync();
-        double s = 0.0;
-        for (int r = 0; r < GM_CLUSTER; ++r) s += *cl.map_shared_rank(&pn, r);
-        const double nrm = sqrt(s), inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
+        if (threadIdx.x < 32) {
+            double s = threadIdx.x < GM_CLUSTER ? *cl.map_shared_rank(&pn, threadIdx.x) : 0.0;
+            for (int o = GM_CLUSTER / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (threadIdx.x == 0) ni = norm_and_inverse(s);
+        }
+        __syncthreads();
+        const double nrm = ni.x, inv = ni.y;
         double *v = gd.V + (size_t)(j + 1) * gd.n + e0;
         for (int e = threadIdx.x; e < len; e += GM_THREADS) {
             const double x = wb[e] * inv;

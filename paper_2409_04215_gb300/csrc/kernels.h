@@ -263,7 +263,7 @@ struct GmresDev {
     double *V;                 // [(m+1)][n] basis
     double *H;                 // [L][m+1][m] Hessenberg, rotated to upper triangular
     double *cs, *sn, *g;       // [L][m], [L][m], [L][m+1]
-    double *beta;              // [L] ||b||
+    double *ibeta;             // [L] 1 / ||b||
     double *hbuf;              // [L][m+1] current column
     double *part;              // [nblk][m+1] block partials of the dots
     double *normp;             // [nblk] block partials of the norm

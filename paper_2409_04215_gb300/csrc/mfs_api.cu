@@ -1246,7 +1246,7 @@ mfs_status ensure_gmres(mfs_ctx *ctx, int nrhs) {
     const int m = std::min(ctx->opt.restart, ctx->opt.max_iter);
     if (ctx->gd.V && ctx->gd_n == (size_t)n && ctx->gd_L == L && ctx->gd_m == m) return MFS_OK;
     GmresDev &gd = ctx->gd;
-    void *olds[] = {gd.V, gd.H, gd.cs, gd.sn, gd.g, gd.beta, gd.hbuf, gd.part, gd.normp, gd.active, (void *)gd.blk_lane,
+    void *olds[] = {gd.V, gd.H, gd.cs, gd.sn, gd.g, gd.ibeta, gd.hbuf, gd.part, gd.normp, gd.active, (void *)gd.blk_lane,
                     (void *)gd.blk_off, (void *)gd.lane_blk, ctx->stat_d, ctx->w_d, ctx->b_d, ctx->x_d, ctx->vin_d};
     ctx->drop_graphs();  // they hold the old buffers' addresses
     for (void *p : olds) ctx->release(p);
@@ -1284,7 +1284,7 @@ mfs_status ensure_gmres(mfs_ctx *ctx, int nrhs) {
     CK(ctx->alloc(&gd.cs, (size_t)L * m));
     CK(ctx->alloc(&gd.sn, (size_t)L * m));
     CK(ctx->alloc(&gd.g, (size_t)L * (m + 1)));
-    CK(ctx->alloc(&gd.beta, L));
+    CK(ctx->alloc(&gd.ibeta, L));
     CK(ctx->alloc(&gd.hbuf, (size_t)L * (m + 1)));
     CK(ctx->alloc(&gd.part, (size_t)gd.nblk * (m + 1)));
     CK(ctx->alloc(&gd.normp, gd.nblk));
