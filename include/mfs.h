@@ -93,7 +93,9 @@ typedef struct {
                              FP32 accumulation over short K runs, double-float sums), operands cut from FP64
                              into TF32 pieces: 1 = three pieces, six products (FP32-level products);
                              2 = two pieces, three products (3xTF32, ~2^-21 products);
-                             0 = CUDA-core split-K FP32 GEMM (TwoSum-compensated slices).  Default 1 */
+                             0 = CUDA-core split-K FP32 GEMM (TwoSum-compensated slices).  Default 1.  With 1 or
+                             2, applies of a few columns (at most 8 bodies of a shape times right-hand sides,
+                             Stokes) run on the CUDA cores in double-FP32 arithmetic, which is faster there */
     int32_t pair_variant; /* >= 0: use this entry of the pair-kernel table (mfs_pair_variant_info) for its
                              (d, nrhs) instead of the autotuner's pick; it must be a forward pair-sum
                              variant of the context's d, else mfs_setup fails with MFS_ERR_INVALID_ARG.

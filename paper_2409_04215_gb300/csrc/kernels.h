@@ -104,8 +104,6 @@ cudaError_t transpose_pieces(const float *src, int rows, int cols, int ld_src, s
 // sum_z P[z] ([rows][cols], (hi, lo) pairs, double-float sums) -> pieces dst[p][rows][ld_dst].
 cudaError_t reduce_pieces(int S, int rows, int cols, const float2 *P, float *dst, int ld_dst, size_t pstride,
                           int pieces, cudaStream_t st);
-// sum_z P[z] ((hi, lo) pairs, double-float sums) -> C (FP64), mn entries.
-cudaError_t reduce_f64(int S, size_t mn, const float2 *P, double *C, cudaStream_t st);
 // gather_rotate with the FP64 values written as pieces dst[p][ncols][ld_dst].
 cudaError_t gather_rotate_pieces(int D, const double *gamma, int sum_MD, const int *col_body, const int *col_rhs,
                                  const int *body_tgt_off, const double *rot, int ncols, int dM, float *dst, int ld_dst,
@@ -117,10 +115,44 @@ cudaError_t gemm_splitk(int m, int n, int k, int S, const float *A, const float 
 int gemm_rm64_chunks(int m, int n, int k, int sm_count);
 cudaError_t gemm_rm64_splitk(int m, int n, int k, int S, const double *A, const double *B, double *P, double *C,
                              cudaStream_t st);
-// Scatter: lambda (FP64 [nrhs][sum_N][D]) at the columns' bodies = R_k * Lcol (rotate back).
-cudaError_t scatter_rotate(int D, const float *L, const double *L64, const int *col_body, const int *col_rhs,
-                           const int *body_src_off, const float *rot, const double *rot64, int ncols, int dN,
-                           int sum_N, double *lambda, cudaStream_t st);
+// ---- one-body apply for few columns, and the scatter of every apply (apply_few.cu) ----
+constexpr int FC_MAX = 8;
+// Whether `ncols` columns of a dM x dN factor go to the warps instead of the tensor cores.  The warps'
+// time grows with columns times elements, the tensor cores' with the factor's bytes from a base of 15 us a
+// product; both sides of the line, whole apply (call included): 600 x 300 points, 8 columns 35 us
+// against 38 on the tensor cores; 1200 x 600, 2 columns 33 against 48, 4 columns 47 against 48, 6 columns 52
+// against 48; 2000 x 1000, 2 columns 62 against 76, 4 columns 87 against 76.  Stokes only: the potentials
+// of a few conductors would move by 1.5e-7 (towards the exact ones, from 1.7e-7 off to 2e-8), which is
+// more than FP64 callers that compare results between versions expect of this path.
+inline bool fc_takes(int D, int ncols, int dM, int dN) {
+    return D == 3 && ncols <= FC_MAX && (ncols <= 2 || (double)ncols * dM * dN <= 16777216.0);
+}
+// out[c][row] = sum_k F[row][k] G[c][k] as (hi, lo) pairs; F the factor's (hi, lo) planes [2][rows][ldk] at
+// pstride, G [ncols][ldk], out [ncols][ldo]; ldk a multiple of 4.
+cudaError_t fc_apply(int ncols, int rows, int ldk, const float *F, size_t pstride, const float2 *G, float2 *out, int ldo,
+                     cudaStream_t st);
+// gather_rotate with the values as (hi, lo) pairs [ncols][ld].
+cudaError_t gather_rotate_hl(int D, const double *gamma, int sum_MD, const int *col_body, const int *col_rhs,
+                             const int *body_off, const double *rot, int ncols, int dM, float2 *out, int ld,
+                             cudaStream_t st);
+struct ScatterArgs {
+    const float2 *P = nullptr;     // (hi, lo) chunk partials [S][ncols][dN], or
+    int S = 0;
+    const double *L64 = nullptr;   // FP64 values [ncols][dN]
+    const int *col_body = nullptr, *col_rhs = nullptr;
+    const int *body_off = nullptr;    // each body's first output point
+    const double *rot64 = nullptr;
+    int ncols = 0, dN = 0, sum_N = 0;
+    double *out = nullptr;         // [nrhs][sum_N][D] at the columns' bodies
+    const double *base = nullptr;  // added when given
+    // source records of the outputs for the pair kernel (layout packed or plain), or null
+    float *rec = nullptr;
+    int rec_floats = 0, packed = 0, nrhs = 1;
+    const int *rec_off = nullptr;
+    const float4 *src_pos = nullptr;
+};
+// out = base + R_k (column values), and the records.
+cudaError_t scatter_rotate(int D, const ScatterArgs &a, cudaStream_t st);
 
 // Completion strengths (Eq. lambda01-02 / Eq. al0) and extraction (Eq. getU / Eq. vkal).
 cudaError_t completion_stokes(const double *F, const double *T, int nrhs, int P, const double *rot64,

@@ -9,6 +9,7 @@
 #include <cstring>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -25,6 +26,23 @@ thread_local std::string g_setup_error;
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
+};
+
+// The treecode's matrices on the unit sphere (FP64, device): check field -> order-0 strengths, each
+// order's strengths -> the next lower order's, local check field -> local sources.  They depend on the
+// kernel's dimension only; the contexts of a process that are alive together share one set per device
+// (ff_matrices), freed with the last of them.
+struct FFMatrices {
+    double *PinvT = nullptr;              // [D FF_NC][D FF_NE]
+    double *ordT[FF_NORD] = {};           // [D FF_ORD_N[o - 1]][D FF_ORD_N[o]], o >= 1
+    double *locT = nullptr;               // [D FF_LOC_NC][D FF_LOC_N]
+    FFMatrices() = default;
+    FFMatrices(const FFMatrices &) = delete;
+    ~FFMatrices() {
+        cudaFree(PinvT);
+        cudaFree(locT);
+        for (double *p : ordT) cudaFree(p);
+    }
 };
 
 struct PairPlan {
@@ -62,7 +80,7 @@ struct ShapeHost {
     double G0inv[36];
     std::vector<int> bodies;     // bodies of this shape
     int *col_body = nullptr, *col_rhs = nullptr;  // device, [max_rhs * nbodies]
-    float *A = nullptr, *Tm = nullptr, *Lm = nullptr;  // GEMM buffers
+    float *A = nullptr, *Tm = nullptr;  // GEMM buffers
     double *Pk = nullptr;                              // split-K chunk results
     size_t Pk_count = 0;
     double *O64 = nullptr, *PkT = nullptr;             // adjoint: transposed-apply output and chunks
@@ -76,6 +94,8 @@ struct ShapeHost {
     std::map<int, std::array<TcMap, 6>> amaps;  // per column count: A pieces, T pieces
     double *A64 = nullptr, *T64 = nullptr, *L64 = nullptr;
     double *Pk64 = nullptr;  // FP64 apply: split-K partials
+    // few columns: [FC_MAX][ld1], [FC_MAX][ld2] twice (forward and transposed), [FC_MAX][dM]
+    float2 *Gf = nullptr, *Tf = nullptr, *Xf = nullptr, *Lf = nullptr;
     // one-body factors per formulation: [0] recompleted S_L (Sec. 3.3), [1] bare self block S^(00)
     // of the Dirichlet problems (Sec. 2.3), built on first use
     FactorSet fs[2];
@@ -186,8 +206,7 @@ struct mfs_ctx {
         FFTree tree;
         int nodes = 0;
         std::vector<double> rsrc, rtgt;              // per body: radius of its proxy / collocation points
-        double *PinvT = nullptr;                     // [D FF_NC][D FF_NE]: transposed pseudo-inverse of the
-                                                     // check <- equivalent map on the unit sphere (FP64)
+        std::shared_ptr<const FFMatrices> mat;       // the fits' matrices
         double *centres = nullptr;                   // [P + nodes][3]: bodies in tree order, then the nodes
         double *re = nullptr;                        // [nodes] equivalent radii
         float4 *eq_pos = nullptr;                    // [nodes FF_NE] equivalent points about their node's centre
@@ -204,15 +223,13 @@ struct mfs_ctx {
         double *mu = nullptr;                        // [max_rhs][nodes FF_NE][D]
         double *fit_chunks = nullptr;                // split-K partials of the fit products
         float *wt = nullptr;                         // [max_rhs][ntgt][3] target weights in tree order (gradient)
-        // lower orders of the equivalent sources (index 1 .. FF_NORD - 1): the map from the next higher
-        // order's strengths, the points about their node's centre, the strengths
-        double *ordT[FF_NORD] = {};                  // [D FF_ORD_N[o - 1]][D FF_ORD_N[o]]
+        // lower orders of the equivalent sources (index 1 .. FF_NORD - 1): the points about their node's
+        // centre, the strengths
         float4 *ord_pos[FF_NORD] = {};               // [nodes FF_ORD_N[o]]
         double *ord_mu[FF_NORD] = {};                // [max_rhs][nodes FF_ORD_N[o]][D]
         size_t ord_rec[FF_NORD] = {};                // first record of the order's segments
         // local expansions of the bodies (tree order)
         bool use_local = false;
-        double *locT = nullptr;                      // [D FF_LOC_NC][D FF_LOC_N]: check -> local sources, unit radius
         double *rloc = nullptr;                      // [P] target radii
         float4 *loc_pos = nullptr, *lchk_pos = nullptr;  // [P FF_LOC_N], [P FF_LOC_NC] about the body's centre
         double *ulocal = nullptr, *nu = nullptr;     // [max_rhs][P FF_LOC_NC][D], [max_rhs][P FF_LOC_N][D]
@@ -657,7 +674,7 @@ mfs_status ff_pair_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const 
                          const double *base, double beta, double scale, int nrhs, int include_self, cudaStream_t st);
 
 mfs_status pair_apply(mfs_ctx *ctx, const double *strength, double *out, const double *base, double beta,
-                      double sign, int nrhs, int include_self, cudaStream_t st) {
+                      double sign, int nrhs, int include_self, cudaStream_t st, bool packed = false) {
     const double scale = sign * kernel_scale(ctx);
     if (ctx->opt.precision == 1) {
         const int S = fp64_chunks(ctx, ctx->sumM);
@@ -680,9 +697,9 @@ mfs_status pair_apply(mfs_ctx *ctx, const double *strength, double *out, const d
         return ff_pair_apply(ctx, ctx->ff, variant, strength, out, base, beta, scale, nrhs, include_self, st);
     PairPlan *plan = nullptr;
     CKS(get_plan(ctx, variant, include_self, &plan));
-    CK(pack_for(ctx, variant, strength, nrhs, st));
+    if (!packed) CK(pack_for(ctx, variant, strength, nrhs, st));
     const PairWork w = work_of(*plan);
-    ctx->launches += 2;
+    ctx->launches += packed ? 1 : 2;
     if (w.total_units > 0) {
         const size_t slot = 2 * (size_t)ctx->pair_launches;
         if (ctx->opt.profile) {
@@ -1044,7 +1061,7 @@ static mfs_status ff_upward(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, con
     const PairWork wu = work_of(pl->p);
     CKS(ff_launch(ctx, variant, g, wu, st));
     CK(pair_epilogue(D, nrhs, wu, nullptr, 0.0, 1.0, F.ucheck, nodes * FF_NC, st));
-    CK(ff_fit(ctx, F, nrhs * nodes, FF_NE, FF_NC, F.ucheck, F.PinvT, F.mu, st));
+    CK(ff_fit(ctx, F, nrhs * nodes, FF_NE, FF_NC, F.ucheck, F.mat->PinvT, F.mu, st));
     CK(ff_scale(F.mu, F.re, nodes, D * FF_NE, nrhs, st));
     ctx->launches += 4;
     return MFS_OK;
@@ -1072,7 +1089,7 @@ mfs_status ff_pair_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const 
     for (int o = 0; o < FF_NORD; ++o) {
         const int n = FF_ORD_N[o];
         if (o > 0)
-            CK(ff_fit(ctx, F, nrhs * nodes, n, FF_ORD_N[o - 1], o == 1 ? F.mu : F.ord_mu[o - 1], F.ordT[o],
+            CK(ff_fit(ctx, F, nrhs * nodes, n, FF_ORD_N[o - 1], o == 1 ? F.mu : F.ord_mu[o - 1], F.mat->ordT[o],
                       F.ord_mu[o], st));
         CK(pack_sources(D, nrhs, layout, o == 0 ? F.eq_pos : F.ord_pos[o], F.eq_pt, o == 0 ? F.mu : F.ord_mu[o],
                         nodes * n, nodes * n, F.rec + F.ord_rec[o] * REC, st));
@@ -1086,7 +1103,7 @@ mfs_status ff_pair_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const 
         const PairWork wl = work_of(ll->p);
         CKS(ff_launch(ctx, variant, g, wl, st));
         CK(pair_epilogue(D, nrhs, wl, nullptr, 0.0, 1.0, F.ulocal, P * FF_LOC_NC, st));
-        CK(ff_fit(ctx, F, nrhs * P, FF_LOC_N, FF_LOC_NC, F.ulocal, F.locT, F.nu, st));
+        CK(ff_fit(ctx, F, nrhs * P, FF_LOC_N, FF_LOC_NC, F.ulocal, F.mat->locT, F.nu, st));
         CK(ff_scale(F.nu, F.rloc, P, D * FF_LOC_N, nrhs, st));
         CK(pack_sources(D, nrhs, layout, F.loc_pos, F.eq_pt, F.nu, P * FF_LOC_N, P * FF_LOC_N, F.rec + F.loc_rec * REC,
                         st));
@@ -1170,22 +1187,52 @@ cudaError_t gemm64(mfs_ctx *ctx, ShapeHost &sh, int cols, int n, int k, const do
 }
 
 // lambda = (I - L) S_L^+ gamma (project) or S_L^+ gamma  (Eq. pseudo, Remark congruent)
+// With pack_variant >= 0 the strengths' source records for that pair-kernel entry too (as pack_for).
 mfs_status precond_apply_dev(mfs_ctx *ctx, const double *gamma, double *lambda, int project, int nrhs,
-                             cudaStream_t st) {
+                             cudaStream_t st, int pack_variant = -1) {
     const int D = ctx->D;
+    int vc = 0;
+    const PairVariant *vv = pair_variants(&vc);
     for (auto &sh : ctx->shapes) {
         const int nb = (int)sh.bodies.size();
         if (nb == 0) continue;
         const int ncols = nb * nrhs;
         const FactorSet &fx = sh.fs[ctx->fset];
         const ShapeDev &sd = fx.dev;
+        ScatterArgs sc;
+        sc.col_body = sh.col_body;
+        sc.col_rhs = sh.col_rhs;
+        sc.body_off = ctx->src_off_d;
+        sc.rot64 = ctx->rot64_d;
+        sc.ncols = ncols;
+        sc.dN = sd.dN;
+        sc.sum_N = ctx->sumN;
+        sc.out = lambda;
+        if (pack_variant >= 0) {
+            sc.rec = ctx->rec_d;
+            sc.packed = vv[pack_variant].packed;
+            sc.rec_floats = pair_record_floats(D, nrhs, sc.packed);
+            sc.nrhs = nrhs;
+            sc.rec_off = ctx->rec_off_d;
+            sc.src_pos = ctx->src_pos_d;
+            if (sc.rec_floats > ctx->rec_floats) {
+                ctx->last_error = "source records larger than their buffer";
+                return MFS_ERR_INVALID_ARG;
+            }
+        }
         if (ctx->opt.precision >= 1) {  // FP64 one-body apply (reference and mixed modes)
             CK(gather_rotate(D, gamma, ctx->sumM * D, sh.col_body, sh.col_rhs, ctx->tgt_off_d, ctx->rot64_d, ncols,
                              sd.dM, sh.A, sh.A64, st));
             CK(gemm64(ctx, sh, ncols, sd.r, sd.dM, sh.A64, sd.U64, sh.T64, st));
             CK(gemm64(ctx, sh, ncols, sd.dN, sd.r, sh.T64, project ? sd.Wp64 : sd.Wr64, sh.L64, st));
-            CK(scatter_rotate(D, nullptr, sh.L64, sh.col_body, sh.col_rhs, ctx->src_off_d, ctx->rot_d, ctx->rot64_d,
-                              ncols, sd.dN, ctx->sumN, lambda, st));
+            sc.L64 = sh.L64;
+        } else if (fx.tc_ready && fc_takes(D, ncols, sd.dM, sd.dN)) {  // few columns: warps on the factor rows
+            CK(gather_rotate_hl(D, gamma, ctx->sumM * D, sh.col_body, sh.col_rhs, ctx->tgt_off_d, ctx->rot64_d, ncols,
+                                sd.dM, sh.Gf, sh.ld1, st));
+            CK(fc_apply(ncols, sd.r, sh.ld1, fx.Utp, fx.ut_stride, sh.Gf, sh.Tf, sh.ld2, st));
+            CK(fc_apply(ncols, sd.dN, sh.ld2, project ? fx.Wptp : fx.Wrtp, fx.wt_stride, sh.Tf, sh.Lf, sd.dN, st));
+            sc.P = sh.Lf;
+            sc.S = 1;
         } else if (fx.tc_ready) {  // tensor cores: multi-piece TF32 tcgen05 GEMMs, double-float chunk sums
             const int np = sh.pieces;
             auto it = sh.amaps.find(ncols);
@@ -1209,13 +1256,12 @@ mfs_status precond_apply_dev(mfs_ctx *ctx, const double *gamma, double *lambda, 
             const int S1 = tc_gemm_chunks(ncols, sd.r, sd.dM, ctx->sm_count, np);
             CK(tc_gemm(np, fx.mU, mp.data(), ncols, sd.r, sd.dM, S1, sh.Ptc, ctx->err_d, st));
             CK(reduce_pieces(tc_gemm_sz(sd.dM, S1), ncols, sd.r, sh.Ptc, sh.Tp, sh.ld2, sh.tp_stride, np, st));
-            // lambda = W t, kept in FP64
+            // lambda = W t, the chunk sums added by the scatter
             const int S2 = tc_gemm_chunks(ncols, sd.dN, sd.r, ctx->sm_count, np);
             CK(tc_gemm(np, project ? fx.mWp : fx.mWr, mp.data() + 3, ncols, sd.dN, sd.r, S2, sh.Ptc, ctx->err_d, st));
-            CK(reduce_f64(tc_gemm_sz(sd.r, S2), (size_t)ncols * sd.dN, sh.Ptc, sh.L64, st));
-            CK(scatter_rotate(D, nullptr, sh.L64, sh.col_body, sh.col_rhs, ctx->src_off_d, ctx->rot_d, ctx->rot64_d,
-                              ncols, sd.dN, ctx->sumN, lambda, st));
-            ctx->launches += 2;
+            sc.P = sh.Ptc;
+            sc.S = tc_gemm_sz(sd.r, S2);
+            ctx->launches += 1;
         } else {
             CK(gather_rotate(D, gamma, ctx->sumM * D, sh.col_body, sh.col_rhs, ctx->tgt_off_d, ctx->rot64_d, ncols,
                              sd.dM, sh.A, nullptr, st));
@@ -1224,10 +1270,10 @@ mfs_status precond_apply_dev(mfs_ctx *ctx, const double *gamma, double *lambda, 
             const int S2 = gemm_splitk_chunks(ncols, sd.dN, sd.r, ctx->sm_count);
             CK(gemm_splitk(ncols, sd.r, sd.dM, S1, sh.A, sd.U, sh.Pk, sh.Tm, nullptr, st));
             CK(gemm_splitk(ncols, sd.dN, sd.r, S2, sh.Tm, project ? sd.Wp : sd.Wr, sh.Pk, nullptr, sh.L64, st));
-            CK(scatter_rotate(D, nullptr, sh.L64, sh.col_body, sh.col_rhs, ctx->src_off_d, ctx->rot_d, ctx->rot64_d,
-                              ncols, sd.dN, ctx->sumN, lambda, st));
+            sc.L64 = sh.L64;
             ctx->launches += 2;
         }
+        CK(scatter_rotate(D, sc, st));
         ctx->launches += 4;
     }
     return MFS_OK;
@@ -1235,8 +1281,11 @@ mfs_status precond_apply_dev(mfs_ctx *ctx, const double *gamma, double *lambda, 
 
 // y = gamma + sum_{k' != k} S^(kk') (I - L^(k')) S_L^(k')+ gamma^(k')  (Eq. 2esysprec)
 mfs_status matvec_dev(mfs_ctx *ctx, const double *gamma, double *y, int nrhs, cudaStream_t st) {
-    CKS(precond_apply_dev(ctx, gamma, ctx->lam_d, 1, nrhs, st));
-    CKS(pair_apply(ctx, ctx->lam_d, y, gamma, 1.0, 1.0, nrhs, 0, st));
+    // direct FP32 sums: the apply's scatter writes the pair kernel's records
+    const bool direct = (ctx->opt.precision == 0 || ctx->opt.precision == 2) && !ctx->ff.ready;
+    const int pack = direct ? forward_variant(ctx, nrhs) : -1;
+    CKS(precond_apply_dev(ctx, gamma, ctx->lam_d, 1, nrhs, st, pack));
+    CKS(pair_apply(ctx, ctx->lam_d, y, gamma, 1.0, 1.0, nrhs, 0, st, pack >= 0));
     return MFS_OK;
 }
 
@@ -1514,27 +1563,43 @@ mfs_status pair_apply_T(mfs_ctx *ctx, const double *w, double *z, int nrhs, int 
 
 // out^(k) = ((I - L^(k)) S_L^(k)+)^T z^(k) = R_M U W_p R_N^T z (project) or (S_L^(k)+)^T z = R_M U W_r R_N^T z,
 // z [nrhs][sum_N][3] -> out [nrhs][sum_M][3] (transposes of the two-step apply, Eq. pseudo).
-mfs_status precondT_dev(mfs_ctx *ctx, const double *z, double *out, int project, int nrhs, cudaStream_t st) {
+// base + that, when base [nrhs][sum_M][3] is given.
+mfs_status precondT_dev(mfs_ctx *ctx, const double *z, double *out, int project, int nrhs, cudaStream_t st,
+                        const double *base = nullptr) {
     for (auto &sh : ctx->shapes) {
         const int nb = (int)sh.bodies.size();
         if (nb == 0) continue;
         const int ncols = nb * nrhs;
         const FactorSet &fx = sh.fs[0];
         const ShapeDev &sd = fx.dev;
+        ScatterArgs sc;
+        sc.col_body = sh.col_body;
+        sc.col_rhs = sh.col_rhs;
+        sc.body_off = ctx->tgt_off_d;
+        sc.rot64 = ctx->rot64_d;
+        sc.ncols = ncols;
+        sc.dN = sd.dM;
+        sc.sum_N = ctx->sumM;
+        sc.out = out;
+        sc.base = base;
         if (ctx->opt.precision == 1) {
             // FP64 reference: out = R_M U (W (R_N^T z)) with the transposed FP64 factors
             CK(gather_rotate(3, z, ctx->sumN * 3, sh.col_body, sh.col_rhs, ctx->src_off_d, ctx->rot64_d, ncols, sd.dN,
                              sh.A, sh.A64, st));
             CK(gemm64(ctx, sh, ncols, sd.r, sd.dN, sh.A64, project ? sd.WpT64 : sd.WrT64, sh.T64, st));
             CK(gemm64(ctx, sh, ncols, sd.dM, sd.r, sh.T64, sd.UT64, sh.O64, st));
-            CK(scatter_rotate(3, nullptr, sh.O64, sh.col_body, sh.col_rhs, ctx->tgt_off_d, ctx->rot_d, ctx->rot64_d,
-                              ncols, sd.dM, ctx->sumM, out, st));
-            ctx->launches += 4;
-            continue;
-        }
-        if (fx.tcT_ready && ctx->opt.precision == 0) {
+            sc.L64 = sh.O64;
+        } else if (fx.tcT_ready && ctx->opt.precision == 0 && fc_takes(3, ncols, sd.dM, sd.dN)) {
+            // few columns, as the forward apply: x = W^T (R_N^T z), out = R_M U x
+            CK(gather_rotate_hl(3, z, ctx->sumN * 3, sh.col_body, sh.col_rhs, ctx->src_off_d, ctx->rot64_d, ncols, sd.dN,
+                                sh.Tf, sh.ld2, st));
+            CK(fc_apply(ncols, sd.r, sh.ld2, project ? fx.WpT : fx.WrT, fx.wt_stride, sh.Tf, sh.Xf, sh.ld2, st));
+            CK(fc_apply(ncols, sd.dM, sh.ld2, fx.Un, fx.un_stride, sh.Xf, sh.Lf, sd.dM, st));
+            sc.P = sh.Lf;
+            sc.S = 1;
+        } else if (fx.tcT_ready && ctx->opt.precision == 0) {
             // tensor cores, as the forward apply: x = W^T (R_N^T z) with the K = dN column pieces in Tp,
-            // x cut back into pieces (same layout, Tp reused), out = R_M U x kept in FP64
+            // x cut back into pieces (same layout, Tp reused), out = R_M U x
             const int np = sh.pieces;
             auto it = sh.amaps.find(ncols);
             if (it == sh.amaps.end()) {
@@ -1558,21 +1623,21 @@ mfs_status precondT_dev(mfs_ctx *ctx, const double *z, double *out, int project,
             CK(reduce_pieces(tc_gemm_sz(sd.dN, S1), ncols, sd.r, sh.PtcT, sh.Tp, sh.ld2, sh.tp_stride, np, st));
             const int S2 = tc_gemm_chunks(ncols, sd.dM, sd.r, ctx->sm_count, np);
             CK(tc_gemm(np, fx.mUn, colmaps, ncols, sd.dM, sd.r, S2, sh.PtcT, ctx->err_d, st));
-            CK(reduce_f64(tc_gemm_sz(sd.r, S2), (size_t)ncols * sd.dM, sh.PtcT, sh.O64, st));
-            CK(scatter_rotate(3, nullptr, sh.O64, sh.col_body, sh.col_rhs, ctx->tgt_off_d, ctx->rot_d, ctx->rot64_d,
-                              ncols, sd.dM, ctx->sumM, out, st));
-            ctx->launches += 6;
-            continue;
+            sc.P = sh.PtcT;
+            sc.S = tc_gemm_sz(sd.r, S2);
+            ctx->launches += 1;
+        } else {
+            CK(gather_rotate(3, z, ctx->sumN * 3, sh.col_body, sh.col_rhs, ctx->src_off_d, ctx->rot64_d, ncols, sd.dN,
+                             sh.A, nullptr, st));
+            const int S1 = gemm_splitk_chunks(ncols, sd.r, sd.dN, ctx->sm_count);
+            const int S2 = gemm_splitk_chunks(ncols, sd.dM, sd.r, ctx->sm_count);
+            CK(gemm_splitk(ncols, sd.r, sd.dN, S1, sh.A, project ? sd.Wp : sd.Wr, sh.PkT, sh.Tm, nullptr, st, true));
+            CK(gemm_splitk(ncols, sd.dM, sd.r, S2, sh.Tm, sd.U, sh.PkT, nullptr, sh.O64, st, true));
+            sc.L64 = sh.O64;
+            ctx->launches += 2;
         }
-        CK(gather_rotate(3, z, ctx->sumN * 3, sh.col_body, sh.col_rhs, ctx->src_off_d, ctx->rot64_d, ncols, sd.dN,
-                         sh.A, nullptr, st));
-        const int S1 = gemm_splitk_chunks(ncols, sd.r, sd.dN, ctx->sm_count);
-        const int S2 = gemm_splitk_chunks(ncols, sd.dM, sd.r, ctx->sm_count);
-        CK(gemm_splitk(ncols, sd.r, sd.dN, S1, sh.A, project ? sd.Wp : sd.Wr, sh.PkT, sh.Tm, nullptr, st, true));
-        CK(gemm_splitk(ncols, sd.dM, sd.r, S2, sh.Tm, sd.U, sh.PkT, nullptr, sh.O64, st, true));
-        CK(scatter_rotate(3, nullptr, sh.O64, sh.col_body, sh.col_rhs, ctx->tgt_off_d, ctx->rot_d, ctx->rot64_d,
-                          ncols, sd.dM, ctx->sumM, out, st));
-        ctx->launches += 6;
+        CK(scatter_rotate(3, sc, st));
+        ctx->launches += 4;
     }
     return MFS_OK;
 }
@@ -1580,12 +1645,7 @@ mfs_status precondT_dev(mfs_ctx *ctx, const double *z, double *out, int project,
 // y = A^T w = w + [((I - L^(k')) S_L^(k')+)^T sum_{k != k'} S^(kk')^T w^(k)]_k'
 mfs_status matvec_T_dev(mfs_ctx *ctx, const double *w, double *y, int nrhs, cudaStream_t st) {
     CKS(pair_apply_T(ctx, w, ctx->lam_d, nrhs, 0, st));
-    CKS(precondT_dev(ctx, ctx->lam_d, ctx->tmpM_d, 1, nrhs, st));
-    const size_t n = (size_t)nrhs * ctx->sumM * 3;
-    combine_raw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ctx->tmpM_d, w, 1.0, 1.0, y, n, 1);
-    CK(cudaGetLastError());
-    ctx->launches += 1;
-    return MFS_OK;
+    return precondT_dev(ctx, ctx->lam_d, y, 1, nrhs, st, w);
 }
 
 struct SolveStats {
@@ -1907,8 +1967,7 @@ static mfs_status alloc_apply_scratch(mfs_ctx *ctx, ShapeHost &sh, cudaStream_t 
         }
     bool ok = ctx->alloc(&sh.col_body, R * nb) == cudaSuccess && ctx->alloc(&sh.col_rhs, R * nb) == cudaSuccess &&
               ctx->alloc(&sh.A, (size_t)R * nb * m) == cudaSuccess &&
-              ctx->alloc(&sh.Tm, (size_t)R * nb * n) == cudaSuccess &&
-              ctx->alloc(&sh.Lm, (size_t)R * nb * n) == cudaSuccess;
+              ctx->alloc(&sh.Tm, (size_t)R * nb * n) == cudaSuccess;
     if (ok && ctx->opt.precision >= 1) {
         size_t need = 1;  // both GEMMs, and the adjoint's second one (n -> m)
         for (int h = 1; h <= R; ++h) {
@@ -1948,6 +2007,15 @@ static mfs_status alloc_apply_scratch(mfs_ctx *ctx, ShapeHost &sh, cudaStream_t 
         if (ok)
             ok = cudaMemsetAsync(sh.Ap, 0, sizeof(float) * np * sh.ap_stride, st) == cudaSuccess &&
                  cudaMemsetAsync(sh.Tp, 0, sizeof(float) * np * sh.tp_stride, st) == cudaSuccess;
+    }
+    if (ok && sh.pieces > 0) {  // few columns (their K padding stays zero, as the pieces')
+        ok = ctx->alloc(&sh.Gf, (size_t)FC_MAX * sh.ld1) == cudaSuccess &&
+             ctx->alloc(&sh.Tf, (size_t)FC_MAX * sh.ld2) == cudaSuccess &&
+             ctx->alloc(&sh.Xf, (size_t)FC_MAX * sh.ld2) == cudaSuccess &&
+             ctx->alloc(&sh.Lf, (size_t)FC_MAX * m) == cudaSuccess &&
+             cudaMemsetAsync(sh.Xf, 0, sizeof(float2) * FC_MAX * sh.ld2, st) == cudaSuccess &&
+             cudaMemsetAsync(sh.Gf, 0, sizeof(float2) * FC_MAX * sh.ld1, st) == cudaSuccess &&
+             cudaMemsetAsync(sh.Tf, 0, sizeof(float2) * FC_MAX * sh.ld2, st) == cudaSuccess;
     }
     if (!ok) {
         cudaGetLastError();
@@ -2021,14 +2089,14 @@ static __global__ void ff_scale_columns_kernel(double *V, const double *s, int n
     V[i] *= s[k] > trunc * s[0] ? 1.0 / s[k] : 0.0;
 }
 
-// The transposed pseudo-inverse [m][n] (device, row-major, owned by the caller through ctx->alloc) of a
+// The transposed pseudo-inverse [m][n] (device, row-major, cudaMalloc'ed, the caller's) of a
 // column-major m x n matrix, m >= n, in FP64, truncated at `trunc` of the largest singular value.
 static mfs_status ff_pinvT(mfs_ctx *ctx, cusolverDnHandle_t solver, int m, int n, const std::vector<double> &A,
                            double trunc, double **out, cudaStream_t st) {
     double *A_d = nullptr, *U_d = nullptr, *S_d = nullptr, *VT_d = nullptr, *work = nullptr, *P_d = nullptr;
     int *info_d = nullptr, lwork = 0, info_h = 0;
     double s0 = 0.0;
-    CK(ctx->alloc(out, (size_t)m * n));
+    CK(cudaMalloc(out, sizeof(double) * (size_t)m * n));
     bool ok = cudaMalloc(&A_d, sizeof(double) * A.size()) == cudaSuccess &&
               cudaMalloc(&U_d, sizeof(double) * (size_t)m * n) == cudaSuccess &&
               cudaMalloc(&S_d, sizeof(double) * n) == cudaSuccess &&
@@ -2059,10 +2127,7 @@ static mfs_status ff_pinvT(mfs_ctx *ctx, cusolverDnHandle_t solver, int m, int n
     return MFS_OK;
 }
 
-// The matrices on the unit sphere: check field -> order-0 strengths (PinvT), each order's strengths ->
-// the next lower order's (ordT), local check field -> local sources (locT).  They depend on the kernel
-// only, so a context computes them once.
-static mfs_status ff_unit_matrices(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStream_t st) {
+static mfs_status ff_build_matrices(mfs_ctx *ctx, FFMatrices &M, cudaStream_t st) {
     const int D = ctx->D;
     cusolverDnHandle_t solver = nullptr;
     if (cusolverDnCreate(&solver) != CUSOLVER_STATUS_SUCCESS) {
@@ -2076,33 +2141,54 @@ static mfs_status ff_unit_matrices(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStrea
             unit_fibonacci(FF_ORD_N[o], e[o]);
             unit_fibonacci(FF_ORD_NC[o], c);
             const int m = D * FF_ORD_NC[o], n = D * FF_ORD_N[o];
-            double *pinvT = nullptr;
-            CKS(ff_pinvT(ctx, solver, m, n, ff_map(D, c, FF_ORD_CHECK[o], e[o], 1.0), FF_ORD_TRUNC[o], &pinvT, st));
-            if (o == 0) {
-                F.PinvT = pinvT;
+            double *pinvT = nullptr, *G_d = nullptr;
+            const mfs_status s = ff_pinvT(ctx, solver, m, n, ff_map(D, c, FF_ORD_CHECK[o], e[o], 1.0),
+                                          FF_ORD_TRUNC[o], o == 0 ? &M.PinvT : &pinvT, st);
+            if (s != MFS_OK || o == 0) {
+                cudaFree(pinvT);
+                CKS(s);
                 continue;
             }
             // ordT = (previous order's field at this order's check points)^T pinvT
             const int np = D * FF_ORD_N[o - 1];
             const std::vector<double> G = ff_map(D, c, FF_ORD_CHECK[o], e[o - 1], 1.0);
-            double *G_d = nullptr;
-            CK(ctx->alloc(&G_d, G.size()));
-            CK(ctx->alloc(&F.ordT[o], (size_t)np * n));
-            CK(cudaMemcpyAsync(G_d, G.data(), sizeof(double) * G.size(), cudaMemcpyHostToDevice, st));
-            CK(gemm_rm64_splitk(np, n, m, 1, G_d, pinvT, nullptr, F.ordT[o], st));
-            CK(cudaStreamSynchronize(st));
-            ctx->release(G_d);
-            ctx->release(pinvT);
+            const bool ok =
+                cudaMalloc(&G_d, sizeof(double) * G.size()) == cudaSuccess &&
+                cudaMalloc(&M.ordT[o], sizeof(double) * (size_t)np * n) == cudaSuccess &&
+                cudaMemcpyAsync(G_d, G.data(), sizeof(double) * G.size(), cudaMemcpyHostToDevice, st) == cudaSuccess &&
+                gemm_rm64_splitk(np, n, m, 1, G_d, pinvT, nullptr, M.ordT[o], st) == cudaSuccess &&
+                cudaStreamSynchronize(st) == cudaSuccess;
+            cudaFree(G_d);
+            cudaFree(pinvT);
+            if (!ok) CK(cudaErrorMemoryAllocation);
         }
         std::vector<double> l;
         unit_fibonacci(FF_LOC_N, l);
         unit_fibonacci(FF_LOC_NC, c);
         return ff_pinvT(ctx, solver, D * FF_LOC_NC, D * FF_LOC_N, ff_map(D, c, FF_LOC_CHECK, l, FF_LOC_EQ),
-                        FF_LOC_TRUNC, &F.locT, st);
+                        FF_LOC_TRUNC, &M.locT, st);
     };
     const mfs_status rc = build();
     cusolverDnDestroy(solver);
     return rc;
+}
+
+// The matrices of this context's kernel on the current device: those of another live context, or built
+// (five small FP64 SVDs, 0.1 s) under the lock and complete on the device before anyone else sees them.
+static mfs_status ff_matrices(mfs_ctx *ctx, std::shared_ptr<const FFMatrices> &out, cudaStream_t st) {
+    static std::mutex mu;
+    static std::weak_ptr<const FFMatrices> kept[64][2];
+    int dev = 0;
+    CK(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev < 64) out = kept[dev][ctx->D == 3].lock();
+    if (out) return MFS_OK;
+    auto M = std::make_shared<FFMatrices>();
+    CKS(ff_build_matrices(ctx, *M, st));
+    CK(cudaStreamSynchronize(st));
+    out = M;
+    if (dev < 64) kept[dev][ctx->D == 3] = out;
+    return MFS_OK;
 }
 
 // Frees the far-field structures that depend on the body centres (all but the pseudo-inverse) and
@@ -2176,16 +2262,7 @@ static mfs_status ff_setup(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStream_t st) 
     std::vector<double> ue, uc;
     unit_fibonacci(FF_NE, ue);
     unit_fibonacci(FF_NC, uc);
-    if (!F.PinvT) {  // independent of the centres (kept across moves) and of the roles (shared)
-        const auto &other = &F == &ctx->ff ? ctx->ffT : ctx->ff;
-        if (other.PinvT) {
-            F.PinvT = other.PinvT;
-            F.locT = other.locT;
-            for (int o = 1; o < FF_NORD; ++o) F.ordT[o] = other.ordT[o];
-        } else {
-            CKS(ff_unit_matrices(ctx, F, st));
-        }
-    }
+    if (!F.mat) CKS(ff_matrices(ctx, F.mat, st));  // independent of the centres
     // Local expansions where a body has clearly more targets than check points: with fewer, the check
     // sums and the match cost more than the lower orders at the targets themselves (ff_cell_lists then
     // weighs each cell).

@@ -1234,7 +1234,7 @@ __global__ void __launch_bounds__(NT, MINB) pair_sum_kernel(PairGeom geo, PairWo
 // result is deterministic; with S = 1 it is the plain sum in CTA order.  Tiles shared by many CTAs
 // (the far-field upward sums of the top nodes) are why S and the y blocks exist.
 template <int D, int NRHS>
-__global__ void __launch_bounds__(1024) pair_epilogue_kernel(PairWork work, const double *base, double beta, double scale, double *out,
+__global__ void __launch_bounds__(256) pair_epilogue_kernel(PairWork work, const double *base, double beta, double scale, double *out,
                                      int ntargets, int S) {
     constexpr int C = D * NRHS;
     constexpr int MAXS = 256;
@@ -1567,13 +1567,14 @@ cudaError_t pair_launch(int vi, const PairGeom &geo, const PairWork &work, int *
 
 cudaError_t pair_epilogue(int D, int nrhs, const PairWork &work, const double *base, double beta, double scale,
                           double *out, int ntargets, cudaStream_t st) {
-    const int threads = 1024;
+    const int threads = 256;
     if (work.ntiles == 0) return cudaSuccess;
-    // lanes per entry from the most CTAs on one tile; blocks per tile so that a tile's entries times
-    // lanes fill about one 1024-thread block each (at most 16)
+    // lanes per entry from the most CTAs on one tile; blocks per tile so that a tile's entries times lanes
+    // fill one block each.  Few tiles are shared by many CTAs (six spheres: 3 tiles, 24 shares an entry),
+    // whose FP64 additions must spread over the SMs: 1024-thread blocks on six SMs took 9 us.
     const int S = work.max_share >= 64 ? 8 : (work.max_share >= 16 ? 4 : 1);
     const long long lanes = (long long)work.tile_targets * D * nrhs * S;
-    const int Y = (int)std::min<long long>(16, std::max<long long>(1, (lanes + threads - 1) / threads));
+    const int Y = (int)std::min<long long>(64, std::max<long long>(1, (lanes + threads - 1) / threads));
     const dim3 grid((unsigned)work.ntiles, (unsigned)Y);
 #define E(D_, R_)                                                                                      \
     if (D == D_ && nrhs == R_) {                                                                       \
@@ -1811,7 +1812,7 @@ extern "C" mfs_status mfs_stokeslet_sum_noalloc(const double *targets, int32_t n
     work.tile_targets = TT;
     work.include_self = 1;
     if (launch_variant<Pol, NT>(geo, work, &meta->err, st) != cudaSuccess) return MFS_ERR_CUDA;
-    pair_epilogue_kernel<3, 1><<<ntiles, 1024, 0, st>>>(work, nullptr, 0.0, 1.0 / (8.0 * MFS_PI * mu), u,
+    pair_epilogue_kernel<3, 1><<<dim3(ntiles, (3 * TT + 255) / 256), 256, 0, st>>>(work, nullptr, 0.0, 1.0 / (8.0 * MFS_PI * mu), u,
                                                        num_targets, 1);
     poison_on_timeout_kernel<<<sms, 256, 0, st>>>(&meta->err, u, 3 * (size_t)num_targets);
     return cudaGetLastError() == cudaSuccess ? MFS_OK : MFS_ERR_CUDA;

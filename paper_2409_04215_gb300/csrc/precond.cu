@@ -232,7 +232,7 @@ cudaError_t build_apply_factors(int kind, int M, int N, const double *Ucm, const
 }
 
 // ---------------------------------------------------------------------------
-// Gather / scatter with per-body rotation
+// Gather with per-body rotation
 // ---------------------------------------------------------------------------
 __global__ void gather_rotate_kernel(int D, const double *gamma, int sum_MD, const int *col_body, const int *col_rhs,
                                      const int *body_tgt_off, const double *rot, int ncols, int dM, float *A,
@@ -267,39 +267,6 @@ cudaError_t gather_rotate(int D, const double *gamma, int sum_MD, const int *col
     dim3 grid((M + 127) / 128, ncols);
     gather_rotate_kernel<<<grid, 128, 0, st>>>(D, gamma, sum_MD, col_body, col_rhs, body_tgt_off, rot, ncols, dM, A,
                                                 A64);
-    return cudaGetLastError();
-}
-
-__global__ void scatter_rotate_kernel(int D, const float *L, const double *L64, const int *col_body,
-                                      const int *col_rhs, const int *body_src_off, const double *rot64, int ncols,
-                                      int dN, int sum_N, double *lambda) {
-    const int col = blockIdx.y;
-    const int N = dN / D;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= N || col >= ncols) return;
-    const int k = col_body[col], h = col_rhs[col];
-    double *out = lambda + ((size_t)h * sum_N + body_src_off[k]) * D;
-    if (D == 1) {
-        out[p] = L64 ? L64[(size_t)col * dN + p] : (double)L[(size_t)col * dN + p];
-    } else {
-        double v[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) v[a] = L64 ? L64[(size_t)col * dN + 3 * p + a] : (double)L[(size_t)col * dN + 3 * p + a];
-        const double *R = rot64 + 9 * k;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) out[3 * p + a] = R[3 * a] * v[0] + R[3 * a + 1] * v[1] + R[3 * a + 2] * v[2];
-    }
-}
-
-cudaError_t scatter_rotate(int D, const float *L, const double *L64, const int *col_body, const int *col_rhs,
-                           const int *body_src_off, const float *rot, const double *rot64, int ncols, int dN,
-                           int sum_N, double *lambda, cudaStream_t st) {
-    (void)rot;
-    if (ncols == 0) return cudaSuccess;
-    const int N = dN / D;
-    dim3 grid((N + 127) / 128, ncols);
-    scatter_rotate_kernel<<<grid, 128, 0, st>>>(D, L, L64, col_body, col_rhs, body_src_off, rot64, ncols, dN, sum_N,
-                                                 lambda);
     return cudaGetLastError();
 }
 

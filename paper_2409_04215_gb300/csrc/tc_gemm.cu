@@ -375,15 +375,6 @@ __global__ void reduce_pieces_kernel(int S, int rows, int cols, const float2 *__
     }
 }
 
-// C = sum_z P[z] as FP64.
-__global__ void reduce_f64_kernel(int S, size_t mn, const float2 *__restrict__ P, double *C) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < mn; i += (size_t)gridDim.x * blockDim.x) {
-        float hi, lo;
-        df_chunk_sum(S, mn, i, P, hi, lo);
-        C[i] = (double)hi + (double)lo;
-    }
-}
-
 // Gather and rotate into the body frame (as gather_rotate), written directly as pieces
 // dst[p][col][ld_dst] of the FP64 values.
 __global__ void gather_rotate_pieces_kernel(int D, const double *gamma, int sum_MD, const int *col_body,
@@ -459,12 +450,6 @@ cudaError_t reduce_pieces(int S, int rows, int cols, const float2 *P, float *dst
     if (pieces < 2 || pieces > 3) return cudaErrorInvalidValue;
     reduce_pieces_kernel<<<(unsigned)std::min<size_t>((mn + 255) / 256, 4096), 256, 0, st>>>(S, rows, cols, P, dst,
                                                                                                ld_dst, pstride, pieces);
-    return cudaGetLastError();
-}
-
-cudaError_t reduce_f64(int S, size_t mn, const float2 *P, double *C, cudaStream_t st) {
-    if (mn == 0) return cudaSuccess;
-    reduce_f64_kernel<<<(unsigned)std::min<size_t>((mn + 255) / 256, 4096), 256, 0, st>>>(S, mn, P, C);
     return cudaGetLastError();
 }
 
