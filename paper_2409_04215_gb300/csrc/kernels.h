@@ -25,6 +25,23 @@ cudaError_t pair_epilogue(int D, int nrhs, const PairWork &work, const double *b
                           double *out, int ntargets, cudaStream_t st);
 cudaError_t pack_sources(int D, int nrhs, int packed, const float4 *src_pos, const int *src_pt_of_rec,
                          const double *strength, int nsrc, int nrec, float *records, cudaStream_t st);
+// Records of several point sets in one launch: set q's n[q] points at pos[q] with strengths
+// strength[q] [nrhs][n[q]][D] to rec[q].
+struct PackSets {
+    static constexpr int MAX = 8;
+    int sets = 0;
+    int n[MAX] = {};
+    const float4 *pos[MAX] = {};
+    const double *strength[MAX] = {};
+    float *rec[MAX] = {};
+    void add(int count, const float4 *p, const double *s, float *r) {
+        n[sets] = count;
+        pos[sets] = p;
+        strength[sets] = s;
+        rec[sets++] = r;
+    }
+};
+cudaError_t pack_sets(int D, int nrhs, int packed, const PackSets &a, cudaStream_t st);
 // Records of the compensated kernels from FP64 body-local positions [nsrc][3] and strengths.
 cudaError_t pack_sources_comp(int D, int nrhs, const double *src_local64, const int *src_pt_of_rec,
                               const double *strength, int nsrc, int nrec, float *records, cudaStream_t st);

@@ -239,6 +239,7 @@ struct mfs_ctx {
             int *seg = nullptr;
             long long *cum = nullptr;
             double pairs = 0.0;                      // target-source pairs one application evaluates
+            int orders = 0;                          // bit o: the lists hold segments of order o
         };
         std::map<int, ListPlan> up;                  // upward sums, key: variant
         std::map<int, ListPlan> ev;                  // order-0 lists at the targets (gradient), key: variant
@@ -249,6 +250,7 @@ struct mfs_ctx {
             std::vector<int> cell_of;                // tree position -> cell
             std::vector<std::vector<int>> local;     // per cell
             std::vector<std::vector<int>> direct;    // per tree position
+            bool any_local = false;
         };
         Cells cells;
     } ff, ffT;                                       // forward sums; transposed sums (adjoint)
@@ -837,6 +839,14 @@ static void ff_segments(const mfs_ctx::FarField &F, std::vector<long long> &bloc
     }
 }
 
+// The orders of equivalent sources among the segments (bit o: order o).
+static int ff_orders(const mfs_ctx *ctx, const mfs_ctx::FarField &F, const std::vector<int> &segs) {
+    int mask = 0;
+    for (int sg : segs)
+        if (sg >= ctx->P && sg < ctx->P + FF_NORD * F.nodes) mask |= 1 << ((sg - ctx->P) / F.nodes);
+    return mask;
+}
+
 static std::vector<int> suspension_of_bodies(const mfs_ctx *ctx) {
     std::vector<int> sus(ctx->P);
     for (int sp = 0; sp < ctx->S; ++sp)
@@ -926,6 +936,7 @@ static const mfs_ctx::FarField::Cells &ff_cells(mfs_ctx *ctx, mfs_ctx::FarField 
             c.local.emplace_back();
             ff_cell_lists(F.tree, F.tree.roots[sp], tb, ctx->centres.data(), F.rtgt.data(),
                           ctx->opt.farfield_separation, (double)F.ntgt / ctx->P, c.local.back(), direct);
+            c.any_local = c.any_local || !c.local.back().empty();
             for (int q = q0; q < q1; ++q) {
                 c.cell_of[q] = (int)c.first.size();
                 c.direct[q].swap(direct[q - q0]);
@@ -948,8 +959,11 @@ mfs_status ff_loc_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, FFListPl
         ff_segments(F, blocks, recs);
         for (int q = 0; q <= P; ++q) toff[q] = q * FF_LOC_NC;
         CKS(build_plan_lists(ctx, variant, 1, toff, 0, cells.first, blocks, recs,
-                             [&](int g0, int, std::vector<int> &segs) { segs = cells.local[cells.cell_of[g0]]; }, lp.p,
-                             &lp.seg, &lp.cum, lp.pairs));
+                             [&](int g0, int, std::vector<int> &segs) {
+                                 segs = cells.local[cells.cell_of[g0]];
+                                 lp.orders |= ff_orders(ctx, F, segs);
+                             },
+                             lp.p, &lp.seg, &lp.cum, lp.pairs));
         it = F.loc.emplace(variant, lp).first;
     }
     *out = &it->second;
@@ -978,6 +992,7 @@ mfs_status ff_direct_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, int i
                                  [&](int g0, int, std::vector<int> &segs) {
                                      segs = cells.direct[g0];
                                      if (include_self) segs.push_back(g0);
+                                     lp.orders |= ff_orders(ctx, F, segs);
                                  },
                                  lp.p, &lp.seg, &lp.cum, lp.pairs));
         } else {
@@ -990,6 +1005,7 @@ mfs_status ff_direct_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, int i
                                      ff_ordered_list(F.tree, F.tree.roots[sus[tb[0]]], tb, ctx->centres.data(),
                                                      F.rtgt.data(), ctx->opt.farfield_separation, !include_self,
                                                      segs);
+                                     lp.orders |= ff_orders(ctx, F, segs);
                                  },
                                  lp.p, &lp.seg, &lp.cum, lp.pairs));
         }
@@ -1085,18 +1101,26 @@ mfs_status ff_pair_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const 
     const PairVariant *vv = pair_variants(&vc);
     const int D = ctx->D, nodes = F.nodes, P = ctx->P, layout = vv[variant].packed;
     const size_t REC = pair_record_floats(D, nrhs, layout);
+    // local expansions, and the orders that the lists hold (a small cluster needs few of them)
+    const bool local = F.use_local && F.cells.any_local;
+    if (local) CKS(ff_loc_plan(ctx, F, variant, &ll));
+    const int orders = pl->orders | (local ? ll->orders : 0);
     CKS(ff_upward(ctx, F, variant, strength, nrhs, st));
-    for (int o = 0; o < FF_NORD; ++o) {
+    PackSets sets;
+    for (int o = 0; o < FF_NORD && (orders >> o) != 0; ++o) {
         const int n = FF_ORD_N[o];
-        if (o > 0)
+        if (o > 0) {
             CK(ff_fit(ctx, F, nrhs * nodes, n, FF_ORD_N[o - 1], o == 1 ? F.mu : F.ord_mu[o - 1], F.mat->ordT[o],
                       F.ord_mu[o], st));
-        CK(pack_sources(D, nrhs, layout, o == 0 ? F.eq_pos : F.ord_pos[o], F.eq_pt, o == 0 ? F.mu : F.ord_mu[o],
-                        nodes * n, nodes * n, F.rec + F.ord_rec[o] * REC, st));
+            ctx->launches += 1;
+        }
+        if ((orders >> o) & 1)
+            sets.add(nodes * n, o == 0 ? F.eq_pos : F.ord_pos[o], o == 0 ? F.mu : F.ord_mu[o],
+                     F.rec + F.ord_rec[o] * REC);
     }
-    ctx->launches += 2 * FF_NORD - 1;
-    if (F.use_local) {
-        CKS(ff_loc_plan(ctx, F, variant, &ll));
+    CK(pack_sets(D, nrhs, layout, sets, st));
+    ctx->launches += 1;
+    if (local) {
         PairGeom g = ff_geom(F, *ll);
         g.tgt = F.lchk_pos;
         g.ntargets = P * FF_LOC_NC;
@@ -1105,8 +1129,9 @@ mfs_status ff_pair_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const 
         CK(pair_epilogue(D, nrhs, wl, nullptr, 0.0, 1.0, F.ulocal, P * FF_LOC_NC, st));
         CK(ff_fit(ctx, F, nrhs * P, FF_LOC_N, FF_LOC_NC, F.ulocal, F.mat->locT, F.nu, st));
         CK(ff_scale(F.nu, F.rloc, P, D * FF_LOC_N, nrhs, st));
-        CK(pack_sources(D, nrhs, layout, F.loc_pos, F.eq_pt, F.nu, P * FF_LOC_N, P * FF_LOC_N, F.rec + F.loc_rec * REC,
-                        st));
+        PackSets loc;
+        loc.add(P * FF_LOC_N, F.loc_pos, F.nu, F.rec + F.loc_rec * REC);
+        CK(pack_sets(D, nrhs, layout, loc, st));
         ctx->launches += 4;
     }
     PairGeom g = ff_geom(F, *pl);
@@ -2264,9 +2289,10 @@ static mfs_status ff_setup(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStream_t st) 
     unit_fibonacci(FF_NC, uc);
     if (!F.mat) CKS(ff_matrices(ctx, F.mat, st));  // independent of the centres
     // Local expansions where a body has clearly more targets than check points: with fewer, the check
-    // sums and the match cost more than the lower orders at the targets themselves (ff_cell_lists then
-    // weighs each cell).
-    F.use_local = F.ntgt >= 160LL * P;
+    // sums, the match and six more launches cost more than the lower orders at the targets themselves
+    // (150 ellipsoids with 200 targets each: 1.15 ms with them, 1.08 without); ff_cell_lists then
+    // weighs each cell.
+    F.use_local = F.ntgt >= 2LL * FF_LOC_NC * P;
     for (int k = 0; k < P; ++k) F.use_local = F.use_local && F.rtgt[k] > 0.0;
     // tree-ordered geometry and segments: proxy segment q (tree position) = body order[q], node segment
     // P + o nodes + node = order o of its equivalent points, local segment P + FF_NORD nodes + q

@@ -1294,19 +1294,14 @@ __global__ void __launch_bounds__(256) pair_epilogue_kernel(PairWork work, const
     }
 }
 
-// Pack proxy strengths (FP64 [nrhs][sum_N][D], body-local rotated positions) into FP32 records.
-// Padding records (beyond N_k in each body) sit at the body centre with zero strength, which
-// contributes exactly zero to every target off that centre.
+// One record: point p's position and strengths (p < 0: padding, all zero).
 template <int D, int NRHS, bool PACKED>
-__global__ void pack_sources_kernel(const float4 *src_pos, const int *src_pt_of_rec, const double *strength, int nsrc,
-                                    int nrec, float *records) {
+__device__ __forceinline__ void pack_record(const float4 *src_pos, int p, const double *strength, int nsrc,
+                                            float *record) {
     constexpr int NV = 3 + D * NRHS, REC = rec_floats(D, NRHS, PACKED);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nrec) return;
     float v[NV];
 #pragma unroll
     for (int c = 0; c < NV; ++c) v[c] = 0.f;
-    const int p = src_pt_of_rec[i];
     if (p >= 0) {
         const float4 y = src_pos[p];
         v[0] = y.x;
@@ -1329,9 +1324,30 @@ __global__ void pack_sources_kernel(const float4 *src_pos, const int *src_pt_of_
             r[c] = v[c];
         }
     }
-    float4 *o = reinterpret_cast<float4 *>(records + (size_t)i * REC);
+    float4 *o = reinterpret_cast<float4 *>(record);
 #pragma unroll
     for (int q = 0; q < REC / 4; ++q) o[q] = make_float4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+}
+
+// Pack proxy strengths (FP64 [nrhs][sum_N][D], body-local rotated positions) into FP32 records.
+// Padding records (beyond N_k in each body) sit at the body centre with zero strength, which
+// contributes exactly zero to every target off that centre.
+template <int D, int NRHS, bool PACKED>
+__global__ void pack_sources_kernel(const float4 *src_pos, const int *src_pt_of_rec, const double *strength, int nsrc,
+                                    int nrec, float *records) {
+    constexpr int REC = rec_floats(D, NRHS, PACKED);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nrec) return;
+    pack_record<D, NRHS, PACKED>(src_pos, src_pt_of_rec[i], strength, nsrc, records + (size_t)i * REC);
+}
+
+// The same for several point sets in one launch (blockIdx.y), record i of a set its point i.
+template <int D, int NRHS, bool PACKED>
+__global__ void pack_sets_kernel(PackSets a) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y;
+    if (i >= a.n[q]) return;
+    pack_record<D, NRHS, PACKED>(a.pos[q], i, a.strength[q], a.n[q],
+                                 a.rec[q] + (size_t)i * rec_floats(D, NRHS, PACKED));
 }
 
 // Records of the compensated policies (layout above) from FP64 body-local positions and strengths.
@@ -1596,6 +1612,24 @@ cudaError_t pack_sources(int D, int nrhs, int packed, const float4 *src_pos, con
         pack_sources_kernel<D_, R_, PA_><<<blocks, threads, 0, st>>>(src_pos, src_pt_of_rec, strength, nsrc, nrec, \
                                                                      records);                         \
         return cudaGetLastError();                                                                      \
+    }
+    PK(3, 1, false) PK(3, 2, false) PK(3, 3, false) PK(3, 4, false)
+    PK(1, 1, false) PK(1, 2, false) PK(1, 3, false) PK(1, 4, false)
+    PK(3, 1, true) PK(3, 2, true) PK(3, 3, true) PK(3, 4, true)
+    PK(1, 1, true) PK(1, 2, true) PK(1, 3, true) PK(1, 4, true)
+#undef PK
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t pack_sets(int D, int nrhs, int packed, const PackSets &a, cudaStream_t st) {
+    int most = 0;
+    for (int q = 0; q < a.sets; ++q) most = std::max(most, a.n[q]);
+    if (most == 0) return cudaSuccess;
+    const dim3 grid((most + 255) / 256, a.sets);
+#define PK(D_, R_, PA_)                                              \
+    if (D == D_ && nrhs == R_ && (packed != 0) == PA_) {             \
+        pack_sets_kernel<D_, R_, PA_><<<grid, 256, 0, st>>>(a);      \
+        return cudaGetLastError();                                   \
     }
     PK(3, 1, false) PK(3, 2, false) PK(3, 3, false) PK(3, 4, false)
     PK(1, 1, false) PK(1, 2, false) PK(1, 3, false) PK(1, 4, false)
