@@ -7,8 +7,8 @@
 // positions, and one warp per chunk places its points in order (so equal keys keep the caller's order
 // and a call's result does not depend on timing).  On the host the same grouping took 6.5 ms for
 // 100 003 points without owners and 60 bodies, and 1 ms for 72 000 points with owners: the velocity call
-// took 9.78 ms and takes 1.41 ms, pressure and traction took 2.61 ms and take 1.38 ms (60 spheres, N = 300;
-// the pair kernels' share is 1.0 ms of either).
+// took 9.78 ms and takes 1.38 ms, pressure and traction took 2.61 ms and take 1.23 ms (60 spheres, N = 300;
+// the pair kernels' share is about 1 ms of either).
 #include <algorithm>
 
 #include "common.cuh"
@@ -18,7 +18,8 @@ namespace mfs {
 
 #define EVAL_THREADS 256
 
-int eval_chunks(int np) { return std::max(1, std::min(1024, (np + 1023) / 1024)); }
+// chunks of 256 points (the placing warp's 8 dependent rounds), longer ones beyond 1024 chunks
+int eval_chunks(int np) { return std::max(1, std::min(1024, (np + 255) / 256)); }
 
 __device__ __forceinline__ int chunk_begin(int np, int nchunks, int c) {
     return (int)((long long)np * c / nchunks);
@@ -87,12 +88,12 @@ __global__ void eval_chunk_scan_kernel(int *counts, int nchunks, int P, int *tot
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= P) return;
     int run = 0;
-    for (int c0 = 0; c0 < nchunks; c0 += 8) {
-        int v[8];
+    for (int c0 = 0; c0 < nchunks; c0 += 32) {  // 32 loads in flight
+        int v[32];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = c0 + u < nchunks ? counts[(size_t)(c0 + u) * P + q] : 0;
+        for (int u = 0; u < 32; ++u) v[u] = c0 + u < nchunks ? counts[(size_t)(c0 + u) * P + q] : 0;
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
+        for (int u = 0; u < 32; ++u)
             if (c0 + u < nchunks) {
                 counts[(size_t)(c0 + u) * P + q] = run;
                 run += v[u];

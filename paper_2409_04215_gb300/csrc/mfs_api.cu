@@ -3734,8 +3734,9 @@ mfs_status mfs_evaluate_stress(mfs_ctx *ctx, const double *points, const double 
         } else {
             PairPlan plan;
             CKS(build_plan_for(ctx, sv, 1, gr.toff, ctx->blk_off, np, plan, &tmp));
-            CK(pack_sources(3, nrhs, 0, ctx->src_pos_d, ctx->rec_pt_d, ctx->lam_d, ctx->sumN, ctx->nrec, ctx->rec_d,
-                            st));
+            int vc = 0;
+            CK(pack_sources(3, nrhs, pair_variants(&vc)[sv].packed, ctx->src_pos_d, ctx->rec_pt_d, ctx->lam_d,
+                            ctx->sumN, ctx->nrec, ctx->rec_d, st));
             PairGeom g = geom_of(ctx);
             g.tgt = gr.t4;
             g.ntargets = np;

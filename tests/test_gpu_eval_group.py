@@ -36,7 +36,7 @@ def _solved(wl, **kw):
 
 
 @pytest.mark.parametrize("farfield", [0, 1])
-@pytest.mark.parametrize("n", [1, 31, 1023, 1025, 4099])
+@pytest.mark.parametrize("n", [1, 31, 257, 1023, 1025, 4099])
 def test_grouping_matches_small_calls(n, farfield):
     wl = sphere_suspension(count=7, m=90, n=40, seed=3)
     ctx = _solved(wl, farfield=farfield)
