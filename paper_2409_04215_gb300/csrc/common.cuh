@@ -33,6 +33,8 @@ struct PairTile {
     int B0, B1;          // source bodies of the suspension [B0, B1)
     long long u0, u1;    // global unit range of this tile
     int gA, gB;          // first and last CTA whose share meets this tile
+    int slotA = 0;       // the slot CTA gA wrote the tile's sum to: 0 when its share starts in the tile, 1 when
+                         // it ends there (every later CTA's share starts in the tile: slot 0)
     int L0, L1;          // L0 >= 0: the tile's sources are the segments of interaction-list entries
                          // [L0, L1) (PairGeom::lst_*) instead of the bodies [B0, B1)
 };

@@ -9,7 +9,7 @@
 // about the same length whatever the lanes' sizes; with a fixed number of blocks per lane, suspensions
 // of 2 to 64 bodies left most SMs waiting for the longest lane).  What bounds the step is latency and
 // the FP64 pipe, not bandwidth: an iteration was ten launches, each a chain of dependent loads, so it is
-// five here (dot, update, dot, update, finish), and one for short lanes (gm_arnoldi_cluster_kernel).  A
+// four here (dot, update and dot, update, finish), and one for short lanes (gm_arnoldi_cluster_kernel).  A
 // warp's FP64 instruction holds its scheduler's FP64 pipe for 64 clocks however many of its lanes are
 // active, so scalar FP64 work (norms, rotations, the tails of reductions) is done by one warp and handed
 // on through shared memory, and no warp runs FP64 instructions on elements or columns that do not exist.
@@ -143,20 +143,35 @@ __device__ __forceinline__ double2 norm_and_inverse(double s) {
     return make_double2(isfinite(s) ? s * inv : sqrt(s), inv);
 }
 
-// The Givens update of column j for lane l (one thread): hcol[0 .. j] the column's entries, hn the norm
-// of the new Krylov vector, cs, sn the earlier rotations (hcol, cs and sn preferably in shared memory).
-__device__ void givens_lane(const GmresDev &gd, int l, int j, const double *hcol, const double *cs_, const double *sn_,
+// The Givens update of column j for lane l, by one warp: hc[0 .. j] the column's entries, hn the norm of
+// the new Krylov vector, cs, sn the earlier rotations (all in shared memory; hc and cs are overwritten).
+// The rotations chain through one value, carry_{i+1} = -sn_i carry_i + cs_i h_{i+1}: the lanes form
+// cs_i h_{i+1} first, one lane walks the chain with a single FMA a step, the lanes finish the entries.
+__device__ void givens_lane(const GmresDev &gd, int l, int j, double *hc, double *cs_, const double *sn_,
                             double h_next) {
-    const int m = gd.m;
+    const int m = gd.m, lane = threadIdx.x & 31;
     double *H = gd.H + (size_t)l * (m + 1) * m;  // H[i][jj] at i*m + jj
     double *cs = gd.cs + (size_t)l * m, *sn = gd.sn + (size_t)l * m, *g = gd.g + (size_t)l * (m + 1);
-    double carry = hcol[0];  // the rotated entry, carried in a register
-    for (int i = 0; i < j; ++i) {
-        const double c = hcol[i + 1];
-        H[i * m + j] = cs_[i] * carry + sn_[i] * c;
-        carry = -sn_[i] * carry + cs_[i] * c;
+    // per step i < j: t = cs_i h_{i+1} and s = sn_i h_{i+1}; H_i = cs_i carry_i + s, carry_{i+1} = t - sn_i carry_i
+    for (int i0 = 0; i0 < j; i0 += 32) {
+        const int i = i0 + lane;
+        const bool in = i < j;
+        const double c1 = in ? hc[i + 1] : 0.0, ci = in ? cs_[i] : 0.0, si = in ? sn_[i] : 0.0;
+        const double first = hc[i0];  // carry_{i0}
+        __syncwarp();
+        const double t = ci * c1;
+        double carry = first, mine = first;  // carry_i of this lane's step
+        const int n = min(32, j - i0);
+        for (int k = 0; k < n; ++k) {  // every lane walks the same chain; lane k keeps its value
+            if (lane == k) mine = carry;
+            carry = fma(-__shfl_sync(0xffffffffu, si, k), carry, __shfl_sync(0xffffffffu, t, k));
+        }
+        if (in) H[(size_t)i * m + j] = fma(ci, mine, si * c1);
+        if (lane == 0) hc[i0 + n] = carry;
+        __syncwarp();
     }
-    const double a = carry, c = h_next;
+    if (lane != 0) return;
+    const double a = hc[j], c = h_next;
     const double r2 = fma(a, a, c * c);
     double den, cj, sj;
     if ((unsigned)__double2hiint(r2) - 0x06000000u < 0x72000000u) {  // r2 well inside the normal range
@@ -224,14 +239,16 @@ __global__ void __launch_bounds__(GM_THREADS) gm_dot_kernel(GmresDev gd, const d
 }
 
 // h = the lane's dots (its blocks' partials added in order, eight threads to a column); hbuf = or += h;
-// w -= V h; in the second pass also the block's share of ||w||^2.
+// w -= V h; then, in the first pass, the second pass's dots of the block's chunk (its V is still near),
+// in the second pass the block's share of ||w||^2.
 template <int PASS>
 __global__ void __launch_bounds__(GM_THREADS) gm_update_kernel(GmresDev gd, double *w) {
     const int b = blockIdx.x, l = gd.blk_lane[b];
     if (!gd.active[l]) return;
     const int cols = *gd.jcur + 1;
     __shared__ double h[1024];
-    __shared__ double red[GM_THREADS];
+    __shared__ double red[PASS ? GM_THREADS : 4 * GM_THREADS];
+    const double *part = gd.part + (PASS ? (size_t)gd.nblk * (gd.m + 1) : 0);
     const int b0 = gd.lane_blk[l], nb = gd.lane_blk[l + 1] - b0;
     const size_t ld = gd.m + 1;
     for (int q0 = 0; q0 < cols; q0 += GM_THREADS / 8) {
@@ -239,7 +256,7 @@ __global__ void __launch_bounds__(GM_THREADS) gm_update_kernel(GmresDev gd, doub
         if ((q & ~3) >= cols) break;  // whole warps: four columns each
         double r = 0.0;
         if (q < cols) {
-            const double *p = gd.part + (size_t)b0 * ld + q;
+            const double *p = part + (size_t)b0 * ld + q;
             int i = s8;
             for (; i + 24 < nb; i += 32) {
                 const double x0 = p[(size_t)i * ld], x1 = p[(size_t)(i + 8) * ld], x2 = p[(size_t)(i + 16) * ld],
@@ -260,7 +277,11 @@ __global__ void __launch_bounds__(GM_THREADS) gm_update_kernel(GmresDev gd, doub
     __syncthreads();
     const long long e0 = gd.blk_off[b];
     const double s = block_update<PASS == 1>(gd.V + e0, gd.n, w + e0, (int)(gd.blk_off[b + 1] - e0), cols, h);
-    if (PASS == 1) {
+    if (PASS == 0) {
+        __syncthreads();
+        block_dots(gd.V + e0, gd.n, w + e0, (int)(gd.blk_off[b + 1] - e0), cols, red,
+                   gd.part + (size_t)(gd.nblk + b) * ld);
+    } else {
         const double t = block_sum(s, GM_THREADS, red);
         if (threadIdx.x == 0) gd.normp[b] = t;
     }
@@ -347,7 +368,7 @@ __global__ void __launch_bounds__(GM_THREADS) gm_finish_kernel(GmresDev gd, cons
         __syncthreads();
         // a block of the lane that starts after its flag was cleared here skips its share of v_{j+1}, which
         // a stopped lane does not use
-        if (first && threadIdx.x == 0) givens_lane(gd, l, j, hs[0], hs[1], hs[2], nrm);
+        if (first && threadIdx.x < 32) givens_lane(gd, l, j, hs[0], hs[1], hs[2], nrm);
     }
     if (advance && last_to_arrive(gd, gridDim.x)) advance_step(gd, j, cudaGraphConditionalHandle(), 0);
 }
@@ -358,12 +379,12 @@ __global__ void gm_advance_kernel(GmresDev gd, cudaGraphConditionalHandle cond, 
 }
 
 // The whole Arnoldi step of one short lane by one cluster of GM_CLUSTER blocks: w stays in shared memory,
-// the dots and the norm are exchanged through distributed shared memory, and the five launches of the
+// the dots and the norm are exchanged through distributed shared memory, and the launches of the
 // long-lane form (each at least a launch and a chain of dependent loads, about 5 us) become one.  For
 // lanes of at most GM_CLUSTER * GM_CHUNK entries: beyond that the FP64 pipes of 16 SMs take longer than
 // the launches saved (at j = 15, 16384 entries: 4 us a pass).
 // Whole solves with this file's kernels against the ten-launch form: two conductors (1200 entries) 692 ->
-// 445 us, six spheres (4320) 1372 -> 942 us; five launches: 40 spheroids (119 640 entries, 76 columns)
+// 445 us, six spheres (4320) 1372 -> 942 us; four launches: 40 spheroids (119 640 entries, 76 columns)
 // 48.1 -> 43.2 ms, 48 uneven lanes 130.7 -> 126.9 ms, solve and gradients of 100 spheres 26.1 -> 25.5 ms.
 __global__ void __launch_bounds__(GM_THREADS) gm_arnoldi_cluster_kernel(GmresDev gd, const double *w, double *vin,
                                                                         int advance) {
@@ -422,7 +443,7 @@ __global__ void __launch_bounds__(GM_THREADS) gm_arnoldi_cluster_kernel(GmresDev
             v[e] = x;
             vin[e0 + e] = x;
         }
-        if (rank == 0 && threadIdx.x == 0) givens_lane(gd, l, j, hc, cs, sn, nrm);
+        if (rank == 0 && threadIdx.x < 32) givens_lane(gd, l, j, hc, cs, sn, nrm);
         cl.sync();  // no block leaves while another reads its shared memory
     }
     if (advance && rank == 0 && last_to_arrive(gd, gd.L)) advance_step(gd, j, cudaGraphConditionalHandle(), 0);
@@ -558,7 +579,7 @@ cudaError_t gmres_init(GmresDev &gd, const double *b, double *vin, cudaStream_t 
     return cudaGetLastError();
 }
 
-int gmres_arnoldi_launches(const GmresDev &gd) { return gd.clusters ? 1 : 5; }
+int gmres_arnoldi_launches(const GmresDev &gd) { return gd.clusters ? 1 : 4; }
 
 cudaError_t gmres_arnoldi(GmresDev &gd, double *w, double *vin, int advance, cudaStream_t st) {
     if (gd.clusters) {
@@ -577,7 +598,6 @@ cudaError_t gmres_arnoldi(GmresDev &gd, double *w, double *vin, int advance, cud
     }
     gm_dot_kernel<<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);  // CGS2
     gm_update_kernel<0><<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
-    gm_dot_kernel<<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
     gm_update_kernel<1><<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
     gm_finish_kernel<<<gd.nblk, GM_THREADS, 0, st>>>(gd, w, vin, advance);
     return cudaGetLastError();

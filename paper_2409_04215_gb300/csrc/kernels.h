@@ -314,7 +314,7 @@ struct GmresDev {
     double *cs, *sn, *g;       // [L][m], [L][m], [L][m+1]
     double *ibeta;             // [L] 1 / ||b||
     double *hbuf;              // [L][m+1] current column
-    double *part;              // [nblk][m+1] block partials of the dots
+    double *part;              // [2][nblk][m+1] block partials of the two passes' dots
     double *normp;             // [nblk] block partials of the norm
     unsigned *arrive;          // [1] blocks done (wraps to 0)
     int *active;               // [L] 1 while the lane iterates

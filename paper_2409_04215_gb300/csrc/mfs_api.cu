@@ -559,6 +559,7 @@ mfs_status build_plan_for(mfs_ctx *ctx, int variant, int include_self, const std
         auto owner = [&](long long u) { return (int)(((u + 1) * G - 1) / W); };
         tl.gA = owner(tl.u0);
         tl.gB = owner(tl.u1 - 1);
+        tl.slotA = (long long)tl.gA * W / G >= tl.u0 ? 0 : 1;
         max_share = std::max(max_share, tl.gB - tl.gA + 1);
     }
     plan.variant = variant;
@@ -798,6 +799,7 @@ mfs_status build_plan_lists(mfs_ctx *ctx, int variant, int include_self, const s
         auto owner = [&](long long u) { return (int)(((u + 1) * G - 1) / W); };
         tl.gA = owner(tl.u0);
         tl.gB = owner(tl.u1 - 1);
+        tl.slotA = (long long)tl.gA * W / G >= tl.u0 ? 0 : 1;
         max_share = std::max(max_share, tl.gB - tl.gA + 1);
     }
     plan.variant = variant;
@@ -1360,7 +1362,7 @@ mfs_status ensure_gmres(mfs_ctx *ctx, int nrhs) {
     CK(ctx->alloc(&gd.g, (size_t)L * (m + 1)));
     CK(ctx->alloc(&gd.ibeta, L));
     CK(ctx->alloc(&gd.hbuf, (size_t)L * (m + 1)));
-    CK(ctx->alloc(&gd.part, (size_t)gd.nblk * (m + 1)));
+    CK(ctx->alloc(&gd.part, 2 * (size_t)gd.nblk * (m + 1)));
     CK(ctx->alloc(&gd.normp, gd.nblk));
     CK(ctx->alloc(&gd.active, L));
     // what a solve reports, in one block (one copy back): resid [L], iters [L], status [L], done, jcur,

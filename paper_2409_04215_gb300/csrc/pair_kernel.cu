@@ -1274,9 +1274,8 @@ __global__ void __launch_bounds__(NT, MINB) pair_sum_kernel(PairGeom geo, PairWo
 }
 
 // Epilogue: out[r][t][d] = beta * base[r][t][d] + scale * (sum of the CTA shares of target t).
-// Blocks (tile, y): the CTAs that share the tile and the slot each wrote (0: the tile is where the
-// CTA's range starts, 1: where it ends) are found once per block; the tile's (target, component)
-// entries, contiguous in every array for one right-hand side, are spread over the gridDim.y blocks,
+// Blocks (tile, y): the tile's (target, component) entries, contiguous in every array for one right-hand
+// side, are spread over the gridDim.y blocks,
 // and S consecutive lanes share an entry: lane k adds shares k, k + S, ... in that order (eight loads
 // in flight), then the S partial sums meet in a fixed xor-shuffle tree.  The order is fixed, so the
 // result is deterministic; with S = 1 it is the plain sum in CTA order.  Tiles shared by many CTAs
@@ -1285,17 +1284,8 @@ template <int D, int NRHS>
 __global__ void __launch_bounds__(256) pair_epilogue_kernel(PairWork work, const double *base, double beta, double scale, double *out,
                                      int ntargets, int S) {
     constexpr int C = D * NRHS;
-    constexpr int MAXS = 256;
-    __shared__ signed char slot_of[MAXS];  // per CTA gA + i: slot 0 / 1, -1 for an empty range
     const PairTile tl = work.tiles[blockIdx.x];
-    const long long W = work.total_units;
     const int ns = (tl.gA >= 0 && tl.gA != tl.gB) ? tl.gB - tl.gA + 1 : 0;
-    for (int i = threadIdx.x; i < ns && i < MAXS; i += blockDim.x) {
-        const int gg = tl.gA + i;
-        const long long b0 = (long long)gg * W / work.G, b1 = (long long)(gg + 1) * W / work.G;
-        slot_of[i] = b0 >= b1 ? -1 : (b0 >= tl.u0 ? 0 : 1);
-    }
-    __syncthreads();
     const int E = (tl.t1 - tl.t0) * C;
     const int per_block = blockDim.x / S, sub = threadIdx.x % S;
     const size_t per_slot = (size_t)work.tile_targets * C;
@@ -1310,15 +1300,7 @@ __global__ void __launch_bounds__(256) pair_epilogue_kernel(PairWork work, const
             } else {
                 const size_t within = (size_t)(t - tl.t0) * C + c;
                 auto share = [&](int i) -> double {
-                    int slot;
-                    if (i < MAXS) {
-                        slot = slot_of[i];
-                    } else {
-                        const int gg = tl.gA + i;
-                        const long long b0 = (long long)gg * W / work.G, b1 = (long long)(gg + 1) * W / work.G;
-                        slot = b0 >= b1 ? -1 : (b0 >= tl.u0 ? 0 : 1);
-                    }
-                    return slot < 0 ? 0.0 : work.partial[(size_t)((tl.gA + i) * 2 + slot) * per_slot + within];
+                    return work.partial[(size_t)((tl.gA + i) * 2 + (i == 0 ? tl.slotA : 0)) * per_slot + within];
                 };
                 int i = sub;
                 for (; i + 7 * S < ns; i += 8 * S) {
@@ -1794,6 +1776,7 @@ __global__ void prep_kernel(const double *targets, int nt, const double *sources
         tl.u1 = tl.u0 + nblk;
         tl.gA = (int)(((tl.u0 + 1) * G - 1) / W);
         tl.gB = (int)((tl.u1 * G - 1) / W);
+        tl.slotA = (long long)tl.gA * W / G >= tl.u0 ? 0 : 1;
         tl.L0 = tl.L1 = -1;
         tiles[t] = tl;
     }
