@@ -8,10 +8,12 @@
 // that of the node's proxy sources outside it.  The equivalent strengths are the least-squares fit
 // of the sources' field on FF_NC check points at radius FF_CHECK * r_e (the "upward" step, run on the
 // device), and a target at least kappa * r_e from a node's centre (kappa = farfield_separation, 3 by
-// default) sees the node through them.
+// default) sees the node through them; further off through fewer points (lower orders, kernels.h), and
+// where it pays through a local expansion: sources around each body that reproduce, at its targets, the
+// field of all nodes well away from it.
 // Targets nearer than that see the node's children, down to the bodies' own proxy points.  Both the
 // fit's right-hand side and the final sums are ordinary pair sums over interaction lists, so the
-// device work is the pair kernel plus one FP64 matrix product per apply.
+// device work is the pair kernel plus a few FP64 matrix products per apply.
 //
 // This file builds, on the host: the tree (8-ary, by median splits of the body centres in x, then y,
 // then z), the nodes' centres and radii, and the interaction list of a set of target bodies.

@@ -750,7 +750,13 @@ mfs_status build_plan_lists(mfs_ctx *ctx, int variant, int include_self, const s
         const int t_end = toff[cuts[ci + 1]];
         int t = toff[cuts[ci]];
         while (t < t_end) {
-            int t1 = std::min(t + TT, t_end);
+            // as few tiles as the range needs, of about equal length in whole target pairs: 839 targets as
+            // 512 + 327 (4 and 3 pairs a thread) rather than 768 + 71 (6 and 1, whose one pair hides no latency).
+            // 2000 ellipsoids, one treecode matvec with tiles of 512 / 768 targets: 32.5 / 33.2 ms after this and
+            // the epilogue's grid cap, 33-34 ms before
+            const int left = (t_end - t + TT - 1) / TT, unit = 2 * v.NT;
+            const int size = std::min(TT, ((t_end - t + left - 1) / left + unit - 1) / unit * unit);
+            int t1 = std::min(t + size, t_end);
             const int g0 = tgroup[t];
             int g1 = tgroup[t1 - 1];
             if (g1 - g0 + 1 > MFS_MAX_TILE_BODIES) {
@@ -1058,13 +1064,29 @@ static cudaError_t ff_fit(mfs_ctx *ctx, mfs_ctx::FarField &F, int rows, int n, i
                             F.fit_chunks, C, st);
 }
 
+// The pair-kernel entry for the sums at check points, whose tiles hold 256 targets (a node, a cell): with one
+// right-hand side the packed entry of exactly that tile, 12 warps per SM where the widest ones keep 8 with
+// two of their six target pairs active; else the entry of the other sums.  2000 ellipsoids, one matvec:
+// 33.2 -> 31.7 ms (entry <1,6,64> for the rest), 600: 5.52 -> 5.26 ms.
+static int ff_check_variant(int D, int nrhs, int variant) {
+    int count = 0;
+    const PairVariant *vv = pair_variants(&count);
+    if (!vv[variant].packed) return variant;
+    for (int i = 0; i < count; ++i)
+        if (!vv[i].grad && !vv[i].comp && vv[i].packed && vv[i].D == D && vv[i].nrhs == nrhs && D == 3 &&
+            vv[i].NT == 64 && vv[i].tile_targets == FF_NC)
+            return i;
+    return variant;
+}
+
 // The upward step of the treecode: the sources (records in the layout of `variant`, packed into
 // F.rec) summed at every node's check points over the node's descendant bodies, then the node's
 // equivalent strengths F.mu = (FP64 product with the pseudo-inverse) scaled by the radius.
 static mfs_status ff_upward(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const double *strength, int nrhs,
                             cudaStream_t st) {
     FFListPlan *pl = nullptr;
-    CKS(ff_up_plan(ctx, F, variant, &pl));
+    const int cv = ff_check_variant(ctx->D, nrhs, variant);
+    CKS(ff_up_plan(ctx, F, cv, &pl));
     int vc = 0;
     const PairVariant *vv = pair_variants(&vc);
     const int D = ctx->D, nodes = F.nodes;
@@ -1077,7 +1099,7 @@ static mfs_status ff_upward(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, con
     g.tgt = F.chk_pos;
     g.ntargets = nodes * FF_NC;
     const PairWork wu = work_of(pl->p);
-    CKS(ff_launch(ctx, variant, g, wu, st));
+    CKS(ff_launch(ctx, cv, g, wu, st));
     CK(pair_epilogue(D, nrhs, wu, nullptr, 0.0, 1.0, F.ucheck, nodes * FF_NC, st));
     CK(ff_fit(ctx, F, nrhs * nodes, FF_NE, FF_NC, F.ucheck, F.mat->PinvT, F.mu, st));
     CK(ff_scale(F.mu, F.re, nodes, D * FF_NE, nrhs, st));
@@ -1105,7 +1127,8 @@ mfs_status ff_pair_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const 
     const size_t REC = pair_record_floats(D, nrhs, layout);
     // local expansions, and the orders that the lists hold (a small cluster needs few of them)
     const bool local = F.use_local && F.cells.any_local;
-    if (local) CKS(ff_loc_plan(ctx, F, variant, &ll));
+    const int cv = ff_check_variant(D, nrhs, variant);
+    if (local) CKS(ff_loc_plan(ctx, F, cv, &ll));
     const int orders = pl->orders | (local ? ll->orders : 0);
     CKS(ff_upward(ctx, F, variant, strength, nrhs, st));
     PackSets sets;
@@ -1127,7 +1150,7 @@ mfs_status ff_pair_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const 
         g.tgt = F.lchk_pos;
         g.ntargets = P * FF_LOC_NC;
         const PairWork wl = work_of(ll->p);
-        CKS(ff_launch(ctx, variant, g, wl, st));
+        CKS(ff_launch(ctx, cv, g, wl, st));
         CK(pair_epilogue(D, nrhs, wl, nullptr, 0.0, 1.0, F.ulocal, P * FF_LOC_NC, st));
         CK(ff_fit(ctx, F, nrhs * P, FF_LOC_N, FF_LOC_NC, F.ulocal, F.mat->locT, F.nu, st));
         CK(ff_scale(F.nu, F.rloc, P, D * FF_LOC_N, nrhs, st));
@@ -2976,7 +2999,8 @@ static mfs_status finish_info(mfs_ctx *ctx, mfs_solve_info *info, const SolveSta
             auto evaluated = [&](int include_self) {
                 const int v = forward_variant(ctx, nrhs);
                 const auto d = ctx->ff.direct.find(v * 2 + include_self);
-                const auto u = ctx->ff.up.find(v), l = ctx->ff.loc.find(v);
+                const int c = ff_check_variant(ctx->D, nrhs, v);
+                const auto u = ctx->ff.up.find(c), l = ctx->ff.loc.find(c);
                 return (d == ctx->ff.direct.end() ? 0.0 : d->second.pairs) +
                        (u == ctx->ff.up.end() ? 0.0 : u->second.pairs) +
                        (l == ctx->ff.loc.end() ? 0.0 : l->second.pairs);

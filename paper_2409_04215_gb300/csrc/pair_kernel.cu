@@ -1541,7 +1541,8 @@ static int occupancy_variant() {
     Q(1, 4, 64)                   \
     Q(2, 3, 64)                   \
     Q(3, 2, 64)                   \
-    Q(4, 2, 64)
+    Q(4, 2, 64)                   \
+    P(PackedStokes, 1, 2, 64)
 
 static const PairVariant kVariants[] = {
 #define S(D_, R_, T_, N_) {D_, R_, T_, N_, N_ * T_, 0, 0, 0, "Scalar<" #D_ "," #R_ "," #T_ "," #N_ ">"},
@@ -1620,7 +1621,10 @@ cudaError_t pair_epilogue(int D, int nrhs, const PairWork &work, const double *b
     // whose FP64 additions must spread over the SMs: 1024-thread blocks on six SMs took 9 us.
     const int S = work.max_share >= 64 ? 8 : (work.max_share >= 16 ? 4 : 1);
     const long long lanes = (long long)work.tile_targets * D * nrhs * S;
-    const int Y = (int)std::min<long long>(64, std::max<long long>(1, (lanes + threads - 1) / threads));
+    // but no more than about 16384 blocks in all (or 4 per tile): with thousands of tiles most are empty
+    // (2585 upward tiles of 2000 ellipsoids, 64 blocks each: 250 us)
+    const long long most = std::max<long long>(4, 16384 / work.ntiles);
+    const int Y = (int)std::min<long long>({64, most, std::max<long long>(1, (lanes + threads - 1) / threads)});
     const dim3 grid((unsigned)work.ntiles, (unsigned)Y);
 #define E(D_, R_)                                                                                      \
     if (D == D_ && nrhs == R_) {                                                                       \
