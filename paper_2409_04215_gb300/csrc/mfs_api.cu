@@ -362,8 +362,10 @@ struct Staged {
     const void *user = nullptr;
     size_t count = 0;
     bool owned = false;
+    bool reading = false;  // the copy from the user's host memory may be in flight (pinned memory)
     cudaStream_t st = nullptr;
     ~Staged() {
+        if (reading) cudaStreamSynchronize(st);  // the caller may reuse its memory once the call returns
         if (owned && d) cudaFreeAsync(d, st);
     }
 };
@@ -379,6 +381,7 @@ mfs_status stage_in(mfs_ctx *ctx, Staged &s, const double *user, size_t count, c
     s.st = st;
     CK(cudaMallocFromPoolAsync((void **)&s.d, sizeof(double) * std::max<size_t>(count, 1), ctx->pool, st));
     s.owned = true;
+    s.reading = true;
     CK(cudaMemcpyAsync(s.d, user, sizeof(double) * count, cudaMemcpyHostToDevice, st));
     return MFS_OK;
 }
@@ -2833,7 +2836,9 @@ mfs_status mfs_setup(mfs_ctx **out, mfs_kind kind, const mfs_bodies *bodies, int
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = dev;
-    unsigned long long keep = ~0ull;
+    // kept between calls: the scratch of evaluations of up to about a million points; more goes back to the
+    // device, where the next context may need it and the calls are long enough to allocate again
+    unsigned long long keep = 256ull << 20;
     if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess ||
         cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
         cudaGetLastError();
@@ -3493,6 +3498,7 @@ static mfs_status group_points(mfs_ctx *ctx, const double *points, const double 
         typename std::remove_const<typename std::remove_pointer<decltype(user)>::type>::type *d = nullptr;
         cudaError_t e = tmp.alloc(&d, count);
         if (e == cudaSuccess) e = cudaMemcpyAsync(d, user, sizeof(*user) * count, cudaMemcpyHostToDevice, st);
+        tmp.host.push_back(nullptr);  // the caller's memory: read before the call returns, errors included
         *out = d;
         return e;
     };
