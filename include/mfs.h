@@ -374,6 +374,15 @@ mfs_status mfs_fp32_fma_rate(int32_t mode, double *tflops, void *stream);
  */
 mfs_status mfs_selftest_bounded_wait(int32_t arrive, int64_t limit, void *stream);
 
+/*
+ * mfs_selftest_fail_alloc -- exercises the out-of-memory path of the context's own buffers (the paper
+ * has no counterpart).  The nth buffer that the context allocates from now on (1 = the next) is
+ * refused as a device without memory would refuse it: the call that asked for it returns MFS_ERR_OOM,
+ * the context stays usable and later calls give the results they would have given.  0 disarms it.
+ * Scratch of a single call does not count.  No device work.
+ */
+mfs_status mfs_selftest_fail_alloc(mfs_ctx *ctx, int32_t nth);
+
 /* Text of the last error on this context (never NULL; "" when none).  Valid until the next call. */
 const char *mfs_last_error(const mfs_ctx *ctx);
 

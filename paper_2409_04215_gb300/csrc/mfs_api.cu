@@ -266,9 +266,16 @@ struct mfs_ctx {
     int pair_launches = 0;   // pair-kernel launches of the current call
     std::vector<cudaEvent_t> pev;  // profile: event pairs around pair-kernel launches
 
+    int fail_alloc = 0;      // mfs_selftest_fail_alloc: the allocation from now that is refused (1 = the next; 0 = none)
+    bool refuse_alloc() {    // a request that no device can serve, so that the runtime reports what it does in earnest
+        void *p = nullptr;
+        return fail_alloc > 0 && --fail_alloc == 0 && cudaMalloc(&p, (size_t)1 << 60) != cudaSuccess;
+    }
+
     template <typename T>
     cudaError_t alloc(T **p, size_t count) {
         *p = nullptr;
+        if (refuse_alloc()) return cudaErrorMemoryAllocation;
         if (count == 0) count = 1;
         cudaError_t e = cudaMalloc((void **)p, sizeof(T) * count);
         if (e == cudaSuccess) allocs.push_back((void *)*p);
@@ -304,6 +311,7 @@ namespace {
         cudaError_t e_ = (call);                                                             \
         if (e_ != cudaSuccess) {                                                             \
             ctx->last_error = std::string(#call) + ": " + cudaGetErrorString(e_);            \
+            cudaGetLastError(); /* the next call's launch checks are not to find it */       \
             return e_ == cudaErrorMemoryAllocation ? MFS_ERR_OOM : MFS_ERR_CUDA;              \
         }                                                                                    \
     } while (0)
@@ -1356,6 +1364,8 @@ mfs_status ensure_gmres(mfs_ctx *ctx, int nrhs) {
     ctx->vin_d = ctx->w_d = ctx->b_d = ctx->x_d = nullptr;
     ctx->stat_d = ctx->stat_h = nullptr;
     gd = GmresDev{};
+    ctx->gd_n = 0;  // until every buffer below exists: a build that runs out of memory half-way is not taken for a whole one
+    ctx->gd_L = ctx->gd_m = 0;
     gd.L = L;
     gd.m = m;
     gd.n = n;
@@ -1373,10 +1383,10 @@ mfs_status ensure_gmres(mfs_ctx *ctx, int nrhs) {
     int *bl = nullptr, *lb = nullptr;
     long long *bo = nullptr;
     CK(ctx->alloc(&bl, blk_lane.size()));
-    CK(ctx->alloc(&bo, blk_off.size()));
-    CK(ctx->alloc(&lb, lane_blk.size()));
     gd.blk_lane = bl;
+    CK(ctx->alloc(&bo, blk_off.size()));
     gd.blk_off = bo;
+    CK(ctx->alloc(&lb, lane_blk.size()));
     gd.lane_blk = lb;
     CK(cudaMemcpy(bl, blk_lane.data(), sizeof(int) * blk_lane.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(bo, blk_off.data(), sizeof(long long) * blk_off.size(), cudaMemcpyHostToDevice));
@@ -1394,7 +1404,7 @@ mfs_status ensure_gmres(mfs_ctx *ctx, int nrhs) {
     // what a solve reports, in one block (one copy back): resid [L], iters [L], status [L], done, jcur,
     // and the blocks' arrival counter
     CK(ctx->alloc(&ctx->stat_d, ctx->stat_bytes(L)));
-    CK(cudaMallocHost((void **)&ctx->stat_h, ctx->stat_bytes(L)));
+    CK(ctx->refuse_alloc() ? cudaErrorMemoryAllocation : cudaMallocHost((void **)&ctx->stat_h, ctx->stat_bytes(L)));
     CK(cudaMemset(ctx->stat_d, 0, ctx->stat_bytes(L)));
     gd.resid = reinterpret_cast<double *>(ctx->stat_d);
     gd.iters = reinterpret_cast<int *>(gd.resid + L);
@@ -1884,6 +1894,12 @@ const char *mfs_pair_variant(const mfs_ctx *ctx, int32_t nrhs) {
 }
 
 const char *mfs_last_error(const mfs_ctx *ctx) { return ctx ? ctx->last_error.c_str() : ""; }
+
+mfs_status mfs_selftest_fail_alloc(mfs_ctx *ctx, int32_t nth) {
+    if (!ctx || nth < 0) return MFS_ERR_INVALID_ARG;
+    ctx->fail_alloc = nth;
+    return MFS_OK;
+}
 
 const char *mfs_setup_error(void) { return g_setup_error.c_str(); }
 
@@ -2950,10 +2966,9 @@ mfs_status mfs_pair_sum(mfs_ctx *ctx, const double *strengths, double *u, int32_
 
 // Where a solve's gamma goes: it is kept for mfs_mobility_vjp and mfs_evaluate.
 static mfs_status keep_buffers(mfs_ctx *ctx) {
+    if (!ctx->keep_gamma) CK(ctx->alloc(&ctx->keep_gamma, (size_t)ctx->opt.max_rhs * ctx->sumM * ctx->D));
+    if (!ctx->keep_lam0) CK(ctx->alloc(&ctx->keep_lam0, (size_t)ctx->opt.max_rhs * ctx->P * 6));
     ctx->last_solve = 0;  // until this one is done
-    if (ctx->keep_gamma) return MFS_OK;
-    CK(ctx->alloc(&ctx->keep_gamma, (size_t)ctx->opt.max_rhs * ctx->sumM * ctx->D));
-    CK(ctx->alloc(&ctx->keep_lam0, (size_t)ctx->opt.max_rhs * ctx->P * 6));
     return MFS_OK;
 }
 
