@@ -383,6 +383,14 @@ mfs_status mfs_selftest_bounded_wait(int32_t arrive, int64_t limit, void *stream
  */
 mfs_status mfs_selftest_fail_alloc(mfs_ctx *ctx, int32_t nth);
 
+/*
+ * mfs_selftest_device_error -- sets the context's device error flag as a kernel whose bounded wait
+ * gave up does (the paper has no counterpart), so that the next call that reads it returns
+ * MFS_ERR_DEVICE_TIMEOUT; a solve that does leaves no solution behind for mfs_evaluate,
+ * mfs_evaluate_stress and mfs_mobility_vjp.  No kernel runs; synchronises `stream`.
+ */
+mfs_status mfs_selftest_device_error(mfs_ctx *ctx, void *stream);
+
 /* Text of the last error on this context (never NULL; "" when none).  Valid until the next call. */
 const char *mfs_last_error(const mfs_ctx *ctx);
 

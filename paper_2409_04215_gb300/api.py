@@ -49,6 +49,7 @@ EXPORTED = [
     "mfs_matvec_transposed",
     "mfs_selftest_bounded_wait",
     "mfs_selftest_fail_alloc",
+    "mfs_selftest_device_error",
     "mfs_dirichlet_apply",
     "mfs_dirichlet_matvec",
     "mfs_solve_capacitance",
@@ -175,6 +176,7 @@ def load_library(path: Optional[str] = None):
     lib.mfs_fp32_fma_rate.argtypes = [i32, ctypes.POINTER(ctypes.c_double), vp]
     lib.mfs_selftest_bounded_wait.argtypes = [i32, ctypes.c_int64, vp]
     lib.mfs_selftest_fail_alloc.argtypes = [vp, i32]
+    lib.mfs_selftest_device_error.argtypes = [vp, vp]
     lib.mfs_pair_variant.restype = ctypes.c_char_p
     lib.mfs_last_error.argtypes = [vp]
     lib.mfs_last_error.restype = ctypes.c_char_p

@@ -1901,6 +1901,14 @@ mfs_status mfs_selftest_fail_alloc(mfs_ctx *ctx, int32_t nth) {
     return MFS_OK;
 }
 
+mfs_status mfs_selftest_device_error(mfs_ctx *ctx, void *stream) {
+    if (!ctx) return MFS_ERR_INVALID_ARG;
+    const int flag = MFS_DEVERR_TIMEOUT;
+    CK(cudaMemcpyAsync(ctx->err_d, &flag, sizeof(int), cudaMemcpyHostToDevice, (cudaStream_t)stream));
+    CK(cudaStreamSynchronize((cudaStream_t)stream));
+    return MFS_OK;
+}
+
 const char *mfs_setup_error(void) { return g_setup_error.c_str(); }
 
 void mfs_destroy(mfs_ctx *ctx) { delete ctx; }
@@ -2972,12 +2980,14 @@ static mfs_status keep_buffers(mfs_ctx *ctx) {
     return MFS_OK;
 }
 
-// Keep the inputs a (and b), n doubles each, of the solve just run (kind: 1 mobility, 2 elastance,
-// 3 resistance, 4 capacitance), whose gamma is in keep_gamma.
-static mfs_status keep_solution(mfs_ctx *ctx, int kind, int nrhs, const double *a, const double *b, size_t n,
-                                cudaStream_t st) {
+// Keep the inputs a (and b), n doubles each, of the solve just enqueued (kind: 1 mobility, 2 elastance,
+// 3 resistance, 4 capacitance), whose gamma is in keep_gamma, and wait for it.  It counts as the last
+// solve only when the device reported no error: what a kernel that gave up left behind is not a solution.
+static mfs_status keep_and_finish(mfs_ctx *ctx, int kind, int nrhs, const double *a, const double *b, size_t n,
+                                  cudaStream_t st, SolveStats &ss) {
     if (a) CK(cudaMemcpyAsync(ctx->keep_lam0, a, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
     if (b) CK(cudaMemcpyAsync(ctx->keep_lam0 + n, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
+    CKS(gmres_finish(ctx, st, ss));
     ctx->last_solve = kind;
     ctx->last_nrhs = nrhs;
     return MFS_OK;
@@ -3074,8 +3084,7 @@ mfs_status mfs_solve_mobility(mfs_ctx *ctx, const double *F, const double *T, do
     ctx->launches += 1;
     CK(cudaEventRecord(ctx->ev1, st));
     // keep gamma, F and T for mfs_mobility_vjp and mfs_evaluate (outside the timed region)
-    CKS(keep_solution(ctx, 1, nrhs, Fi.d, Ti.d, nb, st));
-    CKS(gmres_finish(ctx, st, ss));
+    CKS(keep_and_finish(ctx, 1, nrhs, Fi.d, Ti.d, nb, st, ss));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
     CKS(stage_out_finish(ctx, Uo, st));
@@ -3112,8 +3121,7 @@ mfs_status mfs_solve_elastance(mfs_ctx *ctx, const double *Q, double *V, int32_t
     CK(extract_laplace(ctx->lam_d, nrhs, ctx->P, ctx->src_off_d, ctx->sumN, Vo.d, st));  // Eq. vkal
     ctx->launches += 1;
     CK(cudaEventRecord(ctx->ev1, st));
-    CKS(keep_solution(ctx, 2, nrhs, Qi.d, nullptr, nb, st));
-    CKS(gmres_finish(ctx, st, ss));
+    CKS(keep_and_finish(ctx, 2, nrhs, Qi.d, nullptr, nb, st, ss));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
     CKS(stage_out_finish(ctx, Vo, st));
@@ -3209,8 +3217,7 @@ mfs_status mfs_solve_resistance(mfs_ctx *ctx, const double *U, const double *Ome
     CK(extract_stokes(ctx->lam_d, nrhs, ctx->P, ctx->src_local64_d, ctx->src_off_d, ctx->sumN, Fo.d, To.d, st, 1.0));
     ctx->launches += 2;
     CK(cudaEventRecord(ctx->ev1, st));
-    CKS(keep_solution(ctx, 3, nrhs, nullptr, nullptr, 0, st));
-    CKS(gmres_finish(ctx, st, ss));
+    CKS(keep_and_finish(ctx, 3, nrhs, nullptr, nullptr, 0, st, ss));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
     CKS(stage_out_finish(ctx, Fo, st));
@@ -3246,8 +3253,7 @@ mfs_status mfs_solve_capacitance(mfs_ctx *ctx, const double *phi, double *q, int
     CK(extract_laplace(ctx->lam_d, nrhs, ctx->P, ctx->src_off_d, ctx->sumN, Qo.d, st, 1));
     ctx->launches += 2;
     CK(cudaEventRecord(ctx->ev1, st));
-    CKS(keep_solution(ctx, 4, nrhs, nullptr, nullptr, 0, st));
-    CKS(gmres_finish(ctx, st, ss));
+    CKS(keep_and_finish(ctx, 4, nrhs, nullptr, nullptr, 0, st, ss));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
     CKS(stage_out_finish(ctx, Qo, st));
