@@ -382,7 +382,7 @@ __global__ void gm_advance_kernel(GmresDev gd, cudaGraphConditionalHandle cond, 
 // the dots and the norm are exchanged through distributed shared memory, and the launches of the
 // long-lane form (each at least a launch and a chain of dependent loads, about 5 us) become one.  For
 // lanes of at most GM_CLUSTER * GM_CHUNK entries: beyond that the FP64 pipes of 16 SMs take longer than
-// the launches saved (at j = 15, 16384 entries: 4 us a pass).
+// the launches saved (at j = 15, 16384 entries: 4 us a pass); and for few of them (gmres_prepare).
 // Whole solves with this file's kernels against the ten-launch form: two conductors (1200 entries) 692 ->
 // 445 us, six spheres (4320) 1372 -> 942 us; four launches: 40 spheroids (119 640 entries, 76 columns)
 // 48.1 -> 43.2 ms, 48 uneven lanes 130.7 -> 126.9 ms, solve and gradients of 100 spheres 26.1 -> 25.5 ms.
@@ -554,7 +554,12 @@ cudaError_t gmres_prepare(GmresDev &gd) {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(gm_arnoldi_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    // the device must be able to hold one such cluster, else the long-lane form serves
+    // The lanes must fit the clusters that the device holds at once (fewer than eight on 152 SMs), twice over at most: a
+    // cluster takes the 16 SMs of a GPC, so lanes beyond that queue, where the long-lane form's blocks share
+    // all SMs.  Time of an iteration, one launch / four, lanes of 4320 entries: 1 lane 67 / 83 us, 8 lanes
+    // 115 / 126, 12 lanes 128 / 136, 16 lanes 138 / 139, 24 lanes 167 / 153, 64 lanes 257 / 211, 256 lanes
+    // 674 / 422; of 16 338 entries: 1 lane 104 / 121, 8 lanes 220 / 223, 12 lanes 271 / 275, 16 lanes
+    // 328 / 319, 64 lanes 940 / 890; of 1800: 8 lanes 222 / 238, 16 lanes 267 / 267, 64 lanes 400 / 315.
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -566,10 +571,11 @@ cudaError_t gmres_prepare(GmresDev &gd) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gm_arnoldi_cluster_kernel, &cfg) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveClusters(&n, gm_arnoldi_cluster_kernel, &cfg) != cudaSuccess) {
         cudaGetLastError();
-        gd.clusters = 0;
+        n = 0;
     }
+    if (gd.L > 2 * n) gd.clusters = 0;
     return cudaSuccess;
 }
 

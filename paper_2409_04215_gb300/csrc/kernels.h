@@ -308,7 +308,7 @@ struct GmresDev {
     const int *blk_lane;       // [nblk] the block's lane
     const long long *blk_off;  // [nblk+1] its first entry (blocks are contiguous)
     const int *lane_blk;       // [L+1] the lane's first block
-    int clusters;              // 1: every lane is short enough for the one-launch Arnoldi step
+    int clusters;              // 1: the lanes are short and few enough for the one-launch Arnoldi step
     double *V;                 // [(m+1)][n] basis
     double *H;                 // [L][m+1][m] Hessenberg, rotated to upper triangular
     double *cs, *sn, *g;       // [L][m], [L][m], [L][m+1]
@@ -329,7 +329,8 @@ struct GmresDev {
 // is short enough for the one-launch step.
 bool gmres_plan_blocks(const std::vector<long long> &seg, int sm_count, std::vector<int> &blk_lane,
                        std::vector<long long> &blk_off, std::vector<int> &lane_blk);
-// Kernel attributes for this basis; clears gd.clusters when the device cannot hold the cluster.
+// Kernel attributes for this basis; clears gd.clusters when the device does not hold the lanes' clusters
+// at about one time.
 cudaError_t gmres_prepare(GmresDev &gd);
 // Start (two launches): v_0 = b / ||b|| per lane, also to vin (the matvec's input at a fixed address),
 // lanes with b = 0 inactive, j = 0, done = (no lane active).
