@@ -84,9 +84,9 @@ __device__ __forceinline__ void block_dots(const double *V, long long n, const d
 }
 
 // w[e] -= sum_{i < cols} h[i] V[i n + e] over e in [0, len); returns the thread's sum of the new w[e]^2
-// (0 unless NORM).  Four elements per thread and eight columns at a time: 32 loads in flight, the last
-// round guarded instead of a remainder loop; each element's sum runs over the columns in order.
-template <bool NORM>
+// (0 unless NORM).  Four elements per thread and G columns at a time: 32 loads in flight with eight, the
+// last round guarded instead of a remainder loop; each element's sum runs over the columns in order.
+template <bool NORM, int G = 8>
 __device__ __forceinline__ double block_update(const double *V, long long n, double *w, int len, int cols,
                                                const double *h) {
     double nrm = 0.0;
@@ -97,10 +97,10 @@ __device__ __forceinline__ double block_update(const double *V, long long n, dou
         bool in[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) in[u] = e + u * GM_THREADS < len;
-        for (int i = 0; i < cols; i += 8) {
-            double v[8][4];
+        for (int i = 0; i < cols; i += G) {
+            double v[G][4];
 #pragma unroll
-            for (int g = 0; g < 8; ++g)
+            for (int g = 0; g < G; ++g)
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                     v[g][u] = (in[u] && i + g < cols) ? V[(size_t)(i + g) * n + e + u * GM_THREADS] : 0.0;
@@ -108,7 +108,7 @@ __device__ __forceinline__ double block_update(const double *V, long long n, dou
             for (int u = 0; u < 4; ++u)
                 if (eb + u * GM_THREADS < len)
 #pragma unroll
-                    for (int g = 0; g < 8; ++g)
+                    for (int g = 0; g < G; ++g)
                         if (i + g < cols) a[u] = fma(h[i + g], v[g][u], a[u]);
         }
 #pragma unroll
@@ -241,8 +241,12 @@ __global__ void __launch_bounds__(GM_THREADS) gm_dot_kernel(GmresDev gd, const d
 // h = the lane's dots (its blocks' partials added in order, eight threads to a column); hbuf = or += h;
 // w -= V h; then, in the first pass, the second pass's dots of the block's chunk (its V is still near),
 // in the second pass the block's share of ||w||^2.
-template <int PASS>
-__global__ void __launch_bounds__(GM_THREADS) gm_update_kernel(GmresDev gd, double *w) {
+// With more blocks than SMs, four columns at a time and two blocks an SM (64 registers), so that one
+// block's FP64 work covers the other's loads and barriers; with at most one block an SM, eight columns at
+// a time (112 registers).  1024 lanes of 4320 entries, mean over 14 steps of the first and second pass:
+// 109 and 74 us, with one block an SM 165 and 121 (the FP64 pipe alone: 108 and 61).
+template <int PASS, int G>
+__global__ void __launch_bounds__(GM_THREADS, G == 8 ? 1 : 2) gm_update_kernel(GmresDev gd, double *w) {
     const int b = blockIdx.x, l = gd.blk_lane[b];
     if (!gd.active[l]) return;
     const int cols = *gd.jcur + 1;
@@ -276,7 +280,7 @@ __global__ void __launch_bounds__(GM_THREADS) gm_update_kernel(GmresDev gd, doub
     }
     __syncthreads();
     const long long e0 = gd.blk_off[b];
-    const double s = block_update<PASS == 1>(gd.V + e0, gd.n, w + e0, (int)(gd.blk_off[b + 1] - e0), cols, h);
+    const double s = block_update<PASS == 1, G>(gd.V + e0, gd.n, w + e0, (int)(gd.blk_off[b + 1] - e0), cols, h);
     if (PASS == 0) {
         __syncthreads();
         block_dots(gd.V + e0, gd.n, w + e0, (int)(gd.blk_off[b + 1] - e0), cols, red,
@@ -603,8 +607,13 @@ cudaError_t gmres_arnoldi(GmresDev &gd, double *w, double *vin, int advance, cud
         return cudaLaunchKernelEx(&cfg, gm_arnoldi_cluster_kernel, gd, (const double *)w, vin, advance);
     }
     gm_dot_kernel<<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);  // CGS2
-    gm_update_kernel<0><<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
-    gm_update_kernel<1><<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
+    if (gd.nblk > gd.sms) {
+        gm_update_kernel<0, 4><<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
+        gm_update_kernel<1, 4><<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
+    } else {
+        gm_update_kernel<0, 8><<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
+        gm_update_kernel<1, 8><<<gd.nblk, GM_THREADS, 0, st>>>(gd, w);
+    }
     gm_finish_kernel<<<gd.nblk, GM_THREADS, 0, st>>>(gd, w, vin, advance);
     return cudaGetLastError();
 }

@@ -304,6 +304,7 @@ cudaError_t ff_scale(double *mu, const double *re, int nodes, int per_node, int 
 struct GmresDev {
     int L, m;                  // lanes, Krylov basis capacity (m <= 1023)
     long long n;               // vector length (all lanes)
+    int sms;                   // SMs of the device
     int nblk;                  // blocks of the long-lane kernels, each within one lane
     const int *blk_lane;       // [nblk] the block's lane
     const long long *blk_off;  // [nblk+1] its first entry (blocks are contiguous)

@@ -1379,6 +1379,7 @@ mfs_status ensure_gmres(mfs_ctx *ctx, int nrhs) {
         }
     seg[L] = n;
     gd.clusters = gmres_plan_blocks(seg, ctx->sm_count, blk_lane, blk_off, lane_blk) ? 1 : 0;
+    gd.sms = ctx->sm_count;
     gd.nblk = (int)blk_lane.size();
     int *bl = nullptr, *lb = nullptr;
     long long *bo = nullptr;
