@@ -45,6 +45,42 @@ struct FFMatrices {
     }
 };
 
+// Where the scratch of single calls comes from: one pool per device, shared by the contexts of a process
+// that are alive together, so that what it keeps between calls does not grow with their number; given back
+// with the last of them.  It keeps 256 MB (an evaluation takes about 150 to 250 bytes a point, the most with
+// several right-hand sides or the stress); more goes back to the device, where the next context may need it
+// and the calls are long enough to allocate again.
+struct CallPool {
+    cudaMemPool_t pool = nullptr;
+    CallPool() = default;
+    CallPool(const CallPool &) = delete;
+    ~CallPool() {
+        if (pool) cudaMemPoolDestroy(pool);
+    }
+};
+
+cudaError_t call_pool(int dev, std::shared_ptr<CallPool> &out) {
+    static std::mutex mu;
+    static std::weak_ptr<CallPool> kept[64];
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev < 64) out = kept[dev].lock();
+    if (out) return cudaSuccess;
+    auto p = std::make_shared<CallPool>();
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    unsigned long long keep = 256ull << 20;
+    int no = 0;  // one stream's call never waits for another's to reuse its memory
+    cudaError_t e = cudaMemPoolCreate(&p->pool, &props);
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(p->pool, cudaMemPoolReuseAllowInternalDependencies, &no);
+    if (e != cudaSuccess) return e;
+    out = p;
+    if (dev < 64) kept[dev] = p;
+    return cudaSuccess;
+}
+
 struct PairPlan {
     int variant = -1;
     int include_self = 0;
@@ -256,7 +292,7 @@ struct mfs_ctx {
     } ff, ffT;                                       // forward sums; transposed sums (adjoint)
 
     int sm_count = 0;
-    cudaMemPool_t pool = nullptr;  // scratch of single calls (Scratch); kept between calls, given back with the context
+    std::shared_ptr<CallPool> pool;  // scratch of single calls (Scratch)
     std::string last_error;
     std::vector<void *> allocs;
     double ms_setup = 0.0;
@@ -278,6 +314,11 @@ struct mfs_ctx {
         if (refuse_alloc()) return cudaErrorMemoryAllocation;
         if (count == 0) count = 1;
         cudaError_t e = cudaMalloc((void **)p, sizeof(T) * count);
+        if (e == cudaErrorMemoryAllocation && pool) {  // what the pool keeps may be enough
+            cudaGetLastError();
+            e = cudaMemPoolTrimTo(pool->pool, 0);
+            if (e == cudaSuccess) e = cudaMalloc((void **)p, sizeof(T) * count);
+        }
         if (e == cudaSuccess) allocs.push_back((void *)*p);
         return e;
     }
@@ -298,7 +339,6 @@ struct mfs_ctx {
         if (evp0) cudaEventDestroy(evp0);
         if (evp1) cudaEventDestroy(evp1);
         for (cudaEvent_t e : pev) cudaEventDestroy(e);
-        if (pool) cudaMemPoolDestroy(pool);
     }
 };
 
@@ -332,7 +372,7 @@ bool is_device_ptr(const void *p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Device scratch of one call on one stream: allocations from the context's pool, freed in stream order
+// Device scratch of one call on one stream: allocations from the device's call pool, freed in stream order
 // when the call returns (no device synchronisation; a cudaMalloc and cudaFree pair per buffer took most
 // of a small evaluation).
 struct Scratch {
@@ -357,7 +397,7 @@ struct Scratch {
     cudaError_t alloc(T **p, size_t count) {
         *p = nullptr;
         const cudaError_t e =
-            cudaMallocFromPoolAsync((void **)p, sizeof(T) * std::max<size_t>(count, 1), ctx->pool, st);
+            cudaMallocFromPoolAsync((void **)p, sizeof(T) * std::max<size_t>(count, 1), ctx->pool->pool, st);
         if (e == cudaSuccess) ps.push_back((void *)*p);
         return e;
     }
@@ -387,7 +427,7 @@ mfs_status stage_in(mfs_ctx *ctx, Staged &s, const double *user, size_t count, c
         return MFS_OK;
     }
     s.st = st;
-    CK(cudaMallocFromPoolAsync((void **)&s.d, sizeof(double) * std::max<size_t>(count, 1), ctx->pool, st));
+    CK(cudaMallocFromPoolAsync((void **)&s.d, sizeof(double) * std::max<size_t>(count, 1), ctx->pool->pool, st));
     s.owned = true;
     s.reading = true;
     CK(cudaMemcpyAsync(s.d, user, sizeof(double) * count, cudaMemcpyHostToDevice, st));
@@ -403,7 +443,7 @@ mfs_status stage_out_alloc(mfs_ctx *ctx, Staged &s, double *user, size_t count, 
         return MFS_OK;
     }
     s.st = st;
-    CK(cudaMallocFromPoolAsync((void **)&s.d, sizeof(double) * std::max<size_t>(count, 1), ctx->pool, st));
+    CK(cudaMallocFromPoolAsync((void **)&s.d, sizeof(double) * std::max<size_t>(count, 1), ctx->pool->pool, st));
     s.owned = true;
     return MFS_OK;
 }
@@ -2857,15 +2897,7 @@ mfs_status mfs_setup(mfs_ctx **out, mfs_kind kind, const mfs_bodies *bodies, int
         return MFS_ERR_CUDA;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    // kept between calls: the scratch of evaluations of up to about a million points; more goes back to the
-    // device, where the next context may need it and the calls are long enough to allocate again
-    unsigned long long keep = 256ull << 20;
-    if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess ||
-        cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    if (call_pool(dev, ctx->pool) != cudaSuccess) {
         cudaGetLastError();
         g_setup_error = "mfs_setup: cannot create a memory pool";
         return MFS_ERR_CUDA;
