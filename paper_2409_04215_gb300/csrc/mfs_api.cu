@@ -1537,8 +1537,8 @@ mfs_status ensure_transposed(mfs_ctx *ctx) {
             need = std::max(need, (size_t)gemm_splitk_chunks(rows, m, n, ctx->sm_count) * rows * m);
         }
         CK(ctx->alloc(&sh.PkT, need));
-        CK(ctx->alloc(&sh.O64, (size_t)R * nb * m));
         FactorSet &fx = sh.fs[0];
+        if (!fx.tc_ready) CK(ctx->alloc(&sh.O64, (size_t)R * nb * m));
         if (fx.tc_ready) {  // tensor cores: the factor planes transposed (exact), their maps, chunk results
             const int np = sh.pieces;
             fx.un_stride = (size_t)m * sh.ld2;
@@ -2097,7 +2097,7 @@ static mfs_status alloc_apply_scratch(mfs_ctx *ctx, ShapeHost &sh, cudaStream_t 
         ok = ctx->alloc(&sh.A64, (size_t)R * nb * m) == cudaSuccess &&
              ctx->alloc(&sh.T64, (size_t)R * nb * n) == cudaSuccess && ctx->alloc(&sh.Pk64, need) == cudaSuccess;
     }
-    if (ok) ok = ctx->alloc(&sh.L64, (size_t)R * nb * n) == cudaSuccess;
+    if (ok && sh.pieces == 0) ok = ctx->alloc(&sh.L64, (size_t)R * nb * n) == cudaSuccess;
     if (ok) {  // split-K chunk results: the largest S * rows * cols over nrhs = 1..R and both GEMMs
         size_t need = 0;
         for (int h = 1; h <= R; ++h) {
