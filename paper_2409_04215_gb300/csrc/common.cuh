@@ -137,3 +137,15 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     float bb = s - a;
     e = (a - (s - bb)) + (b - bb);
 }
+
+// 1/sqrt(x) in FP64: the hardware's FP64 rsqrt estimate y0 (relative error at most 2^-20) and one
+// third-order Householder step, y = y0 (1 + h/2 + 3 h^2/8) with h = 1 - x y0^2, whose remainder
+// 5 h^3/16 lies below 2^-58: five FP64 instructions instead of a square root and a division.  Outside
+// the normal range (zero, subnormal, infinite, NaN; an integer test) the plain expression is taken.
+__device__ __forceinline__ double rsqrt64(double x) {
+    if ((unsigned)__double2hiint(x) - 0x00100000u >= 0x7fe00000u) return 1.0 / sqrt(x);
+    double y0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+    const double h = fma(-x * y0, y0, 1.0);
+    return fma(y0 * h, fma(0.375, h, 0.5), y0);
+}

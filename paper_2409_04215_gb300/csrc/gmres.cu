@@ -139,7 +139,7 @@ __device__ __forceinline__ double block_sum(double v, int threads, double *sh) {
 // (||x||, 1 / ||x||) from s = ||x||^2, (0, 0) for 0.
 __device__ __forceinline__ double2 norm_and_inverse(double s) {
     if (s == 0.0) return make_double2(0.0, 0.0);
-    const double inv = rsqrt(s);
+    const double inv = rsqrt64(s);
     return make_double2(isfinite(s) ? s * inv : sqrt(s), inv);
 }
 
@@ -175,7 +175,7 @@ __device__ void givens_lane(const GmresDev &gd, int l, int j, double *hc, double
     const double r2 = fma(a, a, c * c);
     double den, cj, sj;
     if ((unsigned)__double2hiint(r2) - 0x06000000u < 0x72000000u) {  // r2 well inside the normal range
-        const double ri = rsqrt(r2);
+        const double ri = rsqrt64(r2);
         den = r2 * ri;
         cj = a * ri;
         sj = c * ri;

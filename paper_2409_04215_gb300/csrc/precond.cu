@@ -657,8 +657,8 @@ cudaError_t extract_laplace(const double *alpha, int nrhs, int P, const int *bod
 // Bound by the FP64 pipe (GB300: 2 DFMA per clock per SM, a warp's DFMA every 64 clocks per scheduler),
 // so what counts is FP64 instructions per pair and that every SM has the same share of them; loads and
 // shared memory do not show.  Per Stokeslet pair: 3 subtractions (the target is taken relative to the
-// source body's centre once per body), r^2 3, 1/r about 5 (CUDA's rsqrt), r.l 3, (r.l)/r^2 2, six FMAs = 22,
-// where divisions and a square root took it above 100.  The grid's y axis cuts each target's
+// source body's centre once per body), r^2 3, 1/r 5 (rsqrt64), r.l 3, (r.l)/r^2 2, six FMAs = 22, where
+// divisions and a square root by the library took it above 100.  The grid's y axis cuts each target's
 // sources into S chunks so that small suspensions fill the GPU too; the partial sums [S][nrhs][nt][D]
 // are added in chunk order by the caller's combine kernel.  24 spheres (M = 600, N = 300), 9.9e7 pairs:
 // 17.8 ms on 113 CTAs with library square roots and divisions; the whole FP64 matvec with this kernel
@@ -675,7 +675,7 @@ int fp64_pair_chunks(int ntargets, int min_sources, int sm_count) {
     return (int)std::max<long long>(1, std::min<long long>(s, 64));
 }
 
-// Body of source s: the fourth value of its record.
+// Body of source s among bodies whose offsets are body_src_off (the body with off[b] <= s).
 __device__ __forceinline__ int body_of_source(const double *src_local4, int s) { return (int)src_local4[4 * (size_t)s + 3]; }
 
 template <int D, int NRHS>
@@ -709,7 +709,7 @@ pair_sum_fp64_kernel(const double *__restrict__ tgt_local, const int *__restrict
         for (; s < e; ++s) {
             const double *yl = src_local4 + 4 * (size_t)s;
             const double r0 = x[0] - yl[0], r1 = x[1] - yl[1], r2_ = x[2] - yl[2];
-            const double ri = rsqrt(fma(r0, r0, fma(r1, r1, r2_ * r2_)));
+            const double ri = rsqrt64(fma(r0, r0, fma(r1, r1, r2_ * r2_)));
             const double ri2 = ri * ri;
 #pragma unroll
             for (int h = 0; h < NRHS; ++h) {
@@ -772,7 +772,7 @@ grad_pair_fp64_kernel(const double *__restrict__ tgt_local, const int *__restric
         for (; s < e; ++s) {
             const double *yl = src_local4 + 4 * (size_t)s;
             const double r[3] = {x[0] - yl[0], x[1] - yl[1], x[2] - yl[2]};
-            const double ri = rsqrt(fma(r[0], r[0], fma(r[1], r[1], r[2] * r[2])));
+            const double ri = rsqrt64(fma(r[0], r[0], fma(r[1], r[1], r[2] * r[2])));
             const double ri2 = ri * ri, ri3 = ri * ri2, ri2_3 = 3.0 * ri2;
 #pragma unroll
             for (int h = 0; h < NRHS; ++h) {

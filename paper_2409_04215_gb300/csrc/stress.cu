@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(128) stress_f64_kernel(const double *__restric
                                      xr[2] - src_local[3 * (size_t)j + 2]};
                 const double *l = lam + ((size_t)h * sum_N + j) * 3;
                 const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
-                const double ir = rsqrt(r2);
+                const double ir = rsqrt64(r2);
                 const double ir3 = ir * ir * ir;
                 const double rl = r[0] * l[0] + r[1] * l[1] + r[2] * l[2];
                 p += rl * ir3;
