@@ -391,6 +391,13 @@ mfs_status mfs_selftest_fail_alloc(mfs_ctx *ctx, int32_t nth);
  */
 mfs_status mfs_selftest_device_error(mfs_ctx *ctx, void *stream);
 
+/*
+ * mfs_selftest_rsqrt64 -- y[i] = x[i]^(-1/2), i < n, by the FP64 path's own routine (the paper has no
+ * counterpart), for its error to be measured.  x and y: device pointers, FP64 [n], may be the same.
+ * Asynchronous on `stream`.
+ */
+mfs_status mfs_selftest_rsqrt64(const double *x, double *y, int64_t n, void *stream);
+
 /* Text of the last error on this context (never NULL; "" when none).  Valid until the next call. */
 const char *mfs_last_error(const mfs_ctx *ctx);
 

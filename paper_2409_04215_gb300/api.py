@@ -50,6 +50,7 @@ EXPORTED = [
     "mfs_selftest_bounded_wait",
     "mfs_selftest_fail_alloc",
     "mfs_selftest_device_error",
+    "mfs_selftest_rsqrt64",
     "mfs_dirichlet_apply",
     "mfs_dirichlet_matvec",
     "mfs_solve_capacitance",
@@ -177,6 +178,7 @@ def load_library(path: Optional[str] = None):
     lib.mfs_selftest_bounded_wait.argtypes = [i32, ctypes.c_int64, vp]
     lib.mfs_selftest_fail_alloc.argtypes = [vp, i32]
     lib.mfs_selftest_device_error.argtypes = [vp, vp]
+    lib.mfs_selftest_rsqrt64.argtypes = [vp, vp, ctypes.c_int64, vp]
     lib.mfs_pair_variant.restype = ctypes.c_char_p
     lib.mfs_last_error.argtypes = [vp]
     lib.mfs_last_error.restype = ctypes.c_char_p
@@ -226,6 +228,19 @@ def selftest_bounded_wait(arrive: bool, limit: int = 1000, stream=None) -> int:
     torch = _torch()
     st = _stream_ptr(stream, torch.device("cuda", torch.cuda.current_device()))
     return int(lib.mfs_selftest_bounded_wait(1 if arrive else 0, int(limit), st))
+
+
+def selftest_rsqrt64(x, stream=None):
+    """x**-0.5 of an FP64 CUDA tensor by the FP64 path's own routine (mfs_selftest_rsqrt64)."""
+    torch = _torch()
+    x = x.contiguous()
+    if x.dtype != torch.float64 or not x.is_cuda:
+        raise ValueError("selftest_rsqrt64: an FP64 CUDA tensor is required")
+    y = torch.empty_like(x)
+    rc = load_library().mfs_selftest_rsqrt64(x.data_ptr(), y.data_ptr(), x.numel(), _stream_ptr(stream, x.device))
+    if rc != MFS_OK:
+        raise MFSError(rc, "mfs_selftest_rsqrt64 failed")
+    return y
 
 
 def default_options(**kw) -> Options:

@@ -138,10 +138,14 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     e = (a - (s - bb)) + (b - bb);
 }
 
-// 1/sqrt(x) in FP64: the hardware's FP64 rsqrt estimate y0 (relative error at most 2^-20) and one
-// third-order Householder step, y = y0 (1 + h/2 + 3 h^2/8) with h = 1 - x y0^2, whose remainder
-// 5 h^3/16 lies below 2^-58: five FP64 instructions instead of a square root and a division.  Outside
-// the normal range (zero, subnormal, infinite, NaN; an integer test) the plain expression is taken.
+// 1/sqrt(x) in FP64: the hardware's FP64 rsqrt estimate y0 and one third-order Householder step,
+// y = y0 (1 + h/2 + 3 h^2/8) with h = 1 - x y0^2: five FP64 instructions instead of a square root and a
+// division.  With y0 good to 2^-20, h is at most 2^-19 and the series' remainder 5 h^3/16 below 2^-58; the
+// rounding of x y0 adds 2^-54 and the last FMA 2^-53, a relative error below 1.51 x 2^-53 in all
+// (test_gpu_rsqrt64.py holds it to that over the whole exponent range, which bears out the estimate's bound
+// too; CUDA's own rsqrt, good to one ulp, is as fast to 1 %: FP64 matvec of 24 spheres 4.53 against 4.58 ms).
+// Outside the normal range (zero, subnormal, infinite, negative, NaN; an integer test) the plain expression
+// is taken.
 __device__ __forceinline__ double rsqrt64(double x) {
     if ((unsigned)__double2hiint(x) - 0x00100000u >= 0x7fe00000u) return 1.0 / sqrt(x);
     double y0;

@@ -10,6 +10,7 @@
 //    alpha_0 = q/N 1 (Eq. al0); extraction U = -K_N^T lambda (Eq. getU), phi = -mean(alpha) (Eq. vkal).
 #include <algorithm>
 
+#include "../../include/mfs.h"
 #include "common.cuh"
 #include "kernels.h"
 
@@ -829,4 +830,17 @@ cudaError_t pair_sum_fp64(int D, int nrhs, int chunks, const double *tgt_local, 
     return cudaErrorInvalidValue;
 }
 
+// Self-test of rsqrt64: y[i] = rsqrt64(x[i]).
+__global__ void rsqrt64_kernel(const double *x, double *y, long long n) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        y[i] = rsqrt64(x[i]);
+}
+
 }  // namespace mfs
+
+extern "C" mfs_status mfs_selftest_rsqrt64(const double *x, double *y, int64_t n, void *stream) {
+    if (n < 0 || (n > 0 && (!x || !y))) return MFS_ERR_INVALID_ARG;
+    if (n == 0) return MFS_OK;
+    mfs::rsqrt64_kernel<<<1024, 256, 0, (cudaStream_t)stream>>>(x, y, n);
+    return cudaGetLastError() == cudaSuccess ? MFS_OK : MFS_ERR_CUDA;
+}
