@@ -74,6 +74,11 @@ struct PairWork {
     double *src_grad = nullptr;  // gradient kernel only: per source body sums, FP64 [P][3] (atomic adds)
     const int *tperm = nullptr;  // epilogue: target t's value goes to (and its base is read at) tperm[t]
     int max_share = 1;           // epilogue: the most CTAs that share one tile
+    // epilogue: linear field per body, [nrhs][nfar][4][D] (constant, d/dx, d/dy, d/dz), that of the tile's body
+    // kb0 added to its sums at the targets far_tgt (about the body's centre)
+    const double *far = nullptr;
+    const float4 *far_tgt = nullptr;
+    int nfar = 0;
 };
 
 // ---------------------------------------------------------------------------

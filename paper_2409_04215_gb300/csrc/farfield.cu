@@ -237,6 +237,77 @@ void ff_cell_lists(const FFTree &t, int root, const std::vector<int> &tbodies, c
     if (!pays) local.clear();
 }
 
+// One block per body (tree position) and right-hand side, one thread per check point.  The constant is the
+// mean over the points; the gradient 3 / (n R^2) sum (u - mean) x, as the points spread evenly over the
+// sphere of radius R, made free of divergence for a velocity (the sources' field is).  It need not be the
+// best fit (its sums are FP32): whatever is taken out here is added at the targets, both in FP64, and the
+// local sources carry the rest.  Bound by FP64 operations (2 per clock per SM).
+template <int D>
+__global__ void __launch_bounds__(FF_LOC_NC)
+ff_take_linear_kernel(double *u, const float4 *chk, const double *radius, int bodies, double *far) {
+    constexpr int W = FF_LOC_NC / 32;
+    __shared__ double mean_w[W][D];
+    __shared__ float grad_w[W][3 * D];
+    const int q = blockIdx.x % bodies, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double *mine = u + ((size_t)blockIdx.x * FF_LOC_NC + threadIdx.x) * D;
+    const float4 p = chk[(size_t)q * FF_LOC_NC + threadIdx.x];
+    const float x[3] = {p.x, p.y, p.z};
+    double v[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        double s = v[d] = mine[d];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) mean_w[warp][d] = s;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        double mean = 0.0;
+        for (int w = 0; w < W; ++w) mean += mean_w[w][d];
+        mean *= 1.0 / FF_LOC_NC;
+        v[d] -= mean;
+        if (threadIdx.x == 0) far[(size_t)blockIdx.x * 4 * D + d] = mean;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            float s = (float)v[d] * x[a];
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) grad_w[warp][a * D + d] = s;
+        }
+    }
+    __syncthreads();
+    const double R = FF_LOC_CHECK * radius[q], f = 3.0 / (FF_LOC_NC * R * R);
+    float g[3 * D];
+#pragma unroll
+    for (int c = 0; c < 3 * D; ++c) {
+        g[c] = 0.f;
+        for (int w = 0; w < W; ++w) g[c] += grad_w[w][c];
+        g[c] = (float)(f * g[c]);
+    }
+    if constexpr (D == 3) {
+        const float third = (g[0] + g[4] + g[8]) / 3.f;
+        g[0] -= third;
+        g[4] -= third;
+        g[8] -= third;
+    }
+#pragma unroll
+    for (int d = 0; d < D; ++d)
+        mine[d] = v[d] - ((double)x[0] * g[d] + (double)x[1] * g[D + d] + (double)x[2] * g[2 * D + d]);
+#pragma unroll
+    for (int c = 0; c < 3 * D; ++c)
+        if (threadIdx.x == c) far[((size_t)blockIdx.x * 4 + 1) * D + c] = g[c];
+}
+
+cudaError_t ff_take_linear(int D, double *u, const float4 *chk, const double *radius, int bodies, int nrhs, double *far,
+                           cudaStream_t st) {
+    const unsigned n = (unsigned)bodies * nrhs;
+    if (n == 0) return cudaSuccess;
+    if (D == 3)
+        ff_take_linear_kernel<3><<<n, FF_LOC_NC, 0, st>>>(u, chk, radius, bodies, far);
+    else
+        ff_take_linear_kernel<1><<<n, FF_LOC_NC, 0, st>>>(u, chk, radius, bodies, far);
+    return cudaGetLastError();
+}
+
 __global__ void ff_scale_kernel(double *mu, const double *re, int nodes, int per_node, size_t n) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         mu[i] *= re[(i / per_node) % nodes];

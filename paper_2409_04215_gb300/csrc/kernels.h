@@ -299,6 +299,11 @@ void ff_cell_lists(const FFTree &t, int root, const std::vector<int> &tbodies, c
 // mu[h][node][e][d] *= re[node] (the fit was made on the unit sphere; the kernels are homogeneous of
 // degree -1).
 cudaError_t ff_scale(double *mu, const double *re, int nodes, int per_node, int nrhs, cudaStream_t st);
+// The constant and linear part of a local check field u [nrhs][bodies][FF_LOC_NC][D] at each body's points
+// (chk [bodies][FF_LOC_NC] about its centre, target radii radius[bodies]) to far [nrhs][bodies][4][D] and out of
+// u: these are fields that the local sources need not carry (mfs_api.cu, ff_pair_apply).
+cudaError_t ff_take_linear(int D, double *u, const float4 *chk, const double *radius, int bodies, int nrhs, double *far,
+                           cudaStream_t st);
 
 // ---- GMRES (gmres.cu): L independent lanes, lane l owns vector entries [seg[l], seg[l+1]) ----
 struct GmresDev {

@@ -269,6 +269,7 @@ struct mfs_ctx {
         double *rloc = nullptr;                      // [P] target radii
         float4 *loc_pos = nullptr, *lchk_pos = nullptr;  // [P FF_LOC_N], [P FF_LOC_NC] about the body's centre
         double *ulocal = nullptr, *nu = nullptr;     // [max_rhs][P FF_LOC_NC][D], [max_rhs][P FF_LOC_N][D]
+        double *ufar = nullptr;                      // [max_rhs][P][4][D]
         size_t loc_rec = 0;
         struct ListPlan {
             PairPlan p;
@@ -1203,18 +1204,28 @@ mfs_status ff_pair_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const 
         const PairWork wl = work_of(ll->p);
         CKS(ff_launch(ctx, cv, g, wl, st));
         CK(pair_epilogue(D, nrhs, wl, nullptr, 0.0, 1.0, F.ulocal, P * FF_LOC_NC, st));
+        // The constant and linear part of the far field at a body stay FP64 and go to the targets in the last
+        // epilogue; the local sources carry the rest.  Strengths of one direction or in long waves give a far
+        // field of little else, and its sum over 96 FP32 records rounded every target by about 5e-8 of it
+        // (one direction, 400 ellipsoids: 5.3e-8 off the exact sums; with this 1.8e-8, without local sources 2.0e-8).
+        CK(ff_take_linear(D, F.ulocal, F.lchk_pos, F.rloc, P, nrhs, F.ufar, st));
         CK(ff_fit(ctx, F, nrhs * P, FF_LOC_N, FF_LOC_NC, F.ulocal, F.mat->locT, F.nu, st));
         CK(ff_scale(F.nu, F.rloc, P, D * FF_LOC_N, nrhs, st));
         PackSets loc;
         loc.add(P * FF_LOC_N, F.loc_pos, F.nu, F.rec + F.loc_rec * REC);
         CK(pack_sets(D, nrhs, layout, loc, st));
-        ctx->launches += 4;
+        ctx->launches += 5;
     }
     PairGeom g = ff_geom(F, *pl);
     g.tgt = F.tgt;
     g.ntargets = F.ntgt;
     PairWork we = work_of(pl->p);
     we.tperm = F.tperm;
+    if (local) {
+        we.far = F.ufar;  // every tile holds one body's targets (ff_direct_plan)
+        we.far_tgt = F.tgt;
+        we.nfar = P;
+    }
     CKS(ff_launch(ctx, variant, g, we, st));
     CK(pair_epilogue(D, nrhs, we, base, beta, scale, out, F.ntgt, st));
     ctx->launches += 2;
@@ -2328,9 +2339,10 @@ static void ff_release_geometry(mfs_ctx *ctx, mfs_ctx::FarField &F) {
         F.ord_pos[o] = nullptr;
         F.ord_mu[o] = nullptr;
     }
-    for (void *p : {(void *)F.rloc, (void *)F.loc_pos, (void *)F.lchk_pos, (void *)F.ulocal, (void *)F.nu})
+    for (void *p : {(void *)F.rloc, (void *)F.loc_pos, (void *)F.lchk_pos, (void *)F.ulocal, (void *)F.nu,
+                    (void *)F.ufar})
         ctx->release(p);
-    F.rloc = F.ulocal = F.nu = nullptr;
+    F.rloc = F.ulocal = F.nu = F.ufar = nullptr;
     F.loc_pos = F.lchk_pos = nullptr;
     ctx->release(F.centres);
     ctx->release(F.re);
@@ -2494,6 +2506,7 @@ static mfs_status ff_setup(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStream_t st) 
         CK(cudaMemcpy(F.rloc, rloc.data(), sizeof(double) * P, cudaMemcpyHostToDevice));
         CK(ctx->alloc(&F.ulocal, (size_t)R * P * FF_LOC_NC * D));
         CK(ctx->alloc(&F.nu, (size_t)R * P * FF_LOC_N * D));
+        CK(ctx->alloc(&F.ufar, (size_t)R * P * 4 * D));
     }
     CK(ctx->alloc(&F.ucheck, (size_t)R * nodes * FF_NC * D));
     CK(ctx->alloc(&F.mu, (size_t)R * nodes * FF_NE * D));

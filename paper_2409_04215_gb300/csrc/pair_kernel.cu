@@ -1280,7 +1280,7 @@ __global__ void __launch_bounds__(NT, MINB) pair_sum_kernel(PairGeom geo, PairWo
 // in flight), then the S partial sums meet in a fixed xor-shuffle tree.  The order is fixed, so the
 // result is deterministic; with S = 1 it is the plain sum in CTA order.  Tiles shared by many CTAs
 // (the far-field upward sums of the top nodes) are why S and the y blocks exist.
-template <int D, int NRHS>
+template <int D, int NRHS, bool FAR = false>
 __global__ void __launch_bounds__(256) pair_epilogue_kernel(PairWork work, const double *base, double beta, double scale, double *out,
                                      int ntargets, int S) {
     constexpr int C = D * NRHS;
@@ -1319,6 +1319,11 @@ __global__ void __launch_bounds__(256) pair_epilogue_kernel(PairWork work, const
             const int h = c / D, d = c % D;
             const size_t o = ((size_t)h * ntargets + (work.tperm ? work.tperm[t] : t)) * D + d;
             const double b = base ? beta * base[o] : 0.0;
+            if constexpr (FAR) {
+                const double *f = work.far + ((size_t)h * work.nfar + tl.kb0) * 4 * D + d;
+                const float4 x = work.far_tgt[t];
+                v += f[0] + (x.x * f[D] + x.y * f[2 * D] + x.z * f[3 * D]);
+            }
             out[o] = b + scale * v;
         }
     }
@@ -1626,13 +1631,16 @@ cudaError_t pair_epilogue(int D, int nrhs, const PairWork &work, const double *b
     const long long most = std::max<long long>(4, 16384 / work.ntiles);
     const int Y = (int)std::min<long long>({64, most, std::max<long long>(1, (lanes + threads - 1) / threads)});
     const dim3 grid((unsigned)work.ntiles, (unsigned)Y);
-#define E(D_, R_)                                                                                      \
-    if (D == D_ && nrhs == R_) {                                                                       \
-        pair_epilogue_kernel<D_, R_><<<grid, threads, 0, st>>>(work, base, beta, scale, out, ntargets, S); \
-        return cudaGetLastError();                                                                     \
+#define E(D_, R_, FAR_)                                                                                      \
+    if (D == D_ && nrhs == R_ && (work.far != nullptr) == FAR_) {                                            \
+        pair_epilogue_kernel<D_, R_, FAR_><<<grid, threads, 0, st>>>(work, base, beta, scale, out, ntargets, S); \
+        return cudaGetLastError();                                                                           \
     }
-    E(3, 1) E(3, 2) E(3, 3) E(3, 4) E(1, 1) E(1, 2) E(1, 3) E(1, 4)
-    E(4, 1) E(4, 2) E(4, 3) E(4, 4)  // pressure and traction
+    E(3, 1, false) E(3, 2, false) E(3, 3, false) E(3, 4, false)
+    E(1, 1, false) E(1, 2, false) E(1, 3, false) E(1, 4, false)
+    E(4, 1, false) E(4, 2, false) E(4, 3, false) E(4, 4, false)  // pressure and traction
+    E(3, 1, true) E(3, 2, true) E(3, 3, true) E(3, 4, true)
+    E(1, 1, true) E(1, 2, true) E(1, 3, true) E(1, 4, true)
 #undef E
     return cudaErrorInvalidValue;
 }
