@@ -94,8 +94,9 @@ typedef struct {
                              into TF32 pieces: 1 = three pieces, six products (FP32-level products);
                              2 = two pieces, three products (3xTF32, ~2^-21 products);
                              0 = CUDA-core split-K FP32 GEMM (TwoSum-compensated slices).  Default 1.  With 1 or
-                             2, applies of a few columns (at most 8 bodies of a shape times right-hand sides,
-                             Stokes) run on the CUDA cores in double-FP32 arithmetic, which is faster there */
+                             2, Stokes applies of a few columns (bodies of a shape times right-hand sides: 1 or
+                             2, and 3 to 8 while columns x 9 M N is at most 2^24) run on the CUDA cores in
+                             double-FP32 arithmetic, which is faster there */
     int32_t pair_variant; /* >= 0: use this entry of the pair-kernel table (mfs_pair_variant_info) for its
                              (d, nrhs) instead of the autotuner's pick; it must be a forward pair-sum
                              variant of the context's d, else mfs_setup fails with MFS_ERR_INVALID_ARG.
@@ -115,10 +116,11 @@ typedef struct {
                              near bodies (direct, FP32 pair kernel).  Targets further away use 128, 96 or 64
                              points matched to the 196 (from 4, 5 and 8 radii on), and bodies with many
                              collocation points receive what lies 5 of their radii away through 96 local
-                             sources fitted around them.  Relative accuracy of the sums about
-                             1e-7; the pair work drops from O(P^2) to about O(P log P).  Needs precision 0 or
-                             2.  Every forward pair sum uses it (the solves, mfs_matvec, mfs_pair_sum); the
-                             transposed sums of mfs_matvec_transposed and mfs_mobility_vjp use a second tree
+                             sources fitted around them (its constant and linear part in FP64).  Relative
+                             accuracy of the sums about 1e-7 (2e-8 for strengths of one direction; 1e-6 where
+                             each body's strengths cancel); the pair work drops from O(P^2) to about
+                             O(P log P).  Needs precision 0 or 2.  Every forward pair sum uses it (the solves,
+                             mfs_matvec, mfs_pair_sum); the transposed sums of mfs_matvec_transposed and mfs_mobility_vjp use a second tree
                              with the roles swapped (collocation points as sources, proxy points as targets,
                              built on first use), and so does the VJP's centre gradient (its target side on
                              the first tree, its source side on the second); mfs_evaluate sums over the first

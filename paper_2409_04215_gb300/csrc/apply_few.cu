@@ -10,7 +10,8 @@
 // products and FP32 accumulation runs on the tensor cores).  Bound by the factor's bytes (8 per element,
 // from L2 between iterations) until eleven FP32 operations per element and column outweigh them.
 // Six spheres (M = 240, N = 120), whole solve of 13 iterations: 942 -> 872 us with the apply, the scatter that
-// also packs and the spread epilogue; velocities 7e-8 from the FP64 solution instead of 1.2e-6.
+// also packs and the spread epilogue (817 us with today's Arnoldi step); velocities 7e-8 from the FP64
+// solution instead of 1.2e-6.
 #include <algorithm>
 
 #include "common.cuh"

@@ -387,9 +387,9 @@ __global__ void gm_advance_kernel(GmresDev gd, cudaGraphConditionalHandle cond, 
 // long-lane form (each at least a launch and a chain of dependent loads, about 5 us) become one.  For
 // lanes of at most GM_CLUSTER * GM_CHUNK entries: beyond that the FP64 pipes of 16 SMs take longer than
 // the launches saved (at j = 15, 16384 entries: 4 us a pass); and for few of them (gmres_prepare).
-// Whole solves with this file's kernels against the ten-launch form: two conductors (1200 entries) 692 ->
-// 445 us, six spheres (4320) 1372 -> 942 us; four launches: 40 spheroids (119 640 entries, 76 columns)
-// 48.1 -> 43.2 ms, 48 uneven lanes 130.7 -> 126.9 ms, solve and gradients of 100 spheres 26.1 -> 25.5 ms.
+// Whole solves with this file's kernels against the ten-launch form, when they came in: two conductors (1200
+// entries) 692 -> 445 us, six spheres (4320) 1372 -> 942 us; four launches: 40 spheroids (119 640 entries, 76
+// columns) 48.1 -> 43.2 ms, 48 uneven lanes 130.7 -> 126.9 ms, solve and gradients of 100 spheres 26.1 -> 25.5.
 __global__ void __launch_bounds__(GM_THREADS) gm_arnoldi_cluster_kernel(GmresDev gd, const double *w, double *vin,
                                                                         int advance) {
     namespace cg = cooperative_groups;

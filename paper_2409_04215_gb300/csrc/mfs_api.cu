@@ -47,9 +47,9 @@ struct FFMatrices {
 
 // Where the scratch of single calls comes from: one pool per device, shared by the contexts of a process
 // that are alive together, so that what it keeps between calls does not grow with their number; given back
-// with the last of them.  It keeps 256 MB (an evaluation takes about 150 to 250 bytes a point, the most with
-// several right-hand sides or the stress); more goes back to the device, where the next context may need it
-// and the calls are long enough to allocate again.
+// with the last of them.  It keeps 256 MB: an evaluation takes from 50 bytes a point (velocities, one
+// right-hand side, device inputs) to 350 (pressure and traction, four of them, host inputs).  More goes back
+// to the device, where the next context may need it and the calls are long enough to allocate again.
 struct CallPool {
     cudaMemPool_t pool = nullptr;
     CallPool() = default;
@@ -977,7 +977,7 @@ mfs_status ff_ev_plan(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, FFListPla
 // better (5 or 6 of them with the widest policies), but a node must be far from all of them: with 6 the
 // bodies' own lists take 6.2e6 pairs a body (2000 ellipsoids, near bodies apart), with 2 they take 3.5e6
 // and the two active target pairs per thread cost the cells' sums little (matvec 38.7 ms with 6, 36.4 with
-// 2, 36.8 with 1; 37.3, 35.8 and 36.3 with the 5-pair policy).
+// 2, 36.8 with 1; 37.3, 35.8 and 36.3 with the 5-pair policy: before the 256-target entry and equal tiles).
 constexpr int FF_CELL = 2;
 
 // The cells of FF_CELL consecutive tree positions (cut at suspensions) and their lists.
@@ -1116,10 +1116,12 @@ static cudaError_t ff_fit(mfs_ctx *ctx, mfs_ctx::FarField &F, int rows, int n, i
                             F.fit_chunks, C, st);
 }
 
-// The pair-kernel entry for the sums at check points, whose tiles hold 256 targets (a node, a cell): with one
-// right-hand side the packed entry of exactly that tile, 12 warps per SM where the widest ones keep 8 with
-// two of their six target pairs active; else the entry of the other sums.  2000 ellipsoids, one matvec:
-// 33.2 -> 31.7 ms (entry <1,6,64> for the rest), 600: 5.52 -> 5.26 ms.
+// The pair-kernel entry for the sums at check points, whose tiles hold 256 targets (a node, a cell): the
+// packed entry of exactly that tile where the table has one (1, 2 and 4 right-hand sides), whose warps have
+// no inactive target pairs; else the entry of the other sums.  One right-hand side: 12 warps per SM where
+// the widest entries keep 8 with two of their six target pairs active; one matvec of 2000 ellipsoids 33.2 ->
+// 31.7 ms (entry <1,6,64> for the rest), 600: 5.52 -> 5.26 ms.  Two and four, one pair sum: 500 ellipsoids
+// (M = 839) 11.48 -> 11.24 and 20.25 -> 20.07 ms, 400 spheres (M = 600) 4.73 -> 4.62 and 8.34 -> 8.26 ms.
 static int ff_check_variant(int D, int nrhs, int variant) {
     int count = 0;
     const PairVariant *vv = pair_variants(&count);
@@ -1167,8 +1169,8 @@ static mfs_status ff_upward(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, con
 // ellipsoids (839 targets) saw about 850 nodes x 196 points: 1.4e8 pairs, 96 % of a matvec's 162 ms.
 // Fewer points for distant nodes (FF_ORD_*) and 128 check points in place of the body's targets for
 // everything beyond FF_LOC_GAP leave 2.1e10 pairs per sum for 1000 ellipsoids (1.0e11 before), and a
-// matvec of 2000 takes 38.5 ms (163.7); the result is as close to the direct sum as before (white-noise
-// strengths, 1000 ellipsoids: 1.3e-7, 1.5e-7 before).
+// matvec of 2000 takes 31.4 ms (162); the result is as close to the exact sums as before (400
+// ellipsoids: white-noise strengths 1.13e-7, 1.28e-7 before; of one direction 1.8e-8, 2.0e-8 before).
 mfs_status ff_pair_apply(mfs_ctx *ctx, mfs_ctx::FarField &F, int variant, const double *strength, double *out,
                          const double *base, double beta, double scale, int nrhs, int include_self, cudaStream_t st) {
     FFListPlan *pl = nullptr, *ll = nullptr;
@@ -2368,8 +2370,8 @@ static void ff_release_geometry(mfs_ctx *ctx, mfs_ctx::FarField &F) {
 }
 
 // The far-field structures (opt.farfield = 1): the tree, the FP64 pseudo-inverse of the map from
-// equivalent strengths on the unit sphere to the field at the check points (ff_unit_pinv, once per
-// context), and the tree-ordered geometry (again after every mfs_update_centers).
+// equivalent strengths on the unit sphere to the field at the check points (ff_matrices, once per
+// process and device), and the tree-ordered geometry (again after every mfs_update_centers).
 static mfs_status ff_setup(mfs_ctx *ctx, mfs_ctx::FarField &F, cudaStream_t st) {
     const int P = ctx->P, D = ctx->D;
     F.rsrc.assign(P, 0.0);

@@ -1549,6 +1549,9 @@ static int occupancy_variant() {
     Q(4, 2, 64)                   \
     P(PackedStokes, 1, 2, 64)
 
+// The stress entries Q: one per number of right-hand sides, with as many target pairs a thread as leave
+// four blocks an SM (4, 3, 2 and 2 pairs: 212, 232, 206 and 244 registers, no spills); other counts
+// were not measured, and the autotuner times velocity sums only.
 static const PairVariant kVariants[] = {
 #define S(D_, R_, T_, N_) {D_, R_, T_, N_, N_ * T_, 0, 0, 0, "Scalar<" #D_ "," #R_ "," #T_ "," #N_ ">"},
 #define P(POL_, R_, TP_, N_) \

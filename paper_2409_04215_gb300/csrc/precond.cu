@@ -676,7 +676,7 @@ int fp64_pair_chunks(int ntargets, int min_sources, int sm_count) {
     return (int)std::max<long long>(1, std::min<long long>(s, 64));
 }
 
-// Body of source s among bodies whose offsets are body_src_off (the body with off[b] <= s).
+// Body of source s: the fourth value of its record.
 __device__ __forceinline__ int body_of_source(const double *src_local4, int s) { return (int)src_local4[4 * (size_t)s + 3]; }
 
 template <int D, int NRHS>
