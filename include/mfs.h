@@ -120,10 +120,11 @@ typedef struct {
                              accuracy of the sums about 1e-7 (2e-8 for strengths of one direction; 1e-6 where
                              each body's strengths cancel); the pair work drops from O(P^2) to about
                              O(P log P).  Needs precision 0 or 2.  Every forward pair sum uses it (the solves,
-                             mfs_matvec, mfs_pair_sum); the transposed sums of mfs_matvec_transposed and mfs_mobility_vjp use a second tree
-                             with the roles swapped (collocation points as sources, proxy points as targets,
-                             built on first use), and so does the VJP's centre gradient (its target side on
-                             the first tree, its source side on the second); mfs_evaluate sums over the first
+                             mfs_matvec, mfs_pair_sum); the transposed sums of mfs_matvec_transposed and
+                             mfs_mobility_vjp use a second tree with the roles swapped (collocation points as
+                             sources, proxy points as targets, built on first use), and so does the VJP's
+                             centre gradient (its target side on the first tree, its source side on the
+                             second); mfs_evaluate sums over the first
                              tree with interaction lists built for each call's points (each owner body's
                              radius that of its farthest point), and mfs_evaluate_stress likewise (the
                              pressure and traction of the equivalent Stokeslets in the far field; these are
